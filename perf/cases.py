@@ -306,6 +306,120 @@ def run(s):
     return {"y": prq.linear(w, codes, sf, 16, prq.F32, out=y), "perm": w.get(prq.FIELD_PERM), "inv_s": w.get(prq.FIELD_INV_S)}
 
 
+# ---- the same results in 64 bits ------------------------------------------------------------------------------
+
+def _mx(v, elem_exp, rounded, search=False):
+    """Blocks of 32 along the last axis: power-of-two scale (floor of the largest magnitude's exponent less `elem_exp`),
+    elements through `rounded`; with `search` the neighbouring scales too, the smaller one first, if strictly better."""
+    b = v.double().reshape(*v.shape[:-1], -1, 32)
+    e0 = (torch.frexp(b.abs().amax(-1, keepdim=True))[1] - 1 - elem_exp).clamp(min=-127)
+    best = torch.ldexp(rounded(torch.ldexp(b, -e0)), e0)
+    if search:
+        err = (b - best).square().sum(-1, keepdim=True)
+        for step in (-1, 1):
+            e = e0 + step
+            q = torch.ldexp(rounded(torch.ldexp(b, -e)), e)
+            d = (b - q).square().sum(-1, keepdim=True)
+            better = (d < err) & (e >= -127)
+            best, err = torch.where(better, q, best), torch.where(better, d, err)
+    return best.reshape(v.shape)
+
+
+def _e2m1(a):
+    m = a.abs()
+    m = torch.where(m < 2, (m * 2).round() / 2, torch.where(m < 4, m.round(), (m / 2).round() * 2)).clamp(max=6)
+    return torch.copysign(m, a)
+
+
+def _e4m3(a):
+    return a.clamp(-448, 448).float().to(torch.float8_e4m3fn).double()
+
+
+def _exact_scales(amax):
+    s = torch.from_numpy(amax).cuda().double().clamp(min=1e-5).sqrt().float()
+    return s, (1.0 / s.double()).float()
+
+
+def _exact_layer(W, amax, k, search=False):
+    """(weights in the permuted order, residual of the tail, permutation, reciprocal scales)"""
+    s, inv_s = _exact_scales(amax)
+    W0 = W.float() * s
+    err = (W0.double() - _mx(W0, 2, _e2m1)).square().sum(0)
+    tail = torch.sort(err, descending=True, stable=True)[1][:k]
+    picked = torch.zeros(W.shape[1], dtype=torch.bool, device="cuda")
+    picked[tail] = True
+    perm = torch.cat([torch.nonzero(~picked)[:, 0], torch.nonzero(picked)[:, 0]])
+    Wt = W0[:, perm]
+    Q = _mx(Wt, 2, _e2m1, search)
+    R = _mx((Wt.double() - Q)[:, W.shape[1] - k:], 2, _e2m1, search) if k else Q[:, :0]
+    return Q, R, perm, inv_s
+
+
+def _exact_linear(layer, x, mode):
+    Q, R, perm, inv_s = layer
+    a = _mx((x.float() * inv_s)[:, perm] if mode == "permute" else x, 2, _e2m1)
+    return a @ Q.T + a[:, a.shape[1] - R.shape[1]:] @ R.T
+
+
+def _exact_block(src, M, k, k_down, mode):
+    out = []
+    for names in SHARED:
+        K = next(K for n, K, _ in BLOCK if n == names[0])
+        gain = src.gain(K)
+        amax = _amax(src, gain)
+        x = src.rows(M, gain)
+        for name, _, N in BLOCK:
+            if name in names:
+                out.append(_exact_linear(_exact_layer(src.weight(N, K), amax, k_down if name == "down" else k), x, mode))
+    return out
+
+
+def exact(c, seed):
+    """What `run` returns for the same inputs: the layer's quantisation rules and the products of the quantised
+    operands in 64 bits, with torch alone."""
+    src, kind = _Source(seed), c["kind"]
+    if kind == "linear":
+        gain = src.gain(c["K"])
+        layer = _exact_layer(src.weight(c["N"], c["K"]), _amax(src, gain), c["k"])
+        return _exact_linear(layer, src.rows(c["M"], gain), c["mode"])
+    if kind == "stack":
+        mode = "identity" if c["form"] == "fused" else "permute"
+        return [y for _ in range(c["layers"]) for y in _exact_block(src, c["M"], c["k"], c["k"], mode)]
+    if kind == "block":
+        return _exact_block(src, c["M"], c["k"], c["k_down"], "permute")
+    if kind == "ffn":
+        H, C = c["H"], c["C"]
+        gain_in, gain_mid = src.gain(H), src.gain(C)
+        down = _exact_layer(src.weight(H, C), _amax(src, gain_mid), c["k"])
+        perm, inv_s = down[2], down[3]
+        up = (src.weight(C, H).float()[perm] * inv_s[perm][:, None]).to(torch.bfloat16)
+        gate = src.weight(C, H)[perm]
+        both = torch.cat([gate.view(C // 32, 32, H), up.view(C // 32, 32, H)], 1).reshape(2 * C, H)
+        layer = _exact_layer(both, _amax(src, gain_in), c["k_gu"])
+        gu = _exact_linear(layer, src.rows(c["M"], gain_in), "permute").view(c["M"], C // 32, 2, 32)
+        h = torch.nn.functional.silu(gu[:, :, 0]) * gu[:, :, 1]
+        return _exact_linear(down, h.reshape(c["M"], C).to(torch.bfloat16), "identity")
+    if kind == "moe":
+        gain = src.gain(c["K"])
+        amax = np.stack([_amax(src, gain, 64) for _ in range(c["E"])])
+        W = src.weight(c["E"], c["N"], c["K"])
+        x, off = src.rows(8 * c["T"], gain), _routing(c, seed)
+        return torch.cat([_exact_linear(_exact_layer(W[e], amax[e], c["k"]), x[off[e]:off[e + 1]], c["mode"])
+                          for e in range(c["E"]) if off[e + 1] > off[e]])
+    if kind == "mxfp8":
+        gain = src.gain(c["K"])
+        Ns = [c["N"] * n // sum(QKV) // 8 * 8 for n in QKV[1:]]
+        Ns = [c["N"] - sum(Ns)] + Ns
+        W = torch.cat([src.weight(n, c["K"]) for n in Ns])
+        s, inv_s = _exact_scales(_amax(src, gain))
+        x = src.rows(c["M"], gain)
+        return _mx(x.float() * inv_s if c["mode"] == "permute" else x, 8, _e4m3) @ _mx(W.float() * s, 8, _e4m3).T
+    gain = src.gain(c["K"])
+    layer = _exact_layer(src.weight(c["N"], c["K"]), _amax(src, gain), c["k"], c["search"])
+    y = _exact_linear(layer, src.rows(16, gain), "permute")
+    return {"y": y, "perm": layer[2].int().cpu().numpy(), "inv_s": layer[3].double().cpu().numpy()}
+
+
 # ---- what a pass cannot do without, and how far results may be apart ------------------------------------------
 
 def _layer_work(M, N, K, k, y_bytes, x_bytes=2.0, w_bytes=17 / 32):
