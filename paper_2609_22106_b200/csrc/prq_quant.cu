@@ -13,13 +13,14 @@
 // written out as one coalesced 512-byte piece; the bytes of tail blocks are also duplicated into the
 // residual stages, which is all the "tail copy" this design needs (the GEMM re-reads the tail codes).
 //
-// The scale + permute mode has two structures.  From 512 rows on (and while two slices of rows fit shared memory)
-// quant_act_rows_kernel runs: persistent CTAs that bring whole rows into shared memory by bulk copies and gather
-// from there (see that kernel).  Smaller batches keep the column-atom CTAs of quant_act_kernel, whose rows can be
-// cut into parts so that a few rows still fill the GPU.
+// The scale + permute mode has two structures.  quant_act_cols_kernel (see there) brings whole rows into shared memory
+// by bulk copies and keeps the columns with the lanes; it runs wherever its rows fit.  The column-atom CTAs of
+// quant_act_kernel are left with what it does not serve better: rows too wide for it, and a handful of atoms of
+// stacked experts.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdlib>
 
 #include "prq_internal.h"
@@ -307,267 +308,368 @@ quant_act_kernel(const QuantBatch b) {
 
 
 // ---------------------------------------------------------------------------------------------------------
-// Scale + permute mode, second structure: whole rows through shared memory.  A persistent CTA takes consecutive
-// slices of kRowsR rows; the rows of the next slices arrive by bulk copies (one per row, no instruction per element)
-// while the current slice is quantised, and every gather of the permutation is a shared-memory read.  The lanes of
-// a warp are 8 different rows reading the SAME source column, for the 4 blocks of one 128-column atom side by side:
-// the staged rows are 16 bytes further apart than a multiple of 128 bytes, so the 8 rows fall into 8 different
-// groups of four banks and a gather costs about one pass however scattered the permutation is -- against one
-// 32-byte sector per 2-byte read when the tail of the permutation is gathered from global memory.  The column's
-// source offset and reciprocal scale are the same for all rows of a warp: they are kept as one 16-byte record per
-// column pair in shared memory (built once per layer and expert) instead of living in registers per lane.  A lane
-// takes one row of one block: 32 values held in registers (no shuffle for the amax), 16 bytes of codes, one scale
-// byte; the four bytes of (row, atom) meet by two shuffles and leave as the one word the GEMM's layout has for them.
-// The tail's bytes are also collected in shared memory and written once more where the residual stages read them;
-// rows and blocks that do not exist get zero bytes; row-major scales are written if asked for.  Several layers that
-// read the same activation are quantised from the one copy of the rows.
-// Threads per CTA: 256 where two CTAs share an SM, 512 where the rows of a wide layer leave room for one only.
-constexpr int kRowsR = 8;                        // rows per slice
-constexpr int kRowsMaxBufs = 8;                  // slices of rows in shared memory at most (at least 2)
-static_assert(32 / kRowsR == 4, "a warp is 8 rows x the 4 blocks of an atom");
-constexpr int kRowsSlices = kGroupRows / kRowsR; // slices per 128-row group
+// Scale + permute mode, second structure: columns stay with their lanes.  A lane owns kCols consecutive destination
+// columns of one layer and keeps their source offsets and reciprocal scales in registers while rows stream past it:
+// whole rows arrive in shared memory by bulk copies (one warp does nothing else), and every gather of the permutation
+// is a 2-byte shared-memory read.
+//
+// Why.  The mode is bound by instruction issue and by a launch's fixed latencies, not by memory (2.53 bytes per element).
+// Gathering from global memory costs about 20 instructions per element (64-bit addresses, one 32-byte sector per
+// scattered 2-byte read).  Rows that stay with their lanes need a 16-byte record per column pair fetched from shared
+// memory for every row (12.7 per element), and the records of a wide layer (K = 9728) do not fit beside its rows.  Here
+// the core is 5 per element -- gather, its address, widening, two packed fp32 products and a conversion per pair, half
+// a three-input maximum -- and 10.7 in all at 4096 x 2560 (ncu), where a CTA sees only three or four slices; a row is
+// all that shared memory holds.  Measured figures stand at the launcher.  Of the 8.9 us at 4096 x 2560 (2.53 B per
+// element: 4.1 us of memory time) about 3 are set-up, the first rows' latency and the last stores.
+//
+// The lanes of a warp read the same row, kCols columns apart: where the permutation is locally the identity, four
+// (eight) lanes would meet in a bank.  A lane therefore walks its columns from another start (`rot`, chosen from its
+// first source column so that the lanes of a bank group read different words), which one rotation of the packed
+// codes undoes.
+//
+// A slice is kRowsC rows of one 128-row group.  The block maxima of two rows travel in one register (only exponents
+// are needed), the four scale bytes of (row, atom) meet by shuffles and leave as the one word the GEMM's layout has
+// for them; tail bytes are stored once more where the residual stages read them.  Rows and blocks that do not exist
+// get zero bytes.  gridDim.y cuts the columns where the warps of one CTA do not cover them, gridDim.z runs over
+// batched layers.
+struct ColsPlan {
+    int n_slices;        // slices of all 128-row groups (grouped: of all groups the launch could need)
+    int n_stages;        // slices of rows in flight per CTA
+    int warps;           // computing warps per CTA (one more loads the rows)
+};
+constexpr int kColsMaxStages = 8;
+constexpr size_t kColsSmem = 220 * 1024;   // shared memory of an SM that the rows in flight may take
 
-template <int kRowsThreads>
-__global__ void __launch_bounds__(kRowsThreads, 512 / kRowsThreads)
-quant_act_rows_kernel(const QuantBatch b, int n_slices, int n_buf) {
-    extern __shared__ __align__(16) uint8_t rows_smem_raw[];
-    // 256-byte aligned in the shared address space (the records are addressed with XORs)
-    uint8_t* const rows_smem = rows_smem_raw + ((256u - (smem_u32(rows_smem_raw) & 255u)) & 255u);
-    __shared__ int s_tile_start[kMaxExperts + 1];
-    __shared__ int s_row_start[kMaxExperts + 1];
-    __shared__ __align__(8) uint64_t bar_rows[kRowsMaxBufs];
+__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+// the largest magnitude of three
+__device__ __forceinline__ float max3_abs(float a, float b, float c) {
+    float d;
+    asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t pack_f32x2(uint32_t lo, uint32_t hi) {
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
+    return d;
+}
+__device__ __forceinline__ void unpack_f32x2(uint64_t a, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a));
+}
+
+// kCols: columns per lane, 8 or 16.  kRowsC: rows per slice, 1, 2 or 4.
+template <int kCols, int kRowsC, bool kGrouped, int kMaxT>
+__global__ void __launch_bounds__(kMaxT, 1)
+quant_act_cols_kernel(const QuantBatch b, const ColsPlan plan_c) {
+    constexpr int kPairs = kCols / 2;
+    constexpr int kBlkLanes = kBlock / kCols;            // lanes per 32-element block: 4 or 2
+    constexpr int kAtomLanes = kAtomK / kCols;           // lanes per scale atom: 16 or 8
+    constexpr int kBankLanes = 64 / kCols;               // lanes whose columns take the 32 banks once: 8 or 4
+    constexpr int kSlicesC = kGroupRows / kRowsC;        // slices per group
+    extern __shared__ __align__(128) uint8_t cols_smem[];
+    __shared__ __align__(8) uint64_t bar_full[kColsMaxStages], bar_empty[kColsMaxStages];
+    __shared__ int s_tile_start[kGrouped ? kMaxExperts + 1 : 1];
+    __shared__ int s_row_start[kGrouped ? kMaxExperts + 1 : 1];
     __shared__ int abort_flag_s;
     volatile int* abort_flag = &abort_flag_s;
     grid_launch_dependents();
     const int K = b.K, nblk = K / kBlock;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t row_bytes = K * 2 + 16;       // staged row: 16 bytes past a multiple of 128
-    const uint32_t buf_bytes = kRowsR * row_bytes;
-    // per pair of destination columns: {byte offsets of the two source columns in a staged row, their two
-    // reciprocal scales}; the records come first so that a block's sixteen are 256 aligned bytes
-    uint4* rec = reinterpret_cast<uint4*>(rows_smem);
-    const uint32_t rec_base = smem_u32(rows_smem);
-    uint8_t* const rows_buf = rows_smem + (K / 2) * 16;
-    uint8_t* sfb = rows_buf + n_buf * buf_bytes;     // 2 x [kRowsR][K / 32]: the tail blocks' scale bytes, per slice parity
-    int rec_lin = -1, rec_expert = -1;           // which layer's constants the records hold
+    const int n_stages = plan_c.n_stages, n_warps = plan_c.warps;
+    const bool loader = warp == n_warps;
+    const uint32_t row_bytes = static_cast<uint32_t>(K) * 2, stage_bytes = kRowsC * row_bytes;
+    const QuantLayer& l = b.lay[blockIdx.z];
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kRowsMaxBufs; ++i) mbar_init(smem_u32(&bar_rows[i]), 1);
+        for (int i = 0; i < kColsMaxStages; ++i) { mbar_init(smem_u32(&bar_full[i]), 1); mbar_init(smem_u32(&bar_empty[i]), n_warps); }
         abort_flag_s = 0;
         fence_mbar_init();
     }
 
-    // The layer's (expert's) permutation and reciprocal scales as one 16-byte record per column pair, so that a
-    // lane fetches them with one shared-memory read (the same for all rows of a warp).  The loads of four records
-    // are in flight together: the build is in front of the first slice.
-    auto build_records = [&](int lin, int expert) {
-        const int2* perm2 = reinterpret_cast<const int2*>(b.lay[lin].perm + static_cast<size_t>(expert) * K);
-        const float2* inv2 = reinterpret_cast<const float2*>(b.lay[lin].inv_s_perm + static_cast<size_t>(expert) * K);
-#pragma unroll 1
-        for (int c0 = threadIdx.x; c0 < K / 2; c0 += 4 * kRowsThreads) {
-            int2 p2[4];
-            float2 s2[4];
+    // this lane's columns, block and place in the block
+    const int my = (static_cast<int>(blockIdx.y) * n_warps + warp) * 32 + lane;   // lane index over the whole row
+    const int col0 = my * kCols;
+    const bool col_ok = !loader && col0 < K;             // K % 32 == 0: a lane is all in or all out
+    uint32_t src[kCols];                                 // byte offsets in a row; slot u = column (u + rot) % kCols
+    uint64_t inv2[kPairs];
+    uint32_t rot = 0;
+    auto load_constants = [&](int expert) {
+        const int4* pp = reinterpret_cast<const int4*>(l.perm + static_cast<size_t>(expert) * K + col0);
+        const uint4* ip = reinterpret_cast<const uint4*>(l.inv_s_perm + static_cast<size_t>(expert) * K + col0);
+        uint32_t inv[kCols];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int c2 = c0 + i * kRowsThreads;
-                if (c2 < K / 2) { p2[i] = __ldg(perm2 + c2); s2[i] = __ldg(inv2 + c2); }
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int c2 = c0 + i * kRowsThreads;
-                if (c2 < K / 2)
-                    rec[c2] = make_uint4(static_cast<uint32_t>(p2[i].x) * 2, static_cast<uint32_t>(p2[i].y) * 2,
-                                         __float_as_uint(s2[i].x), __float_as_uint(s2[i].y));
-            }
+        for (int i = 0; i < kCols / 4; ++i) {
+            int4 p4 = make_int4(0, 0, 0, 0);
+            uint4 s4 = make_uint4(0, 0, 0, 0);
+            if (col_ok) { p4 = __ldg(pp + i); s4 = __ldg(ip + i); }
+            src[4 * i] = p4.x; src[4 * i + 1] = p4.y; src[4 * i + 2] = p4.z; src[4 * i + 3] = p4.w;
+            inv[4 * i] = s4.x; inv[4 * i + 1] = s4.y; inv[4 * i + 2] = s4.z; inv[4 * i + 3] = s4.w;
         }
-        rec_lin = lin; rec_expert = expert;
+        rot = (2u * (lane / kBankLanes) - src[0]) % kCols;
+#pragma unroll
+        for (int d = 1; d < kCols; d <<= 1) {
+            uint32_t a[kCols], c[kCols];
+#pragma unroll
+            for (int u = 0; u < kCols; ++u) { a[u] = (rot & d) ? src[(u + d) % kCols] : src[u]; c[u] = (rot & d) ? inv[(u + d) % kCols] : inv[u]; }
+#pragma unroll
+            for (int u = 0; u < kCols; ++u) { src[u] = a[u]; inv[u] = c[u]; }
+        }
+#pragma unroll
+        for (int u = 0; u < kCols; ++u) src[u] *= 2;
+#pragma unroll
+        for (int t = 0; t < kPairs; ++t) inv2[t] = pack_f32x2(inv[2 * t], inv[2 * t + 1]);
     };
-    const bool dense = b.expert_offsets == nullptr;
-    // a dense layer's constants belong to the prepared weights, not to an earlier kernel of the stream: fetch them
-    // while that kernel may still be running
-    if (dense) build_records(0, 0);
-    grid_dependency_wait();
-    if (!dense) {
-        // the experts' row ranges, once per CTA: every slice looks its expert up, and a dependent global load
-        // there would sit in front of each of them
-        for (int e = threadIdx.x; e <= b.n_experts; e += kRowsThreads) s_row_start[e] = b.expert_offsets[e];
+    __syncthreads();
+    if (!kGrouped) {
+        // a dense layer's constants belong to the prepared weights, not to an earlier kernel of the stream
+        if (!loader) load_constants(0);
+        grid_dependency_wait();
+    } else {
+        grid_dependency_wait();
+        // the experts' row ranges, once per CTA
+        for (int e = threadIdx.x; e <= b.n_experts; e += blockDim.x) s_row_start[e] = b.expert_offsets[e];
         __syncthreads();
         if (threadIdx.x < 32) warp_expert_starts(s_row_start, b.n_experts, kGroupRows, s_tile_start, nullptr);
+        __syncthreads();
+    }
+    const int n_slices = kGrouped ? min(plan_c.n_slices, s_tile_start[b.n_experts] * kSlicesC) : plan_c.n_slices;
+
+    // A CTA's slices are consecutive (with stacked experts the constants then change a few times, not per slice), and
+    // the CTAs' shares differ by one slice at most.
+    const int G = static_cast<int>(gridDim.x), g = static_cast<int>(blockIdx.x);
+    const int base = n_slices / G, extra = n_slices - base * G;
+    const int sl_begin = g * base + min(g, extra), n_mine = base + (g < extra ? 1 : 0);
+    // where a slice sits: its group, its first row inside the group, the expert and the rows (in x) of the group
+    int group = sl_begin / kSlicesC, r_first = (sl_begin % kSlicesC) * kRowsC, expert = 0, g_row0 = 0, g_end = 0;
+    auto enter_group = [&]() {
+        if (!kGrouped) {
+            g_row0 = group * kGroupRows; g_end = min(b.M, g_row0 + kGroupRows);
+        } else {
+            while (s_tile_start[expert + 1] <= group) ++expert;   // last expert whose first group is <= group
+            g_row0 = s_row_start[expert] + (group - s_tile_start[expert]) * kGroupRows;
+            g_end = min(s_row_start[expert + 1], g_row0 + kGroupRows);
+        }
+    };
+    auto next_slice = [&]() {
+        r_first += kRowsC;
+        if (r_first == kGroupRows) { r_first = 0; ++group; return true; }
+        return false;
+    };
+    if (n_mine > 0) {
+        if (kGrouped) {
+            int lo = 0, hi = b.n_experts - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (s_tile_start[mid] <= group) lo = mid; else hi = mid - 1;
+            }
+            expert = lo;
+        }
+        enter_group();
+    }
+
+    int it = 0;   // slices whose rows were asked for (the loading warp)
+    if (loader) {
+        int st = 0;
+        uint32_t ph = 0;
+        for (int i = 0; i < n_mine; ++i) {
+            const int row0 = g_row0 + r_first, n_rows = min(kRowsC, g_end - row0);
+            if (n_rows > 0) {
+                if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_empty[st]), ph ^ 1, abort_flag))) break;
+                const uint32_t full = smem_u32(&bar_full[st]);
+                if (lane == 0) mbar_arrive_expect_tx(full, n_rows * row_bytes);
+                __syncwarp();
+                if (lane < n_rows)
+                    bulk_load(smem_u32(cols_smem) + st * stage_bytes + lane * row_bytes, b.x + static_cast<size_t>(row0 + lane) * b.ldx, row_bytes, full);
+                ++it;
+                if (++st == n_stages) { st = 0; ph ^= 1; }
+            }
+            if (next_slice() && i + 1 < n_mine) enter_group();
+        }
+    } else {
+        const StagePlan plan(K, l.k_tail);
+        const int blk = my / kBlkLanes, sub = my % kBlkLanes, ba = blk & 3;   // block of the row, lane in it, block of its atom
+        const int atom = blk >> 2;
+        const int n_tail_blk = l.k_tail / kBlock, tail_t = blk - (nblk - n_tail_blk);   // >= 0: a tail block
+        const int n_res = (plan.S - plan.S1) * (kStageK / kBlock);                      // block positions of the residual stages
+        const size_t sf_stage_stride = static_cast<size_t>(b.act_groups) * kSfGroupBytes;
+        // the pointers that every slice needs, held in registers (the layer is looked up with an index)
+        uint8_t* codes = l.codes + col0 / 2;
+        uint8_t* sf_atom = l.scales_sf + (atom >> 1) * sf_stage_stride + (atom & 1) * 512;
+        uint8_t* sf_tail = l.scales_sf + (plan.S1 + (max(tail_t, 0) >> 3)) * sf_stage_stride + ((tail_t >> 2) & 1) * 512 + (tail_t & 3);
+        asm volatile("" : "+l"(codes), "+l"(sf_atom), "+l"(sf_tail));
+        const bool has_row_scales = l.scales_row != nullptr;
+        const bool word_lane = ba == 0 && atom < 2 * plan.S1;   // an odd atom count leaves half a stage that must read as zeros
+        const bool tail_lane = col_ok && tail_t >= 0;
+        const bool fill = n_res > n_tail_blk && blockIdx.y == 0;
+        const uint32_t smem0 = smem_u32(cols_smem), code_row = K / 2;
+        int st = 0, expert_now = kGrouped ? -1 : 0;
+        uint32_t ph = 0;
+        for (int i_sl = 0; i_sl < n_mine; ++i_sl) {
+            const int row0 = g_row0 + r_first, n_rows = min(kRowsC, g_end - row0);   // n_rows <= 0: padding of the group
+            uint32_t bytes[kRowsC];
+#pragma unroll
+            for (int r = 0; r < kRowsC; ++r) bytes[r] = 0;
+            if (n_rows > 0) {
+                if (kGrouped && expert != expert_now) { load_constants(expert); expert_now = expert; }
+                if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_full[st]), ph, abort_flag))) break;
+                const uint32_t sbase = smem0 + st * stage_bytes;
+                uint64_t v[kRowsC][kPairs];
+                float am[kRowsC];
+#pragma unroll
+                for (int r = 0; r < kRowsC; ++r) {
+                    // rows that do not exist read the last one that does; their results are dropped below
+                    const uint32_t rb = sbase + min(r, n_rows - 1) * row_bytes;
+#pragma unroll
+                    for (int p = 0; p < kPairs; ++p) {
+                        uint32_t x0, x1;
+                        asm volatile("{\n\t.reg .b16 h;\n\tld.shared.b16 h, [%1];\n\tmov.b32 %0, {0, h};\n\t}" : "=r"(x0) : "r"(rb + src[2 * p]));
+                        asm volatile("{\n\t.reg .b16 h;\n\tld.shared.b16 h, [%1];\n\tmov.b32 %0, {0, h};\n\t}" : "=r"(x1) : "r"(rb + src[2 * p + 1]));
+                        v[r][p] = mul_f32x2(pack_f32x2(x0, x1), inv2[p]);
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&bar_empty[st]));   // every value of the slice is in registers
+                if (++st == n_stages) { st = 0; ph ^= 1; }
+#pragma unroll
+                for (int r = 0; r < kRowsC; ++r) {
+                    am[r] = 0.f;
+#pragma unroll
+                    for (int p = 0; p < kPairs; ++p) {
+                        float lo, hi;
+                        unpack_f32x2(v[r][p], lo, hi);
+                        am[r] = max3_abs(am[r], lo, hi);
+                    }
+                }
+                // largest exponent over the block's lanes, two rows per register
+#pragma unroll
+                for (int r = 0; r < kRowsC; r += 2) {
+                    uint32_t e = __float_as_uint(am[r]) >> 23;
+                    if (r + 1 < kRowsC) e |= (__float_as_uint(am[r + 1]) >> 23) << 16;
+#pragma unroll
+                    for (int d = 1; d < kBlkLanes; d <<= 1) e = __vmaxu2(e, __shfl_xor_sync(0xffffffffu, e, d));
+                    bytes[r] = max(static_cast<int>(e & 0xffffu) - 2, 0);
+                    if (r + 1 < kRowsC) bytes[r + 1] = max(static_cast<int>(e >> 16) - 2, 0);
+                }
+                uint8_t* cp = codes + static_cast<size_t>(row0) * code_row;
+#pragma unroll
+                for (int r = 0; r < kRowsC; ++r) {
+                    const uint32_t up = (254u - bytes[r]) << 23;   // 2^(127 - byte), exact multiply
+                    const uint64_t up2 = pack_f32x2(up, up);
+                    uint32_t pk[kCols / 8];
+#pragma unroll
+                    for (int h = 0; h < kCols / 8; ++h) {
+                        float f[8];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) unpack_f32x2(mul_f32x2(v[r][4 * h + i], up2), f[2 * i], f[2 * i + 1]);
+                        pk[h] = cvt_e2m1x8(f[0], f[1], f[2], f[3], f[4], f[5], f[6], f[7]);
+                    }
+                    // nibble u holds column (u + rot) % kCols: put them in order by a rotation of the packed word(s)
+                    const bool live = col_ok && r < n_rows;
+                    if (kCols == 8) {
+                        pk[0] = __funnelshift_l(pk[0], pk[0], 4 * rot);
+                        if (live) *reinterpret_cast<uint32_t*>(cp) = pk[0];
+                    } else {
+                        const uint32_t lo = (rot & 8) ? pk[kCols / 8 - 1] : pk[0], hi = (rot & 8) ? pk[0] : pk[kCols / 8 - 1];
+                        const uint2 w = make_uint2(__funnelshift_l(hi, lo, 4 * (rot & 7)), __funnelshift_l(lo, hi, 4 * (rot & 7)));
+                        if (live) *reinterpret_cast<uint2*>(cp) = w;
+                    }
+                    cp += code_row;
+                    bytes[r] = live ? bytes[r] : 0u;
+                }
+                if (has_row_scales && sub == 0 && col_ok) {
+#pragma unroll
+                    for (int r = 0; r < kRowsC; ++r)
+                        if (r < n_rows) l.scales_row[static_cast<size_t>(row0 + r) * nblk + blk] = static_cast<uint8_t>(bytes[r]);
+                }
+            }
+            const size_t group_off = static_cast<size_t>(group) * kSfGroupBytes;
+            // the lanes of a block share out the slice's rows: lane `sub` brings the words of rows sub, sub + lanes, ...
+#pragma unroll
+            for (int r0 = 0; r0 < kRowsC; r0 += kBlkLanes) {
+                uint32_t mine = bytes[r0];
+#pragma unroll
+                for (int i = 1; i < kBlkLanes; ++i)
+                    if (r0 + i < kRowsC) mine = sub == i ? bytes[r0 + i] : mine;
+                const int r = r0 + sub;
+                const int gr = r_first + r, off = (gr & 31) * 16 + (gr >> 5) * 4;   // row inside its group
+                uint32_t w = mine << (8 * ba);
+#pragma unroll
+                for (int d = kBlkLanes; d < kAtomLanes; d <<= 1) w |= __shfl_xor_sync(0xffffffffu, w, d);
+                if (r < kRowsC && word_lane) *reinterpret_cast<uint32_t*>(sf_atom + group_off + off) = w;
+                if (r < kRowsC && tail_lane) sf_tail[group_off + off] = static_cast<uint8_t>(mine);
+            }
+            // residual block positions past the tail
+            if (fill) {
+                uint8_t* const sf_res = l.scales_sf + group_off + plan.S1 * sf_stage_stride;
+                for (int i = static_cast<int>(threadIdx.x); i < (n_res - n_tail_blk) * kRowsC; i += n_warps * 32) {
+                    const int p = n_tail_blk + i / kRowsC, gr = r_first + i % kRowsC;
+                    sf_res[(p >> 3) * sf_stage_stride + sf_offset_in_group(gr, p & 7)] = 0;
+                }
+            }
+            if (next_slice() && i_sl + 1 < n_mine) enter_group();
+        }
     }
     __syncthreads();
-    const int n_groups = dense ? b.groups_per_lin : s_tile_start[b.n_experts];
-
-    // where a slice sits: its group, its first row (in x) and how many of its rows exist
-    struct Slice { int group, expert, r_first, row0, n_rows; };
-    auto slice_at = [&](int sl) {
-        Slice t;
-        t.group = sl / kRowsSlices; t.r_first = (sl % kRowsSlices) * kRowsR; t.expert = 0;
-        int g_row0, g_end;
-        if (dense) {
-            g_row0 = t.group * kGroupRows; g_end = min(b.M, g_row0 + kGroupRows);
-        } else if (t.group >= n_groups) {   // padding of the launch grid
-            g_row0 = 0; g_end = 0;
-        } else {
-            int lo = 0, hi = b.n_experts - 1;
-            while (lo < hi) {  // last expert whose first group is <= group
-                const int mid = (lo + hi + 1) >> 1;
-                if (s_tile_start[mid] <= t.group) lo = mid; else hi = mid - 1;
-            }
-            t.expert = lo;
-            g_row0 = s_row_start[lo] + (t.group - s_tile_start[lo]) * kGroupRows;
-            g_end = min(s_row_start[lo + 1], g_row0 + kGroupRows);
-        }
-        t.row0 = g_row0 + t.r_first;
-        t.n_rows = max(0, min(kRowsR, g_end - t.row0));
-        return t;
-    };
-    auto request = [&](const Slice& t, int buf) {   // one thread
-        if (t.n_rows == 0) return;
-        const uint32_t bar = smem_u32(&bar_rows[buf]);
-        mbar_arrive_expect_tx(bar, t.n_rows * K * 2);
-        for (int r = 0; r < t.n_rows; ++r)
-            bulk_load(smem_u32(rows_buf + buf * buf_bytes + r * row_bytes), b.x + static_cast<size_t>(t.row0 + r) * b.ldx, K * 2, bar);
-    };
-
-    const int rl = lane % kRowsR, side = lane / kRowsR;
-    const uint32_t byte_sel = side == 0 ? 0x3210u : side == 1 ? 0x2301u : side == 2 ? 0x1032u : 0x0123u;
-    const size_t sf_stage_stride = static_cast<size_t>(b.act_groups) * kSfGroupBytes;
-    uint32_t phases = 0;                         // bit i: parity of buffer i's next completion
-    // a CTA's slices are consecutive: with stacked experts its records then change a few times, not per slice.  The
-    // rows of the next n_buf - 1 slices are on their way while a slice is quantised: a narrow layer's slice is
-    // quantised in a fraction of the time its rows take to arrive.
-    const int per_cta = (n_slices + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x);
-    int sl = min(n_slices, static_cast<int>(blockIdx.x) * per_cta);
-    const int sl_end = min(n_slices, sl + per_cta);
-    if (threadIdx.x == 0)
-        for (int d = 0; d < n_buf - 1 && sl + d < sl_end; ++d) request(slice_at(sl + d), d);
-    for (int it = 0; sl < sl_end; ++it, ++sl) {
-        const int buf = it % n_buf;
-        // the buffer of the slice before this one: its readers passed the barrier of their slice
-        if (threadIdx.x == 0 && sl + n_buf - 1 < sl_end) request(slice_at(sl + n_buf - 1), (it + n_buf - 1) % n_buf);
-        const Slice cur = slice_at(sl);
-        if (!dense && cur.group >= n_groups) continue;
-        if (cur.n_rows > 0) {
-            if (!mbar_wait(smem_u32(&bar_rows[buf]), (phases >> buf) & 1u, abort_flag)) break;
-            phases ^= 1u << buf;
-        }
-        const bool row_ok = rl < cur.n_rows;
-        const uint32_t xrow_a = smem_u32(rows_buf + buf * buf_bytes + rl * row_bytes);
-        const size_t row = static_cast<size_t>(cur.row0 + rl);
-        const int g = cur.r_first + rl;                        // row inside its 128-row group
-        const int sf_row_off = (g & 31) * 16 + (g >> 5) * 4;
-        uint8_t* tailb = sfb + (it & 1) * (kRowsR * nblk);     // [kRowsR][tail blocks] of this slice
-        for (int lin = 0; lin < b.n_lin; ++lin) {
-            const QuantLayer& l = b.lay[lin];
-            if (rec_lin != lin || rec_expert != cur.expert) {
-                if (rec_lin >= 0) __syncthreads();             // the old records are still being read
-                build_records(lin, cur.expert);
-                __syncthreads();
-            }
-            const StagePlan plan(K, l.k_tail);
-            const int tail_blk0 = (K - l.k_tail) / kBlock, n_tail_blk = l.k_tail / kBlock;
-            uint8_t* sf_group = l.scales_sf + static_cast<size_t>(cur.group) * kSfGroupBytes;
-            uint8_t* crow = l.codes + row * (K / 2);
-            // A warp takes whole 128-column atoms, its four sides one block each: the four scale bytes of
-            // (row, atom) meet by two shuffles and go out as the one word the GEMM's layout has for them.  Rows
-            // and blocks that do not exist contribute zero bytes (an odd atom count leaves half a stage of them).
-#pragma unroll 1
-            for (int a = warp; a < 2 * plan.S1; a += kRowsThreads / 32) {
-                const int blk = a * 4 + side;
-                const int j0 = blk * kBlock;
-                uint32_t byte = 0;
-                if (row_ok && blk < nblk) {
-                    // At step t a lane visits the block's column pair t ^ side: where the permutation is (nearly)
-                    // the identity, the four blocks side by side would otherwise read the same banks.  (A block's
-                    // records are 256 aligned bytes, so the exchange is one XOR on the address.)
-                    const uint32_t rec_blk = rec_base + (blk * 256 ^ (side << 4));
-                    float v[32];
-#pragma unroll
-                    for (int t = 0; t < 16; ++t) {
-                        uint4 rc;
-                        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(rc.x), "=r"(rc.y), "=r"(rc.z), "=r"(rc.w) : "r"(rec_blk ^ (t << 4)));
-                        uint16_t x0, x1;
-                        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(x0) : "r"(xrow_a + rc.x));
-                        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(x1) : "r"(xrow_a + rc.y));
-                        v[2 * t] = __uint_as_float(static_cast<uint32_t>(x0) << 16) * __uint_as_float(rc.z);
-                        v[2 * t + 1] = __uint_as_float(static_cast<uint32_t>(x1) << 16) * __uint_as_float(rc.w);
-                    }
-                    float am;
-                    {
-                        float m[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            m[i] = fmaxf(fmaxf(fabsf(v[4 * i]), fabsf(v[4 * i + 1])), fmaxf(fabsf(v[4 * i + 2]), fabsf(v[4 * i + 3])));
-                        am = fmaxf(fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])), fmaxf(fmaxf(m[4], m[5]), fmaxf(m[6], m[7])));
-                    }
-                    byte = scale_byte(__float_as_uint(am));
-                    const float inv = __uint_as_float((254u - byte) << 23);  // 2^(127 - byte), exact multiply
-                    uint32_t pk[4];
-#pragma unroll
-                    for (int h = 0; h < 4; ++h)
-                        pk[h] = cvt_e2m1x8(v[8 * h] * inv, v[8 * h + 1] * inv, v[8 * h + 2] * inv, v[8 * h + 3] * inv,
-                                           v[8 * h + 4] * inv, v[8 * h + 5] * inv, v[8 * h + 6] * inv, v[8 * h + 7] * inv);
-                    // byte t of pk holds pair t ^ side: exchange the bytes inside every word accordingly
-                    *reinterpret_cast<uint4*>(crow + j0 / 2) =
-                        make_uint4(__byte_perm(pk[0], 0, byte_sel), __byte_perm(pk[1], 0, byte_sel),
-                                   __byte_perm(pk[2], 0, byte_sel), __byte_perm(pk[3], 0, byte_sel));
-                    if (l.scales_row) l.scales_row[row * nblk + blk] = static_cast<uint8_t>(byte);
-                    if (blk >= tail_blk0) tailb[rl * nblk + blk - tail_blk0] = static_cast<uint8_t>(byte);
-                }
-                uint32_t w = byte << (8 * side);
-                w |= __shfl_xor_sync(0xffffffffu, w, 8);
-                w |= __shfl_xor_sync(0xffffffffu, w, 16);
-                if (side == 0)
-                    *reinterpret_cast<uint32_t*>(sf_group + (a >> 1) * sf_stage_stride + (a & 1) * 512 + sf_row_off) = w;
-            }
-            // every warp is through with this slice's rows (their buffer may be refilled from now on) and the tail's
-            // bytes are in shared memory
-            __syncthreads();
-            if (n_tail_blk > 0) {
-                // the tail's bytes once more, where the residual stages read them (zeros past the tail and the rows)
-                for (int idx = threadIdx.x; idx < kRowsR * (plan.S - plan.S1) * 2; idx += kRowsThreads) {
-                    const int r = idx % kRowsR, sa = idx / kRowsR, ts = sa >> 1, ah = sa & 1;
-                    const int t0 = ts * 8 + ah * 4;
-                    uint32_t w = 0;
-                    if (r < cur.n_rows) {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            if (t0 + i < n_tail_blk) w |= static_cast<uint32_t>(tailb[r * nblk + t0 + i]) << (8 * i);
-                    }
-                    const int gr = cur.r_first + r;
-                    *reinterpret_cast<uint32_t*>(sf_group + (plan.S1 + ts) * sf_stage_stride + ah * 512 + (gr & 31) * 16 + (gr >> 5) * 4) = w;
-                }
-            }
-        }
-    }
-    if (abort_flag_s) {
-        // copies may still be on their way into this CTA's shared memory: give them one more bounded wait
-        for (int i = 0; i < n_buf; ++i) mbar_wait_after_abort(smem_u32(&bar_rows[i]), (phases >> i) & 1u);
-        if (threadIdx.x == 0 && b.status) atomicExch(b.status, static_cast<int>(PRQ_ERR_TIMEOUT));
-    }
+    // gave up: let the copies in flight land before the CTA's shared memory is given up (bounded)
+    if (loader && lane == 0 && abort_flag_s)
+        for (int j = max(0, it - n_stages); j < it; ++j)
+            mbar_wait_after_abort(smem_u32(&bar_full[j % n_stages]), (j / n_stages) & 1);
+    if (threadIdx.x == 0 && abort_flag_s && b.status) atomicExch(b.status, static_cast<int>(PRQ_ERR_TIMEOUT));
 }
 
-template <int kRowsThreads>
-cudaError_t launch_rows_impl(const QuantBatch& b, size_t smem, int n_buf, int sm_count, cudaStream_t stream) {
-    static size_t configured = 0;   // the attribute is per function; raise it when a larger K comes
-    if (smem > configured) {
-        cudaError_t e = cudaFuncSetAttribute(quant_act_rows_kernel<kRowsThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(smem));
+// Registers of one instance as built (they decide how many of its CTAs an SM holds).
+template <int kCols, int kRowsC, bool kGrouped, int kMaxT>
+cudaError_t launch_cols_impl(const QuantBatch& b, int sm_count, cudaStream_t stream) {
+    auto kernel = quant_act_cols_kernel<kCols, kRowsC, kGrouped, kMaxT>;
+    const int lanes = (b.K + kStageK - 1) / kStageK * (kStageK / kCols);
+    const int all_warps = (lanes + 31) / 32, max_warps = kMaxT / 32 - 1;
+    const int chunks = (all_warps + max_warps - 1) / max_warps, warps = (all_warps + chunks - 1) / chunks;
+    static std::atomic<int> regs{0};   // the same on every device; the attribute is set per device below
+    static std::atomic<unsigned long long> configured{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 64 || !((configured.load(std::memory_order_acquire) >> dev) & 1)) {
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kColsSmem - (kGrouped ? 9216 : 0));
         if (e != cudaSuccess) return e;
-        configured = smem;
+        cudaFuncAttributes fa;
+        e = cudaFuncGetAttributes(&fa, kernel);
+        if (e != cudaSuccess) return e;
+        regs.store(fa.numRegs);
+        if (dev < 64) configured.fetch_or(1ull << dev, std::memory_order_release);
     }
-    const int n_slices = b.groups_per_lin * kRowsSlices;
-    const int per_sm = 512 / kRowsThreads;
+    const int threads = 32 * (warps + 1);
+    const size_t stage = static_cast<size_t>(kRowsC) * b.K * 2;
+    // CTAs per SM: as many as the registers hold, while each still has room for three slices of rows
+    int per_sm = 65536 / (((regs.load() + 7) / 8 * 8) * threads);
+    per_sm = per_sm < 1 ? 1 : per_sm > 16 ? 16 : per_sm;
+    const size_t fixed = 1024 + (kGrouped ? 8 * (kMaxExperts + 1) : 0) + 256;
+    while (per_sm > 1 && kColsSmem / per_sm < 3 * stage + fixed) --per_sm;
+    // slices in flight: about 100 KB per SM hide the memory latency
+    size_t n_stages = (kColsSmem / per_sm - fixed) / stage;
+    const size_t in_flight = (98304 / per_sm + stage - 1) / stage;
+    n_stages = n_stages > in_flight ? in_flight : n_stages;
+    n_stages = n_stages > kColsMaxStages ? kColsMaxStages : n_stages < 2 ? 2 : n_stages;
+    ColsPlan cp;
+    cp.n_slices = b.groups_per_lin * (kGroupRows / kRowsC);
+    cp.n_stages = static_cast<int>(n_stages);
+    cp.warps = warps;
+    int want = per_sm * sm_count / (chunks * b.n_lin);
+    // a CTA of a grouped launch first looks the experts up: two slices at least, or that is all it does
+    if (kGrouped && want > cp.n_slices / 2) want = cp.n_slices / 2;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(n_slices < per_sm * sm_count ? n_slices : per_sm * sm_count);
-    cfg.blockDim = dim3(kRowsThreads);
-    cfg.dynamicSmemBytes = smem;
+    cfg.gridDim = dim3(want < 1 ? 1 : want < cp.n_slices ? want : cp.n_slices, chunks, b.n_lin);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = n_stages * stage;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, quant_act_rows_kernel<kRowsThreads>, b, n_slices, n_buf);
+    return cudaLaunchKernelEx(&cfg, kernel, b, cp);
 }
 
 }  // namespace
@@ -593,29 +695,30 @@ cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, cudaStr
         while (parts < 4 && tiles * parts < 8LL * sm_count[dev]) parts *= 2;   // 3 CTAs per SM: keep the last wave short
         if (parts == 4 && tiles * parts < 4LL * sm_count[dev]) parts = 8;
         if (const char* ev = dev_knobs_enabled() ? getenv("PRQ_QUANT_PARTS") : nullptr) { const int v = atoi(ev); if (v == 1 || v == 2 || v == 4 || v == 8) parts = v; }
-        // Whole rows through shared memory when there are rows enough to fill the GPU that way, a slice's rows fit
-        // twice, and the rows can be fetched by bulk copies (16-byte aligned).
-        // (dense layers: with stacked experts of K = 768 the row structure measured 25-40 % slower than the column atoms
-        // at 128 experts -- 26.7 against 19.0 us at 1024 tokens, 78.7 against 63.5 at 8192 -- also with the experts' row
-        // ranges cached in shared memory and seven slices in flight: narrow rows leave two of the eight warps without
-        // an atom, and a slice of 8 rows is little work per barrier)
-        int rows = b.M >= 512 && b.expert_offsets == nullptr ? 1 : 0;
-        if (const char* ev = dev_knobs_enabled() ? getenv("PRQ_QUANT_ROWS") : nullptr) rows = atoi(ev);
-        const size_t buf_bytes = static_cast<size_t>(kRowsR) * (p.K * 2 + 16);
-        const size_t fixed = static_cast<size_t>(p.K) * 8 + 2 * static_cast<size_t>(kRowsR) * (p.K / 32) + 256;   // + alignment slack
-        if (rows && 2 * buf_bytes + fixed <= 200 * 1024 && (reinterpret_cast<uintptr_t>(b.x) & 15) == 0 && b.ldx % 8 == 0) {
-            QuantBatch br = b;
-            br.n_atoms = n_atoms; br.n_tail = 0; br.tail_split = 1;
-            // Two CTAs per SM where two slices of rows fit twice (8.7 KB of static shared memory and 1 KB reserved per
-            // CTA beside the dynamic part); then as many slices in flight as the CTA's share of the SM holds.
-            const size_t half_sm = 227 * 1024 / 2 - 10 * 1024;
-            const bool two = 2 * buf_bytes + fixed <= half_sm;
-            const size_t budget = two ? half_sm : 200 * 1024;
-            int n_buf = static_cast<int>((budget - fixed) / buf_bytes);
-            n_buf = n_buf > kRowsMaxBufs ? kRowsMaxBufs : n_buf;
-            const size_t smem = n_buf * buf_bytes + fixed;
-            return two ? launch_rows_impl<256>(br, smem, n_buf, sm_count[dev], stream)
-                       : launch_rows_impl<512>(br, smem, n_buf, sm_count[dev], stream);
+        // The column-stationary structure, in the instance that measured best (microseconds in a chain of launches, K and
+        // k as given; column atoms -> this structure):
+        //   up to 128 rows of K <= 4096: one row per slice, CTAs of at most five computing warps (64 x 2560: 2.7 -> 2.0);
+        //   large batches: four rows per slice amortise a slice's bookkeeping (4096 x 2560: 15.3 -> 8.9, four rows against
+        //   two: 8.9 / 9.8; 4096 x 4096: 22.6 -> 11.0); beyond 8192 columns two rows, so that one CTA's registers hold the
+        //   whole width (4096 x 9728: 46.7 -> 20.9, against 22.0 with the columns cut in two);
+        //   in between two rows per slice (600 x 2560: 5.5 -> 3.6, 1000 x 6144: 11.5 -> 6.7, 16 x 9728: 2.9 -> 2.8);
+        //   stacked experts: eight columns per lane, more warps for narrow rows (K = 768, 128 experts: 1024 tokens 19.5 -> 11.5,
+        //   8192 tokens 62 -> 34), except for a handful of atoms, where looking the experts up is all there is to it
+        //   (16 experts of K = 256, 64 rows: 3.1 against 3.6).
+        // What does not fit twice (K beyond about 13 000, 27 000, 55 000 columns at 4, 2, 1 rows) takes the next smaller
+        // slice and finally the column atoms.
+        const bool grouped = b.expert_offsets != nullptr;
+        auto fits = [&](int rows) { return 4 * static_cast<size_t>(rows) * p.K + 10240 <= kColsSmem - 9216; };
+        bool cols = !(grouped && static_cast<long long>(grid_groups) * n_atoms <= 64);
+        if (const char* ev = dev_knobs_enabled() ? getenv("PRQ_QUANT_ROWS") : nullptr) cols = atoi(ev) != 0;
+        if (cols && grouped && fits(4)) return launch_cols_impl<8, 4, true, 544>(b, sm_count[dev], stream);
+        if (cols && !grouped) {
+            const bool large = b.M >= 1500 && p.K >= 2048;
+            if (b.M <= 128 && p.K <= 4096) return launch_cols_impl<16, 1, false, 192>(b, sm_count[dev], stream);
+            if (large && p.K <= 8192) return launch_cols_impl<16, 4, false, 384>(b, sm_count[dev], stream);
+            if (large && fits(2)) return launch_cols_impl<16, 2, false, 640>(b, sm_count[dev], stream);
+            if (fits(2)) return launch_cols_impl<16, 2, false, 320>(b, sm_count[dev], stream);
+            if (fits(1)) return launch_cols_impl<16, 1, false, 192>(b, sm_count[dev], stream);
         }
     }
     // the tail atoms of the scale + permute mode in shares of 16 rows (128 / 8), see the kernel

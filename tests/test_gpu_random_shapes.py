@@ -240,6 +240,24 @@ def test_permuting_quantiser_structures_against_oracle(prq, oracle, monkeypatch,
         w.free()
 
 
+@pytest.mark.parametrize("M,K,k", [(128, 4096, 96), (129, 4128, 32), (1499, 2048, 64), (1500, 2016, 2016), (1501, 2080, 160),
+                                   (1502, 8192, 0), (1505, 8224, 288), (9, 9760, 64), (3, 13760, 96), (2, 27040, 32)])
+def test_permuting_quantiser_instances_against_oracle(prq, oracle, M, K, k):
+    """Both sides of every line of the launcher's rule (rows, columns, what fits shared memory), with partial slices,
+    odd block counts and tails that straddle atoms: codes and scale bytes are whole numbers, so nothing may differ."""
+    ch = synth.HeavyTailChannels(4000 + M, K)
+    W = synth.weights(4100 + M, 32, K)
+    w = prq.prepare_weights(W, oracle.channel_amax(ch.rows(4200 + M, 32)), 0.5, k)
+    x = ch.rows(4300 + M, M)
+    codes, _, sf = prq.quantize_act(w, dev_bf16(x), prq.ACT_SCALE_PERM)
+    assert prq.last_device_status() == 0
+    oc, osc = oracle.quantize_act(x, w.get(prq.FIELD_PERM), w.get(prq.FIELD_INV_S))
+    assert np.array_equal(codes.cpu().numpy()[: M * K // 2].reshape(M, K // 2), oc)
+    want = prq_ref.expected_sf(oracle.augment_act(oc, osc, k)[1], K, k)
+    assert np.array_equal(sf.cpu().numpy()[: want.size], want)
+    w.free()
+
+
 @pytest.mark.parametrize("gbn", [0, 64, 128])
 def test_many_experts_beyond_the_row_cache(prq, oracle, monkeypatch, gbn):
     """300 stacked experts (more than the kernels cache row ranges for), most with a handful of rows and many with
