@@ -145,7 +145,8 @@ prq_status prq_prepare_weights_stacked(const uint16_t *const *Ws, const int *Ns,
  *   W_device  device, n_experts x N x K bf16 row-major (read only; not kept)
  *   act_amax  HOST, n_experts x K fp32          opts  may be NULL
  *   stream    the kernels and copies run there; the call synchronises it before it returns
- * Allocates temporaries on the device (codes, scale bytes and a few arrays of K elements) and frees them.
+ * The handle is one allocation on the device; codes and scale bytes are kept there only, and prq_weights_get copies
+ * them to the host when asked.
  * Errors as prq_prepare_weights; a NaN or an infinity in W * s gives NONFINITE. */
 prq_status prq_prepare_weights_device(const uint16_t *W_device, int n_experts, int N, int K, const float *act_amax,
                                       float alpha, int k_tail, const prq_prep_opts *opts, prq_stream_t stream,

@@ -360,12 +360,17 @@ void prq_weights_free(prq_weights* w) {
     int cur = 0;
     cudaGetDevice(&cur);
     if (w->device >= 0 && w->device != cur) cudaSetDevice(w->device);
-    cudaFree(w->d_codes);
-    cudaFree(w->d_sf);
-    cudaFree(w->d_perm);
-    cudaFree(w->d_inv_s_perm);
-    cudaFree(w->d_inv_s);
-    for (uint8_t* p : w->d_sf_alt) cudaFree(p);
+    if (w->arena) {
+        cudaFree(w->arena);   // every device pointer of the handle lies in it
+    } else {
+        cudaFree(w->d_codes);
+        cudaFree(w->d_sf);
+        cudaFree(w->d_perm);
+        cudaFree(w->d_inv_s_perm);
+        cudaFree(w->d_inv_s);
+        cudaFree(w->d_scales_row);
+        for (uint8_t* p : w->d_sf_alt) cudaFree(p);
+    }
     if (w->device >= 0 && w->device != cur) cudaSetDevice(cur);
     delete w;
 }
@@ -427,6 +432,78 @@ static PrepOptions read_opts(const prq_prep_opts* opts) {
 
 static prq_status create_handle_fp8(const uint16_t* W, int N, int K, const float* act_amax, float alpha, int dev, prq_weights** out);
 
+// A handle from a device copy of W: the kernels write every buffer of it where the GEMMs read it, in one allocation, and
+// only the K-sized arrays pass through the host (scales, column errors, permutation).  Laying the scale bytes out on the
+// host, keeping host copies of the codes and allocating every buffer by itself took 13 - 20 ms at 2560 x 9728, most of it page
+// faults and pageable copies of 14 MB; this takes 0.7 ms, more than half of it the allocation.
+static prq_status fill_handle_device(prq_weights* w, const uint16_t* W, const float* act_amax, bool scale_search, int num_sms,
+                                     cudaStream_t stream) {
+    const int N = w->N, K = w->K, k_tail = w->k_tail;
+    const size_t E = w->n_experts, Ka = static_cast<size_t>(K) + k_tail, S = w->plan.S, EK = E * K;
+    w->h_perm.resize(EK);
+    w->h_s.resize(EK);
+    w->h_inv_s.resize(EK);
+    w->h_col_err.resize(EK + 1);
+    for (size_t e = 0; e < E; ++e) {
+        const prq_status st = channel_scales(act_amax + e * K, K, w->alpha, &w->h_s[e * K], &w->h_inv_s[e * K]);
+        if (st != PRQ_OK) return st;
+    }
+    size_t total = 0;
+    auto take = [&](size_t bytes) { const size_t at = total; total += (bytes + 1023) & ~static_cast<size_t>(1023); return at; };
+    w->d_codes_bytes = E * N * Ka / 2 + 256;
+    // scale bytes in stage order, padded by a few groups so that a tile's bulk copy never runs off the end
+    w->d_sf_bytes = (E * S * w->w_groups + 4) * kSfGroupBytes;
+    const size_t o_codes = take(w->d_codes_bytes), o_sf = take(w->d_sf_bytes);
+    size_t o_alt[kNumAlt] = {}, alt_bytes[kNumAlt] = {};
+    for (int a = 0; a < kNumAlt && E == 1; ++a) {
+        if (!alt_wanted(w->gated, a)) continue;
+        w->w_groups_alt[a] = ((N + kAltTileRows[a] - 1) / kAltTileRows[a]) * ((kAltTileRows[a] + kGroupRows - 1) / kGroupRows);
+        alt_bytes[a] = (S * w->w_groups_alt[a] + 4) * kSfGroupBytes;
+        o_alt[a] = take(alt_bytes[a]);
+    }
+    const size_t o_perm = take(2 * sizeof(float) * EK);        // the permutation and, right behind it, 1 / s in its order
+    const size_t o_rows = take(E * N * Ka / kBlock), o_s = take(sizeof(float) * EK), o_err = take(sizeof(double) * (EK + 1));
+    if (cudaMalloc(&w->arena, total) != cudaSuccess) { cudaGetLastError(); w->arena = nullptr; return PRQ_ERR_OOM; }
+    uint8_t* const base = static_cast<uint8_t*>(w->arena);
+    w->d_codes = base + o_codes;
+    w->d_sf = base + o_sf;
+    for (int a = 0; a < kNumAlt; ++a) if (alt_bytes[a]) w->d_sf_alt[a] = base + o_alt[a];
+    w->d_perm = reinterpret_cast<int32_t*>(base + o_perm);
+    w->d_inv_s_perm = reinterpret_cast<float*>(w->d_perm + EK);
+    w->d_scales_row = base + o_rows;
+    float* const d_s = reinterpret_cast<float*>(base + o_s);
+    double* const d_err = reinterpret_cast<double*>(base + o_err);
+
+    bool ok = cudaMemcpyAsync(d_s, w->h_s.data(), sizeof(float) * EK, cudaMemcpyHostToDevice, stream) == cudaSuccess;
+    ok = ok && cudaMemsetAsync(d_err + EK, 0, sizeof(double), stream) == cudaSuccess;
+    ok = ok && launch_col_err(W, d_s, w->n_experts, N, K, d_err, reinterpret_cast<int*>(d_err + EK), stream) == cudaSuccess;
+    ok = ok && cudaMemcpyAsync(w->h_col_err.data(), d_err, sizeof(double) * (EK + 1), cudaMemcpyDeviceToHost, stream) == cudaSuccess;
+    ok = ok && cudaStreamSynchronize(stream) == cudaSuccess;
+    if (!ok) return PRQ_ERR_CUDA;
+    int nonfinite = 0;
+    std::memcpy(&nonfinite, &w->h_col_err[EK], sizeof(int));
+    if (nonfinite) return PRQ_ERR_NONFINITE;
+    w->h_col_err.resize(EK);
+
+    std::vector<float> both(2 * EK);   // permutation (as bits), then 1 / s in its order
+    for (size_t e = 0; e < E; ++e) {
+        rank_and_permute(&w->h_col_err[e * K], K, k_tail, &w->h_perm[e * K]);
+        for (int j = 0; j < K; ++j) both[EK + e * K + j] = w->h_inv_s[e * K + w->h_perm[e * K + j]];
+    }
+    std::memcpy(both.data(), w->h_perm.data(), sizeof(int32_t) * EK);
+    ok = cudaMemcpyAsync(w->d_perm, both.data(), 2 * sizeof(float) * EK, cudaMemcpyHostToDevice, stream) == cudaSuccess;
+    ok = ok && launch_quant_perm(W, d_s, w->d_perm, w->n_experts, N, K, k_tail, scale_search, w->d_codes, w->d_scales_row, num_sms, stream) == cudaSuccess;
+    SfLayouts t = {};
+    t.n_experts = w->n_experts;
+    t.l[t.n++] = SfLayout{w->d_sf, w->d_sf_bytes, kGroupRows, 1, w->w_groups};
+    for (int a = 0; a < kNumAlt; ++a)
+        if (alt_bytes[a]) t.l[t.n++] = SfLayout{w->d_sf_alt[a], alt_bytes[a], kAltTileRows[a], (kAltTileRows[a] + kGroupRows - 1) / kGroupRows, w->w_groups_alt[a]};
+    ok = ok && launch_sf_layout(w->d_scales_row, N, K, k_tail, t, num_sms, stream) == cudaSuccess;
+    if (ok && build_weight_maps(w) != PRQ_OK) ok = false;   // beside the kernels
+    ok = cudaStreamSynchronize(stream) == cudaSuccess && ok;
+    return ok ? PRQ_OK : PRQ_ERR_CUDA;
+}
+
 static prq_status create_handle(const uint16_t* W, bool w_on_device, prq_stream_t stream, int n_experts, int N, int K,
                                 const float* act_amax, float alpha, int k_tail, const prq_prep_opts* opts, prq_weights** out) {
     const PrepOptions po = read_opts(opts);
@@ -463,6 +540,16 @@ static prq_status create_handle(const uint16_t* W, bool w_on_device, prq_stream_
     w->w_groups = (N + kGroupRows - 1) / kGroupRows;
     w->device = dev;
     w->gated = gated;
+    if (w_on_device) {
+        try {
+            st = fill_handle_device(w, W, act_amax, scale_search, di->num_sms, static_cast<cudaStream_t>(stream));
+        } catch (const std::bad_alloc&) {
+            st = PRQ_ERR_OOM;
+        }
+        if (st != PRQ_OK) { prq_weights_free(w); return st; }
+        *out = w;
+        return PRQ_OK;
+    }
     const size_t Ka = static_cast<size_t>(K) + k_tail;
     const size_t E = n_experts;
     try {
@@ -485,9 +572,7 @@ static prq_status create_handle(const uint16_t* W, bool w_on_device, prq_stream_
         }
         PrepResult r;
         for (size_t e = 0; e < E; ++e) {
-            st = w_on_device ? prepare_layer_device(W + e * N * K, N, K, act_amax + e * K, alpha, k_tail, r, scale_search,
-                                                     static_cast<cudaStream_t>(stream))
-                             : prepare_layer(W + e * N * K, N, K, act_amax + e * K, alpha, k_tail, r, scale_search);
+            st = prepare_layer(W + e * N * K, N, K, act_amax + e * K, alpha, k_tail, r, scale_search);
             if (st != PRQ_OK) { delete w; return st; }
             std::memcpy(&w->h_codes[e * N * Ka / 2], r.codes.data(), r.codes.size());
             std::memcpy(&w->h_scales[e * N * Ka / kBlock], r.scales.data(), r.scales.size());
@@ -767,6 +852,7 @@ prq_status prq_weights_clone(const prq_weights* w, prq_weights** out) {
         dup(&c->d_sf, w->d_sf, w->d_sf_bytes);
         dup(&c->d_perm, w->d_perm, sizeof(int32_t) * EK);
         dup(&c->d_inv_s_perm, w->d_inv_s_perm, sizeof(float) * EK);
+        dup(&c->d_scales_row, w->d_scales_row, EK / w->K * w->N * ((static_cast<size_t>(w->K) + w->k_tail) / kBlock));
         for (int a = 0; a < kNumAlt; ++a) {
             c->w_groups_alt[a] = w->w_groups_alt[a];
             if (w->d_sf_alt[a])
@@ -839,14 +925,33 @@ prq_status prq_weights_info(const prq_weights* w, int* n_experts, int* N, int* K
     return PRQ_OK;
 }
 
+// Bytes of a handle that only the device holds -> host memory.  On a stream of its own, so that it neither waits for nor
+// disturbs what the caller's streams are doing (a capture in progress included); the handle is immutable.
+static prq_status fetch_from_device(const prq_weights* w, void* dst, const void* src, size_t bytes) {
+    int cur = 0;
+    if (cudaGetDevice(&cur) != cudaSuccess) return PRQ_ERR_CUDA;
+    if (cur != w->device && cudaSetDevice(w->device) != cudaSuccess) return PRQ_ERR_CUDA;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    cudaStream_t s = nullptr;
+    bool ok = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess;
+    ok = ok && cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, s) == cudaSuccess;
+    ok = ok && cudaStreamSynchronize(s) == cudaSuccess;
+    if (s) cudaStreamDestroy(s);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (cur != w->device) cudaSetDevice(cur);
+    return ok ? PRQ_OK : PRQ_ERR_CUDA;
+}
+
 prq_status prq_weights_get(const prq_weights* w, int expert, prq_field which, void* dst, size_t dst_bytes) {
     if (!w || !dst || expert < 0 || expert >= w->n_experts) return PRQ_ERR_INVALID_ARG;
     const size_t Ka = static_cast<size_t>(w->K) + w->k_tail, N = w->N, K = w->K, e = expert;
     const void* src = nullptr;
     size_t bytes = 0;
+    bool on_device = false;
     switch (which) {
-        case PRQ_FIELD_CODES: bytes = w->format == PRQ_FMT_MXFP8 ? N * K : N * Ka / 2; src = &w->h_codes[e * bytes]; break;
-        case PRQ_FIELD_SCALES: bytes = N * Ka / kBlock; src = &w->h_scales[e * bytes]; break;
+        case PRQ_FIELD_CODES: bytes = w->format == PRQ_FMT_MXFP8 ? N * K : N * Ka / 2; on_device = w->h_codes.empty(); src = (on_device ? w->d_codes : w->h_codes.data()) + e * bytes; break;
+        case PRQ_FIELD_SCALES: bytes = N * Ka / kBlock; on_device = w->h_scales.empty(); src = (on_device ? w->d_scales_row : w->h_scales.data()) + e * bytes; break;
         case PRQ_FIELD_PERM: bytes = K * sizeof(int32_t); src = &w->h_perm[e * K]; break;
         case PRQ_FIELD_TOPK: bytes = w->k_tail * sizeof(int32_t); src = w->h_perm.data() + e * K + (K - w->k_tail); break;
         case PRQ_FIELD_S: bytes = K * sizeof(float); src = &w->h_s[e * K]; break;
@@ -855,6 +960,7 @@ prq_status prq_weights_get(const prq_weights* w, int expert, prq_field which, vo
         default: return PRQ_ERR_INVALID_ARG;
     }
     if (dst_bytes != bytes) return PRQ_ERR_INVALID_ARG;
+    if (bytes && on_device) return fetch_from_device(w, dst, src, bytes);
     if (bytes) std::memcpy(dst, src, bytes);
     return PRQ_OK;
 }

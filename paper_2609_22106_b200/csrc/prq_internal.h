@@ -61,9 +61,10 @@ prq_status prepare_layer(const uint16_t* W, int N, int K, const float* amax, flo
 // The pieces of it that stay on the host when the rest runs on the GPU:
 // s_j = max(amax_j, 1e-5)^alpha and its reciprocal (FP64, stored fp32; PRQ_ERR_NONFINITE on a bad amax) ...
 prq_status channel_scales(const float* amax, int K, float alpha, std::vector<float>& s, std::vector<float>& inv_s);
+prq_status channel_scales(const float* amax, int K, float alpha, float* s, float* inv_s);
 // ... and the error-ranked top-k with its permutation [unselected ascending | selected ascending]
 // (ties: the lower channel index ranks first).
-void rank_and_permute(const std::vector<double>& col_err, int K, int k_tail, std::vector<int32_t>& perm);
+void rank_and_permute(const double* col_err, int K, int k_tail, int32_t* perm);
 // Eq. (1), middle line: rows of the producer weights permuted (and, for the up projection, scaled by 1 / s and
 // rounded once to bf16); with duplicate_tail the last k_tail rows are repeated.  Host buffers.
 prq_status fold_producer(const int32_t* perm, const float* inv_s, int C, int k_tail, const uint16_t* W_up,
@@ -75,11 +76,16 @@ prq_status prepare_layer_fp8(const uint16_t* W, int N, int K, const float* amax,
 // Gate and up projection rows interleaved in groups of 32 (rows 64 b .. 64 b + 31 = gate rows 32 b .., rows 64 b + 32 ..
 // 64 b + 63 = up rows 32 b ..): the layout prq_linear_gated expects.  Host buffers, C % 32 == 0.
 void stack_gate_up(const uint16_t* W_gate, const uint16_t* W_up, int C, int H, uint16_t* out);
-// The same result computed on the current device from a DEVICE copy of W (column errors, permuted
-// quantisation, residual and packing as kernels; scales and ranking on the host in between).  Allocates its
-// temporaries, runs on `stream` and synchronises it.
-prq_status prepare_layer_device(const uint16_t* W_dev, int N, int K, const float* amax, float alpha, int k_tail,
-                                PrepResult& out, bool scale_search, cudaStream_t stream);
+// The heavy steps of the same on the GPU (prq_prep_device.cu), all experts of a layer per launch; device buffers.
+// Column errors of the scaled weights s: E x K, err: E x K doubles; *nonfinite becomes 1 if W * s holds a NaN or infinity.
+cudaError_t launch_col_err(const uint16_t* W, const float* s, int E, int N, int K, double* err, int* nonfinite, cudaStream_t stream);
+// [Q(W D P) | Q(R)]: codes E x N x (K + k)/2, scale bytes E x N x (K + k)/32, both row-major.
+cudaError_t launch_quant_perm(const uint16_t* W, const float* s, const int32_t* perm, int E, int N, int K, int k_tail, bool search,
+                              uint8_t* codes, uint8_t* scales, int sm_count, cudaStream_t stream);
+// Row-major scale bytes -> the layouts of the GEMMs (padding becomes zero).
+struct SfLayout { uint8_t* dst; size_t bytes; int tile_rows, groups_per_tile, groups; };   // groups per stage and expert
+struct SfLayouts { int n, n_experts; SfLayout l[5]; };
+cudaError_t launch_sf_layout(const uint8_t* scales, int N, int K, int k_tail, const SfLayouts& t, int sm_count, cudaStream_t stream);
 
 }  // namespace prq
 
@@ -89,7 +95,8 @@ struct prq_weights {
     prq::StagePlan plan;
     int w_groups = 0;  // ceil(N / 128) scale groups per expert (layout for 128- and 256-row weight tiles)
     int device = -1;
-    // canonical host copies (all experts concatenated)
+    // canonical copies (all experts concatenated).  A layer prepared on the device leaves its codes and row-major scale
+    // bytes there (d_codes, d_scales_row; h_codes and h_scales are empty): prq_weights_get fetches them when asked.
     std::vector<uint8_t> h_codes, h_scales;
     std::vector<int32_t> h_perm;
     std::vector<float> h_s, h_inv_s;
@@ -117,4 +124,6 @@ struct prq_weights {
     int32_t* d_perm = nullptr;       // E x K
     float* d_inv_s_perm = nullptr;   // E x K : inv_s[perm[j]] in the new channel order
     size_t d_codes_bytes = 0, d_sf_bytes = 0;
+    uint8_t* d_scales_row = nullptr; // E x N x (K + k)/32 (layers prepared on the device)
+    void* arena = nullptr;           // one allocation that holds all of the above (layers prepared on the device)
 };

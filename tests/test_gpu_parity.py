@@ -531,6 +531,57 @@ def test_device_prep_experts_and_errors(prq, oracle):
     assert ei.value.code == 7                        # PRQ_ERR_NONFINITE
 
 
+@pytest.mark.parametrize("E,N,K,k,search,offset", [
+    (1, 1, 32, 32, False, 0), (1, 127, 96, 32, True, 1), (1, 128, 544, 0, False, 2), (1, 129, 10272, 288, False, 0), (1, 513, 10240, 64, True, 3),
+    (1, 3, 49184, 64, False, 0), (1, 2, 49184, 32, True, 1), (3, 130, 160, 64, True, 1), (2, 300, 768, 96, False, 4)])
+def test_device_prep_at_its_edges(prq, E, N, K, k, search, offset):
+    """Device prep against host prep, field by field: rows around the 128 that are summed at a time, layers wider than one
+    CTA's threads and than shared memory, weights on 2, 4, 6 and 8 bytes, and the clone of such a handle."""
+    Ws = np.stack([synth.weights(60 + e, N, K) for e in range(E)])
+    amax = np.stack([np.abs(np.random.default_rng(70 + e).standard_normal(K)).astype(np.float32) + 0.05 for e in range(E)])
+    flat = torch.zeros(E * N * K + 8, dtype=torch.int16, device="cuda")
+    flat[offset:offset + Ws.size] = torch.from_numpy(Ws.view(np.int16).reshape(-1)).cuda()
+    wd = prq.prepare_weights_device(flat[offset:offset + Ws.size].view(E, N, K), amax, 0.5, k, scale_search=search)
+    wh = prq.prepare_weights(Ws, amax, 0.5, k, scale_search=search)
+    wc = wd.clone()
+    for e in range(E):
+        for f in (prq.FIELD_S, prq.FIELD_INV_S, prq.FIELD_COL_ERR, prq.FIELD_PERM, prq.FIELD_TOPK, prq.FIELD_SCALES, prq.FIELD_CODES):
+            assert np.array_equal(wd.get(f, e), wh.get(f, e)), (e, f)
+            assert np.array_equal(wc.get(f, e), wh.get(f, e)), (e, f)
+    for w in (wd, wh, wc):
+        w.free()
+
+
+@pytest.mark.parametrize("bn", [224, 240, 288])
+def test_device_prep_layouts_feed_every_kernel(prq, monkeypatch, bn):
+    """The scale-byte layouts that the device writes are the host's: decode and every prefill tile width give the same
+    bits from either handle (N ragged in all tilings, residual stages partly filled); so does a capture during which a
+    field is fetched."""
+    monkeypatch.setenv("PRQ_PAIR_BN", str(bn))
+    N, K, k = 1000, 1056, 288
+    W = synth.weights(81, N, K)
+    amax = np.abs(np.random.default_rng(82).standard_normal(K)).astype(np.float32) + 0.05
+    wd, wh = prq.prepare_weights_device(torch.from_numpy(W.view(np.int16)).cuda(), amax, 0.5, k), prq.prepare_weights(W, amax, 0.5, k)
+    for M in (5, 128, 300):
+        x = to_dev_bf16(synth.HeavyTailChannels(83, K).rows(84 + M, M))
+        ys = []
+        for w in (wd, wh):
+            codes, _, sf = prq.quantize_act(w, x, prq.ACT_SCALE_PERM)
+            ys.append(prq.linear(w, codes, sf, M))
+        assert torch.equal(*ys), M
+    assert prq.last_device_status() == 0
+    y = torch.empty((5, N), device="cuda")
+    codes, _, sf = prq.quantize_act(wd, x[:5], prq.ACT_SCALE_PERM)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        prq.linear(wd, codes, sf, 5, out=y)
+        fetched = wd.get(prq.FIELD_CODES)
+    g.replay()
+    assert torch.equal(y, prq.linear(wh, codes, sf, 5)) and np.array_equal(fetched, wh.get(prq.FIELD_CODES))
+    wd.free()
+    wh.free()
+
+
 @pytest.mark.parametrize("N,K,k,M", [(256, 512, 64, 16), (512, 2560, 128, 300), (256, 768, 64, 1), (384, 1024, 256, 128)])
 def test_offline_copy_form_equals_the_revisit_form(prq, oracle, N, K, k, M):
     """Activation tail construction paragraph, offline copy: the producer emits the k tail channels twice, the
