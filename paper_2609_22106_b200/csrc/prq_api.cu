@@ -31,6 +31,7 @@ struct DeviceInfo {
     int max_clusters[4][9] = {};  // decode kernel: [token-tile index][cluster size], 0 = not queried yet
     int max_pairs = 0;            // prefill pair kernel: co-resident CTA pairs, 0 = not queried yet
     int max_pairs_gated = 0;      // the same for its gated-producer instance
+    int max_pairs_fp8 = 0;        // ... and for its instances of the second format
 };
 std::mutex g_dev_mutex;
 DeviceInfo g_dev[64];
@@ -277,6 +278,35 @@ PairSchedule choose_pair_schedule(int M, int N, int S, int max_pairs) {
     return best;
 }
 
+// Second format: CTA pairs on 256-row tiles, or the tile-per-CTA kernel (bn = 0).  A 128 x 128 tile needs 33 KB of fresh
+// operands per 358 cycles of E4M3 MMAs, more than L2 gives 148 SMs at once; the pair's tile halves the bytes per MMA (q / k / v
+// stacked, 6144 x 2560 at 4096 tokens: 65.8 -> 52.6 us; o, 2560 x 4096: 46.0 -> 37.7).  A wave of pairs takes about as long
+// as a wave of small tiles, so the pairs are taken where they need fewer waves (512 x 6144 x 2560: one against two, 13.9 /
+// 16.1 us; 1024 x 6144: two against three, 20.6 / 22.5) and not where both need one (300 x 1024 x 1024: 9.5 / 8.6 us).  The
+// width is the one whose waves move the fewest operand bytes; 288 columns only in a single wave.
+struct Fp8Schedule { int bn, pairs; long long tiles, waves; };
+Fp8Schedule fp8_schedule(int M, int N, DeviceInfo* di) {
+    Fp8Schedule best = {};
+    if (di->max_pairs_fp8 == 0) di->max_pairs_fp8 = std::min(prefill_pair_max_clusters_fp8(), di->num_sms / 2);
+    if (di->max_pairs_fp8 < 1) return best;
+    // developer switch: 0 = the tile-per-CTA kernel, 224 / 240 / 288 = that width where it can run
+    const int forced = env_int("PRQ_FP8_BN", -1);
+    if (forced == 0) return best;
+    const int bns[3] = {kPrefillTileN, kPrefillTileWide, kPrefillTileOneWave}, bytes[3] = {32256, 33280, 37376};
+    long long best_cost = 1ll << 60;
+    for (int i = 0; i < 3; ++i) {
+        const long long tiles = ((M + 255ll) / 256) * ((N + bns[i] - 1) / bns[i]);
+        const int pairs = static_cast<int>(std::min<long long>(tiles, di->max_pairs_fp8));
+        const long long waves = (tiles + pairs - 1) / pairs;
+        if (bns[i] == kPrefillTileOneWave && waves > 1) continue;
+        if (forced > 0 && bns[i] != forced) continue;
+        if (waves * bytes[i] < best_cost) { best_cost = waves * bytes[i]; best = Fp8Schedule{bns[i], pairs, tiles, waves}; }
+    }
+    const long long units = ((M + 127ll) / 128) * ((N + 127ll) / 128), unit_waves = (units + di->num_sms - 1) / di->num_sms;
+    if (forced < 0 && best.waves >= unit_waves) best.bn = 0;
+    return best;
+}
+
 // Two counters ("arrived", "finished") per 128-row half of a 256 x 224 pair tile: first all the "arrived"
 // counters, then all the "finished" ones.
 size_t prefill_flag_count(const prq_weights* w, int M) {
@@ -494,7 +524,7 @@ static prq_status fill_handle_device(prq_weights* w, const uint16_t* W, const fl
     ok = cudaMemcpyAsync(w->d_perm, both.data(), 2 * sizeof(float) * EK, cudaMemcpyHostToDevice, stream) == cudaSuccess;
     ok = ok && launch_quant_perm(W, d_s, w->d_perm, w->n_experts, N, K, k_tail, scale_search, w->d_codes, w->d_scales_row, num_sms, stream) == cudaSuccess;
     SfLayouts t = {};
-    t.n_experts = w->n_experts;
+    t.n_experts = w->n_experts; t.group_bytes = kSfGroupBytes;
     t.l[t.n++] = SfLayout{w->d_sf, w->d_sf_bytes, kGroupRows, 1, w->w_groups};
     for (int a = 0; a < kNumAlt; ++a)
         if (alt_bytes[a]) t.l[t.n++] = SfLayout{w->d_sf_alt[a], alt_bytes[a], kAltTileRows[a], (kAltTileRows[a] + kGroupRows - 1) / kGroupRows, w->w_groups_alt[a]};
@@ -645,24 +675,46 @@ static prq_status create_handle_fp8(const uint16_t* W, int N, int K, const float
         w->h_perm.resize(K);
         for (int j = 0; j < K; ++j) w->h_perm[j] = j;
         w->h_col_err.assign(K, 0.0);
-        const int S8 = (K + 127) / 128, nblk = K / kBlock;
+        const int S8 = (K + 127) / 128;
         w->d_sf_bytes = (static_cast<size_t>(S8) * w->w_groups + 4) * 512;
-        std::vector<uint8_t> sf(w->d_sf_bytes, 0);
-        for (int n = 0; n < N; ++n)
-            for (int b = 0; b < nblk; ++b)
-                sf[(static_cast<size_t>(b / 4) * w->w_groups + n / kGroupRows) * 512 + sf_offset_in_group(n % kGroupRows, b % 4)] =
-                    w->h_scales[static_cast<size_t>(n) * nblk + b];
         w->d_codes_bytes = w->h_codes.size() + 256;
-        if (cudaMalloc(&w->d_codes, w->d_codes_bytes) != cudaSuccess || cudaMalloc(&w->d_sf, w->d_sf_bytes) != cudaSuccess ||
-            cudaMalloc(&w->d_inv_s, sizeof(float) * K) != cudaSuccess) {
+        size_t alt_bytes[kNumAlt] = {};
+        bool mem = cudaMalloc(&w->d_codes, w->d_codes_bytes) == cudaSuccess && cudaMalloc(&w->d_sf, w->d_sf_bytes) == cudaSuccess &&
+                   cudaMalloc(&w->d_inv_s, sizeof(float) * K) == cudaSuccess && cudaMalloc(&w->d_scales_row, w->h_scales.size()) == cudaSuccess;
+        for (int a = 0; a < kNumAlt && mem; ++a) {
+            if (!alt_wanted(false, a)) continue;
+            w->w_groups_alt[a] = ((N + kAltTileRows[a] - 1) / kAltTileRows[a]) * ((kAltTileRows[a] + kGroupRows - 1) / kGroupRows);
+            alt_bytes[a] = (static_cast<size_t>(S8) * w->w_groups_alt[a] + 4) * 512;
+            mem = cudaMalloc(&w->d_sf_alt[a], alt_bytes[a]) == cudaSuccess;
+        }
+        if (!mem) {
             cudaGetLastError();
             prq_weights_free(w);
             return PRQ_ERR_OOM;
         }
-        bool ok = cudaMemcpy(w->d_codes, w->h_codes.data(), w->h_codes.size(), cudaMemcpyHostToDevice) == cudaSuccess;
-        ok = ok && cudaMemcpy(w->d_sf, sf.data(), sf.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+        // the tile-per-CTA kernel's layout and the three tilings of the pair kernel, from one upload of the row-major bytes
+        SfLayouts t = {};
+        t.n_experts = 1; t.group_bytes = 512;
+        t.l[t.n++] = SfLayout{w->d_sf, w->d_sf_bytes, kGroupRows, 1, w->w_groups};
+        for (int a = 0; a < kNumAlt; ++a)
+            if (alt_bytes[a]) t.l[t.n++] = SfLayout{w->d_sf_alt[a], alt_bytes[a], kAltTileRows[a], (kAltTileRows[a] + kGroupRows - 1) / kGroupRows, w->w_groups_alt[a]};
+        DeviceInfo* di;
+        bool ok = device_info(dev, &di) == PRQ_OK;
+        ok = ok && cudaMemcpy(w->d_codes, w->h_codes.data(), w->h_codes.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+        ok = ok && cudaMemcpy(w->d_scales_row, w->h_scales.data(), w->h_scales.size(), cudaMemcpyHostToDevice) == cudaSuccess;
         ok = ok && cudaMemcpy(w->d_inv_s, w->h_inv_s.data(), sizeof(float) * K, cudaMemcpyHostToDevice) == cudaSuccess;
-        if (!ok || make_code_map(&w->tm_w_fp8, w->d_codes, static_cast<uint64_t>(K), N, 128) != PRQ_OK) {
+        ok = ok && launch_sf_layout(w->d_scales_row, N, K, 0, t, di->num_sms, nullptr) == cudaSuccess;
+        ok = ok && cudaStreamSynchronize(nullptr) == cudaSuccess;
+        cudaFree(w->d_scales_row);   // the canonical bytes of a host preparation stay on the host
+        w->d_scales_row = nullptr;
+        ok = ok && make_code_map(&w->tm_w_fp8, w->d_codes, static_cast<uint64_t>(K), N, 128) == PRQ_OK;
+        for (int a = 0; a < kNumAlt && ok; ++a) {
+            if (!alt_bytes[a]) continue;
+            const int rows = kAltTileRows[a], gpt = (rows + kGroupRows - 1) / kGroupRows;
+            ok = make_code_map(&w->tm_w_pair[a], w->d_codes, static_cast<uint64_t>(K), N, rows / 2) == PRQ_OK &&
+                 make_sf_map(&w->tm_sfw_pair[a], w->d_sf_alt[a], static_cast<uint64_t>(S8) * w->w_groups_alt[a] * 512, 2 * gpt * (a == 2 ? 2 : 1)) == PRQ_OK;
+        }
+        if (!ok) {
             prq_weights_free(w);
             return PRQ_ERR_CUDA;
         }
@@ -1093,16 +1145,37 @@ prq_status prq_linear(const prq_weights* w, const void* codes, const void* scale
     p.n_experts = 1;
     p.act_groups = dense_groups(M);
     if (w->format == PRQ_FMT_MXFP8) {
-        // second format: the tile-per-CTA kernel (128 output features x 128 tokens) over the layer as one expert
-        p.w_groups = w->w_groups;
-        p.act_sf = static_cast<const uint8_t*>(scales_sf);
-        p.w_sf = w->d_sf;
-        p.y = y; p.ldy = ldy; p.y_bf16 = y_dtype == PRQ_BF16;
-        p.status = di->status_ptr;
-        CUtensorMap tm_act8;
-        st = make_code_map(&tm_act8, codes, static_cast<uint64_t>(w->K), M, 128);
-        if (st != PRQ_OK) return st;
-        cudaError_t e8 = launch_gemm_fp8(tm_act8, w->tm_w_fp8, p, di->num_sms, static_cast<cudaStream_t>(stream));
+        const cudaError_t e8 = [&]() -> cudaError_t {
+            const Fp8Schedule fs = fp8_schedule(M, w->N, di);
+            if (fs.bn) {
+                // the pair kernel, whole tiles wave after wave
+                const int v = fs.bn == kPrefillTileOneWave ? 2 : fs.bn == kPrefillTileWide ? 1 : 0;
+                PrefillParams q;
+                std::memset(&q, 0, sizeof(q));
+                q.M = M; q.N = w->N; q.K = w->K;
+                q.m_tiles = (M + 255) / 256; q.n_tiles = (w->N + fs.bn - 1) / fs.bn;
+                q.total_tiles = static_cast<int>(fs.tiles); q.whole_tiles = static_cast<int>(fs.waves);
+                q.act_groups = p.act_groups; q.w_groups = w->w_groups_alt[v];
+                q.y = y; q.ldy = ldy; q.y_bf16 = y_dtype == PRQ_BF16;
+                q.status = di->status_ptr; q.trace = trace_ptr();
+                q.wait_limit = kDefaultWaitLimitCycles;
+                CUtensorMap tm_a, tm_sfa, tm_y;
+                const size_t sf_bytes = static_cast<size_t>((w->K + 127) / 128) * p.act_groups * 512;
+                if (make_code_map(&tm_a, codes, static_cast<uint64_t>(w->K), M, 128) != PRQ_OK || make_sf_map(&tm_sfa, scales_sf, sf_bytes, 2) != PRQ_OK ||
+                    make_out_map(&tm_y, y, M, w->N, ldy, y_dtype == PRQ_BF16) != PRQ_OK)
+                    return cudaErrorInvalidValue;
+                return launch_prefill_pair_fp8(fs.bn, tm_a, w->tm_w_pair[v], tm_sfa, w->tm_sfw_pair[v], tm_y, q, fs.pairs, static_cast<cudaStream_t>(stream));
+            }
+            // the tile-per-CTA kernel (128 output features x 128 tokens) over the layer as one expert
+            p.w_groups = w->w_groups;
+            p.act_sf = static_cast<const uint8_t*>(scales_sf);
+            p.w_sf = w->d_sf;
+            p.y = y; p.ldy = ldy; p.y_bf16 = y_dtype == PRQ_BF16;
+            p.status = di->status_ptr;
+            CUtensorMap tm_act8;
+            if (make_code_map(&tm_act8, codes, static_cast<uint64_t>(w->K), M, 128) != PRQ_OK) return cudaErrorInvalidValue;
+            return launch_gemm_fp8(tm_act8, w->tm_w_fp8, p, di->num_sms, static_cast<cudaStream_t>(stream));
+        }();
         g_launches.fetch_add(1);
         return e8 == cudaSuccess ? PRQ_OK : PRQ_ERR_CUDA;
     }

@@ -10,6 +10,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cmath>
 #include <cstring>
 
@@ -137,27 +138,31 @@ prq_status prepare_layer_fp8(const uint16_t* W, int N, int K, const float* amax,
     if (st != PRQ_OK) return st;
     codes.assign(static_cast<size_t>(N) * K, 0);
     scales.assign(static_cast<size_t>(N) * K / kBlock, 0);
-    for (int n = 0; n < N; ++n)
-        for (int b = 0; b < K / kBlock; ++b) {
-            float v[kBlock], am = 0.f;
-            for (int i = 0; i < kBlock; ++i) {
-                const int j = b * kBlock + i;
-                const uint32_t u = static_cast<uint32_t>(W[static_cast<size_t>(n) * K + j]) << 16;
-                float w;
-                std::memcpy(&w, &u, 4);
-                if (!std::isfinite(w)) return PRQ_ERR_NONFINITE;
-                v[i] = w * s[j];                               // bf16 x fp32 -> fp32, one rounding
-                am = std::fmax(am, std::fabs(v[i]));
+    std::atomic<bool> finite{true};
+    parallel_for(N, [&](long lo, long hi) {
+        for (long n = lo; n < hi; ++n)
+            for (int b = 0; b < K / kBlock; ++b) {
+                float v[kBlock], am = 0.f;
+                bool ok = true;
+                for (int i = 0; i < kBlock; ++i) {
+                    const int j = b * kBlock + i;
+                    const uint32_t u = static_cast<uint32_t>(W[static_cast<size_t>(n) * K + j]) << 16;
+                    float w;
+                    std::memcpy(&w, &u, 4);
+                    ok = ok && std::isfinite(w);
+                    v[i] = w * s[j];                           // bf16 x fp32 -> fp32, one rounding
+                    am = std::fmax(am, std::fabs(v[i]));
+                }
+                if (!ok || !std::isfinite(am)) { finite.store(false); return; }
+                uint32_t ab;
+                std::memcpy(&ab, &am, 4);
+                const int eb = static_cast<int>(ab >> 23) - 8;
+                const int byte = am == 0.f ? 0 : (eb < 0 ? 0 : eb);
+                scales[static_cast<size_t>(n) * (K / kBlock) + b] = static_cast<uint8_t>(byte);
+                for (int i = 0; i < kBlock; ++i) codes[static_cast<size_t>(n) * K + b * kBlock + i] = e4m3_code(v[i], byte - 127);
             }
-            if (!std::isfinite(am)) return PRQ_ERR_NONFINITE;
-            uint32_t ab;
-            std::memcpy(&ab, &am, 4);
-            const int eb = static_cast<int>(ab >> 23) - 8;
-            const int byte = am == 0.f ? 0 : (eb < 0 ? 0 : eb);
-            scales[static_cast<size_t>(n) * (K / kBlock) + b] = static_cast<uint8_t>(byte);
-            for (int i = 0; i < kBlock; ++i) codes[static_cast<size_t>(n) * K + b * kBlock + i] = e4m3_code(v[i], byte - 127);
-        }
-    return PRQ_OK;
+    });
+    return finite.load() ? PRQ_OK : PRQ_ERR_NONFINITE;
 }
 
 }  // namespace prq

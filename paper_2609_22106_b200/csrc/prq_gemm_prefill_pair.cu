@@ -52,7 +52,6 @@ namespace {
 
 constexpr int kThreads = 192;
 constexpr int kPTile = 128 * 128;                 // activation tile bytes (128 rows x 256 codes)
-constexpr int kSfp = kSfGroupBytes;               // 1 group of 128 activation rows
 constexpr int kStages = 5;
 constexpr int kStagingPerWarp = 2 * 4096;         // two 32-row x 128-byte chunks per epilogue warp
 constexpr int kTmemCols = 512;
@@ -68,22 +67,30 @@ constexpr int kChunkCols = 32;                    // accumulator columns per epi
 //   much as one of 64: 256 + 32 measured 9 % slower than 144 + 144 predicts); each CTA loads 72 + 72 weight rows -- rows
 //   [72 r, +72) and [144 + 72 r, +72) of the tile -- so that the accumulator's columns are the tile's weight rows in
 //   order, and the scale bytes are tiled per 144-row half (two groups each).
-template <int BN>
+// kFp8: the second format (MXFP8, one byte per element).  A stage is still one 128-byte swizzled row per operand row,
+// which then holds 128 elements = four blocks = ONE 512-byte scale atom per 128-row group, and an MMA takes 32 of them.
+template <int BN, bool kFp8 = false>
 struct PCfg {
+    static constexpr int kStageElems = kFp8 ? 128 : kStageK;
+    static constexpr int kSfGroup = kFp8 ? 512 : kSfGroupBytes;   // scale bytes per (stage, 128-row group)
+    static constexpr int kSfRows = kSfGroup / 256;                // rows of the scale tensor maps per group
+    static constexpr int kSfp = kSfGroup;                         // one group of 128 activation rows
     static constexpr bool kWide = BN > 256;
     static constexpr int kHalfN = BN / 2;                    // weight rows each CTA of the pair loads
     static constexpr int kQTile = kHalfN * 128;              // half weight tile bytes
     static constexpr int kHalfGroups = kWide ? (BN / 2 + 127) / 128 : 0;                    // scale groups per 144-row half
     static constexpr int kSfqGroups = kWide ? 2 * kHalfGroups : (BN + 127) / 128;           // 128-row scale groups of a weight tile
-    static constexpr int kSfq = kSfqGroups * kSfGroupBytes;
-    static constexpr int kStageBytes = kPTile + kQTile + kSfp + kSfq;  // 33792 / 34816 / 39936
+    static constexpr int kSfq = kSfqGroups * kSfGroup;
+    static constexpr int kTxBytes = kPTile + kQTile + kSfp + kSfq;     // 33792 / 34816 / 39936; MXFP8 32256 / 33280 / 37376
+    static constexpr int kStageBytes = (kTxBytes + 1023) / 1024 * 1024;
     // the alternating staging buffers serve epilogues that run under a main loop; the one-wave tile has only a last
     // epilogue, which stages in the idle ring
     static constexpr int kStagingBytes = kWide ? 0 : 4 * kStagingPerWarp;
     static constexpr int kSmemBytes = kStages * kStageBytes + kStagingBytes + 1024;
     static constexpr int kAccBufs = kWide ? 1 : 2;
     static constexpr int kSfCol = kAccBufs * BN;             // scale columns start behind the accumulator(s)
-    static constexpr int kSfSetCols = 8 + 8 * kSfqGroups;    // 8 activation + 8 per weight group
+    static constexpr int kSfCols = kFp8 ? 4 : 8;             // scale columns per group: 4 per atom
+    static constexpr int kSfSetCols = kSfCols * (1 + kSfqGroups);
     static constexpr int kChunks = (BN + kChunkCols - 1) / kChunkCols;   // 7, 7 and a 16-column one, or 9
     static constexpr int kLastCols = BN - (kChunks - 1) * kChunkCols;    // 32 or 16
     static constexpr int kSlotUnits = kChunks * 8 * 128;     // float4 per workspace slot (128 rows)
@@ -200,10 +207,10 @@ __device__ __forceinline__ uint64_t desc64(uint32_t hi, uint32_t lo) { return (s
 // 288-column tile two (256 columns, then the 32 columns of the third weight group into accumulator
 // columns 256 ..).  The copies and the MMAs are issued by one thread, so tensor memory sees them in order
 // and one set of scale columns is enough.  `rem` = reduction elements this stage still covers.
-template <int BN, int Q>
+template <int BN, bool kFp8, int Q>
 __device__ __forceinline__ void issue_stage(uint32_t lo_base, uint32_t d_tmem, uint32_t sf_t, int rem,
                                             uint32_t accumulate, uint32_t empty_bar0) {
-    using C = PCfg<BN>;
+    using C = PCfg<BN, kFp8>;
     constexpr int kStageBytes = C::kStageBytes, kQTile = C::kQTile, G = C::kSfqGroups;
     constexpr uint32_t so = (Q * kStageBytes) >> 4;  // stage offset in 16-byte units
     constexpr uint32_t sfo = so + ((kPTile + kQTile) >> 4);
@@ -214,7 +221,29 @@ __device__ __forceinline__ void issue_stage(uint32_t lo_base, uint32_t d_tmem, u
     constexpr uint32_t jdesc0 = (1u << 7) | (1u << 10) | (((N2 > 0 ? N2 : 16) >> 3) << 17) | (1u << 23) | ((256u >> 4) << 24);
     constexpr uint32_t jdesc2 = jdesc0 | (2u << 4) | (2u << 29);
     const uint32_t plo = lo_base + so, qlo = lo_base + so + (kPTile >> 4), slo = lo_base + sfo;
-    const uint32_t sfp_t = sf_t, sfq_t = sf_t + 8;
+    constexpr int kSfp = C::kSfp;
+    const uint32_t sfp_t = sf_t, sfq_t = sf_t + C::kSfCols;
+    // the second instruction of a step reads the CTA's weight rows from row N1 / 2 on and the scale columns of
+    // the second half's groups
+    constexpr uint32_t q2 = ((N1 / 2) * 128) >> 4, s2 = 4 * C::kHalfGroups;
+    if constexpr (kFp8) {
+        // E4M3 x E4M3 (format 0); step j takes byte j of the scale words
+        constexpr uint32_t id = ((N1 >> 3) << 17) | (1u << 23) | ((256u >> 4) << 24);
+        constexpr uint32_t jd = (((N2 > 0 ? N2 : 16) >> 3) << 17) | (1u << 23) | ((256u >> 4) << 24);
+        tc_copy_sf_atom_pair(sfp_t, desc64(kHiPlain, slo));
+#pragma unroll
+        for (int g = 0; g < G; ++g) tc_copy_sf_atom_pair(sfq_t + 4 * g, desc64(kHiPlain, slo + ((kSfp + g * C::kSfGroup) >> 4)));
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (rem > 32 * j) {
+                const uint32_t sid = (static_cast<uint32_t>(j) << 4) | (static_cast<uint32_t>(j) << 29), acc = j ? 1u : accumulate;
+                tc_mma_mxf8_pair(d_tmem, desc64(kHiSw128, plo + 2 * j), desc64(kHiSw128, qlo + 2 * j), id | sid, sfp_t, sfq_t, acc);
+                if (N2 > 0) tc_mma_mxf8_pair(d_tmem + N1, desc64(kHiSw128, plo + 2 * j), desc64(kHiSw128, qlo + q2 + 2 * j), jd | sid, sfp_t, sfq_t + s2, acc);
+            }
+        }
+        tc_commit_pair(empty_bar0 + Q * 8, 3);
+        return;
+    }
     tc_copy_sf_atom_pair(sf_t, desc64(kHiPlain, slo));
 #pragma unroll
     for (int g = 0; g < G; ++g)
@@ -225,9 +254,6 @@ __device__ __forceinline__ void issue_stage(uint32_t lo_base, uint32_t d_tmem, u
         for (int g = 0; g < G; ++g)
             tc_copy_sf_atom_pair(sfq_t + 4 * G + 4 * g, desc64(kHiPlain, slo + ((kSfp + g * kSfGroupBytes + 512) >> 4)));
     }
-    // the second instruction of a step reads the CTA's weight rows from row N1 / 2 on and the scale columns of
-    // the second half's groups
-    constexpr uint32_t q2 = ((N1 / 2) * 128) >> 4, s2 = 4 * C::kHalfGroups;
     tc_mma_mxf4_pair(d_tmem, desc64(kHiSw128, plo), desc64(kHiSw128, qlo), idesc0, sfp_t, sfq_t, accumulate);
     if (N2 > 0) tc_mma_mxf4_pair(d_tmem + N1, desc64(kHiSw128, plo), desc64(kHiSw128, qlo + q2), jdesc0, sfp_t, sfq_t + s2, accumulate);
     if (rem > 64) {
@@ -245,12 +271,13 @@ __device__ __forceinline__ void issue_stage(uint32_t lo_base, uint32_t d_tmem, u
     tc_commit_pair(empty_bar0 + Q * 8, 3);
 }
 
-template <int BN, bool kGated = false>
+template <int BN, bool kGated = false, bool kFp8 = false>
 __global__ void __launch_bounds__(kThreads, 1)
 prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_constant__ CUtensorMap tm_w,
                     const __grid_constant__ CUtensorMap tm_sfa, const __grid_constant__ CUtensorMap tm_sfw,
                     const __grid_constant__ CUtensorMap tm_y, const PrefillParams p) {
-    using C = PCfg<BN>;
+    using C = PCfg<BN, kFp8>;
+    constexpr int kSfp = C::kSfp;
     constexpr int kHalfN = C::kHalfN, kQTile = C::kQTile, kStageBytes = C::kStageBytes, kSfCol = C::kSfCol;
     constexpr int kChunks = C::kChunks, kLastCols = C::kLastCols;
     extern __shared__ uint8_t smem_raw[];
@@ -265,8 +292,9 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_con
     const uint32_t staging_base = smem_base + kStages * kStageBytes;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();          // 0 = leader of the pair
-    const StagePlan plan(p.K, p.k_tail);
-    const int S = plan.S, S1 = plan.S1;
+    // reduction stages: the K main columns, then the k tail columns (MXFP4 only; the second format has no tail)
+    const int S1 = (p.K + C::kStageElems - 1) / C::kStageElems;
+    const int S = S1 + (kFp8 ? 0 : (p.k_tail + C::kStageElems - 1) / C::kStageElems);
     const int G = gridDim.x >> 1, g = blockIdx.x >> 1;   // pairs
     const uint32_t W = static_cast<uint32_t>(p.sk_tiles) * S;   // stream-K units, shared out over all pairs
     const SkPlan plan_sk{p.sk_aligned, p.sk_base, p.sk_extra, S, G, W};
@@ -342,7 +370,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_con
             } else {
                 tma_load_2d_pair(sb + kPTile, &tm_w, xw, ni * BN + static_cast<int>(rank) * kHalfN, full);
             }
-            tma_load_2d_pair(sb + kPTile + kQTile + kSfp, &tm_sfw, 0, ni * 4 * C::kSfqGroups + s * p.w_groups * 4, full);
+            tma_load_2d_pair(sb + kPTile + kQTile + kSfp, &tm_sfw, 0, (ni * C::kSfqGroups + s * p.w_groups) * C::kSfRows, full);
         };
         int pre = 0;
         {
@@ -362,13 +390,13 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_con
         }
         while (ok && r.next(sg)) {
             const int mi = sg.tile % p.m_tiles, ni = sg.tile / p.m_tiles;
-            // scale bytes: rows of 256 bytes, 4 per 128-row group
-            const int sfa_row0 = (mi * 2 + static_cast<int>(rank)) * 4, sfa_stride = p.act_groups * 4;
+            // scale bytes: rows of 256 bytes, 4 (2) per 128-row group
+            const int sfa_row0 = (mi * 2 + static_cast<int>(rank)) * C::kSfRows, sfa_stride = p.act_groups * C::kSfRows;
             for (int s = sg.s0; s < sg.s1; ++s, ++it) {
                 if (!mbar_wait(smem_u32(&bar_empty[st]), ph ^ 1, abort_flag, p.wait_limit)) { ok = false; break; }
                 if (trace && lane == 0 && it < 64) trace[it] = clock64();
                 if (elect_one()) {
-                    if (rank == 0) mbar_arrive_expect_tx(smem_u32(&bar_full[st]), 2 * kStageBytes);
+                    if (rank == 0) mbar_arrive_expect_tx(smem_u32(&bar_full[st]), 2 * C::kTxBytes);
                     const uint32_t full = leader_full0 + st * 8;
                     const int xa = s < S1 ? s * 128 : (p.K - p.k_tail) / 2 + (s - S1) * 128;
                     const uint32_t sb = smem_base + st * kStageBytes;
@@ -408,18 +436,18 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_con
                 for (int s = sg.s0; s < sg.s1; ++s, ++it) {
                     if (!ready && !mbar_wait(smem_u32(&bar_full[st]), ph, abort_flag, p.wait_limit)) { ok = false; break; }
                     if (trace && lane == 0 && it < 64) trace[64 + it] = clock64();
-                    const int rem = s < S1 ? p.K - s * kStageK : p.k_tail - (s - S1) * kStageK;
+                    const int rem = s < S1 ? p.K - s * C::kStageElems : p.k_tail - (s - S1) * C::kStageElems;
                     const int nst = st + 1 == kStages ? 0 : st + 1;
                     const uint32_t nph = nst == 0 ? ph ^ 1 : ph;
                     ready = mbar_test_wait(smem_u32(&bar_full[nst]), nph);
                     if (leader) {
                         const uint32_t eb = smem_u32(&bar_empty[0]);
                         switch (st) {
-                            case 0: issue_stage<BN, 0>(lo_base, d_tmem, sf_t, rem, accumulate, eb); break;
-                            case 1: issue_stage<BN, 1>(lo_base, d_tmem, sf_t, rem, accumulate, eb); break;
-                            case 2: issue_stage<BN, 2>(lo_base, d_tmem, sf_t, rem, accumulate, eb); break;
-                            case 3: issue_stage<BN, 3>(lo_base, d_tmem, sf_t, rem, accumulate, eb); break;
-                            default: issue_stage<BN, 4>(lo_base, d_tmem, sf_t, rem, accumulate, eb); break;
+                            case 0: issue_stage<BN, kFp8, 0>(lo_base, d_tmem, sf_t, rem, accumulate, eb); break;
+                            case 1: issue_stage<BN, kFp8, 1>(lo_base, d_tmem, sf_t, rem, accumulate, eb); break;
+                            case 2: issue_stage<BN, kFp8, 2>(lo_base, d_tmem, sf_t, rem, accumulate, eb); break;
+                            case 3: issue_stage<BN, kFp8, 3>(lo_base, d_tmem, sf_t, rem, accumulate, eb); break;
+                            default: issue_stage<BN, kFp8, 4>(lo_base, d_tmem, sf_t, rem, accumulate, eb); break;
                         }
                     }
                     accumulate = 1;
@@ -763,12 +791,12 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_con
     if (threadIdx.x == 0 && abort_flag_s) atomicExch(p.status, static_cast<int>(PRQ_ERR_TIMEOUT));
 }
 
-template <int BN, bool kGated = false>
+template <int BN, bool kGated = false, bool kFp8 = false>
 int max_clusters_bn() {
-    constexpr int kSmemBytes = PCfg<BN>::kSmemBytes;
+    constexpr int kSmemBytes = PCfg<BN, kFp8>::kSmemBytes;
     static int cached = -1;
     if (cached >= 0) return cached;
-    if (cudaFuncSetAttribute(prefill_pair_kernel<BN, kGated>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess) return 0;
+    if (cudaFuncSetAttribute(prefill_pair_kernel<BN, kGated, kFp8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2);
     cfg.blockDim = dim3(kThreads);
@@ -781,19 +809,19 @@ int max_clusters_bn() {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, prefill_pair_kernel<BN, kGated>, &cfg) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveClusters(&n, prefill_pair_kernel<BN, kGated, kFp8>, &cfg) != cudaSuccess) return 0;
     cached = n;
     return n;
 }
 
-template <int BN, bool kGated = false>
+template <int BN, bool kGated = false, bool kFp8 = false>
 cudaError_t launch_bn(const CUtensorMap& tm_act, const CUtensorMap& tm_w, const CUtensorMap& tm_sfa,
                       const CUtensorMap& tm_sfw, const CUtensorMap& tm_y, const PrefillParams& p,
                       int pairs, cudaStream_t stream) {
-    constexpr int kSmemBytes = PCfg<BN>::kSmemBytes;
+    constexpr int kSmemBytes = PCfg<BN, kFp8>::kSmemBytes;
     static bool configured = false;
     if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(prefill_pair_kernel<BN, kGated>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+        cudaError_t e = cudaFuncSetAttribute(prefill_pair_kernel<BN, kGated, kFp8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
         if (e != cudaSuccess) return e;
         configured = true;
     }
@@ -811,10 +839,27 @@ cudaError_t launch_bn(const CUtensorMap& tm_act, const CUtensorMap& tm_w, const 
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, prefill_pair_kernel<BN, kGated>, tm_act, tm_w, tm_sfa, tm_sfw, tm_y, p);
+    return cudaLaunchKernelEx(&cfg, prefill_pair_kernel<BN, kGated, kFp8>, tm_act, tm_w, tm_sfa, tm_sfw, tm_y, p);
 }
 
 }  // namespace
+
+// The second format: whole tiles only, wave after wave (there is no workspace for pieces); one tile per pair at 288 columns.
+cudaError_t launch_prefill_pair_fp8(int bn, const CUtensorMap& tm_act, const CUtensorMap& tm_w, const CUtensorMap& tm_sfa,
+                                    const CUtensorMap& tm_sfw, const CUtensorMap& tm_y, const PrefillParams& p, int pairs,
+                                    cudaStream_t stream) {
+    if (p.sk_tiles != 0 || p.k_tail != 0 || (bn == kPrefillTileOneWave && p.whole_tiles > 1)) return cudaErrorInvalidValue;
+    if (bn == kPrefillTileOneWave) return launch_bn<kPrefillTileOneWave, false, true>(tm_act, tm_w, tm_sfa, tm_sfw, tm_y, p, pairs, stream);
+    if (bn == kPrefillTileWide) return launch_bn<kPrefillTileWide, false, true>(tm_act, tm_w, tm_sfa, tm_sfw, tm_y, p, pairs, stream);
+    if (bn == kPrefillTileN) return launch_bn<kPrefillTileN, false, true>(tm_act, tm_w, tm_sfa, tm_sfw, tm_y, p, pairs, stream);
+    return cudaErrorInvalidValue;
+}
+
+int prefill_pair_max_clusters_fp8() {
+    const int a = max_clusters_bn<kPrefillTileN, false, true>(), b = max_clusters_bn<kPrefillTileWide, false, true>();
+    const int c = max_clusters_bn<kPrefillTileOneWave, false, true>();
+    return a < b ? (a < c ? a : c) : (b < c ? b : c);
+}
 
 int prefill_pair_max_clusters(int bn) {
     if (bn == kPrefillTileGated) return max_clusters_bn<kPrefillTileGated, true>();

@@ -1,8 +1,11 @@
 // Internal declarations shared by the translation units of libprq.
 #pragma once
+#include <algorithm>
 #include <cstdlib>
 #include <cstddef>
 #include <cstdint>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include <cuda.h>
@@ -42,6 +45,25 @@ struct StagePlan {
 // 4 bytes per (r / 32), one per block.  This is the order the tensor-memory scale copy consumes.
 __host__ __device__ inline int sf_offset_in_group(int r, int blk_in_stage) {
     return (blk_in_stage >> 2) * 512 + (r & 31) * 16 + (r >> 5) * 4 + (blk_in_stage & 3);
+}
+
+// body(lo, hi) over [0, n) on the host's threads.  A thread that cannot be started leaves its share to the caller.
+template <class F>
+void parallel_for(long n, F&& body) {
+    const unsigned hw = std::thread::hardware_concurrency();
+    const long nt = std::min<long>(std::max(1u, std::min(hw, 64u)), std::max<long>(1, n));
+    std::vector<std::thread> th;
+    th.reserve(nt);
+    for (long t = 1; t < nt; ++t) {
+        const long lo = n * t / nt, hi = n * (t + 1) / nt;
+        try {
+            th.emplace_back([=, &body] { body(lo, hi); });
+        } catch (const std::system_error&) {
+            body(lo, hi);
+        }
+    }
+    body(0, n / nt);
+    for (auto& x : th) x.join();
 }
 
 struct PrepResult {
@@ -84,7 +106,7 @@ cudaError_t launch_quant_perm(const uint16_t* W, const float* s, const int32_t* 
                               uint8_t* codes, uint8_t* scales, int sm_count, cudaStream_t stream);
 // Row-major scale bytes -> the layouts of the GEMMs (padding becomes zero).
 struct SfLayout { uint8_t* dst; size_t bytes; int tile_rows, groups_per_tile, groups; };   // groups per stage and expert
-struct SfLayouts { int n, n_experts; SfLayout l[5]; };
+struct SfLayouts { int n, n_experts, group_bytes; SfLayout l[5]; };   // group_bytes: 1024, second format 512
 cudaError_t launch_sf_layout(const uint8_t* scales, int N, int K, int k_tail, const SfLayouts& t, int sm_count, cudaStream_t stream);
 
 }  // namespace prq
@@ -111,8 +133,8 @@ struct prq_weights {
     uint8_t* d_sf_alt[4] = {nullptr, nullptr, nullptr, nullptr};
     int w_groups_alt[4] = {0, 0, 0, 0};
     bool gated = false;
-    // Second format (prq_prep_opts::format = PRQ_FMT_MXFP8): d_codes holds N x K bytes of E4M3 codes, d_sf the scale
-    // bytes as [128-element stage][128-row group][512]; k_tail is 0, perm the identity; none of the MXFP4 tilings exist.
+    // Second format (prq_prep_opts::format = PRQ_FMT_MXFP8): d_codes holds N x K bytes of E4M3 codes, d_sf and d_sf_alt the
+    // scale bytes as [128-element stage][128-row group][512]; k_tail is 0, perm the identity.
     int format = 0;
     CUtensorMap tm_w_fp8;
     float* d_inv_s = nullptr;        // K: the activation side's factors (original = permuted order)

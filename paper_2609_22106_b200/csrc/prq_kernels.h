@@ -184,8 +184,14 @@ struct PrefillParams {
 cudaError_t launch_prefill_pair(int bn, const CUtensorMap& tm_act, const CUtensorMap& tm_w,
                                 const CUtensorMap& tm_sfa, const CUtensorMap& tm_sfw, const CUtensorMap& tm_y,
                                 const PrefillParams& p, int pairs, cudaStream_t stream);
+// The same kernel for the second format (MXFP8): `bn` = 224, 240 or 288 columns, whole tiles only; codes are K-byte rows,
+// `tm_sfa` / `tm_sfw` have boxes of 2 rows per 128-row group.
+cudaError_t launch_prefill_pair_fp8(int bn, const CUtensorMap& tm_act, const CUtensorMap& tm_w, const CUtensorMap& tm_sfa,
+                                    const CUtensorMap& tm_sfw, const CUtensorMap& tm_y, const PrefillParams& p, int pairs,
+                                    cudaStream_t stream);
 // How many pairs of the pair kernel can be resident at once on the current device.
 int prefill_pair_max_clusters(int bn);
+int prefill_pair_max_clusters_fp8();
 
 // Benchmark utility: `grid` CTAs each issuing n_mma block-scaled FP4 MMAs (128 x 256 x 64) from shared memory.
 cudaError_t launch_mxf4_peak_probe(int n_mma, int grid, int* status, cudaStream_t stream);

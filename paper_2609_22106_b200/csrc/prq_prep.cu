@@ -113,23 +113,6 @@ inline uint8_t quantize_block_search(const float* v, uint8_t* codes) {
     return best;
 }
 
-template <class F>
-void parallel_for(long n, F&& body) {
-    unsigned hw = std::thread::hardware_concurrency();
-    long nt = std::max(1u, std::min(hw ? hw : 1u, 64u));
-    nt = std::min<long>(nt, std::max<long>(1, n));
-    if (nt <= 1) {
-        body(0, n);
-        return;
-    }
-    std::vector<std::thread> th;
-    for (long t = 0; t < nt; ++t) {
-        long lo = n * t / nt, hi = n * (t + 1) / nt;
-        th.emplace_back([=, &body] { body(lo, hi); });
-    }
-    for (auto& x : th) x.join();
-}
-
 double scale_power(double a, float alpha) {
     if (alpha == 0.f) return 1.0;
     if (alpha == 1.f) return a;

@@ -254,27 +254,28 @@ __global__ void __launch_bounds__(kPermThreads) quant_perm_kernel(const uint16_t
 }
 
 // ---------------------------------------------------------------------------------------------- scale-byte layouts
-// Every layout is [expert][stage][128-row group][1024 bytes]; a weight tile of `tile_rows` rows has `groups_per_tile`
-// groups of its own, the last one partly empty.  One thread per word: the four blocks of one (row, atom).  Words that
+// Every layout is [expert][stage][128-row group][1024 bytes] (second format: 512, four blocks per stage); a weight tile of
+// `tile_rows` rows has `groups_per_tile` groups of its own, the last one partly empty.  One thread per word: the four blocks of one (row, atom).  Words that
 // hold no row or block are zero bytes (2^-127, finite).
 __global__ void __launch_bounds__(256) sf_layout_kernel(const uint8_t* __restrict__ scales, int N, int K, int k_tail, SfLayouts t) {
     const SfLayout l = t.l[blockIdx.y];
-    const StagePlan plan(K, k_tail);
+    const int nb = t.group_bytes / 128;   // blocks per stage: 8 or 4
     const int nblk = K / kBlock, n_all = nblk + k_tail / kBlock;
+    const int S1 = (nblk + nb - 1) / nb, S = S1 + (k_tail / kBlock + nb - 1) / nb;
     for (size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < l.bytes / 4; i += static_cast<size_t>(gridDim.x) * blockDim.x) {
-        const int off = static_cast<int>(i & 255) * 4;
-        size_t g = i >> 8;
+        const int off = static_cast<int>(i % (t.group_bytes / 4)) * 4;
+        size_t g = i / (t.group_bytes / 4);
         uint32_t w = 0;
         const int group = static_cast<int>(g % l.groups);
         g /= l.groups;
-        const int stage = static_cast<int>(g % plan.S);
-        const size_t expert = g / plan.S;
+        const int stage = static_cast<int>(g % S);
+        const size_t expert = g / S;
         const int in_tile = (group % l.groups_per_tile) * kGroupRows + (off & 12) * 8 + ((off & 511) >> 4);
         const int n = group / l.groups_per_tile * l.tile_rows + in_tile;
         if (expert < static_cast<size_t>(t.n_experts) && in_tile < l.tile_rows && n < N) {
             const int bis = (off >> 9) * 4;
-            const int b = stage < plan.S1 ? stage * (kStageK / kBlock) + bis : nblk + (stage - plan.S1) * (kStageK / kBlock) + bis;
-            const int end = stage < plan.S1 ? nblk : n_all;
+            const int b = stage < S1 ? stage * nb + bis : nblk + (stage - S1) * nb + bis;
+            const int end = stage < S1 ? nblk : n_all;
             const uint8_t* p = scales + (expert * N + n) * n_all + b;
 #pragma unroll
             for (int j = 0; j < 4; ++j)

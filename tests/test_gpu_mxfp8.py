@@ -52,6 +52,22 @@ def test_mxfp8_layers(prq, oracle, shape):
     fp8_case(prq, oracle, N, K, M, 0.5, seed=N + M)
 
 
+@pytest.mark.parametrize("bn", [0, 224, 240, 288])
+@pytest.mark.parametrize("shape", [(8, 32, 1), (225, 128, 129), (241, 160, 256), (289, 992, 257), (577, 96, 700), (480, 2080, 512)])
+def test_mxfp8_every_tile_width(prq, oracle, monkeypatch, bn, shape):
+    """The tile-per-CTA kernel and the three widths of the CTA-pair kernel on the same layers: N and M just past a tile or
+    half a tile, reductions with 1 to 4 MMA steps in the last stage and more stages than the ring has slots."""
+    monkeypatch.setenv("PRQ_FP8_BN", str(bn))
+    N, K, M = shape
+    fp8_case(prq, oracle, N, K, M, 0.5, seed=5 * N + M)
+
+
+def test_mxfp8_several_waves_of_pairs(prq, oracle):
+    """As the rule chooses: three waves of pair tiles, the last one short, against sampled rows."""
+    rows = np.concatenate([np.arange(0, 2100, 97), np.arange(2040, 2100)])
+    fp8_case(prq, oracle, 4104, 96, 2100, 0.5, seed=9, rows=rows)
+
+
 def test_mxfp8_decision_boundaries_and_unit_scales(prq, oracle):
     rows = []
     for vals in ([448, 1, .5, -3, 2 ** -9, 296], [256, 17, 19, 272, 304], [500, 464, 462, -510], [512, 3, 1],
