@@ -340,26 +340,6 @@ struct ColsPlan {
 constexpr int kColsMaxStages = 8;
 constexpr size_t kColsSmem = 220 * 1024;   // shared memory of an SM that the rows in flight may take
 
-__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
-    uint64_t d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-// the largest magnitude of three
-__device__ __forceinline__ float max3_abs(float a, float b, float c) {
-    float d;
-    asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-__device__ __forceinline__ uint64_t pack_f32x2(uint32_t lo, uint32_t hi) {
-    uint64_t d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
-    return d;
-}
-__device__ __forceinline__ void unpack_f32x2(uint64_t a, float& lo, float& hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a));
-}
-
 // kCols: columns per lane, 8 or 16.  kRowsC: rows per slice, 1, 2 or 4.
 template <int kCols, int kRowsC, bool kGrouped, int kMaxT>
 __global__ void __launch_bounds__(kMaxT, 1)
