@@ -273,6 +273,10 @@ prq_status prq_quantize_act(const prq_weights *w, prq_act_mode mode, const void 
  * half of an output tile and two fp32 partial tiles per SM (about 34 MB on a B200).  Calls on different
  * streams that may overlap need separate workspaces. */
 size_t prq_linear_workspace_bytes(const prq_weights *w, int M);
+/* Leading bytes of such a workspace that must be zero before ONE prq_linear call on M tokens (0 where the call counts
+ * nothing).  For a caller that takes a fresh workspace for every call; one that keeps its workspace zero-fills all of it
+ * once, as above. */
+size_t prq_linear_workspace_clear_bytes(const prq_weights *w, int M);
 
 /* Eq. (3): y = [Q(x) | Q(x)_tail] [Q(W D P) | Q(R)]^T, one block-scaled FP4 GEMM over K + k with fp32
  * accumulation.  Reads activation columns [0, K) and then [K - k, K) again; no M x (K + k) buffer exists.

@@ -68,6 +68,8 @@ def lib():
         L.prq_quantize_act.argtypes = [vp, ci, vp, ci, ci, vp, vp, vp, vp, vp]
         L.prq_linear_workspace_bytes.argtypes = [vp, ci]
         L.prq_linear_workspace_bytes.restype = cs
+        L.prq_linear_workspace_clear_bytes.argtypes = [vp, ci]
+        L.prq_linear_workspace_clear_bytes.restype = cs
         L.prq_linear.argtypes = [vp, vp, vp, ci, vp, ci, ci, vp, cs, vp]
         L.prq_linear_static_scratch.argtypes = [vp, vp, vp, ci, vp, ci, ci, vp]
         L.prq_linear_fused.argtypes = [vp, ci, vp, ci, ci, vp, ci, ci, vp]
@@ -108,15 +110,26 @@ def _np_ptr(a: np.ndarray):
     return a.ctypes.data_as(ctypes.c_void_p)
 
 
+# A call on a few tokens takes the GPU less time than Python's part of it takes the host, so that part is kept short: the
+# current stream as a number (torch.cuda.current_stream() builds an object, 3.6 us of the 9 us that a call took), pointers as
+# numbers (ctypes converts them by the declared argument types).
+_raw_stream = None
+
+
 def _stream_ptr(stream=None):
+    global _raw_stream
+    if stream is not None:
+        return stream.cuda_stream
     import torch
 
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if _raw_stream is None:
+        get, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        _raw_stream = (lambda: get(device())) if get and device else (lambda: torch.cuda.current_stream().cuda_stream)
+    return _raw_stream() if torch.cuda.is_initialized() else torch.cuda.current_stream().cuda_stream
 
 
 def _dptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 class Weights:
@@ -319,7 +332,12 @@ def linear(w: Weights, codes, scales_sf, M: int, y_dtype: int = F32, workspace=N
     if out is None:
         out = torch.empty((M, w.N), dtype=torch.float32 if y_dtype == F32 else torch.bfloat16, device=codes.device)
     if workspace is None and M > 128:   # up to 128 tokens the kernel needs no scratch: nothing to allocate or clear
-        workspace = new_workspace(w, M, codes.device)
+        # a workspace for this call alone: only what this call counts on is cleared (the partial tiles behind the counters
+        # are written before they are read), not tens of megabytes
+        workspace = torch.empty(max(linear_workspace_bytes(w, M), 16), dtype=torch.uint8, device=codes.device)
+        clear = int(lib().prq_linear_workspace_clear_bytes(w.handle, M))
+        if clear:
+            workspace[:clear].zero_()
     _check(lib().prq_linear(w.handle, _dptr(codes), _dptr(scales_sf), M, _dptr(out), out.stride(0) if M else w.N,
                             y_dtype, _dptr(workspace), workspace.numel() if workspace is not None else 0,
                             _stream_ptr(stream)), "prq_linear")

@@ -1118,6 +1118,21 @@ size_t prq_linear_workspace_bytes(const prq_weights* w, int M) {
     return 0;  // decode: the split-K partial sums meet in distributed shared memory
 }
 
+static PairSchedule schedule_prefill(const prq_weights* w, int M, DeviceInfo* di) {
+    if (di->max_pairs == 0)
+        di->max_pairs = std::min(std::min(std::min(prefill_pair_max_clusters(kPrefillTileN), prefill_pair_max_clusters(kPrefillTileWide)),
+                                          prefill_pair_max_clusters(kPrefillTileOneWave)), di->num_sms / 2);
+    return choose_pair_schedule(M, w->N, w->plan.S, std::min(di->max_pairs, env_int("PRQ_GRID", 1 << 20)));
+}
+
+size_t prq_linear_workspace_clear_bytes(const prq_weights* w, int M) {
+    DeviceInfo* di;
+    if (!w || M <= 128 || w->format != PRQ_FMT_MXFP4 || device_info(w->device, &di) != PRQ_OK) return 0;
+    // the counters are touched only where a tile is cut into pieces
+    const PairSchedule ps = schedule_prefill(w, M, di);
+    return ps.sk > 0 && (ps.base > 1 || env_int("PRQ_SK_RANGES", 0)) ? prefill_flag_bytes(w, M) : 0;
+}
+
 static prq_status check_linear_common(const prq_weights* w, const void* codes, const void* scales_sf, void* y, int ldy,
                                       prq_dtype y_dtype) {
     if (!w || !codes || !scales_sf || !y) return PRQ_ERR_INVALID_ARG;
@@ -1209,10 +1224,7 @@ prq_status prq_linear(const prq_weights* w, const void* codes, const void* scale
         if (w->gated) return PRQ_ERR_INVALID_ARG;   // a gated-producer handle has the tiling of prq_linear_gated only
         PrefillParams q;
         std::memset(&q, 0, sizeof(q));
-        if (di->max_pairs == 0)
-            di->max_pairs = std::min(std::min(std::min(prefill_pair_max_clusters(kPrefillTileN), prefill_pair_max_clusters(kPrefillTileWide)),
-                                              prefill_pair_max_clusters(kPrefillTileOneWave)), di->num_sms / 2);
-        const PairSchedule ps = choose_pair_schedule(M, w->N, w->plan.S, std::min(di->max_pairs, env_int("PRQ_GRID", 1 << 20)));
+        const PairSchedule ps = schedule_prefill(w, M, di);
         const int pair_bn = ps.bn, variant = pair_bn == kPrefillTileOneWave ? 2 : pair_bn == kPrefillTileWide ? 1 : 0, pairs = ps.pairs;
         if (pairs < 1) return PRQ_ERR_CUDA;
         q.M = M; q.N = w->N; q.K = w->K; q.k_tail = w->k_tail;

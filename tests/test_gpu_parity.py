@@ -192,6 +192,22 @@ def test_prefill_stream_k_splits(prq, oracle, shape):
     layer_case(prq, oracle, N=N, K=K, M=M, k=k, alpha=0.5, mode=prq.ACT_IDENTITY, seed=M)
 
 
+@pytest.mark.parametrize("M,N,K,k", [(200, 256, 9728, 256), (129, 520, 4096, 128), (1500, 1024, 2560, 128), (300, 640, 512, 0)])
+def test_linear_without_a_workspace(prq, M, N, K, k):
+    """linear() with no workspace takes memory as it finds it and clears only the counters that the call uses: same bits
+    from memory full of ones as with a zero-filled workspace, tiles cut into pieces or not."""
+    W = synth.weights(90 + M, N, K)
+    w = prq.prepare_weights(W, np.full(K, 2.0, np.float32), 0.5, k)
+    x = to_dev_bf16(synth.HeavyTailChannels(91, K).rows(92 + M, M))
+    codes, _, sf = prq.quantize_act(w, x, prq.ACT_SCALE_PERM)
+    want = prq.linear(w, codes, sf, M, workspace=prq.new_workspace(w, M))
+    torch.full((prq.linear_workspace_bytes(w, M),), 255, dtype=torch.uint8, device="cuda")   # what the next allocation finds
+    for _ in range(2):
+        assert torch.equal(prq.linear(w, codes, sf, M), want)
+    assert prq.last_device_status() == 0
+    w.free()
+
+
 def test_k0_runs_the_same_kernels_as_plain_mxfp4(prq, oracle):
     """k = 0: the product is plain W4A4 MXFP4 of (x, W D); with alpha = 0 of (x, W) themselves."""
     L = synth.layer(93, 256, 1024, 200, T_cal=32)
