@@ -130,25 +130,25 @@ constexpr int kNumAlt = 4;
 // (the one-wave tile is tiled per 144-row half: its two MMAs per step take 144 columns each)
 constexpr int kAltTileRows[kNumAlt] = {kPrefillTileN, kPrefillTileWide, kPrefillTileOneWave / 2, kPrefillTileGated};
 constexpr int kAltGated = 3;
-bool alt_wanted(bool gated, int a) { return gated ? a == kAltGated : a != kAltGated; }
+constexpr int kAltWide = 1;
+bool alt_wanted(bool gated, int n_experts, int a) { return n_experts > 1 ? a == kAltWide : gated ? a == kAltGated : a != kAltGated; }
 
-// Weight-side tensor maps of a dense handle, encoded once at creation (cloning re-encodes: other addresses).
+// Weight-side tensor maps of a handle, encoded once at creation (cloning re-encodes: other addresses).
 prq_status build_weight_maps(prq_weights* w) {
     w->maps_ready = false;
-    if (w->n_experts != 1) return PRQ_OK;
-    const uint64_t Ka = static_cast<uint64_t>(w->K) + w->k_tail;
-    prq_status st = make_code_map(&w->tm_w_decode, w->d_codes, Ka / 2, w->N, 128);
+    const uint64_t Ka = static_cast<uint64_t>(w->K) + w->k_tail, E = w->n_experts;
+    prq_status st = make_code_map(&w->tm_w_decode, w->d_codes, Ka / 2, E * w->N, 128);
     for (int v = 0; v < kNumAlt; ++v) {   // 224-, 240- and 288-row tilings, or the 192-row one
-        if (!alt_wanted(w->gated, v)) continue;
+        if (!alt_wanted(w->gated, w->n_experts, v)) continue;
         const int rows = kAltTileRows[v], gpt = (rows + kGroupRows - 1) / kGroupRows;
         const bool one_wave = v == 2;   // a 288-row tile = two 144-row halves: boxes of 72 weight rows, four scale groups
         // each CTA of a pair loads half a tile (the 288-row tile: a quarter, twice)
-        if (st == PRQ_OK) st = make_code_map(&w->tm_w_pair[v], w->d_codes, Ka / 2, w->N, rows / 2);
+        if (st == PRQ_OK) st = make_code_map(&w->tm_w_pair[v], w->d_codes, Ka / 2, E * w->N, rows / 2);
         if (st == PRQ_OK && w->d_sf_alt[v])
             st = make_sf_map(&w->tm_sfw_pair[v], w->d_sf_alt[v],
-                             static_cast<uint64_t>(w->plan.S) * w->w_groups_alt[v] * kSfGroupBytes, 4 * gpt * (one_wave ? 2 : 1));
+                             E * w->plan.S * w->w_groups_alt[v] * kSfGroupBytes, 4 * gpt * (one_wave ? 2 : 1));
     }
-    if (st == PRQ_OK) w->maps_ready = true;
+    if (st == PRQ_OK && E == 1) w->maps_ready = true;   // (the dense calls refuse stacked experts)
     return st;
 }
 
@@ -462,6 +462,17 @@ static PrepOptions read_opts(const prq_prep_opts* opts) {
 
 static prq_status create_handle_fp8(const uint16_t* W, int N, int K, const float* act_amax, float alpha, int dev, prq_weights** out);
 
+// Where the handle's scale bytes go: the 128-row groups, and the tilings it keeps (alt_bytes[a] > 0).
+static SfLayouts sf_layouts(const prq_weights* w, const size_t (&alt_bytes)[kNumAlt]) {
+    SfLayouts t = {};
+    t.n_experts = w->n_experts;
+    t.group_bytes = w->format == PRQ_FMT_MXFP8 ? 512 : kSfGroupBytes;
+    t.l[t.n++] = SfLayout{w->d_sf, w->d_sf_bytes, kGroupRows, 1, w->w_groups};
+    for (int a = 0; a < kNumAlt; ++a)
+        if (alt_bytes[a]) t.l[t.n++] = SfLayout{w->d_sf_alt[a], alt_bytes[a], kAltTileRows[a], (kAltTileRows[a] + kGroupRows - 1) / kGroupRows, w->w_groups_alt[a]};
+    return t;
+}
+
 // A handle from a device copy of W: the kernels write every buffer of it where the GEMMs read it, in one allocation, and
 // only the K-sized arrays pass through the host (scales, column errors, permutation).  Laying the scale bytes out on the
 // host, keeping host copies of the codes and allocating every buffer by itself took 13 - 20 ms at 2560 x 9728, most of it page
@@ -485,10 +496,10 @@ static prq_status fill_handle_device(prq_weights* w, const uint16_t* W, const fl
     w->d_sf_bytes = (E * S * w->w_groups + 4) * kSfGroupBytes;
     const size_t o_codes = take(w->d_codes_bytes), o_sf = take(w->d_sf_bytes);
     size_t o_alt[kNumAlt] = {}, alt_bytes[kNumAlt] = {};
-    for (int a = 0; a < kNumAlt && E == 1; ++a) {
-        if (!alt_wanted(w->gated, a)) continue;
+    for (int a = 0; a < kNumAlt; ++a) {
+        if (!alt_wanted(w->gated, w->n_experts, a)) continue;
         w->w_groups_alt[a] = ((N + kAltTileRows[a] - 1) / kAltTileRows[a]) * ((kAltTileRows[a] + kGroupRows - 1) / kGroupRows);
-        alt_bytes[a] = (S * w->w_groups_alt[a] + 4) * kSfGroupBytes;
+        alt_bytes[a] = (E * S * w->w_groups_alt[a] + 4) * kSfGroupBytes;
         o_alt[a] = take(alt_bytes[a]);
     }
     const size_t o_perm = take(2 * sizeof(float) * EK);        // the permutation and, right behind it, 1 / s in its order
@@ -523,12 +534,7 @@ static prq_status fill_handle_device(prq_weights* w, const uint16_t* W, const fl
     std::memcpy(both.data(), w->h_perm.data(), sizeof(int32_t) * EK);
     ok = cudaMemcpyAsync(w->d_perm, both.data(), 2 * sizeof(float) * EK, cudaMemcpyHostToDevice, stream) == cudaSuccess;
     ok = ok && launch_quant_perm(W, d_s, w->d_perm, w->n_experts, N, K, k_tail, scale_search, w->d_codes, w->d_scales_row, num_sms, stream) == cudaSuccess;
-    SfLayouts t = {};
-    t.n_experts = w->n_experts; t.group_bytes = kSfGroupBytes;
-    t.l[t.n++] = SfLayout{w->d_sf, w->d_sf_bytes, kGroupRows, 1, w->w_groups};
-    for (int a = 0; a < kNumAlt; ++a)
-        if (alt_bytes[a]) t.l[t.n++] = SfLayout{w->d_sf_alt[a], alt_bytes[a], kAltTileRows[a], (kAltTileRows[a] + kGroupRows - 1) / kGroupRows, w->w_groups_alt[a]};
-    ok = ok && launch_sf_layout(w->d_scales_row, N, K, k_tail, t, num_sms, stream) == cudaSuccess;
+    ok = ok && launch_sf_layout(w->d_scales_row, N, K, k_tail, sf_layouts(w, alt_bytes), num_sms, stream) == cudaSuccess;
     if (ok && build_weight_maps(w) != PRQ_OK) ok = false;   // beside the kernels
     ok = cudaStreamSynchronize(stream) == cudaSuccess && ok;
     return ok ? PRQ_OK : PRQ_ERR_CUDA;
@@ -589,16 +595,15 @@ static prq_status create_handle(const uint16_t* W, bool w_on_device, prq_stream_
         w->h_s.resize(E * K);
         w->h_inv_s.resize(E * K);
         w->h_col_err.resize(E * K);
-        const int S = w->plan.S, S1 = w->plan.S1, nb = kStageK / kBlock;
+        const size_t S = w->plan.S;
         // scale bytes in stage order, padded by a few groups so that a tile's bulk copy never runs off the end
         w->d_sf_bytes = (E * S * w->w_groups + 4) * kSfGroupBytes;
-        std::vector<uint8_t> sf(w->d_sf_bytes, 0);
         std::vector<float> inv_s_perm(E * K);
-        std::vector<uint8_t> sf_alt[kNumAlt];
-        for (int a = 0; a < kNumAlt && E == 1; ++a) {
-            if (!alt_wanted(gated, a)) continue;
+        size_t alt_bytes[kNumAlt] = {};
+        for (int a = 0; a < kNumAlt; ++a) {
+            if (!alt_wanted(gated, n_experts, a)) continue;
             w->w_groups_alt[a] = ((N + kAltTileRows[a] - 1) / kAltTileRows[a]) * ((kAltTileRows[a] + kGroupRows - 1) / kGroupRows);
-            sf_alt[a].assign((static_cast<size_t>(S) * w->w_groups_alt[a] + 4) * kSfGroupBytes, 0);
+            alt_bytes[a] = (E * S * w->w_groups_alt[a] + 4) * kSfGroupBytes;
         }
         PrepResult r;
         for (size_t e = 0; e < E; ++e) {
@@ -611,45 +616,26 @@ static prq_status create_handle(const uint16_t* W, bool w_on_device, prq_stream_
             std::memcpy(&w->h_inv_s[e * K], r.inv_s.data(), sizeof(float) * K);
             std::memcpy(&w->h_col_err[e * K], r.col_err.data(), sizeof(double) * K);
             for (int j = 0; j < K; ++j) inv_s_perm[e * K + j] = r.inv_s[r.perm[j]];
-            const int nblk_main = K / kBlock, nblk = static_cast<int>(Ka / kBlock);
-            for (int n = 0; n < N; ++n) {
-                const uint8_t* srow = &r.scales[static_cast<size_t>(n) * nblk];
-                const int g = n / kGroupRows, rr = n % kGroupRows;
-                for (int b = 0; b < nblk; ++b) {
-                    const int stage = b < nblk_main ? b / nb : S1 + (b - nblk_main) / nb;
-                    const int bis = b < nblk_main ? b % nb : (b - nblk_main) % nb;
-                    sf[((e * S + stage) * w->w_groups + g) * kSfGroupBytes + sf_offset_in_group(rr, bis)] = srow[b];
-                    for (int a = 0; a < kNumAlt && E == 1; ++a) {
-                        if (!alt_wanted(gated, a)) continue;
-                        const int tile_rows = kAltTileRows[a], gpt = (tile_rows + kGroupRows - 1) / kGroupRows;
-                        const int ga = (n / tile_rows) * gpt + (n % tile_rows) / kGroupRows;
-                        sf_alt[a][(static_cast<size_t>(stage) * w->w_groups_alt[a] + ga) * kSfGroupBytes +
-                                  sf_offset_in_group((n % tile_rows) % kGroupRows, bis)] = srow[b];
-                    }
-                }
-            }
         }
         w->d_codes_bytes = w->h_codes.size() + 256;
-        if (cudaMalloc(&w->d_codes, w->d_codes_bytes) != cudaSuccess || cudaMalloc(&w->d_sf, w->d_sf_bytes) != cudaSuccess ||
-            cudaMalloc(&w->d_perm, sizeof(int32_t) * E * K) != cudaSuccess ||
-            cudaMalloc(&w->d_inv_s_perm, sizeof(float) * E * K) != cudaSuccess) {
+        bool mem = cudaMalloc(&w->d_codes, w->d_codes_bytes) == cudaSuccess && cudaMalloc(&w->d_sf, w->d_sf_bytes) == cudaSuccess &&
+                   cudaMalloc(&w->d_perm, sizeof(int32_t) * E * K) == cudaSuccess &&
+                   cudaMalloc(&w->d_inv_s_perm, sizeof(float) * E * K) == cudaSuccess && cudaMalloc(&w->d_scales_row, w->h_scales.size()) == cudaSuccess;
+        for (int a = 0; a < kNumAlt && mem; ++a)
+            if (alt_bytes[a]) mem = cudaMalloc(&w->d_sf_alt[a], alt_bytes[a]) == cudaSuccess;
+        if (!mem) {
             cudaGetLastError();
             prq_weights_free(w);
             return PRQ_ERR_OOM;
         }
         bool ok = cudaMemcpy(w->d_codes, w->h_codes.data(), w->h_codes.size(), cudaMemcpyHostToDevice) == cudaSuccess;
-        ok = ok && cudaMemcpy(w->d_sf, sf.data(), sf.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+        ok = ok && cudaMemcpy(w->d_scales_row, w->h_scales.data(), w->h_scales.size(), cudaMemcpyHostToDevice) == cudaSuccess;
         ok = ok && cudaMemcpy(w->d_perm, w->h_perm.data(), sizeof(int32_t) * E * K, cudaMemcpyHostToDevice) == cudaSuccess;
         ok = ok && cudaMemcpy(w->d_inv_s_perm, inv_s_perm.data(), sizeof(float) * E * K, cudaMemcpyHostToDevice) == cudaSuccess;
-        for (int a = 0; a < kNumAlt && E == 1 && ok; ++a) {
-            if (!alt_wanted(gated, a)) continue;
-            if (cudaMalloc(&w->d_sf_alt[a], sf_alt[a].size()) != cudaSuccess) {
-                cudaGetLastError();
-                prq_weights_free(w);
-                return PRQ_ERR_OOM;
-            }
-            ok = cudaMemcpy(w->d_sf_alt[a], sf_alt[a].data(), sf_alt[a].size(), cudaMemcpyHostToDevice) == cudaSuccess;
-        }
+        ok = ok && launch_sf_layout(w->d_scales_row, N, K, k_tail, sf_layouts(w, alt_bytes), di->num_sms, nullptr) == cudaSuccess;
+        ok = ok && cudaStreamSynchronize(nullptr) == cudaSuccess;
+        cudaFree(w->d_scales_row);   // the canonical bytes of a host preparation stay on the host
+        w->d_scales_row = nullptr;
         if (!ok) { prq_weights_free(w); return PRQ_ERR_CUDA; }
         if (build_weight_maps(w) != PRQ_OK) { prq_weights_free(w); return PRQ_ERR_CUDA; }
     } catch (const std::bad_alloc&) {
@@ -682,7 +668,7 @@ static prq_status create_handle_fp8(const uint16_t* W, int N, int K, const float
         bool mem = cudaMalloc(&w->d_codes, w->d_codes_bytes) == cudaSuccess && cudaMalloc(&w->d_sf, w->d_sf_bytes) == cudaSuccess &&
                    cudaMalloc(&w->d_inv_s, sizeof(float) * K) == cudaSuccess && cudaMalloc(&w->d_scales_row, w->h_scales.size()) == cudaSuccess;
         for (int a = 0; a < kNumAlt && mem; ++a) {
-            if (!alt_wanted(false, a)) continue;
+            if (!alt_wanted(false, 1, a)) continue;
             w->w_groups_alt[a] = ((N + kAltTileRows[a] - 1) / kAltTileRows[a]) * ((kAltTileRows[a] + kGroupRows - 1) / kGroupRows);
             alt_bytes[a] = (static_cast<size_t>(S8) * w->w_groups_alt[a] + 4) * 512;
             mem = cudaMalloc(&w->d_sf_alt[a], alt_bytes[a]) == cudaSuccess;
@@ -693,17 +679,12 @@ static prq_status create_handle_fp8(const uint16_t* W, int N, int K, const float
             return PRQ_ERR_OOM;
         }
         // the tile-per-CTA kernel's layout and the three tilings of the pair kernel, from one upload of the row-major bytes
-        SfLayouts t = {};
-        t.n_experts = 1; t.group_bytes = 512;
-        t.l[t.n++] = SfLayout{w->d_sf, w->d_sf_bytes, kGroupRows, 1, w->w_groups};
-        for (int a = 0; a < kNumAlt; ++a)
-            if (alt_bytes[a]) t.l[t.n++] = SfLayout{w->d_sf_alt[a], alt_bytes[a], kAltTileRows[a], (kAltTileRows[a] + kGroupRows - 1) / kGroupRows, w->w_groups_alt[a]};
         DeviceInfo* di;
         bool ok = device_info(dev, &di) == PRQ_OK;
         ok = ok && cudaMemcpy(w->d_codes, w->h_codes.data(), w->h_codes.size(), cudaMemcpyHostToDevice) == cudaSuccess;
         ok = ok && cudaMemcpy(w->d_scales_row, w->h_scales.data(), w->h_scales.size(), cudaMemcpyHostToDevice) == cudaSuccess;
         ok = ok && cudaMemcpy(w->d_inv_s, w->h_inv_s.data(), sizeof(float) * K, cudaMemcpyHostToDevice) == cudaSuccess;
-        ok = ok && launch_sf_layout(w->d_scales_row, N, K, 0, t, di->num_sms, nullptr) == cudaSuccess;
+        ok = ok && launch_sf_layout(w->d_scales_row, N, K, 0, sf_layouts(w, alt_bytes), di->num_sms, nullptr) == cudaSuccess;
         ok = ok && cudaStreamSynchronize(nullptr) == cudaSuccess;
         cudaFree(w->d_scales_row);   // the canonical bytes of a host preparation stay on the host
         w->d_scales_row = nullptr;
@@ -908,7 +889,7 @@ prq_status prq_weights_clone(const prq_weights* w, prq_weights** out) {
         for (int a = 0; a < kNumAlt; ++a) {
             c->w_groups_alt[a] = w->w_groups_alt[a];
             if (w->d_sf_alt[a])
-                dup(&c->d_sf_alt[a], w->d_sf_alt[a], (static_cast<size_t>(w->plan.S) * w->w_groups_alt[a] + 4) * kSfGroupBytes);
+                dup(&c->d_sf_alt[a], w->d_sf_alt[a], (static_cast<size_t>(w->n_experts) * w->plan.S * w->w_groups_alt[a] + 4) * kSfGroupBytes);
         }
     } catch (const std::bad_alloc&) {
         st = PRQ_ERR_OOM;
@@ -1416,7 +1397,27 @@ prq_status prq_linear_grouped(const prq_weights* w, const void* codes, const voi
     // token tile: 64 rows when the experts hold a handful of tokens each (the smaller tile leaves room for a deeper
     // ring of weight tiles in flight), 128 otherwise (every extra token tile of an expert re-reads its weight tiles)
     int bn = static_cast<long long>(M_total) <= 64LL * w->n_experts ? 64 : 128;
-    bn = env_int("PRQ_GROUPED_BN", bn);   // developer switch
+    // ... and CTA pairs on 256 x 240 tiles from 224 tokens per expert on, unless the 240-column tiles cover half as much
+    // again as N: less operand traffic per output, but an expert's last tile is padded to 256 (E x N x K + k, tokens per
+    // expert, microseconds 128-token tiles / pairs: 128 x 2048 x 832, 512: 116 / 104, 256: 64.7 / 64.3, 128: 43.3 / 47.3;
+    // 16 x 2048 x 832, 250: 13.3 / 12.0; 32 x 1400 x 672, 750: 41.9 / 32.7; 16 x 512 x 256, 4096: 24.6 / 19.9)
+    const long long wide_cols = static_cast<long long>((w->N + kPrefillTileWide - 1) / kPrefillTileWide) * kPrefillTileWide;
+    const bool pairs_fit = w->d_sf_alt[kAltWide] && (static_cast<long long>(M_total) / 256 + w->n_experts) * (wide_cols / kPrefillTileWide) < (1ll << 30);
+    if (pairs_fit && M_total >= 224LL * w->n_experts && 2 * wide_cols <= 3LL * w->N) bn = kPrefillTileWide;
+    const int forced = env_int("PRQ_GROUPED_BN", 0);   // developer switch
+    if (forced) bn = forced;
+    if (bn == kPrefillTileWide) {
+        // CTA pairs
+        if (!pairs_fit) return PRQ_ERR_INVALID_ARG;
+        p.w_groups = w->w_groups_alt[kAltWide];
+        CUtensorMap tm_a, tm_sfa;
+        st = make_code_map(&tm_a, codes, w->K / 2, M_total, 128);
+        if (st == PRQ_OK) st = make_sf_map(&tm_sfa, scales_sf, static_cast<uint64_t>(w->plan.S) * p.act_groups * kSfGroupBytes, 4);
+        if (st != PRQ_OK) return st;
+        const cudaError_t e = launch_gemm_grouped_pair(tm_a, w->tm_w_pair[kAltWide], tm_sfa, w->tm_sfw_pair[kAltWide], p, di->num_sms / 2, static_cast<cudaStream_t>(stream));
+        g_launches.fetch_add(1);
+        return e == cudaSuccess ? PRQ_OK : PRQ_ERR_CUDA;
+    }
     if (bn == 0) bn = 128;
     if (bn != 64 && bn != 128) return PRQ_ERR_INVALID_ARG;
     CUtensorMap tm_act, tm_w;

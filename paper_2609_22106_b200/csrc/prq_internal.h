@@ -128,6 +128,7 @@ struct prq_weights {
     uint8_t* d_sf = nullptr;         // E x S x w_groups x 1024 (+ padding)
     // Dense layers also keep the scale bytes grouped per 224-, 240- and 288-row weight tile of the prefill kernel
     // (two or three 128-row groups per tile, the last partly empty) so that those tile widths need no re-alignment.
+    // Stacked experts keep the 240-row tiling alone, expert after expert (the grouped kernel on CTA pairs).
     // A handle prepared as a gated producer (prq_prep_opts::gated_producer) keeps the 192-row tiling instead, the
     // one prq_linear_gated runs.
     uint8_t* d_sf_alt[4] = {nullptr, nullptr, nullptr, nullptr};

@@ -85,6 +85,11 @@ cudaError_t launch_gemm_grouped(int bn, const CUtensorMap& tm_act, const CUtenso
                                 cudaStream_t stream);
 
 
+// The same product on CTA pairs, 256 tokens x 240 output features per tile: `tm_act` has 128-row boxes, `tm_w` 120-row boxes,
+// `tm_sfa` / `tm_sfw` boxes of 4 / 8 rows of 256 scale bytes; `p.w_groups` and the weights' scale bytes in the 240-row tiling.
+cudaError_t launch_gemm_grouped_pair(const CUtensorMap& tm_act, const CUtensorMap& tm_w, const CUtensorMap& tm_sfa,
+                                     const CUtensorMap& tm_sfw, const GemmParams& p, int pairs, cudaStream_t stream);
+
 // The same kernel for the second format (MXFP8), dense layers of any M: `p.expert_offsets` null, `p.n_experts` 1;
 // scale bytes in 512-byte groups per (128-element stage, 128-row group); code maps over K-byte rows.
 cudaError_t launch_gemm_fp8(const CUtensorMap& tm_act, const CUtensorMap& tm_w, const GemmParams& p, int grid,

@@ -185,8 +185,12 @@ __device__ __forceinline__ uint32_t cluster_map(uint32_t local_addr, uint32_t ra
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(local_addr), "r"(rank));
     return ra;
 }
+// Arrives on a barrier of any CTA of the cluster, relaxed.  What it hands over is tensor memory whose reads are complete
+// (tcgen05.wait::ld has returned; tcgen05.fence::before_thread_sync orders them), no data in memory: with release semantics
+// towards another CTA the arrive would first wait until the thread's earlier global stores have been performed, microseconds
+// behind an epilogue's stores.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }

@@ -258,6 +258,39 @@ def test_permuting_quantiser_instances_against_oracle(prq, oracle, M, K, k):
     w.free()
 
 
+@pytest.mark.parametrize("seed", [23, 24, 25])
+def test_random_grouped_shapes_on_cta_pairs(prq, oracle, monkeypatch, seed):
+    test_random_grouped_shapes_against_oracle(prq, oracle, monkeypatch, seed, 240)
+
+
+def test_many_experts_on_cta_pairs(prq, oracle, monkeypatch):
+    test_many_experts_beyond_the_row_cache(prq, oracle, monkeypatch, 240)
+
+
+@pytest.mark.parametrize("N,K,k", [(248, 320, 64), (1000, 768, 0), (8, 96, 96), (480, 2080, 288)])
+def test_grouped_tiles_of_cta_pairs(prq, oracle, N, K, k):
+    """Experts whose rows end at, one before and one past a 256-token tile and its halves, features that leave a ragged
+    last tile, more stages than the ring has slots: same bits as the tile-per-CTA kernel, whose sums are the same."""
+    counts = [256, 0, 257, 511, 128, 129, 1, 767, 300]
+    offsets = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
+    E, M = len(counts), int(offsets[-1])
+    Ws = np.stack([synth.weights(2100 + e, N, K) for e in range(E)])
+    w = prq.prepare_weights(Ws, np.full((E, K), 1.5, np.float32), 0.5, k)
+    x, off = dev_bf16(synth.HeavyTailChannels(2200, K).rows(2201, M)), torch.from_numpy(offsets).cuda()
+    codes, _, sf = prq.quantize_act(w, x, prq.ACT_SCALE_PERM, expert_offsets=off)
+    for dt, td in ((prq.F32, torch.float32), (prq.BF16, torch.bfloat16)):
+        ys = []
+        for bn in ("128", "240"):
+            with pytest.MonkeyPatch.context() as mp:
+                mp.setenv("PRQ_GROUPED_BN", bn)
+                full = torch.full((M + 2, (N + 7) // 8 * 8 + 8), 7.0, dtype=td, device="cuda")
+                prq.linear_grouped(w, codes, sf, off, M, dt, out=full[1: M + 1, :N])
+            assert prq.last_device_status() == 0
+            ys.append(full)
+        assert torch.equal(*ys)
+    w.free()
+
+
 @pytest.mark.parametrize("gbn", [0, 64, 128])
 def test_many_experts_beyond_the_row_cache(prq, oracle, monkeypatch, gbn):
     """300 stacked experts (more than the kernels cache row ranges for), most with a handful of rows and many with
