@@ -28,7 +28,7 @@ EXPORTS = [
     "prq_linear_grouped", "prq_forward_host_scratch_bytes", "prq_forward_host",
     "prq_status_string", "prq_last_device_status", "prq_kernel_launch_count", "prq_mxf4_peak_probe",
     "prq_handover_probe", "prq_stack_gate_up", "prq_linear_gated", "prq_weights_format", "prq_act_bytes_for",
-    "prq_prepare_weights_stacked",
+    "prq_prepare_weights_stacked", "prq_linear_workspace_clear_bytes",
 ]
 
 
