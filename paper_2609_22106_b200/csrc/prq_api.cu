@@ -860,6 +860,32 @@ prq_status prq_prepare_weights_host_opts(const uint16_t* W, int N, int K, const 
     return PRQ_OK;
 }
 
+// A stream for copies of a handle's own memory, which no work on the caller's streams touches: they neither wait for that work
+// nor disturb a capture in progress.  finish() waits for them; a handle must not leave the library with bytes on their way
+// (a device-to-device cudaMemcpy returns before it has run, and the caller's next call may be on any stream).
+class CopyStream {
+public:
+    CopyStream() {
+        cudaThreadExchangeStreamCaptureMode(&mode_);
+        ok_ = cudaStreamCreateWithFlags(&s_, cudaStreamNonBlocking) == cudaSuccess;
+    }
+    ~CopyStream() {
+        if (s_) cudaStreamDestroy(s_);
+        cudaThreadExchangeStreamCaptureMode(&mode_);
+    }
+    CopyStream(const CopyStream&) = delete;
+    CopyStream& operator=(const CopyStream&) = delete;
+    bool copy(void* dst, const void* src, size_t bytes, cudaMemcpyKind kind) {
+        return ok_ = ok_ && cudaMemcpyAsync(dst, src, bytes, kind, s_) == cudaSuccess;
+    }
+    bool finish() { return (!s_ || cudaStreamSynchronize(s_) == cudaSuccess) && ok_; }
+
+private:
+    cudaStreamCaptureMode mode_ = cudaStreamCaptureModeRelaxed;
+    cudaStream_t s_ = nullptr;
+    bool ok_ = false;
+};
+
 prq_status prq_weights_clone(const prq_weights* w, prq_weights** out) {
     if (!w || !out || w->format != PRQ_FMT_MXFP4) return PRQ_ERR_INVALID_ARG;
     prq_weights* c = new (std::nothrow) prq_weights;
@@ -868,6 +894,7 @@ prq_status prq_weights_clone(const prq_weights* w, prq_weights** out) {
     cudaGetDevice(&cur);
     if (cur != w->device) cudaSetDevice(w->device);
     prq_status st = PRQ_OK;
+    CopyStream copies;
     try {
         c->n_experts = w->n_experts; c->N = w->N; c->K = w->K; c->k_tail = w->k_tail; c->alpha = w->alpha;
         c->plan = w->plan; c->w_groups = w->w_groups; c->device = w->device; c->gated = w->gated;
@@ -879,7 +906,7 @@ prq_status prq_weights_clone(const prq_weights* w, prq_weights** out) {
             void** pp = static_cast<void**>(dst_pp);
             if (st != PRQ_OK || !src) return;
             if (cudaMalloc(pp, bytes) != cudaSuccess) { cudaGetLastError(); st = PRQ_ERR_OOM; return; }
-            if (cudaMemcpy(*pp, src, bytes, cudaMemcpyDeviceToDevice) != cudaSuccess) st = PRQ_ERR_CUDA;
+            if (!copies.copy(*pp, src, bytes, cudaMemcpyDeviceToDevice)) st = PRQ_ERR_CUDA;
         };
         dup(&c->d_codes, w->d_codes, w->d_codes_bytes);
         dup(&c->d_sf, w->d_sf, w->d_sf_bytes);
@@ -894,6 +921,7 @@ prq_status prq_weights_clone(const prq_weights* w, prq_weights** out) {
     } catch (const std::bad_alloc&) {
         st = PRQ_ERR_OOM;
     }
+    if (!copies.finish() && st == PRQ_OK) st = PRQ_ERR_CUDA;
     if (st == PRQ_OK) st = build_weight_maps(c);
     if (cur != w->device) cudaSetDevice(cur);
     if (st != PRQ_OK) { prq_weights_free(c); return st; }
@@ -914,6 +942,7 @@ prq_status prq_weights_offline_copy(const prq_weights* w, prq_weights** out) {
     int cur = 0;
     cudaGetDevice(&cur);
     if (cur != c->device) cudaSetDevice(c->device);
+    CopyStream copies;
     try {
         c->K = Kw; c->k_tail = 0; c->plan = StagePlan(Kw, 0);
         // the activation arrives permuted, scaled and with its tail columns doubled: nothing is left to apply
@@ -928,12 +957,13 @@ prq_status prq_weights_offline_copy(const prq_weights* w, prq_weights** out) {
         bool ok = cudaMalloc(&c->d_perm, sizeof(int32_t) * E * Kw) == cudaSuccess &&
                   cudaMalloc(&c->d_inv_s_perm, sizeof(float) * E * Kw) == cudaSuccess;
         if (!ok) { cudaGetLastError(); st = PRQ_ERR_OOM; }
-        ok = ok && cudaMemcpy(c->d_perm, c->h_perm.data(), sizeof(int32_t) * E * Kw, cudaMemcpyHostToDevice) == cudaSuccess;
-        ok = ok && cudaMemcpy(c->d_inv_s_perm, c->h_inv_s.data(), sizeof(float) * E * Kw, cudaMemcpyHostToDevice) == cudaSuccess;
+        ok = ok && copies.copy(c->d_perm, c->h_perm.data(), sizeof(int32_t) * E * Kw, cudaMemcpyHostToDevice);
+        ok = ok && copies.copy(c->d_inv_s_perm, c->h_inv_s.data(), sizeof(float) * E * Kw, cudaMemcpyHostToDevice);
         if (!ok && st == PRQ_OK) st = PRQ_ERR_CUDA;
     } catch (const std::bad_alloc&) {
         st = PRQ_ERR_OOM;
     }
+    if (!copies.finish() && st == PRQ_OK) st = PRQ_ERR_CUDA;
     if (st == PRQ_OK) st = build_weight_maps(c);
     if (cur != c->device) cudaSetDevice(cur);
     if (st != PRQ_OK) { prq_weights_free(c); return st; }
@@ -958,20 +988,17 @@ prq_status prq_weights_info(const prq_weights* w, int* n_experts, int* N, int* K
     return PRQ_OK;
 }
 
-// Bytes of a handle that only the device holds -> host memory.  On a stream of its own, so that it neither waits for nor
-// disturbs what the caller's streams are doing (a capture in progress included); the handle is immutable.
+// Bytes of a handle that only the device holds -> host memory (the handle is immutable).
 static prq_status fetch_from_device(const prq_weights* w, void* dst, const void* src, size_t bytes) {
     int cur = 0;
     if (cudaGetDevice(&cur) != cudaSuccess) return PRQ_ERR_CUDA;
     if (cur != w->device && cudaSetDevice(w->device) != cudaSuccess) return PRQ_ERR_CUDA;
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    cudaStream_t s = nullptr;
-    bool ok = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess;
-    ok = ok && cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, s) == cudaSuccess;
-    ok = ok && cudaStreamSynchronize(s) == cudaSuccess;
-    if (s) cudaStreamDestroy(s);
-    cudaThreadExchangeStreamCaptureMode(&mode);
+    bool ok;
+    {
+        CopyStream copies;
+        copies.copy(dst, src, bytes, cudaMemcpyDeviceToHost);
+        ok = copies.finish();
+    }
     if (cur != w->device) cudaSetDevice(cur);
     return ok ? PRQ_OK : PRQ_ERR_CUDA;
 }

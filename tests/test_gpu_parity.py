@@ -598,6 +598,33 @@ def test_device_prep_layouts_feed_every_kernel(prq, monkeypatch, bn):
     wh.free()
 
 
+def test_a_clone_is_complete_when_the_call_returns(prq):
+    """A clone of a layer prepared on the device (40 MB of codes), taken while the default stream is busy: its bytes, read
+    back first thing, and its product on another stream are the original's."""
+    w = prq.prepare_weights_device(torch.randn(8192, 9728, device="cuda").to(torch.bfloat16), np.ones(9728, np.float32), 0.5, 256)
+    codes = w.get(prq.FIELD_CODES)
+    x = to_dev_bf16(synth.HeavyTailChannels(71, 9728).rows(72, 16))
+    want = prq.linear_fused(w, x)
+    busy = torch.randn(8192, 8192, device="cuda")
+    torch.cuda.synchronize()
+    for _ in range(8):
+        busy @ busy
+    c = w.clone()
+    assert np.array_equal(c.get(prq.FIELD_CODES), codes)
+    assert np.array_equal(c.get(prq.FIELD_SCALES), w.get(prq.FIELD_SCALES))
+    side = torch.cuda.Stream()
+    y = torch.empty_like(want)
+    for _ in range(8):
+        busy @ busy
+    d = w.clone()
+    prq.linear_fused(d, x, out=y, stream=side)
+    side.synchronize()
+    assert torch.equal(y, want)
+    assert prq.last_device_status() == 0
+    for h in (w, c, d):
+        h.free()
+
+
 @pytest.mark.parametrize("N,K,k,M", [(256, 512, 64, 16), (512, 2560, 128, 300), (256, 768, 64, 1), (384, 1024, 256, 128)])
 def test_offline_copy_form_equals_the_revisit_form(prq, oracle, N, K, k, M):
     """Activation tail construction paragraph, offline copy: the producer emits the k tail channels twice, the
