@@ -29,7 +29,8 @@ struct DeviceInfo {
     int num_sms = 0;
     int* status_ptr = nullptr;
     int max_clusters[4][9] = {};  // decode kernel: [token-tile index][cluster size], 0 = not queried yet
-    int max_pairs = 0;            // prefill pair kernel: co-resident CTA pairs, 0 = not queried yet
+    // co-resident CTA pairs, 0 = not queried yet (read through co_resident_pairs, which holds g_dev_mutex):
+    int max_pairs = 0;            // prefill pair kernel
     int max_pairs_gated = 0;      // the same for its gated-producer instance
     int max_pairs_fp8 = 0;        // ... and for its instances of the second format
 };
@@ -59,6 +60,14 @@ prq_status device_info(int dev, DeviceInfo** out) {
     }
     *out = &d;
     return PRQ_OK;
+}
+
+// One of the pair counts, queried on first use (on the current device, which must be the one `di` describes).
+template <class Query>
+int co_resident_pairs(DeviceInfo* di, int DeviceInfo::*field, Query query) {
+    std::lock_guard<std::mutex> lock(g_dev_mutex);
+    if (di->*field == 0) di->*field = std::min<int>(query(), di->num_sms / 2);
+    return di->*field;
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -287,8 +296,8 @@ PairSchedule choose_pair_schedule(int M, int N, int S, int max_pairs) {
 struct Fp8Schedule { int bn, pairs; long long tiles, waves; };
 Fp8Schedule fp8_schedule(int M, int N, DeviceInfo* di) {
     Fp8Schedule best = {};
-    if (di->max_pairs_fp8 == 0) di->max_pairs_fp8 = std::min(prefill_pair_max_clusters_fp8(), di->num_sms / 2);
-    if (di->max_pairs_fp8 < 1) return best;
+    const int max_pairs = co_resident_pairs(di, &DeviceInfo::max_pairs_fp8, prefill_pair_max_clusters_fp8);
+    if (max_pairs < 1) return best;
     // developer switch: 0 = the tile-per-CTA kernel, 224 / 240 / 288 = that width where it can run
     const int forced = env_int("PRQ_FP8_BN", -1);
     if (forced == 0) return best;
@@ -296,7 +305,7 @@ Fp8Schedule fp8_schedule(int M, int N, DeviceInfo* di) {
     long long best_cost = 1ll << 60;
     for (int i = 0; i < 3; ++i) {
         const long long tiles = ((M + 255ll) / 256) * ((N + bns[i] - 1) / bns[i]);
-        const int pairs = static_cast<int>(std::min<long long>(tiles, di->max_pairs_fp8));
+        const int pairs = static_cast<int>(std::min<long long>(tiles, max_pairs));
         const long long waves = (tiles + pairs - 1) / pairs;
         if (bns[i] == kPrefillTileOneWave && waves > 1) continue;
         if (forced > 0 && bns[i] != forced) continue;
@@ -1127,15 +1136,17 @@ size_t prq_linear_workspace_bytes(const prq_weights* w, int M) {
 }
 
 static PairSchedule schedule_prefill(const prq_weights* w, int M, DeviceInfo* di) {
-    if (di->max_pairs == 0)
-        di->max_pairs = std::min(std::min(std::min(prefill_pair_max_clusters(kPrefillTileN), prefill_pair_max_clusters(kPrefillTileWide)),
-                                          prefill_pair_max_clusters(kPrefillTileOneWave)), di->num_sms / 2);
-    return choose_pair_schedule(M, w->N, w->plan.S, std::min(di->max_pairs, env_int("PRQ_GRID", 1 << 20)));
+    const int max_pairs = co_resident_pairs(di, &DeviceInfo::max_pairs, [] {
+        return std::min(std::min(prefill_pair_max_clusters(kPrefillTileN), prefill_pair_max_clusters(kPrefillTileWide)),
+                        prefill_pair_max_clusters(kPrefillTileOneWave));
+    });
+    return choose_pair_schedule(M, w->N, w->plan.S, std::min(max_pairs, env_int("PRQ_GRID", 1 << 20)));
 }
 
 size_t prq_linear_workspace_clear_bytes(const prq_weights* w, int M) {
     DeviceInfo* di;
     if (!w || M <= 128 || w->format != PRQ_FMT_MXFP4 || device_info(w->device, &di) != PRQ_OK) return 0;
+    if (!handle_device_is_current(w)) return prefill_flag_bytes(w, M);   // the schedule is the handle's device's
     // the counters are touched only where a tile is cut into pieces
     const PairSchedule ps = schedule_prefill(w, M, di);
     return ps.sk > 0 && (ps.base > 1 || env_int("PRQ_SK_RANGES", 0)) ? prefill_flag_bytes(w, M) : 0;
@@ -1334,8 +1345,7 @@ prq_status prq_linear_gated(const prq_weights* w, const void* codes, const void*
     DeviceInfo* di;
     prq_status st = device_info(w->device, &di);
     if (st != PRQ_OK) return st;
-    if (di->max_pairs_gated == 0)
-        di->max_pairs_gated = std::max(1, std::min(prefill_pair_max_clusters(kPrefillTileGated), di->num_sms / 2));
+    const int max_pairs = std::max(1, co_resident_pairs(di, &DeviceInfo::max_pairs_gated, [] { return prefill_pair_max_clusters(kPrefillTileGated); }));
 
     PrefillParams q;
     std::memset(&q, 0, sizeof(q));
@@ -1344,7 +1354,7 @@ prq_status prq_linear_gated(const prq_weights* w, const void* codes, const void*
     const long long tiles = static_cast<long long>(q.m_tiles) * q.n_tiles;
     if (tiles >= (1ll << 30)) return PRQ_ERR_INVALID_ARG;
     // whole tiles only, wave after wave (a piece of a tile has no gate and up sums to put through the activation)
-    const int pairs = static_cast<int>(std::min<long long>(tiles, di->max_pairs_gated));
+    const int pairs = static_cast<int>(std::min<long long>(tiles, max_pairs));
     q.sk_tiles = 0; q.whole_tiles = static_cast<int>((tiles + pairs - 1) / pairs); q.total_tiles = static_cast<int>(tiles);
     q.act_groups = dense_groups(M); q.w_groups = w->w_groups_alt[kAltGated];
     q.act_sf = static_cast<const uint8_t*>(scales_sf); q.w_sf = w->d_sf_alt[kAltGated];

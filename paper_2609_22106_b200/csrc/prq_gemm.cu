@@ -479,12 +479,9 @@ cudaError_t launch_grouped_impl(const CUtensorMap& tm_act, const CUtensorMap& tm
                                 cudaStream_t stream) {
     using C = Cfg<kFp8, BN>;
     constexpr int smem = C::kStages * C::kStageBytes + 1024 + C::kEpiWarps * C::kStagingBytes;  // + store staging
-    static bool configured = false;  // the attribute is per function, setting it twice is harmless
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(gemm_grouped_kernel<kFp8, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static OncePerDevice opt_in;
+    const cudaError_t e = opt_in([] { return cudaFuncSetAttribute(gemm_grouped_kernel<kFp8, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(C::kThreads);

@@ -492,12 +492,9 @@ cudaError_t launch_one(const DecodeMaps& maps, const DecodeBatch& b, cudaStream_
     const int n_tiles = b.lay[b.n_lin - 1].tile_end;
     using C = DCfg<BN, kDense>;
     if (kDense && p.splits != 1) return cudaErrorInvalidValue;   // the dense variant has no receive buffer
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(decode_kernel<BN, kFused, kBatch, kDense>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static OncePerDevice opt_in;
+    const cudaError_t e = opt_in([] { return cudaFuncSetAttribute(decode_kernel<BN, kFused, kBatch, kDense>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes); });
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_tiles * p.splits);
     cfg.blockDim = dim3(C::kThreads);
@@ -518,14 +515,12 @@ cudaError_t launch_one(const DecodeMaps& maps, const DecodeBatch& b, cudaStream_
 // more weight tiles than SMs, no K split, 64 tokens or more: the two-CTAs-per-SM variant
 bool wants_dense(int bn, const DecodeBatch& b) {
     if (bn < 64 || b.splits != 1) return false;
-    static int sm_count[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
-    if (sm_count[dev] == 0 && cudaDeviceGetAttribute(&sm_count[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    int sms = 0;
+    if (current_sm_count(&sms) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return b.lay[b.n_lin - 1].tile_end > sm_count[dev];
+    return b.lay[b.n_lin - 1].tile_end > sms;
 }
 
 template <int BN>

@@ -23,8 +23,6 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
-#include <atomic>
-
 #include "prq_kernels.h"
 #include "prq_pair.cuh"
 #include "prq_ptx.cuh"
@@ -308,15 +306,9 @@ gemm_grouped_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __gri
 cudaError_t launch_gemm_grouped_pair(const CUtensorMap& tm_act, const CUtensorMap& tm_w, const CUtensorMap& tm_sfa,
                                      const CUtensorMap& tm_sfw, const GemmParams& p, int pairs, cudaStream_t stream) {
     constexpr int BN = kPrefillTileWide;
-    static std::atomic<unsigned long long> configured{0};   // the attribute is set once per device
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    static OncePerDevice opt_in;
+    const cudaError_t e = opt_in([] { return cudaFuncSetAttribute(gemm_grouped_pair_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, gp_smem<BN>()); });
     if (e != cudaSuccess) return e;
-    if (dev >= 64 || !((configured.load(std::memory_order_acquire) >> dev) & 1)) {
-        e = cudaFuncSetAttribute(gemm_grouped_pair_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, gp_smem<BN>());
-        if (e != cudaSuccess) return e;
-        if (dev < 64) configured.fetch_or(1ull << dev, std::memory_order_release);
-    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * pairs);
     cfg.blockDim = dim3(kGpThreads);

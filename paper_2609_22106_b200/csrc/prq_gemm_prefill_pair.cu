@@ -663,8 +663,6 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_con
 template <int BN, bool kGated = false, bool kFp8 = false>
 int max_clusters_bn() {
     constexpr int kSmemBytes = PCfg<BN, kFp8>::kSmemBytes;
-    static int cached = -1;
-    if (cached >= 0) return cached;
     if (cudaFuncSetAttribute(prefill_pair_kernel<BN, kGated, kFp8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2);
@@ -678,9 +676,7 @@ int max_clusters_bn() {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, prefill_pair_kernel<BN, kGated, kFp8>, &cfg) != cudaSuccess) return 0;
-    cached = n;
-    return n;
+    return cudaOccupancyMaxActiveClusters(&n, prefill_pair_kernel<BN, kGated, kFp8>, &cfg) == cudaSuccess ? n : 0;
 }
 
 template <int BN, bool kGated = false, bool kFp8 = false>
@@ -688,12 +684,9 @@ cudaError_t launch_bn(const CUtensorMap& tm_act, const CUtensorMap& tm_w, const 
                       const CUtensorMap& tm_sfw, const CUtensorMap& tm_y, const PrefillParams& p,
                       int pairs, cudaStream_t stream) {
     constexpr int kSmemBytes = PCfg<BN, kFp8>::kSmemBytes;
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(prefill_pair_kernel<BN, kGated, kFp8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static OncePerDevice opt_in;
+    const cudaError_t e = opt_in([] { return cudaFuncSetAttribute(prefill_pair_kernel<BN, kGated, kFp8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes); });
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * pairs);
     cfg.blockDim = dim3(kThreads);

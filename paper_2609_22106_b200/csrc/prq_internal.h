@@ -1,6 +1,7 @@
 // Internal declarations shared by the translation units of libprq.
 #pragma once
 #include <algorithm>
+#include <atomic>
 #include <cstdlib>
 #include <cstddef>
 #include <cstdint>
@@ -23,6 +24,39 @@ inline bool dev_knobs_enabled() {
     return on;
 }
 
+// Runs `set` (a kernel's shared-memory opt-in and the like) once per device: such attributes belong to the device that is
+// current, and one process may hold handles on several.  Any thread may come first; running `set` twice is harmless.
+class OncePerDevice {
+public:
+    template <class F>
+    cudaError_t operator()(F&& set) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        if (dev < 64 && ((done_.load(std::memory_order_acquire) >> dev) & 1)) return cudaSuccess;
+        e = set();
+        if (e == cudaSuccess && dev < 64) done_.fetch_or(1ull << dev, std::memory_order_release);
+        return e;
+    }
+
+private:
+    std::atomic<unsigned long long> done_{0};
+};
+
+// SM count of the current device, looked up once per device.
+inline cudaError_t current_sm_count(int* n) {
+    static std::atomic<int> count[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    *n = count[dev].load(std::memory_order_relaxed);
+    if (*n == 0) {
+        e = cudaDeviceGetAttribute(n, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) count[dev].store(*n, std::memory_order_relaxed);
+    }
+    return e;
+}
 
 constexpr int kBlock = 32;        // MXFP4 block length
 constexpr int kStageK = 256;      // reduction elements per pipeline stage (one 128-byte swizzled row)

@@ -7,7 +7,7 @@
 // clock higher than real data) with unit block scales.
 #include <cuda_runtime.h>
 
-#include "prq.h"
+#include "prq_internal.h"
 #include "prq_ptx.cuh"
 
 namespace prq {
@@ -101,12 +101,9 @@ cudaError_t launch_handover_probe(int n, int grid, int threads, int cluster, int
 }
 
 cudaError_t launch_mxf4_peak_probe(int n_mma, int grid, int* status, cudaStream_t stream) {
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(mxf4_peak_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static OncePerDevice opt_in;
+    const cudaError_t e = opt_in([] { return cudaFuncSetAttribute(mxf4_peak_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem); });
+    if (e != cudaSuccess) return e;
     mxf4_peak_kernel<<<grid, 64, kSmem, stream>>>(n_mma, status);
     return cudaGetLastError();
 }

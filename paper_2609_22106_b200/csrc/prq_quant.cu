@@ -606,20 +606,16 @@ cudaError_t launch_cols_impl(const QuantBatch& b, int sm_count, cudaStream_t str
     const int lanes = (b.K + kStageK - 1) / kStageK * (kStageK / kCols);
     const int all_warps = (lanes + 31) / 32, max_warps = kMaxT / 32 - 1;
     const int chunks = (all_warps + max_warps - 1) / max_warps, warps = (all_warps + chunks - 1) / chunks;
-    static std::atomic<int> regs{0};   // the same on every device; the attribute is set per device below
-    static std::atomic<unsigned long long> configured{0};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev >= 64 || !((configured.load(std::memory_order_acquire) >> dev) & 1)) {
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kColsSmem - (kGrouped ? 9216 : 0));
-        if (e != cudaSuccess) return e;
+    static std::atomic<int> regs{0};   // the same on every device
+    static OncePerDevice opt_in;
+    const cudaError_t e = opt_in([&] {
+        cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kColsSmem - (kGrouped ? 9216 : 0));
         cudaFuncAttributes fa;
-        e = cudaFuncGetAttributes(&fa, kernel);
-        if (e != cudaSuccess) return e;
-        regs.store(fa.numRegs);
-        if (dev < 64) configured.fetch_or(1ull << dev, std::memory_order_release);
-    }
+        if (r == cudaSuccess) r = cudaFuncGetAttributes(&fa, kernel);
+        if (r == cudaSuccess) regs.store(fa.numRegs);
+        return r;
+    });
+    if (e != cudaSuccess) return e;
     const int threads = 32 * (warps + 1);
     const size_t stage = static_cast<size_t>(kRowsC) * b.K * 2;
     // CTAs per SM: as many as the registers hold, while each still has room for three slices of rows
@@ -662,18 +658,12 @@ cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, cudaStr
     int parts = 1;
     if (scale_perm) {
         // split the rows of a group (a CTA has a fixed cost of about a microsecond, so no further than needed)
-        static int sm_count[64] = {};
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-        if (sm_count[dev] == 0) {
-            int n = 0;
-            cudaError_t e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-            if (e != cudaSuccess) return e;
-            sm_count[dev] = n;
-        }
+        int sms = 0;
+        const cudaError_t e = current_sm_count(&sms);
+        if (e != cudaSuccess) return e;
         const long long tiles = static_cast<long long>(n_atoms) * grid_groups;
-        while (parts < 4 && tiles * parts < 8LL * sm_count[dev]) parts *= 2;   // 3 CTAs per SM: keep the last wave short
-        if (parts == 4 && tiles * parts < 4LL * sm_count[dev]) parts = 8;
+        while (parts < 4 && tiles * parts < 8LL * sms) parts *= 2;   // 3 CTAs per SM: keep the last wave short
+        if (parts == 4 && tiles * parts < 4LL * sms) parts = 8;
         if (const char* ev = dev_knobs_enabled() ? getenv("PRQ_QUANT_PARTS") : nullptr) { const int v = atoi(ev); if (v == 1 || v == 2 || v == 4 || v == 8) parts = v; }
         // The column-stationary structure, in the instance that measured best (microseconds in a chain of launches, K and
         // k as given; column atoms -> this structure):
@@ -691,14 +681,14 @@ cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, cudaStr
         auto fits = [&](int rows) { return 4 * static_cast<size_t>(rows) * p.K + 10240 <= kColsSmem - 9216; };
         bool cols = !(grouped && static_cast<long long>(grid_groups) * n_atoms <= 64);
         if (const char* ev = dev_knobs_enabled() ? getenv("PRQ_QUANT_ROWS") : nullptr) cols = atoi(ev) != 0;
-        if (cols && grouped && fits(4)) return launch_cols_impl<8, 4, true, 544>(b, sm_count[dev], stream);
+        if (cols && grouped && fits(4)) return launch_cols_impl<8, 4, true, 544>(b, sms, stream);
         if (cols && !grouped) {
             const bool large = b.M >= 1500 && p.K >= 2048;
-            if (b.M <= 128 && p.K <= 4096) return launch_cols_impl<16, 1, false, 192>(b, sm_count[dev], stream);
-            if (large && p.K <= 8192) return launch_cols_impl<16, 4, false, 384>(b, sm_count[dev], stream);
-            if (large && fits(2)) return launch_cols_impl<16, 2, false, 640>(b, sm_count[dev], stream);
-            if (fits(2)) return launch_cols_impl<16, 2, false, 320>(b, sm_count[dev], stream);
-            if (fits(1)) return launch_cols_impl<16, 1, false, 192>(b, sm_count[dev], stream);
+            if (b.M <= 128 && p.K <= 4096) return launch_cols_impl<16, 1, false, 192>(b, sms, stream);
+            if (large && p.K <= 8192) return launch_cols_impl<16, 4, false, 384>(b, sms, stream);
+            if (large && fits(2)) return launch_cols_impl<16, 2, false, 640>(b, sms, stream);
+            if (fits(2)) return launch_cols_impl<16, 2, false, 320>(b, sms, stream);
+            if (fits(1)) return launch_cols_impl<16, 1, false, 192>(b, sms, stream);
         }
     }
     // the tail atoms of the scale + permute mode in shares of 16 rows (128 / 8), see the kernel

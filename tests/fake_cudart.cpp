@@ -20,6 +20,7 @@
 namespace {
 std::mutex g_mu;
 thread_local int t_device = 0;
+thread_local cudaError_t t_last = cudaSuccess;
 struct Stream {
     bool blocking;
     std::vector<std::function<void()>> work;
@@ -64,7 +65,7 @@ cudaError_t copy(void* dst, const void* src, size_t n, cudaMemcpyKind kind, Stre
 cudaError_t launch(const void* func, size_t dynamic_smem) {
     std::lock_guard<std::mutex> lock(g_mu);
     auto it = g_dynamic_smem.find({t_device, func});
-    if (dynamic_smem > static_cast<size_t>(it == g_dynamic_smem.end() ? 48 * 1024 : it->second)) return cudaErrorInvalidValue;
+    if (dynamic_smem > static_cast<size_t>(it == g_dynamic_smem.end() ? 48 * 1024 : it->second)) return t_last = cudaErrorInvalidValue;
     ++g_launches[t_device];
     return cudaSuccess;
 }
@@ -85,7 +86,7 @@ cudaError_t cudaGetDevice(int* d) { *d = t_device; return cudaSuccess; }
 cudaError_t cudaSetDevice(int d) { if (d < 0 || d > 1) return cudaErrorInvalidDevice; t_device = d; return cudaSuccess; }
 cudaError_t cudaGetDeviceProperties_v2(cudaDeviceProp* p, int) { std::memset(p, 0, sizeof(*p)); p->major = 10; p->multiProcessorCount = 148; return cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { *v = 148; return cudaSuccess; }
-cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaGetLastError() { const cudaError_t e = t_last; t_last = cudaSuccess; return e; }
 cudaError_t cudaMalloc(void** p, size_t n) {   // fresh memory: different bytes every time
     std::lock_guard<std::mutex> lock(g_mu);
     *p = std::aligned_alloc(1024, (n + 1023) / 1024 * 1024);

@@ -58,3 +58,63 @@ def test_a_copy_of_a_handle_is_complete_when_the_call_returns(fake, form, where)
     assert np.array_equal(c.get(fake.FIELD_SCALES), w.get(fake.FIELD_SCALES))
     c.free()
     w.free()
+
+
+def _aligned(n_bytes):
+    """Host bytes on a 256-byte boundary (device memory to the stand-in)."""
+    a = np.zeros(n_bytes + 256, np.uint8)
+    return a[-a.ctypes.data % 256:][:n_bytes]
+
+
+def _every_kernel(fake):
+    """Calls that between them launch every kernel with a shared-memory opt-in, on the current device."""
+    L, p = fake.lib(), lambda a: a.ctypes.data
+    for N, K, M in ((256, 512, 1), (256, 512, 32), (256, 512, 64), (256, 512, 128), (19456, 32, 64), (19456, 32, 128), (256, 512, 300),
+                    (2560, 512, 2048), (2560, 512, 4096), (32, 9728, 2048)):
+        w = fake.prepare_weights(np.zeros((N, K), np.uint16), np.ones(K, np.float32), 0.5, 0)
+        x, codes, sf, y = (_aligned(n) for n in (M * K * 2, fake.act_bytes(M, K, 0, 1, fake.BUF_CODES), fake.act_bytes(M, K, 0, 1, fake.BUF_SCALES_SF), M * N * 4))
+        ws = _aligned(max(16, fake.linear_workspace_bytes(w, M)))
+        fake._check(L.prq_quantize_act(w.handle, fake.ACT_SCALE_PERM, p(x), M, K, None, p(codes), None, p(sf), None), f"quantize {N} {K} {M}")
+        fake._check(L.prq_linear(w.handle, p(codes), p(sf), M, p(y), N, fake.F32, p(ws), ws.size, None), f"linear {N} {K} {M}")
+        if M <= 128:
+            two = (ctypes.c_void_p * 2)
+            fake._check(L.prq_linear_multi(2, two(w.handle.value, w.handle.value), two(p(codes), p(codes)), two(p(sf), p(sf)), M, two(p(y), p(y)),
+                                           (ctypes.c_int * 2)(N, N), fake.F32, None), f"multi {N} {K} {M}")
+        if M <= fake.FUSED_MAX_M:
+            fake._check(L.prq_linear_fused(w.handle, fake.ACT_IDENTITY, p(x), M, K, p(y), N, fake.F32, None), "fused")
+        w.free()
+    for N, M in ((128, 64), (1024, 1300), (2048, 1500), (6144, 700), (6144, 4096)):   # MXFP8: both kernels, several widths
+        w = fake.prepare_weights(np.zeros((N, 256), np.uint16), np.ones(256, np.float32), 0.5, 0, fmt=fake.FMT_MXFP8)
+        codes, sf, y = _aligned(M * 256), _aligned(L.prq_act_bytes_for(w.handle, M, fake.BUF_SCALES_SF)), _aligned(M * N * 4)
+        fake._check(L.prq_linear(w.handle, p(codes), p(sf), M, p(y), N, fake.F32, None, 0, None), f"mxfp8 {N} {M}")
+        w.free()
+    E, N, K = 2, 512, 256   # stacked experts: quantiser, 64- and 128-token tiles, CTA pairs
+    w = fake.prepare_weights(np.zeros((E, N, K), np.uint16), np.ones((E, K), np.float32), 0.5, 0)
+    for M in (100, 300, 60000):
+        codes, sf, x, y = _aligned(M * K // 2), _aligned(fake.act_bytes(M, K, 0, E, fake.BUF_SCALES_SF)), _aligned(M * K * 2), _aligned(M * N * 2)
+        off = np.array([0, M // 2, M], np.int32)
+        fake._check(L.prq_quantize_act(w.handle, fake.ACT_SCALE_PERM, p(x), M, K, p(off), p(codes), None, p(sf), None), f"grouped quantize {M}")
+        fake._check(L.prq_linear_grouped(w.handle, p(codes), p(sf), p(off), M, p(y), N, fake.BF16, None), f"grouped {M}")
+    w.free()
+    gu = fake.prepare_weights(np.zeros((512, 256), np.uint16), np.ones(256, np.float32), 0.5, 0, gated_producer=True)
+    down = fake.prepare_weights(np.zeros((64, 256), np.uint16), np.ones(256, np.float32), 0.5, 0)
+    M = 300
+    b = [_aligned(fake.act_bytes(M, 256, 0, 1, k)) for k in (fake.BUF_CODES, fake.BUF_SCALES_SF)]
+    fake._check(L.prq_linear_gated(gu.handle, p(b[0]), p(b[1]), M, down.handle, p(b[0]), None, p(b[1]), None, None), "gated")
+    gu.free()
+    down.free()
+    fake._check(L.prq_mxf4_peak_probe(4, None, None), "probe")
+
+
+def test_every_kernel_runs_on_a_second_device(fake):
+    """The shared-memory opt-in of a kernel belongs to a device: a process with handles on two GPUs needs it on both."""
+    launches = []
+    for device in (0, 1):
+        assert fake.lib().cudaSetDevice(device) == 0
+        try:
+            before = fake.lib().fake_launches(device)
+            _every_kernel(fake)
+            launches.append(fake.lib().fake_launches(device) - before)
+        finally:
+            fake.lib().cudaSetDevice(0)
+    assert launches[0] == launches[1]
