@@ -336,6 +336,7 @@ struct ColsPlan {
     int n_slices;        // slices of all 128-row groups (grouped: of all groups the launch could need)
     int n_stages;        // slices of rows in flight per CTA
     int warps;           // computing warps per CTA (one more loads the rows)
+    int strided;         // a CTA takes slices g, g + G, ... instead of consecutive ones (one 128-row group only)
 };
 constexpr int kColsMaxStages = 8;
 constexpr size_t kColsSmem = 220 * 1024;   // shared memory of an SM that the rows in flight may take
@@ -417,10 +418,13 @@ quant_act_cols_kernel(const QuantBatch b, const ColsPlan plan_c) {
     const int n_slices = kGrouped ? min(plan_c.n_slices, s_tile_start[b.n_experts] * kSlicesC) : plan_c.n_slices;
 
     // A CTA's slices are consecutive (with stacked experts the constants then change a few times, not per slice), and
-    // the CTAs' shares differ by one slice at most.
+    // the CTAs' shares differ by one slice at most.  A few rows of one dense group are dealt out in turn instead: the
+    // group's padding follows its rows, and nobody then has two slices of rows beside others that have none.
     const int G = static_cast<int>(gridDim.x), g = static_cast<int>(blockIdx.x);
     const int base = n_slices / G, extra = n_slices - base * G;
-    const int sl_begin = g * base + min(g, extra), n_mine = base + (g < extra ? 1 : 0);
+    const bool strided = !kGrouped && plan_c.strided;
+    const int sl_begin = strided ? g : g * base + min(g, extra), n_mine = base + (g < extra ? 1 : 0);
+    const int step_rows = strided ? G * kRowsC : kRowsC;
     // where a slice sits: its group, its first row inside the group, the expert and the rows (in x) of the group
     int group = sl_begin / kSlicesC, r_first = (sl_begin % kSlicesC) * kRowsC, expert = 0, g_row0 = 0, g_end = 0;
     auto enter_group = [&]() {
@@ -433,8 +437,8 @@ quant_act_cols_kernel(const QuantBatch b, const ColsPlan plan_c) {
         }
     };
     auto next_slice = [&]() {
-        r_first += kRowsC;
-        if (r_first == kGroupRows) { r_first = 0; ++group; return true; }
+        r_first += step_rows;
+        if (r_first >= kGroupRows) { r_first -= kGroupRows; ++group; return true; }
         return false;
     };
     if (n_mine > 0) {
@@ -632,9 +636,20 @@ cudaError_t launch_cols_impl(const QuantBatch& b, int sm_count, cudaStream_t str
     cp.n_slices = b.groups_per_lin * (kGroupRows / kRowsC);
     cp.n_stages = static_cast<int>(n_stages);
     cp.warps = warps;
+    cp.strided = 0;
     int want = per_sm * sm_count / (chunks * b.n_lin);
     // a CTA of a grouped launch first looks the experts up: two slices at least, or that is all it does
     if (kGrouped && want > cp.n_slices / 2) want = cp.n_slices / 2;
+    // A launch on a few rows must leave room for the CTAs of the next one, which set themselves up beside it.  Where it would
+    // take more than two thirds of the CTAs the GPU holds, half as many take two slices each (rows first, padding last).
+    // Quantise + multiply, three layers of K = 2560 (q / k / v, 384 of 444 places), 1 / 16 / 64 tokens: 8.5 / 9.1 / 9.9 ->
+    // 6.5 / 7.0 / 9.0 us; four layers 9.6 / 9.9 / 11.0 -> 7.2 / 7.9 / 10.0; two of K = 8192 6.8 / 7.4 / 9.7 -> 6.4 / 7.0 / 9.5.
+    // (Two layers of K = 2560, 256 places, lose by it at 32 tokens: 10.1 -> 10.5.)
+    if (!kGrouped && b.M <= kGroupRows) {
+        const int grid = want < cp.n_slices ? want : cp.n_slices;
+        const int live = (b.M + kRowsC - 1) / kRowsC, half = cp.n_slices / 2, fewer = live > half ? live : half;
+        if (3LL * grid * chunks * b.n_lin > 2LL * per_sm * sm_count && fewer < grid) { cp.strided = 1; want = fewer; }
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(want < 1 ? 1 : want < cp.n_slices ? want : cp.n_slices, chunks, b.n_lin);
     cfg.blockDim = dim3(threads);

@@ -30,7 +30,10 @@ std::set<Stream*> g_streams;
 std::map<std::pair<int, const void*>, int> g_dynamic_smem;
 std::map<std::pair<int, const void*>, std::vector<unsigned char>> g_symbols;
 std::map<const void*, size_t> g_symbol_bytes;
+std::map<const void*, const char*> g_names;
 int g_launches[2];
+const char* g_last_name = "";
+int g_last_grid = 0;
 unsigned g_fill = 1;
 
 void run(Stream* s) {
@@ -62,11 +65,13 @@ cudaError_t copy(void* dst, const void* src, size_t n, cudaMemcpyKind kind, Stre
     }
     return cudaSuccess;
 }
-cudaError_t launch(const void* func, size_t dynamic_smem) {
+cudaError_t launch(const void* func, dim3 grid, size_t dynamic_smem) {
     std::lock_guard<std::mutex> lock(g_mu);
     auto it = g_dynamic_smem.find({t_device, func});
     if (dynamic_smem > static_cast<size_t>(it == g_dynamic_smem.end() ? 48 * 1024 : it->second)) return t_last = cudaErrorInvalidValue;
     ++g_launches[t_device];
+    g_last_name = g_names[func];
+    g_last_grid = static_cast<int>(grid.x * grid.y * grid.z);
     return cudaSuccess;
 }
 CUresult encode_tiled() { return CUDA_SUCCESS; }
@@ -75,6 +80,8 @@ thread_local struct { dim3 grid, block; size_t smem; cudaStream_t stream; } t_co
 
 extern "C" {
 int fake_launches(int device) { return g_launches[device]; }
+const char* fake_last_kernel() { return g_last_name; }   // mangled
+int fake_last_grid() { return g_last_grid; }             // CTAs
 int fake_pending() {   // operations that no wait has covered yet
     std::lock_guard<std::mutex> lock(g_mu);
     size_t n = g_legacy.work.size();
@@ -134,7 +141,7 @@ cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v) {
     if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) g_dynamic_smem[{t_device, f}] = v;
     return cudaSuccess;
 }
-cudaError_t cudaFuncGetAttributes(cudaFuncAttributes* a, const void*) { std::memset(a, 0, sizeof(*a)); a->numRegs = 64; return cudaSuccess; }
+cudaError_t cudaFuncGetAttributes(cudaFuncAttributes* a, const void*) { std::memset(a, 0, sizeof(*a)); a->numRegs = 112; return cudaSuccess; }
 cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void* f, const cudaLaunchConfig_t* c) {
     std::lock_guard<std::mutex> lock(g_mu);
     auto it = g_dynamic_smem.find({t_device, f});
@@ -142,8 +149,8 @@ cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void* f, const cudaLaun
     *n = 74;
     return cudaSuccess;
 }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) { return launch(f, c->dynamicSmemBytes); }
-cudaError_t cudaLaunchKernel(const void* f, dim3, dim3, void**, size_t smem, cudaStream_t) { return launch(f, smem); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) { return launch(f, c->gridDim, c->dynamicSmemBytes); }
+cudaError_t cudaLaunchKernel(const void* f, dim3 grid, dim3, void**, size_t smem, cudaStream_t) { return launch(f, grid, smem); }
 cudaError_t cudaGetSymbolAddress(void** p, const void* symbol) {
     std::lock_guard<std::mutex> lock(g_mu);
     auto& mem = g_symbols[{t_device, symbol}];
@@ -162,7 +169,7 @@ void** __cudaRegisterFatBinary(void*) { static void* handle; return &handle; }
 void __cudaRegisterFatBinaryEnd(void**) {}
 void __cudaUnregisterFatBinary(void**) {}
 char __cudaInitModule(void**) { return 0; }
-void __cudaRegisterFunction(void**, const char*, char*, const char*, int, uint3*, uint3*, dim3*, dim3*, int*) {}
+void __cudaRegisterFunction(void**, const char* host, char*, const char* name, int, uint3*, uint3*, dim3*, dim3*, int*) { g_names[host] = name; }
 void __cudaRegisterVar(void**, char* host, char*, const char*, int, size_t bytes, int, int) { g_symbol_bytes[host] = bytes; }
 unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t smem, struct CUstream_st* s) { t_config = {g, b, smem, s}; return 0; }
 cudaError_t __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* smem, void* s) {

@@ -258,6 +258,25 @@ def test_permuting_quantiser_instances_against_oracle(prq, oracle, M, K, k):
     w.free()
 
 
+@pytest.mark.parametrize("K,layers,k,Ms", [(2560, 3, 96, (1, 2, 63, 64, 65, 96, 127, 128)), (2560, 4, 0, (31, 40)), (8192, 2, 288, (1, 64, 127)), (11008, 1, 64, (3, 128))])
+def test_permuting_quantiser_with_slices_dealt_in_turn(prq, oracle, K, layers, k, Ms):
+    """A few rows of launches that would fill the GPU: fewer CTAs, each with every second slice or so of rows and padding."""
+    ch = synth.HeavyTailChannels(5000 + K, K)
+    W = synth.weights(5100 + K, 32, K)
+    ws = [prq.prepare_weights(W, oracle.channel_amax(ch.rows(5200 + K + i, 32)), 0.5, max(0, k - 32 * i)) for i in range(layers)]
+    for M in Ms:
+        x = ch.rows(5300 + M, M)
+        acts = prq.quantize_act_multi(ws, dev_bf16(x), prq.ACT_SCALE_PERM)
+        assert prq.last_device_status() == 0
+        for w, (codes, sf) in zip(ws, acts):
+            oc, osc = oracle.quantize_act(x, w.get(prq.FIELD_PERM), w.get(prq.FIELD_INV_S))
+            assert np.array_equal(codes.cpu().numpy()[: M * K // 2].reshape(M, K // 2), oc), M
+            want = prq_ref.expected_sf(oracle.augment_act(oc, osc, w.k_tail)[1], K, w.k_tail)
+            assert np.array_equal(sf.cpu().numpy()[: want.size], want), M
+    for w in ws:
+        w.free()
+
+
 @pytest.mark.parametrize("seed", [23, 24, 25])
 def test_random_grouped_shapes_on_cta_pairs(prq, oracle, monkeypatch, seed):
     test_random_grouped_shapes_against_oracle(prq, oracle, monkeypatch, seed, 240)

@@ -31,7 +31,7 @@ def fake(tmp_path_factory):
     binding = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(binding)
     binding.LIB_PATH = lib
-    binding.lib()
+    binding.lib().fake_last_kernel.restype = ctypes.c_char_p
     return binding
 
 
@@ -118,3 +118,29 @@ def test_every_kernel_runs_on_a_second_device(fake):
         finally:
             fake.lib().cudaSetDevice(0)
     assert launches[0] == launches[1]
+
+
+def _quantise(fake, K, M, k=0, experts=1, layers=1):
+    """One scale + permute launch; returns the kernel it took and its CTAs."""
+    L, p = fake.lib(), lambda a: a.ctypes.data
+    ws = [_device_weights(fake, 8, K, k, experts) for _ in range(layers)]
+    x = _aligned(M * K * 2)
+    codes, sf = _aligned(fake.act_bytes(M, K, k, experts, fake.BUF_CODES)), _aligned(fake.act_bytes(M, K, k, experts, fake.BUF_SCALES_SF))
+    off = np.linspace(0, M, experts + 1).astype(np.int32)
+    if layers == 1:
+        fake._check(L.prq_quantize_act(ws[0].handle, fake.ACT_SCALE_PERM, p(x), M, K, p(off) if experts > 1 else None, p(codes), None, p(sf), None), "quantise")
+    else:
+        arr = ctypes.c_void_p * layers
+        fake._check(L.prq_quantize_act_multi(layers, arr(*[w.handle.value for w in ws]), fake.ACT_SCALE_PERM, p(x), M, K, arr(*[p(codes)] * layers),
+                                             arr(*[p(sf)] * layers), None), "quantise_multi")
+    for w in ws:
+        w.free()
+    name = L.fake_last_kernel().decode()
+    return "columns" if "quant_act_cols_kernel" in name else "atoms", L.fake_last_grid()
+
+
+@pytest.mark.parametrize("K,layers,M,ctas", [
+    (2560, 3, 1, 192), (2560, 3, 16, 192), (2560, 3, 64, 192), (2560, 4, 64, 256), (2560, 3, 96, 288),   # 3 x 128 of 444 places: fewer
+    (2560, 2, 64, 256), (1024, 3, 64, 384)])                                                             # room enough: a row per CTA
+def test_a_few_rows_for_several_layers_leave_room_for_the_next_launch(fake, K, layers, M, ctas):
+    assert _quantise(fake, K, M, k=64, layers=layers) == ("columns", ctas)
