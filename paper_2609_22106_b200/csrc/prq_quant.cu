@@ -14,9 +14,8 @@
 // residual stages, which is all the "tail copy" this design needs (the GEMM re-reads the tail codes).
 //
 // The scale + permute mode has two structures.  quant_act_cols_kernel (see there) brings whole rows into shared memory
-// by bulk copies and keeps the columns with the lanes; it runs wherever its rows fit.  The column-atom CTAs of
-// quant_act_kernel are left with what it does not serve better: rows too wide for it, and a handful of atoms of
-// stacked experts.
+// by bulk copies and keeps the columns with the lanes.  The column-atom CTAs of quant_act_kernel serve what it does not serve
+// better: very wide rows, and some calls on few rows (the launcher has the lines and what both measured there).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -78,9 +77,9 @@ quant_act_kernel(const QuantBatch b) {
     // atoms of the tail are some twenty times slower than the others: their source columns are scattered over the
     // whole row, every 2-byte read is a 32-byte sector of its own, and the CTA runs at the rate at which its SM's L1
     // takes sectors (about 20 us for 128 rows against 1 us for a head atom, whose window is nearly contiguous).  A
-    // launch could not end before its slowest CTA, which the next kernel of the stream then waited for (8 - 11 us
-    // per call at 4096 tokens).  So the tail atoms are cut into `tail_split` shares of the rows each and come first
-    // in the grid, the head atoms after them.
+    // launch could not end before its slowest CTA, which the next kernel of the stream then waited for.  So the tail
+    // atoms are cut into `tail_split` shares of the rows each and come first in the grid, the head atoms after them
+    // (quantise + multiply, K = 28672, k = 256, without / with: 300 rows 43.5 / 30.2 us, 1024: 88 / 60, 4096: 198 / 183).
     // (counted over the whole layer: the tail units of ALL row groups precede every head atom.)
     int group = static_cast<int>(blockIdx.y) - lin * b.groups_per_lin;
     int atom = blockIdx.x, tail_share = 0, tail_split = 1;
@@ -670,7 +669,8 @@ cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, cudaStr
     const int grid_groups = b.groups_per_lin * b.n_lin;
     cudaLaunchConfig_t cfg = {};
     const int n_atoms = (p.K + kAtomK - 1) / kAtomK;
-    int parts = 1;
+    int parts = 1, k_max = 0;
+    for (int i = 0; i < b.n_lin; ++i) k_max = b.lay[i].k_tail > k_max ? b.lay[i].k_tail : k_max;
     if (scale_perm) {
         // split the rows of a group (a CTA has a fixed cost of about a microsecond, so no further than needed)
         int sms = 0;
@@ -688,13 +688,31 @@ cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, cudaStr
         //   whole width (4096 x 9728: 46.7 -> 20.9, against 22.0 with the columns cut in two);
         //   in between two rows per slice (600 x 2560: 5.5 -> 3.6, 1000 x 6144: 11.5 -> 6.7, 16 x 9728: 2.9 -> 2.8);
         //   stacked experts: eight columns per lane, more warps for narrow rows (K = 768, 128 experts: 1024 tokens 19.5 -> 11.5,
-        //   8192 tokens 62 -> 34), except for a handful of atoms, where looking the experts up is all there is to it
-        //   (16 experts of K = 256, 64 rows: 3.1 against 3.6).
-        // What does not fit twice (K beyond about 13 000, 27 000, 55 000 columns at 4, 2, 1 rows) takes the next smaller
-        // slice and finally the column atoms.
+        //   8192 tokens 62 -> 34).
+        // ... and the column atoms where they are the better ones, judged with the product behind them (quantise + multiply,
+        // column atoms / this structure):
+        //   rows of which two do not fit twice (K > 25728; stacked experts, four rows, 12864).  With one row per slice a CTA has
+        //   five warps for a whole row in shared memory, and every one of the 12 - 21 cuts of the columns brings all of it:
+        //   K = 28672, 16 / 300 / 4096 rows 10.6 / 27 / 149 against 13.9 / 37 / 271; K = 51456 16 / 36 / 263 against 22 / 58 / 464;
+        //   2 to 32 rows where the atoms alone have a CTA per SM (K = 22016, 8 / 32 rows: 8.6 / 9.5 against 9.4 / 10.7;
+        //   K = 18432, below that line: 8.9 / 9.8 against 8.8 / 9.7);
+        //   no tail, or one block of it, and 41 (65) to 128 rows of a narrow layer: there are no scattered reads to save (k = 0,
+        //   64 / 128 rows: K = 2560 7.5 / 8.5 against 7.7 / 9.2, K = 6144 8.2 / 9.8 against 8.7 / 10.4; K = 8192 8.0 / 10.2 against 7.7 /
+        //   9.8; k = 128, K = 2560: 9.2 / 10.0 against 7.7 / 9.2);
+        //   stacked experts of one atom (128 experts of K = 128, 4096 / 65536 rows: 14.4 / 45 against 16.0 / 50); up to 64 atoms, where
+        //   looking the experts up is all there is to it; up to 128 rows while the atoms' launch stays within 768 CTAs (2 experts
+        //   of K = 3072, 8 / 128 rows: 10.2 / 11.0 against 10.7 / 12.1; 8 of K = 2048, beyond that line: 11.3 / 12.2 against 9.7 / 10.8).
         const bool grouped = b.expert_offsets != nullptr;
         auto fits = [&](int rows) { return 4 * static_cast<size_t>(rows) * p.K + 10240 <= kColsSmem - 9216; };
-        bool cols = !(grouped && static_cast<long long>(grid_groups) * n_atoms <= 64);
+        bool cols;
+        if (grouped) {
+            cols = n_atoms > 1 && tiles > 64 && !(b.M <= 128 && tiles * parts <= 768);
+        } else {
+            const bool wide_few = b.M > 1 && b.M <= 32 && tiles >= sms;
+            const bool narrow_flat = b.M <= 128 && p.K <= 6144 && tiles >= 16 && tiles <= 80 &&
+                                     ((k_max == 0 && b.M > 40) || (k_max <= kBlock && b.M > 64));
+            cols = !wide_few && !narrow_flat;
+        }
         if (const char* ev = dev_knobs_enabled() ? getenv("PRQ_QUANT_ROWS") : nullptr) cols = atoi(ev) != 0;
         if (cols && grouped && fits(4)) return launch_cols_impl<8, 4, true, 544>(b, sms, stream);
         if (cols && !grouped) {
@@ -703,7 +721,6 @@ cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, cudaStr
             if (large && p.K <= 8192) return launch_cols_impl<16, 4, false, 384>(b, sms, stream);
             if (large && fits(2)) return launch_cols_impl<16, 2, false, 640>(b, sms, stream);
             if (fits(2)) return launch_cols_impl<16, 2, false, 320>(b, sms, stream);
-            if (fits(1)) return launch_cols_impl<16, 1, false, 192>(b, sms, stream);
         }
     }
     // the tail atoms of the scale + permute mode in shares of 16 rows (128 / 8), see the kernel
@@ -714,8 +731,6 @@ cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, cudaStr
     // cost of finding its expert -- eight times as many tail CTAs made the 128-expert quantiser 35-50 % slower, and its
     // launches are long enough for a 20 us CTA not to be their end)
     if (scale_perm && b.expert_offsets == nullptr) {
-        int k_max = 0;
-        for (int i = 0; i < b.n_lin; ++i) k_max = b.lay[i].k_tail > k_max ? b.lay[i].k_tail : k_max;
         bb.n_tail = (k_max + kAtomK - 1) / kAtomK < n_atoms ? (k_max + kAtomK - 1) / kAtomK : n_atoms;
         bb.tail_split = 8 / parts;
     }

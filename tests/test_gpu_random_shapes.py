@@ -241,7 +241,8 @@ def test_permuting_quantiser_structures_against_oracle(prq, oracle, monkeypatch,
 
 
 @pytest.mark.parametrize("M,K,k", [(128, 4096, 96), (129, 4128, 32), (1499, 2048, 64), (1500, 2016, 2016), (1501, 2080, 160),
-                                   (1502, 8192, 0), (1505, 8224, 288), (9, 9760, 64), (3, 13760, 96), (2, 27040, 32)])
+                                   (1502, 8192, 0), (1505, 8224, 288), (9, 9760, 64), (3, 13760, 96), (2, 27040, 32),
+                                   (130, 25760, 160), (33, 18976, 0), (7, 18976, 96), (1, 51488, 64), (65, 4128, 32), (41, 6112, 0)])
 def test_permuting_quantiser_instances_against_oracle(prq, oracle, M, K, k):
     """Both sides of every line of the launcher's rule (rows, columns, what fits shared memory), with partial slices,
     odd block counts and tails that straddle atoms: codes and scale bytes are whole numbers, so nothing may differ."""
@@ -255,6 +256,24 @@ def test_permuting_quantiser_instances_against_oracle(prq, oracle, M, K, k):
     assert np.array_equal(codes.cpu().numpy()[: M * K // 2].reshape(M, K // 2), oc)
     want = prq_ref.expected_sf(oracle.augment_act(oc, osc, k)[1], K, k)
     assert np.array_equal(sf.cpu().numpy()[: want.size], want)
+    w.free()
+
+
+@pytest.mark.parametrize("counts,K,k", [([70, 0, 90], 12896, 96), ([40] * 4, 12864, 64), ([1, 2, 0, 5], 3072, 32), ([300, 500], 128, 96)])
+def test_permuting_quantiser_of_stacked_experts_at_the_lines(prq, oracle, counts, K, k):
+    """Both structures for stacked experts at the edges of the launcher's rule: rows too wide, few rows, one atom."""
+    E, M = len(counts), sum(counts)
+    off = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
+    ch = synth.HeavyTailChannels(6000 + K, K)
+    w = prq.prepare_weights(np.stack([synth.weights(6100 + e, 8, K) for e in range(E)]), np.stack([oracle.channel_amax(ch.rows(6200 + e, 16)) for e in range(E)]), 0.5, k)
+    x = ch.rows(6300, M)
+    codes, srow, _ = prq.quantize_act(w, dev_bf16(x), prq.ACT_SCALE_PERM, expert_offsets=torch.from_numpy(off).cuda(), row_scales=True)
+    assert prq.last_device_status() == 0
+    for e in range(E):
+        r = slice(int(off[e]), int(off[e + 1]))
+        oc, osc = oracle.quantize_act(x[r], w.get(prq.FIELD_PERM, e), w.get(prq.FIELD_INV_S, e))
+        assert np.array_equal(codes.cpu().numpy()[: M * K // 2].reshape(M, K // 2)[r], oc)
+        assert np.array_equal(srow.cpu().numpy()[: M * K // 32].reshape(M, K // 32)[r], osc)
     w.free()
 
 

@@ -144,3 +144,18 @@ def _quantise(fake, K, M, k=0, experts=1, layers=1):
     (2560, 2, 64, 256), (1024, 3, 64, 384)])                                                             # room enough: a row per CTA
 def test_a_few_rows_for_several_layers_leave_room_for_the_next_launch(fake, K, layers, M, ctas):
     assert _quantise(fake, K, M, k=64, layers=layers) == ("columns", ctas)
+
+
+@pytest.mark.parametrize("want,K,M,k,experts", [
+    # rows of which two do not fit twice, up to the widest that one did
+    ("columns", 25728, 300, 64, 1), ("atoms", 25760, 300, 64, 1), ("atoms", 28672, 4096, 64, 1), ("atoms", 51456, 16, 0, 1),
+    # a CTA per SM from the atoms alone, two to 32 rows
+    ("columns", 18816, 8, 64, 1), ("atoms", 18944, 8, 64, 1), ("columns", 18944, 1, 64, 1), ("atoms", 22016, 32, 0, 1), ("columns", 22016, 33, 64, 1),
+    # nothing scattered to gather, 41 (65) to 128 rows of a narrow layer
+    ("columns", 2560, 40, 0, 1), ("atoms", 2560, 41, 0, 1), ("atoms", 2560, 128, 0, 1), ("columns", 2560, 129, 0, 1), ("columns", 2560, 64, 32, 1),
+    ("atoms", 2560, 65, 32, 1), ("columns", 2560, 65, 64, 1), ("columns", 1024, 64, 0, 1), ("atoms", 6144, 64, 0, 1), ("columns", 8192, 64, 0, 1),
+    # stacked experts: one atom, a handful of atoms, a few rows, and what the structure is for
+    ("atoms", 128, 2000, 32, 8), ("columns", 160, 9000, 32, 8), ("atoms", 256, 3800, 32, 2), ("columns", 256, 4000, 32, 2), ("atoms", 3072, 128, 64, 2),
+    ("columns", 3072, 129, 64, 2), ("columns", 2048, 64, 64, 8), ("columns", 12864, 600, 64, 2), ("atoms", 12896, 600, 64, 2)])
+def test_which_structure_quantises(fake, want, K, M, k, experts):
+    assert _quantise(fake, K, M, k, experts)[0] == want
