@@ -316,6 +316,16 @@ Fp8Schedule fp8_schedule(int M, int N, DeviceInfo* di) {
     return best;
 }
 
+// Grouped product: CTA pairs on 256 x 240 tiles instead of a CTA per 128-token tile (the measurements stand at the call).
+// An expert's last tile is counted as half full.
+bool grouped_pairs_pay(int M, int n_experts, int N, long long wide_cols, int S, bool y_bf16, int pairs) {
+    const long long half_tiles = (2LL * M + 256LL * n_experts) / 256 * (wide_cols / kPrefillTileWide);   // twice the tiles
+    auto tokens = [&](int t) { return M >= static_cast<long long>(t) * n_experts; };
+    if (2 * wide_cols > 3LL * N || half_tiles < 5LL * pairs) return false;
+    if (!y_bf16) return tokens(768) && S >= 5;
+    return tokens(512) || (tokens(224) && S <= 5 && 4 * wide_cols <= 5LL * N && half_tiles >= 8LL * pairs);
+}
+
 // Two counters ("arrived", "finished") per 128-row half of a 256 x 224 pair tile: first all the "arrived"
 // counters, then all the "finished" ones.
 size_t prefill_flag_count(const prq_weights* w, int M) {
@@ -1434,13 +1444,19 @@ prq_status prq_linear_grouped(const prq_weights* w, const void* codes, const voi
     // token tile: 64 rows when the experts hold a handful of tokens each (the smaller tile leaves room for a deeper
     // ring of weight tiles in flight), 128 otherwise (every extra token tile of an expert re-reads its weight tiles)
     int bn = static_cast<long long>(M_total) <= 64LL * w->n_experts ? 64 : 128;
-    // ... and CTA pairs on 256 x 240 tiles from 224 tokens per expert on, unless the 240-column tiles cover half as much
-    // again as N: less operand traffic per output, but an expert's last tile is padded to 256 (E x N x K + k, tokens per
-    // expert, microseconds 128-token tiles / pairs: 128 x 2048 x 832, 512: 116 / 104, 256: 64.7 / 64.3, 128: 43.3 / 47.3;
-    // 16 x 2048 x 832, 250: 13.3 / 12.0; 32 x 1400 x 672, 750: 41.9 / 32.7; 16 x 512 x 256, 4096: 24.6 / 19.9)
-    const long long wide_cols = static_cast<long long>((w->N + kPrefillTileWide - 1) / kPrefillTileWide) * kPrefillTileWide;
-    const bool pairs_fit = w->d_sf_alt[kAltWide] && (static_cast<long long>(M_total) / 256 + w->n_experts) * (wide_cols / kPrefillTileWide) < (1ll << 30);
-    if (pairs_fit && M_total >= 224LL * w->n_experts && 2 * wide_cols <= 3LL * w->N) bn = kPrefillTileWide;
+    // ... and CTA pairs on 256 x 240 tiles where experts hold many tokens and the pairs get several tiles each: less operand
+    // traffic per output, but an expert's last tile is padded to 256 tokens, few tiles leave most pairs idle, and fp32 output
+    // leaves the epilogue in front of a short reduction (quantise + product, operands rotated over more than L2, E x N x K + k,
+    // tokens per expert, microseconds 128-token tiles / pairs):
+    //   bf16, taken from 512 tokens on and 2.5 tiles per pair: 16 x 2048 x 1600, 768: 53.1 / 45.5, 32 x 1000 x 4160, 512: 85.0 / 72.5;
+    //     left alone: 4 x 1024 x 256, 512 (0.7 tiles): 7.8 / 9.1, 2 x 1408 x 832, 224 (0.3): 10.3 / 11.7;
+    //   bf16 with fewer tokens, taken while the reduction is short, the padding of N at most a quarter and 4 tiles per pair are
+    //     there: 128 x 1408 x 832, 256: 58.3 / 50.6, 16 x 4096 x 256, 384: 24.3 / 20.9; left alone: 64 x 2048 x 2048, 384: 90 / 99;
+    //   fp32, taken from 768 tokens on with five stages or more: 32 x 2560 x 4096, 768: 261 / 224; left alone:
+    //     64 x 1408 x 1536, 640: 105 / 119, 32 x 768 x 576, 640: 29.5 / 32.2, 4 x 1024 x 320, 1024: 11.4 / 14.6.
+    const long long wide_tiles = (w->N + kPrefillTileWide - 1) / kPrefillTileWide, wide_cols = wide_tiles * kPrefillTileWide;
+    const bool pairs_fit = w->d_sf_alt[kAltWide] && (static_cast<long long>(M_total) / 256 + w->n_experts) * wide_tiles < (1ll << 30);
+    if (pairs_fit && grouped_pairs_pay(M_total, w->n_experts, w->N, wide_cols, w->plan.S, y_dtype == PRQ_BF16, di->num_sms / 2)) bn = kPrefillTileWide;
     const int forced = env_int("PRQ_GROUPED_BN", 0);   // developer switch
     if (forced) bn = forced;
     if (bn == kPrefillTileWide) {

@@ -159,3 +159,22 @@ def test_a_few_rows_for_several_layers_leave_room_for_the_next_launch(fake, K, l
     ("columns", 3072, 129, 64, 2), ("columns", 2048, 64, 64, 8), ("columns", 12864, 600, 64, 2), ("atoms", 12896, 600, 64, 2)])
 def test_which_structure_quantises(fake, want, K, M, k, experts):
     assert _quantise(fake, K, M, k, experts)[0] == want
+
+
+@pytest.mark.parametrize("want,E,N,K,M,bf16", [
+    # the benchmark's expert projection at prefill; few tiles for the pairs; the padding of N
+    ("pairs", 128, 2048, 768, 65536, True), ("tiles", 4, 1024, 256, 2048, True), ("tiles", 2, 1408, 768, 448, True), ("tiles", 128, 256, 768, 65536, True),
+    ("pairs", 16, 1000, 2048, 8192, True), ("tiles", 16, 1000, 2048, 8191, True), ("tiles", 8, 1000, 2048, 5000, True),
+    # 224 to 511 tokens per expert: short reductions, little padding, four tiles per pair
+    ("pairs", 128, 1408, 768, 32768, True), ("tiles", 128, 1408, 1312, 32768, True), ("tiles", 16, 1408, 768, 4096, True), ("tiles", 128, 1408, 768, 28671, True),
+    ("tiles", 128, 512, 768, 32768, True),
+    # fp32 output: long reductions and many tokens only
+    ("tiles", 128, 2048, 768, 65536, False), ("pairs", 32, 2560, 1280, 24576, False), ("tiles", 32, 2560, 1280, 24575, False), ("tiles", 32, 2560, 1024, 24576, False)])
+def test_which_tiles_the_grouped_product_takes(fake, want, E, N, K, M, bf16):
+    W, amax, h = np.zeros((E, N, K), np.uint16), np.ones((E, K), np.float32), ctypes.c_void_p()
+    fake._check(fake.lib().prq_prepare_weights_device(W.ctypes.data, E, N, K, amax.ctypes.data, 0.5, 0, None, None, ctypes.byref(h)), "prepare")
+    w, off, some = fake.Weights(h), np.linspace(0, M, E + 1).astype(np.int32), _aligned(16)   # (nothing is read or written: the kernels do not run)
+    fake._check(fake.lib().prq_linear_grouped(w.handle, some.ctypes.data, some.ctypes.data, off.ctypes.data, M, some.ctypes.data, (N + 7) // 8 * 8,
+                                              fake.BF16 if bf16 else fake.F32, None), "grouped")
+    assert ("pairs" if "grouped_pair" in fake.lib().fake_last_kernel().decode() else "tiles") == want
+    w.free()
