@@ -326,18 +326,30 @@ def new_workspace(w: Weights, M: int, device="cuda"):
     return torch.zeros(max(linear_workspace_bytes(w, M), 16), dtype=torch.uint8, device=device)
 
 
+def _workspace_for_one_call(w: Weights, M: int, device):
+    """Only what one call counts on is cleared (the partial tiles behind the counters are written before they are read), not
+    tens of megabytes."""
+    import torch
+
+    workspace = torch.empty(max(linear_workspace_bytes(w, M), 16), dtype=torch.uint8, device=device)
+    clear = int(lib().prq_linear_workspace_clear_bytes(w.handle, M))
+    if clear:
+        workspace[:clear].zero_()
+    return workspace
+
+
 def linear(w: Weights, codes, scales_sf, M: int, y_dtype: int = F32, workspace=None, out=None, stream=None):
     import torch
 
     if out is None:
         out = torch.empty((M, w.N), dtype=torch.float32 if y_dtype == F32 else torch.bfloat16, device=codes.device)
     if workspace is None and M > 128:   # up to 128 tokens the kernel needs no scratch: nothing to allocate or clear
-        # a workspace for this call alone: only what this call counts on is cleared (the partial tiles behind the counters
-        # are written before they are read), not tens of megabytes
-        workspace = torch.empty(max(linear_workspace_bytes(w, M), 16), dtype=torch.uint8, device=codes.device)
-        clear = int(lib().prq_linear_workspace_clear_bytes(w.handle, M))
-        if clear:
-            workspace[:clear].zero_()
+        if stream is None:
+            workspace = _workspace_for_one_call(w, M, codes.device)
+        else:   # on the stream of the call: cleared in front of the kernel, and given back behind it
+            on = stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(stream.cuda_stream, device=codes.device)
+            with torch.cuda.stream(on):
+                workspace = _workspace_for_one_call(w, M, codes.device)
     _check(lib().prq_linear(w.handle, _dptr(codes), _dptr(scales_sf), M, _dptr(out), out.stride(0) if M else w.N,
                             y_dtype, _dptr(workspace), workspace.numel() if workspace is not None else 0,
                             _stream_ptr(stream)), "prq_linear")

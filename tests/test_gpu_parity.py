@@ -208,6 +208,29 @@ def test_linear_without_a_workspace(prq, M, N, K, k):
     w.free()
 
 
+def test_linear_without_a_workspace_on_another_stream(prq):
+    """The workspace that linear() takes for itself belongs to the stream of the call: right while the current stream is
+    busy, with memory that held other bytes before, and while later tensors of the current stream are written."""
+    N, K, k, M = 256, 9728, 256, 200   # every tile is cut along K
+    w = prq.prepare_weights_device(torch.randn(N, K, device="cuda").to(torch.bfloat16), np.ones(K, np.float32), 0.5, k)
+    x = to_dev_bf16(synth.HeavyTailChannels(73, K).rows(74, M))
+    codes, _, sf = prq.quantize_act(w, x)
+    want = prq.linear(w, codes, sf, M, workspace=prq.new_workspace(w, M))
+    side, busy, y = torch.cuda.Stream(), torch.randn(8192, 8192, device="cuda"), torch.empty_like(want)
+    for _ in range(3):
+        dirty = [torch.full((prq.linear_workspace_bytes(w, M),), 0x55, dtype=torch.uint8, device="cuda") for _ in range(2)]
+        torch.cuda.synchronize()
+        del dirty
+        busy @ busy
+        prq.linear(w, codes, sf, M, out=y, stream=side)
+        later = [torch.full((prq.linear_workspace_bytes(w, M),), 0x77, dtype=torch.uint8, device="cuda") for _ in range(2)]
+        side.synchronize()
+        assert prq.last_device_status() == 0
+        assert torch.equal(y, want)
+        del later
+    w.free()
+
+
 def test_k0_runs_the_same_kernels_as_plain_mxfp4(prq, oracle):
     """k = 0: the product is plain W4A4 MXFP4 of (x, W D); with alpha = 0 of (x, W) themselves."""
     L = synth.layer(93, 256, 1024, 200, T_cal=32)

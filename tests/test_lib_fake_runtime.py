@@ -178,3 +178,36 @@ def test_which_tiles_the_grouped_product_takes(fake, want, E, N, K, M, bf16):
                                               fake.BF16 if bf16 else fake.F32, None), "grouped")
     assert ("pairs" if "grouped_pair" in fake.lib().fake_last_kernel().decode() else "tiles") == want
     w.free()
+
+
+def test_a_workspace_of_its_own_belongs_to_the_stream_of_the_call(fake, monkeypatch):
+    """linear() without a workspace on a stream that is not the current one: the workspace comes from that stream's memory
+    pool and is cleared there, in front of the kernel that counts on it; it goes back to that pool when the call returns."""
+    import contextlib
+
+    import torch
+
+    current, done = [None], []
+
+    @contextlib.contextmanager
+    def on(stream):
+        current.append(stream)
+        yield
+        current.pop()
+
+    class Side:
+        cuda_stream = 0
+
+    side, real_empty, real_zero = Side(), torch.empty, torch.Tensor.zero_
+    monkeypatch.setattr(torch.cuda, "stream", on)
+    monkeypatch.setattr(torch.cuda, "ExternalStream", lambda number, device: side)
+    monkeypatch.setattr(torch, "empty", lambda *a, **k: (done.append(("empty", current[-1])), real_empty(*a, **k))[1])
+    monkeypatch.setattr(torch.Tensor, "zero_", lambda t: (done.append(("zero", current[-1])), real_zero(t))[1])
+    N, K, M = 256, 9728, 200        # a call that cuts its tiles along K
+    w = fake.prepare_weights(np.zeros((N, K), np.uint16), np.ones(K, np.float32), 0.5, 0)
+    t = lambda n: torch.frombuffer(memoryview(_aligned(n)), dtype=torch.uint8)
+    codes, sf, y = t(M * K // 2), t(fake.act_bytes(M, K, 0, 1, fake.BUF_SCALES_SF)), t(M * N * 4).view(torch.float32).view(M, N)
+    fake.linear(w, codes, sf, M, out=y, stream=side)
+    assert done == [("empty", side), ("zero", side)]
+    monkeypatch.undo()
+    w.free()
