@@ -5,7 +5,8 @@
 #include <cstdlib>
 #include <cstddef>
 #include <cstdint>
-#include <system_error>
+#include <exception>
+#include <new>
 #include <thread>
 #include <vector>
 
@@ -81,23 +82,32 @@ __host__ __device__ inline int sf_offset_in_group(int r, int blk_in_stage) {
     return (blk_in_stage >> 2) * 512 + (r & 31) * 16 + (r >> 5) * 4 + (blk_in_stage & 3);
 }
 
-// body(lo, hi) over [0, n) on the host's threads.  A thread that cannot be started leaves its share to the caller.
+// body(lo, hi) over [0, n) on the host's threads.  Threads that cannot be had (no memory, no more of them) leave their shares
+// to the caller; an exception of the caller's own share leaves only when the others are through.
 template <class F>
 void parallel_for(long n, F&& body) {
+    struct Threads {
+        std::vector<std::thread> list;
+        ~Threads() { for (auto& t : list) t.join(); }
+    } th;
     const unsigned hw = std::thread::hardware_concurrency();
-    const long nt = std::min<long>(std::max(1u, std::min(hw, 64u)), std::max<long>(1, n));
-    std::vector<std::thread> th;
-    th.reserve(nt);
+    long nt = std::min<long>(std::max(1u, std::min(hw, 64u)), std::max<long>(1, n));
+    try {
+        th.list.reserve(nt);
+    } catch (const std::bad_alloc&) {
+        nt = 1;
+    }
     for (long t = 1; t < nt; ++t) {
         const long lo = n * t / nt, hi = n * (t + 1) / nt;
+        bool started = true;
         try {
-            th.emplace_back([=, &body] { body(lo, hi); });
-        } catch (const std::system_error&) {
-            body(lo, hi);
+            th.list.emplace_back([=, &body] { body(lo, hi); });
+        } catch (const std::exception&) {   // std::system_error or std::bad_alloc
+            started = false;
         }
+        if (!started) body(lo, hi);
     }
     body(0, n / nt);
-    for (auto& x : th) x.join();
 }
 
 struct PrepResult {

@@ -214,3 +214,15 @@ def test_mxfp8_host_prep_is_bit_exact(prq, oracle):
     # the format carries no tail
     with pytest.raises(prq.PrqError):
         prq.prepare_weights_host(Wb, np.ones(32, np.float32), 0.0, 32, fmt=prq.FMT_MXFP8)
+
+
+def test_host_threads_that_cannot_be_had(tmp_path):
+    """The host preparation's work sharing when memory for its threads runs out: done by the caller, no abort."""
+    import subprocess
+
+    exe = str(tmp_path / "parallel_for")
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-I", os.path.join(ROOT, "paper_2609_22106_b200", "csrc"), "-I", os.path.join(ROOT, "include"),
+                           "-I", "/usr/local/cuda/include", "-o", exe, os.path.join(ROOT, "tests", "parallel_for_out_of_memory.cpp"), "-lpthread",
+                           "-L/usr/local/cuda/lib64", "-lcudart_static", "-ldl", "-lrt"])
+    r = subprocess.run([exe], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, (r.returncode, r.stdout[-500:], r.stderr[-500:])
