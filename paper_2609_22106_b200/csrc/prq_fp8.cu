@@ -181,7 +181,7 @@ prq_status prepare_layer_fp8(const uint16_t* W, int N, int K, const float* amax,
                 scales[static_cast<size_t>(n) * (K / kBlock) + b] = static_cast<uint8_t>(byte);
                 for (int i = 0; i < kBlock; ++i) codes[static_cast<size_t>(n) * K + b * kBlock + i] = e4m3_code(v[i], byte - 127);
             }
-    });
+    }, 1 + 16384 / K);   // 12 ns per element: 0.2 ms to a thread (8 x 64: 0.33 ms with a thread per row, 0.03 as now)
     return finite.load() ? PRQ_OK : PRQ_ERR_NONFINITE;
 }
 

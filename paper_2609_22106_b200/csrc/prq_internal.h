@@ -82,16 +82,16 @@ __host__ __device__ inline int sf_offset_in_group(int r, int blk_in_stage) {
     return (blk_in_stage >> 2) * 512 + (r & 31) * 16 + (r >> 5) * 4 + (blk_in_stage & 3);
 }
 
-// body(lo, hi) over [0, n) on the host's threads.  Threads that cannot be had (no memory, no more of them) leave their shares
+// body(lo, hi) over [0, n) on the host's threads, `at_least` items to a thread (starting one costs some 40 us).  Threads that cannot be had (no memory, no more of them) leave their shares
 // to the caller; an exception of the caller's own share leaves only when the others are through.
 template <class F>
-void parallel_for(long n, F&& body) {
+void parallel_for(long n, F&& body, long at_least = 1) {
     struct Threads {
         std::vector<std::thread> list;
         ~Threads() { for (auto& t : list) t.join(); }
     } th;
     const unsigned hw = std::thread::hardware_concurrency();
-    long nt = std::min<long>(std::max(1u, std::min(hw, 64u)), std::max<long>(1, n));
+    long nt = std::min<long>(std::max(1u, std::min(hw, 64u)), std::max<long>(1, n / std::max(1l, at_least)));
     try {
         th.list.reserve(nt);
     } catch (const std::bad_alloc&) {

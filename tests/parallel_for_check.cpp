@@ -1,5 +1,5 @@
 // parallel_for when threads cannot be had: every allocation from the n-th on fails.  The work must be done all the same, and
-// nothing may end the process (the callers are C entry points).
+// nothing may end the process (the callers are C entry points).  And no thread for less than `at_least` items.
 #include <cstdio>
 #include <cstdlib>
 #include <new>
@@ -25,6 +25,9 @@ int main() {
         g_fail = false;
         if (done != 1000) { std::printf("%d allocations: %ld of 1000\n", left, done.load()); return 1; }
     }
+    std::atomic<int> shares{0};
+    prq::parallel_for(599, [&](long, long) { ++shares; }, 300);
+    if (shares != 1) return 1;
     // an exception of the caller's own share arrives after the other shares are through
     std::atomic<long> done{0};
     bool caught = false;

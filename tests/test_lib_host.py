@@ -222,7 +222,7 @@ def test_host_threads_that_cannot_be_had(tmp_path):
 
     exe = str(tmp_path / "parallel_for")
     subprocess.check_call(["g++", "-std=c++17", "-O1", "-I", os.path.join(ROOT, "paper_2609_22106_b200", "csrc"), "-I", os.path.join(ROOT, "include"),
-                           "-I", "/usr/local/cuda/include", "-o", exe, os.path.join(ROOT, "tests", "parallel_for_out_of_memory.cpp"), "-lpthread",
+                           "-I", "/usr/local/cuda/include", "-o", exe, os.path.join(ROOT, "tests", "parallel_for_check.cpp"), "-lpthread",
                            "-L/usr/local/cuda/lib64", "-lcudart_static", "-ldl", "-lrt"])
     r = subprocess.run([exe], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, (r.returncode, r.stdout[-500:], r.stderr[-500:])
