@@ -321,9 +321,9 @@ Fp8Schedule fp8_schedule(int M, int N, DeviceInfo* di) {
 bool grouped_pairs_pay(int M, int n_experts, int N, long long wide_cols, int S, bool y_bf16, int pairs) {
     const long long half_tiles = (2LL * M + 256LL * n_experts) / 256 * (wide_cols / kPrefillTileWide);   // twice the tiles
     auto tokens = [&](int t) { return M >= static_cast<long long>(t) * n_experts; };
-    if (2 * wide_cols > 3LL * N || half_tiles < 5LL * pairs) return false;
-    if (!y_bf16) return tokens(768) && S >= 5;
-    return tokens(512) || (tokens(224) && S <= 5 && 4 * wide_cols <= 5LL * N && half_tiles >= 8LL * pairs);
+    if (2 * wide_cols > 3LL * N) return false;
+    if (!y_bf16) return tokens(768) && S >= 5 && half_tiles >= 5LL * pairs;
+    return (tokens(224) && S <= 5 && half_tiles >= 3LL * pairs) || (tokens(512) && half_tiles >= 4LL * pairs);
 }
 
 // Two counters ("arrived", "finished") per 128-row half of a 256 x 224 pair tile: first all the "arrived"
@@ -1448,10 +1448,11 @@ prq_status prq_linear_grouped(const prq_weights* w, const void* codes, const voi
     // traffic per output, but an expert's last tile is padded to 256 tokens, few tiles leave most pairs idle, and fp32 output
     // leaves the epilogue in front of a short reduction (quantise + product, operands rotated over more than L2, E x N x K + k,
     // tokens per expert, microseconds 128-token tiles / pairs):
-    //   bf16, taken from 512 tokens on and 2.5 tiles per pair: 16 x 2048 x 1600, 768: 53.1 / 45.5, 32 x 1000 x 4160, 512: 85.0 / 72.5;
-    //     left alone: 4 x 1024 x 256, 512 (0.7 tiles): 7.8 / 9.1, 2 x 1408 x 832, 224 (0.3): 10.3 / 11.7;
-    //   bf16 with fewer tokens, taken while the reduction is short, the padding of N at most a quarter and 4 tiles per pair are
-    //     there: 128 x 1408 x 832, 256: 58.3 / 50.6, 16 x 4096 x 256, 384: 24.3 / 20.9; left alone: 64 x 2048 x 2048, 384: 90 / 99;
+    //   bf16 and up to five stages, taken from 224 tokens on and 1.5 tiles per pair: 128 x 1408 x 832, 256: 58.3 / 50.6, 16 x 1424 x 800,
+    //     422: 25.1 / 21.9, 32 x 720 x 480, 255: 20.5 / 18.8; left alone: 4 x 1024 x 256, 512 (0.7 tiles): 7.8 / 9.1, 2 x 1408 x 832,
+    //     224 (0.3): 10.3 / 11.7;
+    //   bf16 and longer reductions, taken from 512 tokens on and two tiles per pair: 16 x 2048 x 1600, 768: 53.1 / 45.5, 32 x 1000 x
+    //     4160, 512: 85.0 / 72.5; left alone: 64 x 2048 x 2048, 384: 90 / 99, 32 x 1536 x 4096, 300: 63.8 / 69.2;
     //   fp32, taken from 768 tokens on with five stages or more: 32 x 2560 x 4096, 768: 261 / 224; left alone:
     //     64 x 1408 x 1536, 640: 105 / 119, 32 x 768 x 576, 640: 29.5 / 32.2, 4 x 1024 x 320, 1024: 11.4 / 14.6.
     const long long wide_tiles = (w->N + kPrefillTileWide - 1) / kPrefillTileWide, wide_cols = wide_tiles * kPrefillTileWide;

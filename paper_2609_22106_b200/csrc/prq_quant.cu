@@ -700,13 +700,17 @@ cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, cudaStr
         //   64 / 128 rows: K = 2560 7.5 / 8.5 against 7.7 / 9.2, K = 6144 8.2 / 9.8 against 8.7 / 10.4; K = 8192 8.0 / 10.2 against 7.7 /
         //   9.8; k = 128, K = 2560: 9.2 / 10.0 against 7.7 / 9.2);
         //   stacked experts of one atom (128 experts of K = 128, 4096 / 65536 rows: 14.4 / 45 against 16.0 / 50); up to 64 atoms, where
-        //   looking the experts up is all there is to it; up to 128 rows while the atoms' launch stays within 768 CTAs (2 experts
-        //   of K = 3072, 8 / 128 rows: 10.2 / 11.0 against 10.7 / 12.1; 8 of K = 2048, beyond that line: 11.3 / 12.2 against 9.7 / 10.8).
+        //   looking the experts up is all there is to it; up to 128 rows while the atoms' launch is small (2 experts of K = 3072,
+        //   8 / 128 rows: 10.2 / 11.0 against 10.7 / 12.1, 32 of K = 256, 64 rows: 8.0 against 8.7; beyond those lines 8 of K = 2048:
+        //   11.3 / 12.2 against 9.7 / 10.8, 16 of K = 640, 64 rows: 9.2 against 9.0); three atoms, which leave every second warp half
+        //   idle, while the atoms' CTAs fit the GPU at once (64 experts of K = 384, 64 / 512 rows: 10.0 / 12.3 against 11.0 / 13.1).
         const bool grouped = b.expert_offsets != nullptr;
         auto fits = [&](int rows) { return 4 * static_cast<size_t>(rows) * p.K + 10240 <= kColsSmem - 9216; };
         bool cols;
         if (grouped) {
-            cols = n_atoms > 1 && tiles > 64 && !(b.M <= 128 && tiles * parts <= 768);
+            const bool few = b.M <= 128 && tiles * parts <= (b.n_experts <= 4 ? 768 : 576);
+            const bool three = n_atoms == 3 && b.M <= 1024 && parts == 4 && tiles <= 216;
+            cols = n_atoms > 1 && tiles > 64 && !few && !three;
         } else {
             const bool wide_few = b.M > 1 && b.M <= 32 && tiles >= sms;
             const bool narrow_flat = b.M <= 128 && p.K <= 6144 && tiles >= 16 && tiles <= 80 &&

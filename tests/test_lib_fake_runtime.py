@@ -156,18 +156,19 @@ def test_a_few_rows_for_several_layers_leave_room_for_the_next_launch(fake, K, l
     ("atoms", 2560, 65, 32, 1), ("columns", 2560, 65, 64, 1), ("columns", 1024, 64, 0, 1), ("atoms", 6144, 64, 0, 1), ("columns", 8192, 64, 0, 1),
     # stacked experts: one atom, a handful of atoms, a few rows, and what the structure is for
     ("atoms", 128, 2000, 32, 8), ("columns", 160, 9000, 32, 8), ("atoms", 256, 3800, 32, 2), ("columns", 256, 4000, 32, 2), ("atoms", 3072, 128, 64, 2),
-    ("columns", 3072, 129, 64, 2), ("columns", 2048, 64, 64, 8), ("columns", 12864, 600, 64, 2), ("atoms", 12896, 600, 64, 2)])
+    ("columns", 3072, 129, 64, 2), ("columns", 2048, 64, 64, 8), ("columns", 640, 128, 64, 16), ("atoms", 256, 128, 64, 32),
+    ("columns", 384, 512, 64, 32), ("atoms", 384, 512, 64, 64), ("columns", 384, 2048, 64, 64), ("columns", 12864, 600, 64, 2), ("atoms", 12896, 600, 64, 2)])
 def test_which_structure_quantises(fake, want, K, M, k, experts):
     assert _quantise(fake, K, M, k, experts)[0] == want
 
 
 @pytest.mark.parametrize("want,E,N,K,M,bf16", [
-    # the benchmark's expert projection at prefill; few tiles for the pairs; the padding of N
+    # the benchmark's expert projection at prefill; few tiles for the pairs; the padding of N; few tokens per expert
     ("pairs", 128, 2048, 768, 65536, True), ("tiles", 4, 1024, 256, 2048, True), ("tiles", 2, 1408, 768, 448, True), ("tiles", 128, 256, 768, 65536, True),
-    ("pairs", 16, 1000, 2048, 8192, True), ("tiles", 16, 1000, 2048, 8191, True), ("tiles", 8, 1000, 2048, 5000, True),
-    # 224 to 511 tokens per expert: short reductions, little padding, four tiles per pair
-    ("pairs", 128, 1408, 768, 32768, True), ("tiles", 128, 1408, 1312, 32768, True), ("tiles", 16, 1408, 768, 4096, True), ("tiles", 128, 1408, 768, 28671, True),
-    ("tiles", 128, 512, 768, 32768, True),
+    ("pairs", 16, 1176, 352, 4688, True), ("tiles", 16, 600, 992, 3784, True), ("pairs", 128, 512, 768, 28672, True), ("tiles", 128, 512, 768, 28671, True),
+    # long reductions: 512 tokens per expert and two tiles per pair
+    ("pairs", 16, 1000, 2048, 8192, True), ("tiles", 16, 1000, 2048, 8191, True), ("tiles", 8, 1000, 2048, 5000, True), ("pairs", 128, 1408, 1280, 32768, True),
+    ("tiles", 128, 1408, 1312, 32768, True),
     # fp32 output: long reductions and many tokens only
     ("tiles", 128, 2048, 768, 65536, False), ("pairs", 32, 2560, 1280, 24576, False), ("tiles", 32, 2560, 1280, 24575, False), ("tiles", 32, 2560, 1024, 24576, False)])
 def test_which_tiles_the_grouped_product_takes(fake, want, E, N, K, M, bf16):
