@@ -146,7 +146,10 @@ prq_status prq_prepare_weights_stacked(const uint16_t *const *Ws, const int *Ns,
  *   act_amax  HOST, n_experts x K fp32          opts  may be NULL
  *   stream    the kernels and copies run there; the call synchronises it before it returns
  * The handle is one allocation on the device; codes and scale bytes are kept there only, and prq_weights_get copies
- * them to the host when asked.
+ * them to the host when asked.  Beside the codes (N x (K + k) / 2 bytes per expert) it holds, for its lifetime, the scale
+ * bytes row-major and once per layout that a kernel reads -- four for a dense layer, two for a gated producer and for stacked
+ * experts, 1 / 16 to 1 / 9 of the codes each -- and 20 bytes per input channel.  A handle prepared on the host holds the same layouts
+ * without the row-major copy (MXFP8: four layouts, 1 / 32 to 1 / 18 of the codes each), and codes and scale bytes in host memory too.
  * Errors as prq_prepare_weights; a NaN or an infinity in W * s gives NONFINITE. */
 prq_status prq_prepare_weights_device(const uint16_t *W_device, int n_experts, int N, int K, const float *act_amax,
                                       float alpha, int k_tail, const prq_prep_opts *opts, prq_stream_t stream,
@@ -180,7 +183,7 @@ void prq_weights_free(prq_weights *w);
 
 /* A second, independent device copy of a handle's prepared weights (same device): serving several
  * streams from separate memory, or benchmarks that rotate over more weight bytes than the L2 holds.
- * Not part of the paper's method.  Free it with prq_weights_free. */
+ * Not part of the paper's method.  The copy is complete when the call returns.  Free it with prq_weights_free. */
 prq_status prq_weights_clone(const prq_weights *w, prq_weights **out);
 
 /* The "offline copy" form of a prepared layer (Activation tail construction paragraph: the producer layers emit the k tail
@@ -227,8 +230,10 @@ prq_status prq_weights_info(const prq_weights *w, int *n_experts, int *N, int *K
 /* Format of a handle (a prq_format).  INVALID_ARG for NULL. */
 prq_status prq_weights_format(const prq_weights *w, int *format);
 
-/* Copy one canonical host-side view of expert `expert` into dst (host, dst_bytes must match).  For an MXFP8 handle
- * PRQ_FIELD_CODES is N x K bytes of E4M3 codes. */
+/* Copy one canonical view of expert `expert` into dst (host, dst_bytes must match).  For an MXFP8 handle PRQ_FIELD_CODES is
+ * N x K bytes of E4M3 codes.  Codes and scale bytes of a layer prepared on the device (and of its copies) are fetched from
+ * there, on a stream of the library's own that waits for none of the caller's; the call returns when dst is written.
+ * Errors: INVALID_ARG, CUDA. */
 prq_status prq_weights_get(const prq_weights *w, int expert, prq_field which, void *dst, size_t dst_bytes);
 
 /* ---- online ------------------------------------------------------------------------------ */
@@ -259,10 +264,10 @@ size_t prq_act_bytes_for(const prq_weights *w, int M, prq_buf which);
  * Precondition: x is finite.  The kernel does not look for NaN or infinities (a scan would cost a second pass
  * over a memory-bound kernel); a block that holds one gets a meaningless scale byte and the product is
  * undefined for that row.  The offline calls do check W and amax (NONFINITE).
- * Errors: INVALID_ARG / ALIGNMENT before anything is enqueued.  In scale + permute mode a dense layer of 512 rows or
- * more is fetched by bulk copies whose waits are bounded like every device wait of this library: if one ran out the
- * kernel returns early and PRQ_ERR_TIMEOUT is recorded in the device status word (prq_last_device_status); the output
- * buffers are then incomplete.
+ * Errors: INVALID_ARG / ALIGNMENT before anything is enqueued.  In scale + permute mode rows of any number, of dense layers
+ * and of stacked experts, may be fetched by bulk copies whose waits are bounded like every device wait of this library: if
+ * one ran out the kernel returns early and PRQ_ERR_TIMEOUT is recorded in the device status word
+ * (prq_last_device_status); the output buffers are then incomplete.
  * M == 0 is a no-op. */
 prq_status prq_quantize_act(const prq_weights *w, prq_act_mode mode, const void *x, int M, int ldx,
                             const int32_t *expert_offsets, void *codes, void *scales_row, void *scales_sf,
@@ -275,7 +280,7 @@ prq_status prq_quantize_act(const prq_weights *w, prq_act_mode mode, const void 
 size_t prq_linear_workspace_bytes(const prq_weights *w, int M);
 /* Leading bytes of such a workspace that must be zero before ONE prq_linear call on M tokens (0 where the call counts
  * nothing).  For a caller that takes a fresh workspace for every call; one that keeps its workspace zero-fills all of it
- * once, as above. */
+ * once, as above.  The clearing must be ordered before the call on the call's stream. */
 size_t prq_linear_workspace_clear_bytes(const prq_weights *w, int M);
 
 /* Eq. (3): y = [Q(x) | Q(x)_tail] [Q(W D P) | Q(R)]^T, one block-scaled FP4 GEMM over K + k with fp32
