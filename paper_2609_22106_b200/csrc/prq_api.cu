@@ -264,9 +264,10 @@ PairSchedule pair_schedule(int bn, int M, int N, int S, int max_pairs) {
     return ps;
 }
 
-// Tile width of the pair kernel: the main loop is bound by the operand bytes an SM takes in per stage
-// (33792 with 224-column tiles, 34816 with 240-column ones), so the width whose busiest pair takes in
-// fewer bytes wins; 224 on a tie.  With the paper's down projection that is 240 from 2048 tokens on
+// Tile width of the pair kernel: where a pair runs several tiles, what an SM takes in weighs on the launch beside the tensor
+// work and the stores of y (4096 tokens of the down projection 44.6 us, with the loads of the steady state left out 37.3),
+// so the width whose busiest pair takes in fewer bytes wins (33792 per stage with 224-column tiles, 34816 with 240-column
+// ones); 224 on a tie.  With the paper's down projection that is 240 from 2048 tokens on
 // (11 instead of 12 column tiles) and 224 below (the tile counts do not fill the pairs either way).
 // Third width, 288 columns with a single accumulator: only where every tile of the call fits ONE wave of pairs at
 // that width while the narrower tilings would leave tiles over (so that they need a second wave or stream-K

@@ -1,12 +1,12 @@
-// Grouped (MoE) block-scaled FP4 GEMM on CTA pairs, for experts with many tokens each: per expert the product of Eq. (3) as
+// Grouped (MoE) block-scaled FP4 GEMM on CTA pairs, for experts with many tokens each (grouped_pairs_pay in prq_api.cu draws the line): per expert the product of Eq. (3) as
 // in prq_gemm.cu, with the prefill kernel's tile -- 256 tokens of one expert x 240 output features, computed by two
 // CTAs of a cluster as one tcgen05 cta_group::2 unit (prq_pair.cuh).
 //
 // Why.  The tile-per-CTA kernel (128 features x 128 tokens) spends 110 KB of operands per 32 KB of output; at the
 // 64 - 70 bytes per cycle that an SM takes in from L2 its main loop alone is 72 us of the 116 us at 8192 tokens x 8
 // experts of 2048 x 768 (k = 64).  The pair's tile needs 113 KB per CTA for 61 KB of output: 104 us, against 63 us of HBM
-// traffic.  Without its stores it takes 70 us: what is left is the sum of operand reads and 268 MB of y on the way through
-// L2, no longer instructions.  With K + k = 832 a tile is only 3.25 stages, so the epilogue must be short: eight warps
+// traffic.  Without its stores it takes 70 us, without the loads of its steady state 70 us too: operand reads and 268 MB of y
+// add up on the way through L2, and neither instructions nor the tensor pipe are what it waits for.  With K + k = 832 a tile is only 3.25 stages, so the epilogue must be short: eight warps
 // per CTA, 32 rows x 128 columns each, write rows of 128 contiguous bytes through a swizzled staging tile of their own.
 // Plain 16-byte stores, not tiled ones: the last rows of an expert are followed by the next expert's, which no tensor map
 // clips.

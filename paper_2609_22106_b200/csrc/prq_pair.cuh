@@ -71,13 +71,14 @@ constexpr uint32_t kHiPlain = (128u >> 4) | (1u << 14);                // SBO 12
 __device__ __forceinline__ uint64_t desc64(uint32_t hi, uint32_t lo) { return (static_cast<uint64_t>(hi) << 32) | lo; }
 
 // One reduction stage of the issue loop with the ring slot Q known at compile time: every
-// shared-memory descriptor is `lo_base` plus a constant.  Scale atoms first -- activation group
-// (columns +0 / +4 for the two halves of the stage), then the weight groups (G = 2 or 3 of them: columns
-// +8 + 4 g for the first half of the stage, +8 + 4 G + 4 g for the second) -- then up to four K = 64 steps,
-// then the commit that frees the slot in both CTAs.  A step is one MMA over all BN columns, or for the
-// 288-column tile two (256 columns, then the 32 columns of the third weight group into accumulator
-// columns 256 ..).  The copies and the MMAs are issued by one thread, so tensor memory sees them in order
-// and one set of scale columns is enough.  `rem` = reduction elements this stage still covers.
+// shared-memory descriptor is `lo_base` plus a constant.  Scale atoms first, then up to four steps, then the commit that
+// frees the slot in both CTAs.  A step is one MMA over all BN columns, or for the 288-column tile two of 144 columns (the
+// second reads the second half of the CTA's weight rows and the scale columns of the second half's groups).  The copies and
+// the MMAs are issued by one thread, so tensor memory sees them in order and one set of scale columns is enough.
+// MXFP4: K = 64 steps, two atoms per 128-row group and stage: the activation's in scale columns +0 / +4 (first / second half of
+// the stage), the weight groups' (G = 2 of them, 288 columns: 4) in +8 + 4 g / +8 + 4 G + 4 g; a step's scale id picks the byte
+// pair.  MXFP8: K = 32 steps, one atom per group: activation +0, weights +4 + 4 g; step j takes byte j.  `rem` = reduction
+// elements this stage still covers.
 template <int BN, bool kFp8, int Q>
 __device__ __forceinline__ void issue_stage(uint32_t lo_base, uint32_t d_tmem, uint32_t sf_t, int rem,
                                             uint32_t accumulate, uint32_t empty_bar0) {

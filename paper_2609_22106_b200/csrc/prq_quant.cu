@@ -317,7 +317,7 @@ quant_act_kernel(const QuantBatch b) {
 // scattered 2-byte read).  Rows that stay with their lanes need a 16-byte record per column pair fetched from shared
 // memory for every row (12.7 per element), and the records of a wide layer (K = 9728) do not fit beside its rows.  Here
 // the core is 5 per element -- gather, its address, widening, two packed fp32 products and a conversion per pair, half
-// a three-input maximum -- and 10.7 in all at 4096 x 2560 (ncu), where a CTA sees only three or four slices; a row is
+// a three-input maximum -- and 10.5 - 10.7 in all at 4096 x 2560 (ncu), where a CTA sees only three or four slices; a row is
 // all that shared memory holds.  Measured figures stand at the launcher.  Of the 8.9 us at 4096 x 2560 (2.53 B per
 // element: 4.1 us of memory time) about 3 are set-up, the first rows' latency and the last stores.
 //
