@@ -426,6 +426,30 @@ def test_linear_fused_small_shapes_and_strides(prq, oracle):
         w.free()
 
 
+@pytest.mark.parametrize("splits", [1, 3])
+def test_decode_several_ring_passes(prq, oracle, splits, monkeypatch):
+    """Reductions of many times the decode kernel's ring (K not a multiple of a stage), at every number of items per group
+    of its quantiser and at the edges of the token tiles."""
+    monkeypatch.setenv("PRQ_DECODE_SPLITS", str(splits))
+    N, K, k = 200, 4384, 96
+    L = synth.layer(0, N, K, 128, T_cal=32, tag=930)
+    amax = oracle.channel_amax(L["zcal"])
+    w = prq.prepare_weights(L["W"], amax, 0.25, k)
+    o = oracle.prepare(L["W"], amax, float(np.float32(0.25)), k)
+    oc, osc = oracle.quantize_act(L["x"])
+    ca, sa = oracle.augment_act(oc, osc, k)
+    y_ref = oracle.matmul(ca, sa, o["wcodes"], o["wscales"])
+    x = to_dev_bf16(L["x"])
+    for M in (1, 2, 3, 4, 5, 8, 15, 16, 17, 32, 33, 64, 65, 128):
+        codes, _, sf = prq.quantize_act(w, x[:M], prq.ACT_IDENTITY)
+        y = prq.linear(w, codes, sf, M)
+        assert np.abs(y.cpu().numpy().astype(np.float64) - y_ref[:M]).max() <= prq_ref.tolerance(y_ref[:M]), M
+        if M <= prq.FUSED_MAX_M:
+            assert torch.equal(prq.linear_fused(w, x[:M], prq.ACT_IDENTITY), y), M
+    assert prq.last_device_status() == 0
+    w.free()
+
+
 def test_linear_fused_rejects_what_it_does_not_cover(prq, oracle):
     L = synth.layer(0, 128, 256, 4, T_cal=16, tag=950)
     w = prq.prepare_weights(L["W"], oracle.channel_amax(L["zcal"]), 0.5, 32)
