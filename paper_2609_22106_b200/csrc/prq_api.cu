@@ -198,23 +198,36 @@ int decode_splits_for(int n_tiles, int S, int M, DeviceInfo* di) {
     const int forced = env_int("PRQ_DECODE_SPLITS", 0);
     const int limit = std::min(8, S);
     if (forced > 0) return std::min(forced, limit);
+    auto resident = [&](int s) {
+        std::lock_guard<std::mutex> lock(g_dev_mutex);
+        int& mc = di->max_clusters[bi][s];
+        if (mc == 0) mc = std::max(1, decode_max_active_clusters(bn, s));
+        return mc;
+    };
     if (bn <= 32) {
-        // Up to 32 tokens two CTAs share an SM, and a few clusters more than fit at once cost less than
-        // a longer reduction per CTA does (measured at 20 tiles: 8 splits beat 6 at every token count):
-        // the largest cluster that oversubscribes the SMs by at most a fifth.
-        int best = 1;
-        for (int s = 1; s <= limit; ++s)
-            if (static_cast<long long>(n_tiles) * s * 5 <= static_cast<long long>(di->num_sms) * 6) best = s;
+        // Up to 32 tokens two CTAs share an SM, so that a launch is set up and has its weights while the one before it runs
+        // -- as far as both fit: clusters that come up late pay set-up and weights behind the dependency.  In hundredths of
+        // a microsecond: a stage costs about 23 and one per token (the quantiser, fused), half as much again beyond the
+        // ring, and late clusters 45 and up to 100 more with their share of the launch.  (us a launch, largest cluster that
+        // oversubscribes the SMs by a fifth at most -> this rule: 4096 x 2560 one / sixteen tokens 3.42 / 4.35 -> 2.74 / 4.21
+        // (5 -> 4 splits), 2560 x 4096 3.37 / 4.35 -> 2.74 / 4.19 (8 -> 6); quantise + multiply 32 tokens 6.34 -> 5.80, 9728 x 2560
+        // 7.76 -> 7.08 (2 -> 3); 2560 x 9728 stays at 8: 4.11, 6 would be 4.47.)
+        const bool two_calls = bn == 32;   // a quantiser stands in front, and hides part of what comes late
+        const int ring = bn == 16 ? 5 : 4;
+        int best = 1, best_cost = 0;
+        for (int s = 1; s <= limit; ++s) {
+            const int mc = resident(s);
+            if (s > 1 && n_tiles > mc) continue;   // more than one wave of clusters: not split (several waves cost far more)
+            const int stages = (S + s - 1) / s, late = std::max(0, 2 * n_tiles - mc);
+            int cost = stages * (two_calls ? 25 : 23 + M) + std::max(0, stages - ring) * (two_calls ? 15 : 18);
+            if (late > 0) cost += two_calls ? 30 + 40 * std::min(late, n_tiles) / n_tiles : 45 + 100 * std::min(late, n_tiles) / n_tiles;
+            if (s == 1 || cost < best_cost) { best_cost = cost; best = s; }
+        }
         return best;
     }
     int best = 1, best_ctas = 0;
     for (int s = 1; s <= limit; ++s) {
-        int mc;
-        {
-            std::lock_guard<std::mutex> lock(g_dev_mutex);
-            if (di->max_clusters[bi][s] == 0) di->max_clusters[bi][s] = std::max(1, decode_max_active_clusters(bn, s));
-            mc = di->max_clusters[bi][s];
-        }
+        const int mc = resident(s);
         const int ctas = std::min(n_tiles, mc) * s;
         const bool one_wave = mc >= n_tiles;
         // prefer configurations that fit in one wave; among them the most CTAs

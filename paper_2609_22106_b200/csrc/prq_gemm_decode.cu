@@ -589,14 +589,24 @@ bool wants_dense(int bn, const DecodeBatch& b) {
     return b.lay[b.n_lin - 1].tile_end > sms;
 }
 
+// The occupancy query counts one CTA per SM for every kernel that allocates tensor memory, however little; two do run beside
+// each other up to 32 tokens (a launch's CTAs enter while the one before it computes).  A kernel without it, of the same
+// threads and shared memory, gives the number that is wanted there.
+template <int kThreads>
+__global__ void __launch_bounds__(kThreads) occupancy_stand_in(int* p) {
+    extern __shared__ int stand_in_smem[];
+    if (p) *p = stand_in_smem[threadIdx.x];
+}
+
 template <int BN>
 int max_clusters(int splits) {
     using C = DCfg<BN>;
-    cudaFuncSetAttribute(decode_kernel<BN, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
+    const void* kernel = C::kCtasPerSm > 1 ? reinterpret_cast<const void*>(occupancy_stand_in<C::kThreads>) : reinterpret_cast<const void*>(decode_kernel<BN, false, false>);
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes + 256) != cudaSuccess) { cudaGetLastError(); return 0; }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(splits);
     cfg.blockDim = dim3(C::kThreads);
-    cfg.dynamicSmemBytes = C::kSmemBytes;
+    cfg.dynamicSmemBytes = C::kSmemBytes + (C::kCtasPerSm > 1 ? 256 : 0);   // (the stand-in has no static shared memory)
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = splits;
@@ -605,7 +615,7 @@ int max_clusters(int splits) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, decode_kernel<BN, false, false>, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
     return n;
 }
 
