@@ -47,6 +47,16 @@ __device__ __forceinline__ uint32_t encode8(const float (&v)[8], uint32_t byte) 
     return cvt_e2m1x8(v[0] * inv, v[1] * inv, v[2] * inv, v[3] * inv, v[4] * inv, v[5] * inv, v[6] * inv, v[7] * inv);
 }
 
+// A launch on few rows leaves the memory idle, and the product behind it then waits for its weights: every CTA asks for its
+// share of them (`part` of `parts`) in L2.  Weights depend on no kernel, so this needs no wait.  Quantise + multiply, k = 256, us:
+// 2560 x 9728 at 16 / 64 / 128 tokens 7.16 / 9.20 / 11.35 -> 6.40 / 8.61 / 10.78, 4096 x 2560 5.33 / 7.06 / 8.92 -> 5.18 / 6.84 /
+// 8.11, 9728 x 2560 6.64 / 7.42 / 9.81 -> 6.33 / 6.95 / 9.01.  (Not for stacked experts: 89 MB keep the memory busy longer than the
+// quantiser runs, and its rows wait behind them; 64 tokens over 128 experts 27.5 -> 29.9.)
+__device__ __forceinline__ void ask_for(const uint8_t* base, uint32_t bytes, int part, int parts) {
+    const uint32_t share = ((bytes + parts - 1) / parts + 127) & ~127u, at = share * part;
+    if (at < bytes) prefetch_l2(base + at, min(share, (bytes - at)) & ~15u);
+}
+
 template <bool kScalePerm, bool kBatch>
 __global__ void __launch_bounds__(kQuantThreads, kScalePerm ? 3 : 4)
 quant_act_kernel(const QuantBatch b) {
@@ -113,6 +123,12 @@ quant_act_kernel(const QuantBatch b) {
         }
     };
     const bool dense = p.expert_offsets == nullptr;
+    if (dense && b.ask && threadIdx.x == 0) {
+        const int parts = static_cast<int>(gridDim.x * gridDim.z) * b.groups_per_lin;
+        const int part = static_cast<int>(blockIdx.x + gridDim.x * (blockIdx.z + gridDim.z * (blockIdx.y - lin * b.groups_per_lin)));
+        ask_for(b.hint[lin].codes, b.hint[lin].code_bytes, part, parts);
+        ask_for(b.hint[lin].sf, b.hint[lin].sf_bytes, part, parts);
+    }
     if (kScalePerm && dense) load_layer_constants(0);
     grid_dependency_wait();
 
@@ -404,7 +420,13 @@ quant_act_cols_kernel(const QuantBatch b, const ColsPlan plan_c) {
     __syncthreads();
     if (!kGrouped) {
         // a dense layer's constants belong to the prepared weights, not to an earlier kernel of the stream
-        if (!loader) load_constants(0);
+        if (!loader) {
+            load_constants(0);
+        } else if (b.ask && lane == 0) {
+            const int part = blockIdx.x + gridDim.x * blockIdx.y, parts = gridDim.x * gridDim.y;
+            ask_for(b.hint[blockIdx.z].codes, b.hint[blockIdx.z].code_bytes, part, parts);
+            ask_for(b.hint[blockIdx.z].sf, b.hint[blockIdx.z].sf_bytes, part, parts);
+        }
         grid_dependency_wait();
     } else {
         grid_dependency_wait();
@@ -648,18 +670,24 @@ cudaError_t launch_cols_impl(const QuantBatch& b, int sm_count, cudaStream_t str
         const int grid = want < cp.n_slices ? want : cp.n_slices;
         const int live = (b.M + kRowsC - 1) / kRowsC, half = cp.n_slices / 2, fewer = live > half ? live : half;
         if (3LL * grid * chunks * b.n_lin > 2LL * per_sm * sm_count && fewer < grid) { cp.strided = 1; want = fewer; }
+        // Where the CTAs ask for weights, no more stages of rows than a CTA has slices: they then come up beside a GEMM that
+        // fills its SMs and ask while it ends.  (Without weights to ask for that only disturbs it: 1024 x 2560 at 16 tokens 4.43 / 4.70.)
+        const int g2 = want < 1 ? 1 : want < cp.n_slices ? want : cp.n_slices, mine = ((cp.strided ? live : cp.n_slices) + g2 - 1) / g2;
+        if (b.hint[0].code_bytes && cp.n_stages > mine) cp.n_stages = mine;
     }
     cudaLaunchConfig_t cfg = {};
+    QuantBatch bb = b;
+    bb.ask = !kGrouped && b.hint[0].code_bytes > 0;
     cfg.gridDim = dim3(want < 1 ? 1 : want < cp.n_slices ? want : cp.n_slices, chunks, b.n_lin);
     cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = n_stages * stage;
+    cfg.dynamicSmemBytes = cp.n_stages * stage;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, b, cp);
+    return cudaLaunchKernelEx(&cfg, kernel, bb, cp);
 }
 
 }  // namespace
@@ -731,6 +759,7 @@ cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, cudaStr
     QuantBatch bb = b;
     bb.n_atoms = n_atoms;
     bb.n_tail = 0; bb.tail_split = 1;
+    bb.ask = b.hint[0].code_bytes > 0;
     // (dense launches only: a grouped launch has a CTA per expert group and column atom already, each with the fixed
     // cost of finding its expert -- eight times as many tail CTAs made the 128-expert quantiser 35-50 % slower, and its
     // launches are long enough for a 20 us CTA not to be their end)
@@ -753,7 +782,7 @@ cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, cudaStr
                       : cudaLaunchKernelEx(&cfg, quant_act_kernel<false, false>, bb);
 }
 
-cudaError_t launch_quant_act(const QuantParams& p, bool scale_perm, int grid_groups, cudaStream_t stream) {
+cudaError_t launch_quant_act(const QuantParams& p, bool scale_perm, int grid_groups, const WeightHint& hint, cudaStream_t stream) {
     QuantBatch b = {};
     b.x = p.x; b.expert_offsets = p.expert_offsets; b.M = p.M; b.ldx = p.ldx; b.K = p.K;
     b.n_experts = p.n_experts; b.act_groups = p.act_groups;
@@ -761,6 +790,7 @@ cudaError_t launch_quant_act(const QuantParams& p, bool scale_perm, int grid_gro
     b.groups_per_lin = grid_groups;
     b.lay[0] = QuantLayer{p.perm, p.inv_s_perm, p.codes, p.scales_row, p.scales_sf, p.k_tail};
     b.status = p.status;
+    b.hint[0] = hint;
     return launch_quant_act_batch(b, scale_perm, stream);
 }
 
