@@ -130,6 +130,15 @@ quant_act_kernel(const QuantBatch b) {
         ask_for(b.hint[lin].sf, b.hint[lin].sf_bytes, part, parts);
     }
     if (kScalePerm && dense) load_layer_constants(0);
+    // Identity mode: this CTA's rows in L2 before the wait, one 128-byte line per thread.  The CTAs that come up beside the GEMM
+    // before this launch (four per SM) thereby read memory while that computes.  A hint only: what an earlier kernel still writes
+    // is read behind the wait.  Quantise + multiply, 2560 x 9728, 512 / 2048 (fp32 y) / 2048 / 4096 tokens: 23.4 / 33.2 / 32.3 / 65.5 ->
+    // 22.2 / 32.0 / 31.2 / 62.0 us, 9728 x 2560 at 3000: 41.7 -> 41.0.  (Asking for the rows of the CTAs behind them too disturbs the
+    // one-wave GEMM: 33.6 with fp32 y.)
+    if (!kScalePerm && dense) {
+        const int row = group * kGroupRows + (threadIdx.x >> 1), col = atom * kAtomK + (threadIdx.x & 1) * 64;
+        if (row < p.M && col < p.K) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.x + static_cast<size_t>(row) * p.ldx + col));
+    }
     grid_dependency_wait();
 
     // Which rows does this CTA own?  Dense: group g covers rows [128 g, 128 g + 128).  Grouped: the
