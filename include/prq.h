@@ -179,6 +179,9 @@ prq_status prq_prepare_weights_search(const uint16_t *W, int N, int K, const uin
                                       const float *alphas, int n_alphas, int k_tail, prq_weights **out,
                                       float *alpha_star, double *nrmse);
 
+/* Waits for the device's work and frees the handle.  Device memory of a layer prepared on the device (up to 96 MB and four
+ * blocks per device) is kept for the next such handle; a null `w` gives all that is kept back to the devices, and so does an
+ * allocation of the library that fails. */
 void prq_weights_free(prq_weights *w);
 
 /* A second, independent device copy of a handle's prepared weights (same device): serving several

@@ -86,6 +86,100 @@ EncodeTiledFn encode_fn() {
     return fn;
 }
 
+// Waits for all work on the current device, as cudaFree does.
+bool device_idle() {
+    typedef CUresult (*SynchronizeFn)();
+    static SynchronizeFn fn = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuCtxSynchronize", &p, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) p = nullptr;
+        return reinterpret_cast<SynchronizeFn>(p);
+    }();
+    return fn && fn() == CUDA_SUCCESS;
+}
+
+// Device memory of freed handles, kept for the next ones: allocating and freeing the 29 MB of a 2560 x 9728 layer takes
+// several times as long as preparing it (2560 x 9728, preparing and first rows, then free: 972 -> 347 us; preparing and freeing alone 0.7 - 5 ms -> 330 us).  A block comes in only when the
+// device is idle -- what cudaFree would have waited for -- so whoever takes it out may write to it on any stream.  At most
+// kPoolBytes and kPoolBlocks per device, the oldest goes first; all of it goes back to the device when an allocation of the
+// library fails, and with prq_weights_free(NULL).  A block serves a request of at least three quarters of its size.
+class ArenaPool {
+public:
+    void* take(int dev, size_t bytes, size_t* got) {
+        {
+            std::lock_guard<std::mutex> lock(m_);
+            size_t best = blocks_.size();
+            for (size_t i = 0; i < blocks_.size(); ++i)
+                if (blocks_[i].dev == dev && blocks_[i].bytes >= bytes && blocks_[i].bytes - blocks_[i].bytes / 4 <= bytes &&
+                    (best == blocks_.size() || blocks_[i].bytes < blocks_[best].bytes))
+                    best = i;
+            if (best < blocks_.size()) {
+                const Block b = blocks_[best];
+                blocks_.erase(blocks_.begin() + best);
+                *got = b.bytes;
+                return b.p;
+            }
+        }
+        void* p = nullptr;
+        *got = bytes;
+        if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+        cudaGetLastError();
+        give_back(dev);
+        if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+        cudaGetLastError();
+        return nullptr;
+    }
+    // `dev` is current.
+    void put(int dev, void* p, size_t bytes) {
+        if (bytes > kPoolBytes || !device_idle()) { cudaFree(p); return; }
+        std::vector<void*> out;
+        try {
+            std::lock_guard<std::mutex> lock(m_);
+            blocks_.reserve(blocks_.size() + 1);
+            out.reserve(blocks_.size());
+            size_t held = bytes, count = 1;
+            for (size_t i = blocks_.size(); i-- > 0;) {   // the newest stay
+                if (blocks_[i].dev != dev) continue;
+                if (held + blocks_[i].bytes <= kPoolBytes && count < kPoolBlocks) { held += blocks_[i].bytes; ++count; continue; }
+                out.push_back(blocks_[i].p);
+                blocks_.erase(blocks_.begin() + i);
+            }
+            blocks_.push_back(Block{p, bytes, dev});
+        } catch (const std::bad_alloc&) {
+            cudaFree(p);
+        }
+        for (void* q : out) cudaFree(q);
+    }
+    // dev < 0: of all devices
+    void give_back(int dev) {
+        for (;;) {
+            Block b = {};
+            {
+                std::lock_guard<std::mutex> lock(m_);
+                for (size_t i = 0; i < blocks_.size() && !b.p; ++i)
+                    if (dev < 0 || blocks_[i].dev == dev) { b = blocks_[i]; blocks_.erase(blocks_.begin() + i); }
+            }
+            if (!b.p) return;
+            int cur = 0;
+            cudaGetDevice(&cur);
+            if (b.dev != cur) cudaSetDevice(b.dev);
+            cudaFree(b.p);
+            if (b.dev != cur) cudaSetDevice(cur);
+        }
+    }
+
+private:
+    static constexpr size_t kPoolBytes = 96u << 20;
+    static constexpr size_t kPoolBlocks = 4;
+    struct Block { void* p; size_t bytes; int dev; };
+    std::mutex m_;
+    std::vector<Block> blocks_;   // oldest first
+};
+ArenaPool& arena_pool() {
+    static ArenaPool* pool = new ArenaPool;   // (never destroyed: handles may be freed during process exit)
+    return *pool;
+}
+
 // Packed E2M1 codes are plain bytes: a row-major (rows x row_bytes) byte matrix, boxes of 128 bytes
 // (256 codes, one swizzle row) x box_rows rows, 128-byte swizzle, zero fill outside the matrix.
 prq_status make_code_map(CUtensorMap* map, const void* base, uint64_t row_bytes, uint64_t rows, uint32_t box_rows) {
@@ -419,12 +513,12 @@ prq_status prq_last_device_status(prq_stream_t stream) {
 }
 
 void prq_weights_free(prq_weights* w) {
-    if (!w) return;
+    if (!w) { arena_pool().give_back(-1); return; }
     int cur = 0;
     cudaGetDevice(&cur);
     if (w->device >= 0 && w->device != cur) cudaSetDevice(w->device);
     if (w->arena) {
-        cudaFree(w->arena);   // every device pointer of the handle lies in it
+        arena_pool().put(w->device, w->arena, w->arena_bytes);   // every device pointer of the handle lies in it
     } else {
         cudaFree(w->d_codes);
         cudaFree(w->d_sf);
@@ -537,7 +631,8 @@ static prq_status fill_handle_device(prq_weights* w, const uint16_t* W, const fl
     }
     const size_t o_perm = take(2 * sizeof(float) * EK);        // the permutation and, right behind it, 1 / s in its order
     const size_t o_rows = take(E * N * Ka / kBlock), o_s = take(sizeof(float) * EK), o_err = take(sizeof(double) * (EK + 1));
-    if (cudaMalloc(&w->arena, total) != cudaSuccess) { cudaGetLastError(); w->arena = nullptr; return PRQ_ERR_OOM; }
+    w->arena = arena_pool().take(w->device, total, &w->arena_bytes);
+    if (!w->arena) return PRQ_ERR_OOM;
     uint8_t* const base = static_cast<uint8_t*>(w->arena);
     w->d_codes = base + o_codes;
     w->d_sf = base + o_sf;

@@ -857,3 +857,49 @@ def test_stacked_preparation_is_the_method_on_the_concatenated_matrix(prq, oracl
     y_k = oracle.matmul(ca, sa, o["wcodes"][r0: r0 + Ns[1]], o["wscales"][r0: r0 + Ns[1]])
     assert np.abs(y[:, r0: r0 + Ns[1]] - y_k).max() <= prq_ref.tolerance(y_k)
     w.free()
+
+
+def test_freed_device_memory_serves_the_next_handle(prq, oracle):
+    """Handles of several sizes prepared, used and freed in turn, on two streams and two threads: whatever memory a handle
+    gets, its fields and products are its own."""
+    import threading
+
+    K, k = 512, 64
+    x = to_dev_bf16(synth.layer(0, 64, K, 5, T_cal=8, tag=980)["x"])
+    layers = []
+    for i, N in enumerate((64, 640, 60, 600)):
+        W = synth.layer(0, N, K, 5, T_cal=8, tag=981 + i)["W"]
+        amax = np.abs(np.random.RandomState(i).randn(K)).astype(np.float32) + 0.1
+        w = prq.prepare_weights(W, amax, 0.5, k)   # host preparation: memory of its own
+        codes, _, sf = prq.quantize_act(w, x, prq.ACT_SCALE_PERM)
+        layers.append((torch.from_numpy(W.view(np.int16)).cuda().view(torch.bfloat16), amax, prq.linear(w, codes, sf, 5), w.get(prq.FIELD_CODES)))
+        w.free()
+    torch.cuda.synchronize()
+    bad = []
+
+    def work(order):
+        torch.cuda.set_device(0)
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for i in order:
+                W, amax, y, c = layers[i]
+                w = prq.prepare_weights_device(W, amax, 0.5, k)
+                codes, _, sf = prq.quantize_act(w, x, prq.ACT_SCALE_PERM)
+                got = prq.linear(w, codes, sf, 5)
+                fields = np.array_equal(w.get(prq.FIELD_CODES), c)
+                w.free()
+                torch.cuda.current_stream().synchronize()
+                if not (fields and torch.equal(got, y)):
+                    bad.append(i)
+
+    threads = [threading.Thread(target=work, args=([j % 4, (j + 1) % 4, 3, 2, 1, 0] * 4,)) for j in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
+    prq.lib().prq_weights_free(None)   # what is kept goes back
+    free0 = torch.cuda.mem_get_info()[0]
+    w = prq.prepare_weights_device(layers[1][0], layers[1][1], 0.5, k)
+    w.free()
+    prq.lib().prq_weights_free(None)
+    assert torch.cuda.mem_get_info()[0] >= free0 - (4 << 20)
