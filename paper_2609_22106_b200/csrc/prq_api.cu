@@ -237,6 +237,7 @@ constexpr int kAltWide = 1;
 bool alt_wanted(bool gated, int n_experts, int a) { return n_experts > 1 ? a == kAltWide : gated ? a == kAltGated : a != kAltGated; }
 
 // Weight-side tensor maps of a handle, encoded once at creation (cloning re-encodes: other addresses).
+int decode_splits_for(int n_tiles, int S, int M, DeviceInfo* di);
 prq_status build_weight_maps(prq_weights* w) {
     w->maps_ready = false;
     const uint64_t Ka = static_cast<uint64_t>(w->K) + w->k_tail, E = w->n_experts;
@@ -251,7 +252,14 @@ prq_status build_weight_maps(prq_weights* w) {
             st = make_sf_map(&w->tm_sfw_pair[v], w->d_sf_alt[v],
                              E * w->plan.S * w->w_groups_alt[v] * kSfGroupBytes, 4 * gpt * (one_wave ? 2 : 1));
     }
-    if (st == PRQ_OK && E == 1) w->maps_ready = true;   // (the dense calls refuse stacked experts)
+    if (st == PRQ_OK && E == 1) {
+        // cluster sizes of the one-token to sixteen-token calls, whose host time is their time (looking them up per call
+        // costs 0.2 of 5.4 us)
+        DeviceInfo* di;
+        st = device_info(w->device, &di);
+        for (int M = 1; M <= 16 && st == PRQ_OK; ++M) w->splits16[M] = static_cast<uint8_t>(decode_splits_for((w->N + 127) / 128, w->plan.S, M, di));
+        w->maps_ready = st == PRQ_OK;   // (the dense calls refuse stacked experts)
+    }
     return st;
 }
 
@@ -292,8 +300,8 @@ int decode_splits_for(int n_tiles, int S, int M, DeviceInfo* di) {
     const int forced = env_int("PRQ_DECODE_SPLITS", 0);
     const int limit = std::min(8, S);
     if (forced > 0) return std::min(forced, limit);
+    std::lock_guard<std::mutex> lock(g_dev_mutex);
     auto resident = [&](int s) {
-        std::lock_guard<std::mutex> lock(g_dev_mutex);
         int& mc = di->max_clusters[bi][s];
         if (mc == 0) mc = std::max(1, decode_max_active_clusters(bn, s));
         return mc;
@@ -332,6 +340,7 @@ int decode_splits_for(int n_tiles, int S, int M, DeviceInfo* di) {
 }
 
 int decode_splits(const prq_weights* w, int M, DeviceInfo* di) {
+    if (M <= 16 && !dev_knobs_enabled()) return w->splits16[M];
     return decode_splits_for((w->N + 127) / 128, w->plan.S, M, di);
 }
 

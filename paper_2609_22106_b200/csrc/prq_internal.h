@@ -188,6 +188,7 @@ struct prq_weights {
     // 224-row [0], 240-row [1], 288-row [2] and 192-row [3] tilings (CTA-pair prefill kernel)
     CUtensorMap tm_w_decode, tm_w_pair[4], tm_sfw_pair[4];
     bool maps_ready = false;
+    uint8_t splits16[17] = {};       // dense layers: cluster size of the decode kernel at 1 .. 16 tokens
     int32_t* d_perm = nullptr;       // E x K
     float* d_inv_s_perm = nullptr;   // E x K : inv_s[perm[j]] in the new channel order
     size_t d_codes_bytes = 0, d_sf_bytes = 0;
