@@ -179,9 +179,9 @@ prq_status prq_prepare_weights_search(const uint16_t *W, int N, int K, const uin
                                       const float *alphas, int n_alphas, int k_tail, prq_weights **out,
                                       float *alpha_star, double *nrmse);
 
-/* Waits for the device's work and frees the handle.  Device memory of a layer prepared on the device (up to 96 MB and four
- * blocks per device) is kept for the next such handle; a null `w` gives all that is kept back to the devices, and so does an
- * allocation of the library that fails. */
+/* Frees the handle; work that still reads it is not disturbed.  Device memory of a layer that was prepared on the device and
+ * used on the legacy default stream alone (up to 96 MB and four blocks per device) is kept for the next such preparation on
+ * that stream; a null `w` gives all that is kept back to the devices, and so does an allocation of the library that fails. */
 void prq_weights_free(prq_weights *w);
 
 /* A second, independent device copy of a handle's prepared weights (same device): serving several

@@ -86,27 +86,18 @@ EncodeTiledFn encode_fn() {
     return fn;
 }
 
-// Waits for all work on the current device, as cudaFree does.
-bool device_idle() {
-    typedef CUresult (*SynchronizeFn)();
-    static SynchronizeFn fn = [] {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuCtxSynchronize", &p, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) p = nullptr;
-        return reinterpret_cast<SynchronizeFn>(p);
-    }();
-    return fn && fn() == CUDA_SUCCESS;
-}
-
 // Device memory of freed handles, kept for the next ones: allocating and freeing the 29 MB of a 2560 x 9728 layer takes
-// several times as long as preparing it (2560 x 9728, preparing and first rows, then free: 972 -> 347 us; preparing and freeing alone 0.7 - 5 ms -> 330 us).  A block comes in only when the
-// device is idle -- what cudaFree would have waited for -- so whoever takes it out may write to it on any stream.  At most
-// kPoolBytes and kPoolBlocks per device, the oldest goes first; all of it goes back to the device when an allocation of the
-// library fails, and with prq_weights_free(NULL).  A block serves a request of at least three quarters of its size.
+// several times as long as preparing it (2560 x 9728, preparing and first rows, then free: 972 -> 347 us; preparing and freeing
+// alone 0.7 - 5 ms -> 330 us).  What cudaFree waits for -- work that still reads the block -- is left to stream order: only
+// handles come in that were prepared and used on the legacy stream alone (see note_use), and a block goes out only to a
+// preparation on that stream, whose writes run behind those reads.  (Waiting for the device instead would break the captures
+// of other threads, which cudaFree does not; the legacy stream cannot be captured, so no graph holds such a handle.)  At
+// most kPoolBytes and kPoolBlocks per device, the oldest goes first; all of it goes back to the device when an allocation of
+// the library fails, and with prq_weights_free(NULL).  A block serves a request of at least three quarters of its size.
 class ArenaPool {
 public:
-    void* take(int dev, size_t bytes, size_t* got) {
-        {
+    void* take(int dev, size_t bytes, cudaStream_t stream, size_t* got) {
+        if (stream == nullptr) {
             std::lock_guard<std::mutex> lock(m_);
             size_t best = blocks_.size();
             for (size_t i = 0; i < blocks_.size(); ++i)
@@ -131,7 +122,7 @@ public:
     }
     // `dev` is current.
     void put(int dev, void* p, size_t bytes) {
-        if (bytes > kPoolBytes || !device_idle()) { cudaFree(p); return; }
+        if (bytes > kPoolBytes) { cudaFree(p); return; }
         std::vector<void*> out;
         try {
             std::lock_guard<std::mutex> lock(m_);
@@ -278,6 +269,11 @@ long long* trace_ptr() {
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
+// Work that reads the handle's memory is about to be queued on `stream` (see ArenaPool).
+void note_use(const prq_weights* w, prq_stream_t stream) {
+    if (stream != nullptr && w->legacy_stream_only.load(std::memory_order_relaxed)) w->legacy_stream_only.store(false, std::memory_order_relaxed);
+}
 
 // Online calls launch on the current device with pointers and tensor maps of the handle's device.
 bool handle_device_is_current(const prq_weights* w) {
@@ -527,7 +523,9 @@ void prq_weights_free(prq_weights* w) {
     cudaGetDevice(&cur);
     if (w->device >= 0 && w->device != cur) cudaSetDevice(w->device);
     if (w->arena) {
-        arena_pool().put(w->device, w->arena, w->arena_bytes);   // every device pointer of the handle lies in it
+        // (every device pointer of the handle lies in it)
+        if (w->legacy_stream_only) arena_pool().put(w->device, w->arena, w->arena_bytes);
+        else cudaFree(w->arena);
     } else {
         cudaFree(w->d_codes);
         cudaFree(w->d_sf);
@@ -640,7 +638,8 @@ static prq_status fill_handle_device(prq_weights* w, const uint16_t* W, const fl
     }
     const size_t o_perm = take(2 * sizeof(float) * EK);        // the permutation and, right behind it, 1 / s in its order
     const size_t o_rows = take(E * N * Ka / kBlock), o_s = take(sizeof(float) * EK), o_err = take(sizeof(double) * (EK + 1));
-    w->arena = arena_pool().take(w->device, total, &w->arena_bytes);
+    w->arena = arena_pool().take(w->device, total, stream, &w->arena_bytes);
+    note_use(w, stream);
     if (!w->arena) return PRQ_ERR_OOM;
     uint8_t* const base = static_cast<uint8_t*>(w->arena);
     w->d_codes = base + o_codes;
@@ -1200,6 +1199,7 @@ prq_status prq_quantize_act(const prq_weights* w, prq_act_mode mode, const void*
         if (expert_offsets) return PRQ_ERR_INVALID_ARG;
         if (!aligned16(x) || !aligned16(codes) || !aligned16(scales_sf) || ldx % 8) return PRQ_ERR_ALIGNMENT;
         if (!handle_device_is_current(w)) return PRQ_ERR_INVALID_ARG;
+        note_use(w, stream);
         cudaError_t e8 = launch_quant_act_fp8(static_cast<const uint16_t*>(x), M, ldx, w->K, mode == PRQ_ACT_SCALE_PERM ? w->d_inv_s : nullptr,
                                               static_cast<uint8_t*>(codes), static_cast<uint8_t*>(scales_row),
                                               static_cast<uint8_t*>(scales_sf), static_cast<cudaStream_t>(stream));
@@ -1210,6 +1210,7 @@ prq_status prq_quantize_act(const prq_weights* w, prq_act_mode mode, const void*
     // (the grouped layout with one group), as prq_linear_grouped accepts it
     if (w->n_experts > 1 && expert_offsets == nullptr) return PRQ_ERR_INVALID_ARG;
     if (!handle_device_is_current(w)) return PRQ_ERR_INVALID_ARG;
+    note_use(w, stream);
     if (!aligned16(x) || !aligned16(codes) || !aligned16(scales_sf) || ldx % 8) return PRQ_ERR_ALIGNMENT;
     QuantParams p;
     p.x = static_cast<const uint16_t*>(x);
@@ -1245,6 +1246,7 @@ prq_status prq_quantize_act_multi(int n, const prq_weights* const* ws, prq_act_m
     if (M == 0) return PRQ_OK;
     if (!x || ldx < ws[0]->K) return PRQ_ERR_INVALID_ARG;
     if (!handle_device_is_current(ws[0])) return PRQ_ERR_INVALID_ARG;
+    for (int i = 0; i < n; ++i) note_use(ws[i], stream);
     if (!aligned16(x) || ldx % 8) return PRQ_ERR_ALIGNMENT;
     for (int i = 0; i < n; ++i)
         if (!aligned16(codes[i]) || !aligned16(scales_sf[i])) return PRQ_ERR_ALIGNMENT;
@@ -1313,6 +1315,7 @@ prq_status prq_linear(const prq_weights* w, const void* codes, const void* scale
     if (st != PRQ_OK) return st;
     if (M < 0 || w->n_experts != 1 || !w->maps_ready) return PRQ_ERR_INVALID_ARG;
     if (!handle_device_is_current(w)) return PRQ_ERR_INVALID_ARG;
+    note_use(w, stream);
     DeviceInfo* di;
     st = device_info(w->device, &di);
     if (st != PRQ_OK) return st;
@@ -1442,6 +1445,7 @@ prq_status prq_linear_multi(int n, const prq_weights* const* ws, const void* con
     }
     if (M == 0) return PRQ_OK;
     if (!handle_device_is_current(ws[0])) return PRQ_ERR_INVALID_ARG;
+    for (int i = 0; i < n; ++i) note_use(ws[i], stream);
     DeviceInfo* di;
     prq_status st = device_info(ws[0]->device, &di);
     if (st != PRQ_OK) return st;
@@ -1486,6 +1490,7 @@ prq_status prq_linear_gated(const prq_weights* w, const void* codes, const void*
     if (!aligned16(codes) || !aligned16(scales_sf) || !aligned16(out_codes) || !aligned16(out_scales_sf) || !aligned16(h_check))
         return PRQ_ERR_ALIGNMENT;
     if (!handle_device_is_current(w)) return PRQ_ERR_INVALID_ARG;
+    note_use(w, stream);
     DeviceInfo* di;
     prq_status st = device_info(w->device, &di);
     if (st != PRQ_OK) return st;
@@ -1530,6 +1535,7 @@ prq_status prq_linear_fused(const prq_weights* w, prq_act_mode mode, const void*
     if (y_dtype != PRQ_F32 && y_dtype != PRQ_BF16) return PRQ_ERR_INVALID_ARG;
     if (!aligned16(x) || !aligned16(y) || ldx % 8 || ldy % (y_dtype == PRQ_F32 ? 4 : 8)) return PRQ_ERR_ALIGNMENT;
     if (!handle_device_is_current(w)) return PRQ_ERR_INVALID_ARG;
+    note_use(w, stream);
     DeviceInfo* di;
     prq_status st = device_info(w->device, &di);
     if (st != PRQ_OK) return st;
@@ -1556,6 +1562,7 @@ prq_status prq_linear_grouped(const prq_weights* w, const void* codes, const voi
     if (st != PRQ_OK) return st;
     if (M_total < 0 || !expert_offsets || w->format != PRQ_FMT_MXFP4) return PRQ_ERR_INVALID_ARG;
     if (!handle_device_is_current(w)) return PRQ_ERR_INVALID_ARG;
+    note_use(w, stream);
     DeviceInfo* di;
     st = device_info(w->device, &di);
     if (st != PRQ_OK) return st;

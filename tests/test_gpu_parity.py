@@ -859,9 +859,11 @@ def test_stacked_preparation_is_the_method_on_the_concatenated_matrix(prq, oracl
     w.free()
 
 
-def test_freed_device_memory_serves_the_next_handle(prq, oracle):
-    """Handles of several sizes prepared, used and freed in turn, on two streams and two threads: whatever memory a handle
-    gets, its fields and products are its own."""
+@pytest.mark.parametrize("side_streams", [False, True])
+def test_freed_device_memory_serves_the_next_handle(prq, oracle, side_streams):
+    """Handles of several sizes prepared, used and freed in turn by two threads, on the default stream or on one each: whatever
+    memory a handle gets, its fields and products are its own.  Freeing one leaves a capture in progress alone."""
+    import contextlib
     import threading
 
     K, k = 512, 64
@@ -879,7 +881,7 @@ def test_freed_device_memory_serves_the_next_handle(prq, oracle):
 
     def work(order):
         torch.cuda.set_device(0)
-        with torch.cuda.stream(torch.cuda.Stream()):
+        with torch.cuda.stream(torch.cuda.Stream()) if side_streams else contextlib.nullcontext():
             for i in order:
                 W, amax, y, c = layers[i]
                 w = prq.prepare_weights_device(W, amax, 0.5, k)
@@ -897,6 +899,18 @@ def test_freed_device_memory_serves_the_next_handle(prq, oracle):
     for t in threads:
         t.join()
     assert not bad
+    w = prq.prepare_weights_device(layers[0][0], layers[0][1], 0.5, k)
+    graph, a = torch.cuda.CUDAGraph(), torch.ones(8, device="cuda")
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, capture_error_mode="thread_local"):
+        b = a + 1
+        t = threading.Thread(target=w.free)
+        t.start()
+        t.join()
+        b = b + 1
+    graph.replay()
+    torch.cuda.synchronize()
+    assert b.sum().item() == 24
     prq.lib().prq_weights_free(None)   # what is kept goes back
     free0 = torch.cuda.mem_get_info()[0]
     w = prq.prepare_weights_device(layers[1][0], layers[1][1], 0.5, k)
