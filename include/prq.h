@@ -179,10 +179,14 @@ prq_status prq_prepare_weights_search(const uint16_t *W, int N, int K, const uin
                                       const float *alphas, int n_alphas, int k_tail, prq_weights **out,
                                       float *alpha_star, double *nrmse);
 
-/* Frees the handle; work that still reads it is not disturbed.  Device memory of a layer that was prepared on the device and
- * used on the legacy default stream alone (up to 96 MB and four blocks per device) is kept for the next such preparation on
- * that stream; a null `w` gives all that is kept back to the devices, and so does an allocation of the library that fails. */
+/* Frees the handle; work that still reads it is not disturbed.  A null `w` is a no-op.  Device memory of a layer that was
+ * prepared on the device and used on the legacy default stream alone (up to 96 MB and four blocks per device) is kept for the
+ * next such preparation on that stream, until prq_release_cached_memory or an allocation of the library that fails. */
 void prq_weights_free(prq_weights *w);
+
+/* Gives the device memory that prq_weights_free keeps back to its devices (cudaFree: waits for work in flight there).  For a
+ * program that needs the memory for something else. */
+void prq_release_cached_memory(void);
 
 /* A second, independent device copy of a handle's prepared weights (same device): serving several
  * streams from separate memory, or benchmarks that rotate over more weight bytes than the L2 holds.

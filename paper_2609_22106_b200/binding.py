@@ -28,7 +28,7 @@ EXPORTS = [
     "prq_linear_grouped", "prq_forward_host_scratch_bytes", "prq_forward_host",
     "prq_status_string", "prq_last_device_status", "prq_kernel_launch_count", "prq_mxf4_peak_probe",
     "prq_handover_probe", "prq_stack_gate_up", "prq_linear_gated", "prq_weights_format", "prq_act_bytes_for",
-    "prq_prepare_weights_stacked", "prq_linear_workspace_clear_bytes",
+    "prq_prepare_weights_stacked", "prq_linear_workspace_clear_bytes", "prq_release_cached_memory",
 ]
 
 
@@ -61,6 +61,7 @@ def lib():
         L.prq_fold_producer.argtypes = [vp, vp, ci, ci, vp, vp, ci, ci, vp, vp]
         L.prq_weights_free.argtypes = [vp]
         L.prq_weights_free.restype = None
+        L.prq_release_cached_memory.restype = None
         L.prq_weights_info.argtypes = [vp] + [ctypes.POINTER(ci)] * 4 + [ctypes.POINTER(cf)]
         L.prq_weights_get.argtypes = [vp, ci, ci, vp, cs]
         L.prq_act_bytes.argtypes = [ci, ci, ci, ci, ci]
@@ -447,6 +448,11 @@ def forward_host(w: Weights, x_host, y_host, mode: int, scratch, y_dtype: int = 
     M = x_host.shape[0]
     _check(lib().prq_forward_host(w.handle, mode, _dptr(x_host), M, _dptr(y_host), y_dtype, _dptr(scratch),
                                   scratch.numel(), _stream_ptr(stream)), "prq_forward_host")
+
+
+def release_cached_memory() -> None:
+    """Gives the device memory that freed layers left to the next ones back to its devices (see include/prq.h)."""
+    lib().prq_release_cached_memory()
 
 
 def last_device_status(stream=None) -> int:

@@ -93,7 +93,7 @@ EncodeTiledFn encode_fn() {
 // preparation on that stream, whose writes run behind those reads.  (Waiting for the device instead would break the captures
 // of other threads, which cudaFree does not; the legacy stream cannot be captured, so no graph holds such a handle.)  At
 // most kPoolBytes and kPoolBlocks per device, the oldest goes first; all of it goes back to the device when an allocation of
-// the library fails, and with prq_weights_free(NULL).  A block serves a request of at least three quarters of its size.
+// the library fails, and with prq_release_cached_memory.  A block serves a request of at least three quarters of its size.
 class ArenaPool {
 public:
     void* take(int dev, size_t bytes, cudaStream_t stream, size_t* got) {
@@ -518,7 +518,7 @@ prq_status prq_last_device_status(prq_stream_t stream) {
 }
 
 void prq_weights_free(prq_weights* w) {
-    if (!w) { arena_pool().give_back(-1); return; }
+    if (!w) return;
     int cur = 0;
     cudaGetDevice(&cur);
     if (w->device >= 0 && w->device != cur) cudaSetDevice(w->device);
@@ -538,6 +538,8 @@ void prq_weights_free(prq_weights* w) {
     if (w->device >= 0 && w->device != cur) cudaSetDevice(cur);
     delete w;
 }
+
+void prq_release_cached_memory(void) { arena_pool().give_back(-1); }
 
 prq_status prq_prepare_weights(const uint16_t* W, int n_experts, int N, int K, const float* act_amax, float alpha,
                                int k_tail, prq_weights** out) {

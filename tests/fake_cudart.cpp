@@ -35,6 +35,7 @@ int g_launches[2];
 const char* g_last_name = "";
 int g_last_grid = 0;
 unsigned g_fill = 1;
+int g_mallocs, g_frees;   // calls; of null pointers not counted
 
 void run(Stream* s) {
     for (auto& w : s->work) w();
@@ -82,6 +83,8 @@ extern "C" {
 int fake_launches(int device) { return g_launches[device]; }
 const char* fake_last_kernel() { return g_last_name; }   // mangled
 int fake_last_grid() { return g_last_grid; }             // CTAs
+int fake_mallocs() { return g_mallocs; }
+int fake_frees() { return g_frees; }
 int fake_pending() {   // operations that no wait has covered yet
     std::lock_guard<std::mutex> lock(g_mu);
     size_t n = g_legacy.work.size();
@@ -99,12 +102,14 @@ cudaError_t cudaMalloc(void** p, size_t n) {   // fresh memory: different bytes 
     *p = std::aligned_alloc(1024, (n + 1023) / 1024 * 1024);
     if (!*p) return cudaErrorMemoryAllocation;
     std::memset(*p, static_cast<int>(g_fill++ * 37 & 0xff), n);
+    ++g_mallocs;
     return cudaSuccess;
 }
 cudaError_t cudaFree(void* p) {
     std::lock_guard<std::mutex> lock(g_mu);
     for (Stream* s : g_streams) run(s);
     run(&g_legacy);
+    if (p) ++g_frees;
     std::free(p);
     return cudaSuccess;
 }

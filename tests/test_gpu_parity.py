@@ -911,9 +911,9 @@ def test_freed_device_memory_serves_the_next_handle(prq, oracle, side_streams):
     graph.replay()
     torch.cuda.synchronize()
     assert b.sum().item() == 24
-    prq.lib().prq_weights_free(None)   # what is kept goes back
+    prq.release_cached_memory()   # what is kept goes back
     free0 = torch.cuda.mem_get_info()[0]
     w = prq.prepare_weights_device(layers[1][0], layers[1][1], 0.5, k)
     w.free()
-    prq.lib().prq_weights_free(None)
+    prq.release_cached_memory()
     assert torch.cuda.mem_get_info()[0] >= free0 - (4 << 20)

@@ -212,3 +212,22 @@ def test_a_workspace_of_its_own_belongs_to_the_stream_of_the_call(fake, monkeypa
     assert done == [("empty", side), ("zero", side)]
     monkeypatch.undo()
     w.free()
+
+
+def test_freeing_nothing_frees_nothing(fake):
+    """prq_weights_free(NULL) is a no-op, also where the library itself calls it (the search's first candidate): what freed
+    layers left to the next ones stays; prq_release_cached_memory gives it back."""
+    L, K, k = fake.lib(), 512, 64
+    fake.release_cached_memory()
+    _device_weights(fake, 640, K, k).free()
+    frees = L.fake_frees()
+    L.prq_weights_free(None)
+    assert L.fake_frees() == frees
+    w, _, _ = fake.prepare_weights_search(synth.weights(3, 64, K), np.ones((8, K), np.uint16), [0.25, 0.5], k)
+    mallocs = L.fake_mallocs()
+    _device_weights(fake, 640, K, k).free()
+    assert L.fake_mallocs() == mallocs       # the block of the first layer of this size was still there
+    w.free()
+    frees = L.fake_frees()
+    fake.release_cached_memory()
+    assert L.fake_frees() == frees + 3       # that layer's, and both candidates'
