@@ -113,12 +113,18 @@ public:
         }
         void* p = nullptr;
         *got = bytes;
-        if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+        return allocate(&p, dev, bytes) ? p : nullptr;
+    }
+    // cudaMalloc on `dev`, which is current; where that fails, once more without what is kept there.
+    bool allocate(void** p, int dev, size_t bytes) {
+        *p = nullptr;
+        if (cudaMalloc(p, bytes) == cudaSuccess) return true;
         cudaGetLastError();
         give_back(dev);
-        if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+        if (cudaMalloc(p, bytes) == cudaSuccess) return true;
         cudaGetLastError();
-        return nullptr;
+        *p = nullptr;
+        return false;
     }
     // `dev` is current.
     void put(int dev, void* p, size_t bytes) {
@@ -169,6 +175,15 @@ private:
 ArenaPool& arena_pool() {
     static ArenaPool* pool = new ArenaPool;   // (never destroyed: handles may be freed during process exit)
     return *pool;
+}
+// Every other allocation of the library, on the current device.
+template <class T>
+bool device_alloc(T** p, size_t bytes) {
+    int dev = 0;
+    void* q = nullptr;
+    if (cudaGetDevice(&dev) != cudaSuccess || !arena_pool().allocate(&q, dev, bytes)) return false;
+    *p = static_cast<T*>(q);
+    return true;
 }
 
 // Packed E2M1 codes are plain bytes: a row-major (rows x row_bytes) byte matrix, boxes of 128 bytes
@@ -756,13 +771,12 @@ static prq_status create_handle(const uint16_t* W, bool w_on_device, prq_stream_
             for (int j = 0; j < K; ++j) inv_s_perm[e * K + j] = r.inv_s[r.perm[j]];
         }
         w->d_codes_bytes = w->h_codes.size() + 256;
-        bool mem = cudaMalloc(&w->d_codes, w->d_codes_bytes) == cudaSuccess && cudaMalloc(&w->d_sf, w->d_sf_bytes) == cudaSuccess &&
-                   cudaMalloc(&w->d_perm, sizeof(int32_t) * E * K) == cudaSuccess &&
-                   cudaMalloc(&w->d_inv_s_perm, sizeof(float) * E * K) == cudaSuccess && cudaMalloc(&w->d_scales_row, w->h_scales.size()) == cudaSuccess;
+        bool mem = device_alloc(&w->d_codes, w->d_codes_bytes) && device_alloc(&w->d_sf, w->d_sf_bytes) &&
+                   device_alloc(&w->d_perm, sizeof(int32_t) * E * K) && device_alloc(&w->d_inv_s_perm, sizeof(float) * E * K) &&
+                   device_alloc(&w->d_scales_row, w->h_scales.size());
         for (int a = 0; a < kNumAlt && mem; ++a)
-            if (alt_bytes[a]) mem = cudaMalloc(&w->d_sf_alt[a], alt_bytes[a]) == cudaSuccess;
+            if (alt_bytes[a]) mem = device_alloc(&w->d_sf_alt[a], alt_bytes[a]);
         if (!mem) {
-            cudaGetLastError();
             prq_weights_free(w);
             return PRQ_ERR_OOM;
         }
@@ -803,16 +817,15 @@ static prq_status create_handle_fp8(const uint16_t* W, int N, int K, const float
         w->d_sf_bytes = (static_cast<size_t>(S8) * w->w_groups + 4) * 512;
         w->d_codes_bytes = w->h_codes.size() + 256;
         size_t alt_bytes[kNumAlt] = {};
-        bool mem = cudaMalloc(&w->d_codes, w->d_codes_bytes) == cudaSuccess && cudaMalloc(&w->d_sf, w->d_sf_bytes) == cudaSuccess &&
-                   cudaMalloc(&w->d_inv_s, sizeof(float) * K) == cudaSuccess && cudaMalloc(&w->d_scales_row, w->h_scales.size()) == cudaSuccess;
+        bool mem = device_alloc(&w->d_codes, w->d_codes_bytes) && device_alloc(&w->d_sf, w->d_sf_bytes) &&
+                   device_alloc(&w->d_inv_s, sizeof(float) * K) && device_alloc(&w->d_scales_row, w->h_scales.size());
         for (int a = 0; a < kNumAlt && mem; ++a) {
             if (!alt_wanted(false, 1, a)) continue;
             w->w_groups_alt[a] = ((N + kAltTileRows[a] - 1) / kAltTileRows[a]) * ((kAltTileRows[a] + kGroupRows - 1) / kGroupRows);
             alt_bytes[a] = (static_cast<size_t>(S8) * w->w_groups_alt[a] + 4) * 512;
-            mem = cudaMalloc(&w->d_sf_alt[a], alt_bytes[a]) == cudaSuccess;
+            mem = device_alloc(&w->d_sf_alt[a], alt_bytes[a]);
         }
         if (!mem) {
-            cudaGetLastError();
             prq_weights_free(w);
             return PRQ_ERR_OOM;
         }
@@ -910,7 +923,7 @@ prq_status prq_prepare_weights_search(const uint16_t* W, int N, int K, const uin
     // the per-alpha pipeline runs on the device from one upload of W (bit-identical to the host path)
     uint16_t* dW = nullptr;
     const size_t w_bytes = sizeof(uint16_t) * static_cast<size_t>(N) * K;
-    if (cudaMalloc(&dW, w_bytes) != cudaSuccess) { cudaGetLastError(); return PRQ_ERR_OOM; }
+    if (!device_alloc(&dW, w_bytes)) return PRQ_ERR_OOM;
     if (cudaMemcpy(dW, W, w_bytes, cudaMemcpyHostToDevice) != cudaSuccess) { cudaFree(dW); return PRQ_ERR_CUDA; }
     for (int a = 0; a < n_alphas && st == PRQ_OK; ++a) {
         prq_weights* w = nullptr;
@@ -918,9 +931,8 @@ prq_status prq_prepare_weights_search(const uint16_t* W, int N, int K, const uin
         if (st != PRQ_OK) break;
         if (!dx) {
             ws_bytes = prq_linear_workspace_bytes(w, T);
-            bool ok = cudaMalloc(&dx, x_bytes) == cudaSuccess && cudaMalloc(&dc, c_bytes) == cudaSuccess &&
-                      cudaMalloc(&dsf, sf_bytes) == cudaSuccess && cudaMalloc(&dy, y_bytes) == cudaSuccess &&
-                      cudaMalloc(&dws, ws_bytes) == cudaSuccess;
+            bool ok = device_alloc(&dx, x_bytes) && device_alloc(&dc, c_bytes) && device_alloc(&dsf, sf_bytes) &&
+                      device_alloc(&dy, y_bytes) && device_alloc(&dws, ws_bytes);
             ok = ok && cudaMemset(dws, 0, ws_bytes) == cudaSuccess;
             ok = ok && cudaMemcpy(dx, Zcal, x_bytes, cudaMemcpyHostToDevice) == cudaSuccess;
             if (!ok) { cudaGetLastError(); prq_weights_free(w); st = PRQ_ERR_OOM; break; }
@@ -1043,7 +1055,7 @@ prq_status prq_weights_clone(const prq_weights* w, prq_weights** out) {
         auto dup = [&](void* dst_pp, const void* src, size_t bytes) {
             void** pp = static_cast<void**>(dst_pp);
             if (st != PRQ_OK || !src) return;
-            if (cudaMalloc(pp, bytes) != cudaSuccess) { cudaGetLastError(); st = PRQ_ERR_OOM; return; }
+            if (!device_alloc(pp, bytes)) { st = PRQ_ERR_OOM; return; }
             if (!copies.copy(*pp, src, bytes, cudaMemcpyDeviceToDevice)) st = PRQ_ERR_CUDA;
         };
         dup(&c->d_codes, w->d_codes, w->d_codes_bytes);
@@ -1092,9 +1104,8 @@ prq_status prq_weights_offline_copy(const prq_weights* w, prq_weights** out) {
         c->h_col_err.assign(E * Kw, 0.0);
         cudaFree(c->d_perm); c->d_perm = nullptr;
         cudaFree(c->d_inv_s_perm); c->d_inv_s_perm = nullptr;
-        bool ok = cudaMalloc(&c->d_perm, sizeof(int32_t) * E * Kw) == cudaSuccess &&
-                  cudaMalloc(&c->d_inv_s_perm, sizeof(float) * E * Kw) == cudaSuccess;
-        if (!ok) { cudaGetLastError(); st = PRQ_ERR_OOM; }
+        bool ok = device_alloc(&c->d_perm, sizeof(int32_t) * E * Kw) && device_alloc(&c->d_inv_s_perm, sizeof(float) * E * Kw);
+        if (!ok) st = PRQ_ERR_OOM;
         ok = ok && copies.copy(c->d_perm, c->h_perm.data(), sizeof(int32_t) * E * Kw, cudaMemcpyHostToDevice);
         ok = ok && copies.copy(c->d_inv_s_perm, c->h_inv_s.data(), sizeof(float) * E * Kw, cudaMemcpyHostToDevice);
         if (!ok && st == PRQ_OK) st = PRQ_ERR_CUDA;

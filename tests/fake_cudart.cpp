@@ -36,6 +36,7 @@ const char* g_last_name = "";
 int g_last_grid = 0;
 unsigned g_fill = 1;
 int g_mallocs, g_frees;   // calls; of null pointers not counted
+int g_fail_in = 0;        // the allocation that fails, counted from the next one (0: none)
 
 void run(Stream* s) {
     for (auto& w : s->work) w();
@@ -85,6 +86,7 @@ const char* fake_last_kernel() { return g_last_name; }   // mangled
 int fake_last_grid() { return g_last_grid; }             // CTAs
 int fake_mallocs() { return g_mallocs; }
 int fake_frees() { return g_frees; }
+void fake_fail_malloc(int nth) { g_fail_in = nth; }
 int fake_pending() {   // operations that no wait has covered yet
     std::lock_guard<std::mutex> lock(g_mu);
     size_t n = g_legacy.work.size();
@@ -99,6 +101,7 @@ cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { *v = 148; retu
 cudaError_t cudaGetLastError() { const cudaError_t e = t_last; t_last = cudaSuccess; return e; }
 cudaError_t cudaMalloc(void** p, size_t n) {   // fresh memory: different bytes every time
     std::lock_guard<std::mutex> lock(g_mu);
+    if (g_fail_in > 0 && --g_fail_in == 0) return t_last = cudaErrorMemoryAllocation;
     *p = std::aligned_alloc(1024, (n + 1023) / 1024 * 1024);
     if (!*p) return cudaErrorMemoryAllocation;
     std::memset(*p, static_cast<int>(g_fill++ * 37 & 0xff), n);

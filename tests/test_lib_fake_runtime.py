@@ -231,3 +231,33 @@ def test_freeing_nothing_frees_nothing(fake):
     frees = L.fake_frees()
     fake.release_cached_memory()
     assert L.fake_frees() == frees + 3       # that layer's, and both candidates'
+
+
+@pytest.mark.parametrize("what", ["host", "mxfp8", "device", "search", "clone", "offline_copy"])
+def test_an_allocation_that_fails_is_tried_again_without_what_is_kept(fake, what):
+    """Memory of freed layers goes back to the device before any allocation of the library gives up -- whichever it is."""
+    L, N, K, k = fake.lib(), 64, 512, 64
+    W, amax = synth.weights(3, N, K), np.ones(K, np.float32)
+    original = _device_weights(fake, N, K, k)
+    call = {"host": lambda: fake.prepare_weights(W, amax, 0.5, k), "mxfp8": lambda: fake.prepare_weights(W, amax, 0.5, 0, fmt=fake.FMT_MXFP8),
+            "device": lambda: _device_weights(fake, N, K, k), "search": lambda: fake.prepare_weights_search(W, np.ones((200, K), np.uint16), [0.25, 0.5], k)[0],
+            "clone": original.clone, "offline_copy": original.offline_copy}[what]
+    nth = 1
+    while True:
+        fake.release_cached_memory()
+        _device_weights(fake, 640, K, k).free()         # a block is kept, too large for anything in the call
+        mallocs = L.fake_mallocs()
+        L.fake_fail_malloc(nth)
+        w = call()
+        done = L.fake_mallocs() - mallocs < nth         # there was no nth allocation to fail
+        L.fake_fail_malloc(0)
+        w.free()
+        if done:
+            break
+        mallocs = L.fake_mallocs()
+        _device_weights(fake, 640, K, k).free()
+        assert L.fake_mallocs() == mallocs + 1          # that block went back
+        nth += 1
+    assert nth > 1
+    original.free()
+    fake.release_cached_memory()
