@@ -1191,14 +1191,17 @@ size_t prq_act_bytes(int M, int K, int k_tail, int n_groups, prq_buf which) {
 // The weights that the decode product behind a quantiser of `n` layers will stream.  From 4 MB on: less than that the product's
 // own CTAs have requested by the time it starts (1024 x 2560, 1.4 MB, 16 / 128 tokens 4.43 / 7.01 without the hint, 4.78 /
 // 7.23 with it); up to 48 MB, a share of L2 that leaves room for what is in use.
-static void weight_hints(int n, const prq_weights* const* ws, int M, WeightHint* hints) {
+static bool weight_hints(int n, const prq_weights* const* ws, int M, WeightHints* hints) {
+    if (M > 128) return false;
     auto code_bytes = [&](const prq_weights* w) { return static_cast<size_t>(w->N) * (static_cast<size_t>(w->K) + w->k_tail) / 2; };
     size_t total = 0;
     for (int i = 0; i < n; ++i) total += code_bytes(ws[i]);
-    if (M > 128 || total < (4u << 20) || total > (48u << 20)) return;
+    if (total < (4u << 20) || total > (48u << 20)) return false;
+    *hints = {};
     for (int i = 0; i < n; ++i)
-        hints[i] = WeightHint{ws[i]->d_codes, ws[i]->d_sf, static_cast<uint32_t>(code_bytes(ws[i])),
-                              static_cast<uint32_t>(static_cast<size_t>(ws[i]->plan.S) * ws[i]->w_groups * kSfGroupBytes)};
+        hints->lay[i] = {ws[i]->d_codes, ws[i]->d_sf, static_cast<uint32_t>(code_bytes(ws[i])),
+                         static_cast<uint32_t>(static_cast<size_t>(ws[i]->plan.S) * ws[i]->w_groups * kSfGroupBytes)};
+    return true;
 }
 
 prq_status prq_quantize_act(const prq_weights* w, prq_act_mode mode, const void* x, int M, int ldx,
@@ -1240,9 +1243,9 @@ prq_status prq_quantize_act(const prq_weights* w, prq_act_mode mode, const void*
     prq_status st = device_info(w->device, &di);
     if (st != PRQ_OK) return st;
     p.status = di->status_ptr;
-    WeightHint hint = {};
-    if (!expert_offsets) weight_hints(1, &w, M, &hint);
-    cudaError_t e = launch_quant_act(p, mode == PRQ_ACT_SCALE_PERM, p.act_groups, hint, static_cast<cudaStream_t>(stream));
+    WeightHints hints;
+    const bool ask = !expert_offsets && weight_hints(1, &w, M, &hints);
+    cudaError_t e = launch_quant_act(p, mode == PRQ_ACT_SCALE_PERM, p.act_groups, ask ? &hints : nullptr, static_cast<cudaStream_t>(stream));
     g_launches.fetch_add(1);
     return e == cudaSuccess ? PRQ_OK : PRQ_ERR_CUDA;
 }
@@ -1277,8 +1280,9 @@ prq_status prq_quantize_act_multi(int n, const prq_weights* const* ws, prq_act_m
     prq_status st = device_info(ws[0]->device, &di);
     if (st != PRQ_OK) return st;
     b.status = di->status_ptr;
-    weight_hints(n, ws, M, b.hint);
-    cudaError_t e = launch_quant_act_batch(b, mode == PRQ_ACT_SCALE_PERM, static_cast<cudaStream_t>(stream));
+    WeightHints hints;
+    const bool ask = weight_hints(n, ws, M, &hints);
+    cudaError_t e = launch_quant_act_batch(b, mode == PRQ_ACT_SCALE_PERM, ask ? &hints : nullptr, static_cast<cudaStream_t>(stream));
     g_launches.fetch_add(1);
     return e == cudaSuccess ? PRQ_OK : PRQ_ERR_CUDA;
 }

@@ -32,18 +32,21 @@ struct QuantParams {
     int* status;             // device status word (a bounded wait that ran out is recorded there)
 };
 
-// What the product with a layer's prepared weights will read, for the quantiser to ask for in L2 while it runs (all zero: it
-// asks for nothing).
-struct WeightHint {
-    const uint8_t* codes;
-    const uint8_t* sf;
-    uint32_t code_bytes, sf_bytes;
-};
-cudaError_t launch_quant_act(const QuantParams& p, bool scale_perm, int grid_groups, const WeightHint& hint, cudaStream_t stream);
-
 // Several dense layers that read the same activation (q / k / v, gate / up), quantised by one launch: the
 // fields that differ per layer; everything else comes from `base`.
 constexpr int kMaxBatch = 4;
+
+// What the product with each layer's prepared weights will read, for the quantiser to ask for in L2 while it runs.
+struct WeightHints {
+    struct {
+        const uint8_t* codes;
+        const uint8_t* sf;
+        uint32_t code_bytes, sf_bytes;
+    } lay[kMaxBatch];
+};
+// `ask` may be null: the launch asks for nothing
+cudaError_t launch_quant_act(const QuantParams& p, bool scale_perm, int grid_groups, const WeightHints* ask, cudaStream_t stream);
+
 struct QuantLayer {                      // what differs per batched layer
     const int32_t* perm;
     const float* inv_s_perm;
@@ -64,13 +67,10 @@ struct QuantBatch {
     int groups_per_lin;                  // blockIdx.y = layer * groups_per_lin + group
     int n_atoms, n_tail, tail_split;     // set by the launcher: 128-column atoms, how many of them are tail atoms
                                          // (scale + permute mode), and into how many row shares each of those is cut
-    int ask;                             // set by the launcher: there are hints (read here, so that a launch without them
-                                         // does not fetch their line of parameters)
     QuantLayer lay[kMaxBatch];
     int* status;                         // device status word
-    WeightHint hint[kMaxBatch];
 };
-cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, cudaStream_t stream);
+cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, const WeightHints* ask, cudaStream_t stream);
 
 struct GemmParams {
     int M;                   // activation rows (all experts)

@@ -21,6 +21,7 @@
 
 #include <atomic>
 #include <cstdlib>
+#include <type_traits>
 
 #include "prq_internal.h"
 #include "prq_kernels.h"
@@ -57,9 +58,16 @@ __device__ __forceinline__ void ask_for(const uint8_t* base, uint32_t bytes, int
     if (at < bytes) prefetch_l2(base + at, min(share, (bytes - at)) & ~15u);
 }
 
-template <bool kScalePerm, bool kBatch>
+// The hints are parameters of instances of their own (kAsk): 100 bytes more in the parameters of every launch made the quantiser
+// 0.06 - 0.1 us slower alone and up to 4 % at 2048 rows (2560 x 9728 10.7 -> 11.1 us, 256 x 256 at 16 tokens 1.54 -> 1.63).
+template <bool kAsk>
+struct AskParam {};
+template <>
+struct AskParam<true> : WeightHints {};
+
+template <bool kScalePerm, bool kBatch, bool kAsk>
 __global__ void __launch_bounds__(kQuantThreads, kScalePerm ? 3 : 4)
-quant_act_kernel(const QuantBatch b) {
+quant_act_kernel(const QuantBatch b, const AskParam<kAsk> ask) {
     __shared__ __align__(16) uint8_t sf_atom[512];
     __shared__ int s_tile_start[kMaxExperts + 1];
 
@@ -123,11 +131,13 @@ quant_act_kernel(const QuantBatch b) {
         }
     };
     const bool dense = p.expert_offsets == nullptr;
-    if (dense && b.ask && threadIdx.x == 0) {
-        const int parts = static_cast<int>(gridDim.x * gridDim.z) * b.groups_per_lin;
-        const int part = static_cast<int>(blockIdx.x + gridDim.x * (blockIdx.z + gridDim.z * (blockIdx.y - lin * b.groups_per_lin)));
-        ask_for(b.hint[lin].codes, b.hint[lin].code_bytes, part, parts);
-        ask_for(b.hint[lin].sf, b.hint[lin].sf_bytes, part, parts);
+    if constexpr (kAsk) {
+        if (threadIdx.x == 0) {
+            const int parts = static_cast<int>(gridDim.x * gridDim.z) * b.groups_per_lin;
+            const int part = static_cast<int>(blockIdx.x + gridDim.x * (blockIdx.z + gridDim.z * (blockIdx.y - lin * b.groups_per_lin)));
+            ask_for(ask.lay[lin].codes, ask.lay[lin].code_bytes, part, parts);
+            ask_for(ask.lay[lin].sf, ask.lay[lin].sf_bytes, part, parts);
+        }
     }
     if (kScalePerm && dense) load_layer_constants(0);
     // Identity mode: this CTA's rows in L2 before the wait, one 128-byte line per thread.  The CTAs that come up beside the GEMM
@@ -365,12 +375,26 @@ struct ColsPlan {
 constexpr int kColsMaxStages = 8;
 constexpr size_t kColsSmem = 220 * 1024;   // shared memory of an SM that the rows in flight may take
 
+// With hints the plan stands in front, so that what every CTA reads first shares two 64-byte lines of parameters (2560 x 9728 at
+// 64 tokens 9.23 -> 8.49 us with the product behind it, 4096 x 2560 7.13 -> 6.78).
+template <bool kAsk>
+struct ColsParam {
+    QuantBatch b;
+    ColsPlan plan;
+};
+template <>
+struct ColsParam<true> {
+    ColsPlan plan;
+    QuantBatch b;
+    WeightHints ask;
+};
+
 // kCols: columns per lane, 8 or 16.  kRowsC: rows per slice, 1, 2 or 4.
-// (The plan stands in front of the batch so that every CTA's first reads share two 64-byte lines of parameters; behind it, and
-// behind the hints, a decoder block of seven launches at 4096 tokens took 1.5 us longer, with the hints as a third parameter 4.5.)
-template <int kCols, int kRowsC, bool kGrouped, int kMaxT>
+template <int kCols, int kRowsC, bool kGrouped, int kMaxT, bool kAsk>
 __global__ void __launch_bounds__(kMaxT, 1)
-quant_act_cols_kernel(const ColsPlan plan_c, const QuantBatch b) {
+quant_act_cols_kernel(const __grid_constant__ ColsParam<kAsk> param) {
+    const QuantBatch& b = param.b;
+    const ColsPlan& plan_c = param.plan;
     constexpr int kPairs = kCols / 2;
     constexpr int kBlkLanes = kBlock / kCols;            // lanes per 32-element block: 4 or 2
     constexpr int kAtomLanes = kAtomK / kCols;           // lanes per scale atom: 16 or 8
@@ -431,12 +455,13 @@ quant_act_cols_kernel(const ColsPlan plan_c, const QuantBatch b) {
     __syncthreads();
     if (!kGrouped) {
         // a dense layer's constants belong to the prepared weights, not to an earlier kernel of the stream
-        if (!loader) {
-            load_constants(0);
-        } else if (b.ask && lane == 0) {
-            const int part = blockIdx.x + gridDim.x * blockIdx.y, parts = gridDim.x * gridDim.y;
-            ask_for(b.hint[blockIdx.z].codes, b.hint[blockIdx.z].code_bytes, part, parts);
-            ask_for(b.hint[blockIdx.z].sf, b.hint[blockIdx.z].sf_bytes, part, parts);
+        if (!loader) load_constants(0);
+        if constexpr (kAsk) {
+            if (loader && lane == 0) {
+                const int part = blockIdx.x + gridDim.x * blockIdx.y, parts = gridDim.x * gridDim.y;
+                ask_for(param.ask.lay[blockIdx.z].codes, param.ask.lay[blockIdx.z].code_bytes, part, parts);
+                ask_for(param.ask.lay[blockIdx.z].sf, param.ask.lay[blockIdx.z].sf_bytes, part, parts);
+            }
         }
         grid_dependency_wait();
     } else {
@@ -636,9 +661,9 @@ quant_act_cols_kernel(const ColsPlan plan_c, const QuantBatch b) {
 }
 
 // Registers of one instance as built (they decide how many of its CTAs an SM holds).
-template <int kCols, int kRowsC, bool kGrouped, int kMaxT>
-cudaError_t launch_cols_impl(const QuantBatch& b, int sm_count, cudaStream_t stream) {
-    auto kernel = quant_act_cols_kernel<kCols, kRowsC, kGrouped, kMaxT>;
+template <int kCols, int kRowsC, bool kGrouped, int kMaxT, bool kAsk = false>
+cudaError_t launch_cols_impl(const QuantBatch& b, int sm_count, cudaStream_t stream, const WeightHints* ask = nullptr) {
+    auto kernel = quant_act_cols_kernel<kCols, kRowsC, kGrouped, kMaxT, kAsk>;
     const int lanes = (b.K + kStageK - 1) / kStageK * (kStageK / kCols);
     const int all_warps = (lanes + 31) / 32, max_warps = kMaxT / 32 - 1;
     const int chunks = (all_warps + max_warps - 1) / max_warps, warps = (all_warps + chunks - 1) / chunks;
@@ -684,11 +709,9 @@ cudaError_t launch_cols_impl(const QuantBatch& b, int sm_count, cudaStream_t str
         // Where the CTAs ask for weights, no more stages of rows than a CTA has slices: they then come up beside a GEMM that
         // fills its SMs and ask while it ends.  (Without weights to ask for that only disturbs it: 1024 x 2560 at 16 tokens 4.43 / 4.70.)
         const int g2 = want < 1 ? 1 : want < cp.n_slices ? want : cp.n_slices, mine = ((cp.strided ? live : cp.n_slices) + g2 - 1) / g2;
-        if (b.hint[0].code_bytes && cp.n_stages > mine) cp.n_stages = mine;
+        if (kAsk && cp.n_stages > mine) cp.n_stages = mine;
     }
     cudaLaunchConfig_t cfg = {};
-    QuantBatch bb = b;
-    bb.ask = !kGrouped && b.hint[0].code_bytes > 0;
     cfg.gridDim = dim3(want < 1 ? 1 : want < cp.n_slices ? want : cp.n_slices, chunks, b.n_lin);
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = cp.n_stages * stage;
@@ -698,12 +721,13 @@ cudaError_t launch_cols_impl(const QuantBatch& b, int sm_count, cudaStream_t str
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, cp, bb);
+    if constexpr (kAsk) return cudaLaunchKernelEx(&cfg, kernel, ColsParam<true>{cp, b, *ask});
+    else return cudaLaunchKernelEx(&cfg, kernel, ColsParam<false>{b, cp});
 }
 
 }  // namespace
 
-cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, cudaStream_t stream) {
+cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, const WeightHints* ask, cudaStream_t stream) {
     const QuantBatch& p = b;
     const int grid_groups = b.groups_per_lin * b.n_lin;
     cudaLaunchConfig_t cfg = {};
@@ -760,17 +784,17 @@ cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, cudaStr
         if (cols && grouped && fits(4)) return launch_cols_impl<8, 4, true, 544>(b, sms, stream);
         if (cols && !grouped) {
             const bool large = b.M >= 1500 && p.K >= 2048;
-            if (b.M <= 128 && p.K <= 4096) return launch_cols_impl<16, 1, false, 192>(b, sms, stream);
+            if (b.M <= 128 && p.K <= 4096)
+                return ask ? launch_cols_impl<16, 1, false, 192, true>(b, sms, stream, ask) : launch_cols_impl<16, 1, false, 192>(b, sms, stream);
             if (large && p.K <= 8192) return launch_cols_impl<16, 4, false, 384>(b, sms, stream);
             if (large && fits(2)) return launch_cols_impl<16, 2, false, 640>(b, sms, stream);
-            if (fits(2)) return launch_cols_impl<16, 2, false, 320>(b, sms, stream);
+            if (fits(2)) return ask ? launch_cols_impl<16, 2, false, 320, true>(b, sms, stream, ask) : launch_cols_impl<16, 2, false, 320>(b, sms, stream);
         }
     }
     // the tail atoms of the scale + permute mode in shares of 16 rows (128 / 8), see the kernel
     QuantBatch bb = b;
     bb.n_atoms = n_atoms;
     bb.n_tail = 0; bb.tail_split = 1;
-    bb.ask = b.hint[0].code_bytes > 0;
     // (dense launches only: a grouped launch has a CTA per expert group and column atom already, each with the fixed
     // cost of finding its expert -- eight times as many tail CTAs made the 128-expert quantiser 35-50 % slower, and its
     // launches are long enough for a 20 us CTA not to be their end)
@@ -786,14 +810,21 @@ cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, cudaStr
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (b.n_lin > 1)
-        return scale_perm ? cudaLaunchKernelEx(&cfg, quant_act_kernel<true, true>, bb)
-                          : cudaLaunchKernelEx(&cfg, quant_act_kernel<false, true>, bb);
-    return scale_perm ? cudaLaunchKernelEx(&cfg, quant_act_kernel<true, false>, bb)
-                      : cudaLaunchKernelEx(&cfg, quant_act_kernel<false, false>, bb);
+    auto launch = [&](auto batch) {
+        constexpr bool kBatch = decltype(batch)::value;
+        if (ask) {
+            AskParam<true> asked;
+            static_cast<WeightHints&>(asked) = *ask;
+            return scale_perm ? cudaLaunchKernelEx(&cfg, quant_act_kernel<true, kBatch, true>, bb, asked)
+                              : cudaLaunchKernelEx(&cfg, quant_act_kernel<false, kBatch, true>, bb, asked);
+        }
+        return scale_perm ? cudaLaunchKernelEx(&cfg, quant_act_kernel<true, kBatch, false>, bb, AskParam<false>{})
+                          : cudaLaunchKernelEx(&cfg, quant_act_kernel<false, kBatch, false>, bb, AskParam<false>{});
+    };
+    return b.n_lin > 1 ? launch(std::true_type{}) : launch(std::false_type{});
 }
 
-cudaError_t launch_quant_act(const QuantParams& p, bool scale_perm, int grid_groups, const WeightHint& hint, cudaStream_t stream) {
+cudaError_t launch_quant_act(const QuantParams& p, bool scale_perm, int grid_groups, const WeightHints* ask, cudaStream_t stream) {
     QuantBatch b = {};
     b.x = p.x; b.expert_offsets = p.expert_offsets; b.M = p.M; b.ldx = p.ldx; b.K = p.K;
     b.n_experts = p.n_experts; b.act_groups = p.act_groups;
@@ -801,8 +832,7 @@ cudaError_t launch_quant_act(const QuantParams& p, bool scale_perm, int grid_gro
     b.groups_per_lin = grid_groups;
     b.lay[0] = QuantLayer{p.perm, p.inv_s_perm, p.codes, p.scales_row, p.scales_sf, p.k_tail};
     b.status = p.status;
-    b.hint[0] = hint;
-    return launch_quant_act_batch(b, scale_perm, stream);
+    return launch_quant_act_batch(b, scale_perm, ask, stream);
 }
 
 }  // namespace prq

@@ -4,6 +4,7 @@ import concurrent.futures
 import ctypes
 import importlib.util
 import os
+import re
 import subprocess
 
 import numpy as np
@@ -261,3 +262,34 @@ def test_an_allocation_that_fails_is_tried_again_without_what_is_kept(fake, what
     assert nth > 1
     original.free()
     fake.release_cached_memory()
+
+
+def _asks(fake, ws, M, mode):
+    """One quantiser launch for the layers `ws`; whether it is an instance that takes hints (its last template argument)."""
+    L, p, K, n = fake.lib(), lambda a: a.ctypes.data, ws[0].K, len(ws)
+    some, arr = _aligned(16), ctypes.c_void_p * n    # (nothing is read or written: the kernels do not run)
+    if n == 1:
+        fake._check(L.prq_quantize_act(ws[0].handle, mode, p(some), M, K, None, p(some), None, p(some), None), "quantise")
+    else:
+        fake._check(L.prq_quantize_act_multi(n, arr(*[w.handle.value for w in ws]), mode, p(some), M, K, arr(*[p(some)] * n), arr(*[p(some)] * n), None), "multi")
+    return re.search(r"quant_act\w*_kernelI\w*?Lb([01])EE", L.fake_last_kernel().decode())[1] == "1"
+
+
+@pytest.mark.parametrize("asks,Ns,K,M", [
+    (True, [2560], 4096, 1), (True, [2560], 4096, 128), (False, [2560], 4096, 129), (False, [2560], 4096, 2048), (False, [256], 256, 16), (False, [1024], 2560, 64),
+    (True, [4096, 1024, 1024], 2560, 64), (False, [512, 256], 1024, 64)])
+def test_which_quantisers_ask_for_weights(fake, asks, Ns, K, M):
+    """Everything else takes the instances without hints, whose launches carry no parameters for them."""
+    ws = [_zero_weights(fake, N, K) for N in Ns]
+    for mode in (fake.ACT_IDENTITY, fake.ACT_SCALE_PERM):
+        assert _asks(fake, ws, M, mode) == asks, mode
+    for w in ws:
+        w.free()
+
+
+def _zero_weights(fake, N, K, k=0, gated=False):
+    W, amax, h = np.zeros((N, K), np.uint16), np.ones(K, np.float32), ctypes.c_void_p()
+    o = fake._opts(False, gated)
+    fake._check(fake.lib().prq_prepare_weights_device(W.ctypes.data, 1, N, K, amax.ctypes.data, 0.5, k, ctypes.cast(ctypes.pointer(o), ctypes.c_void_p), None,
+                                                      ctypes.byref(h)), "prepare")
+    return fake.Weights(h)
