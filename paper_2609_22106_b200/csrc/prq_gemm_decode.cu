@@ -8,7 +8,10 @@
 // token t (t mod cluster size); the owner adds up what it received and writes its tokens to y.  The pushes are asynchronous
 // stores whose bytes are counted on an mbarrier of the owner, which therefore waits for exactly its own tokens (the 32 KB
 // of a 64-token tile among seven CTAs: 1500 cycles, with plain stores and a cluster barrier 2800; one bulk copy per
-// owner 2170).  No global scratch, no atomics, and the summation order is fixed (peer 0, 1, ...), so
+// owner 2170).  Two CTAs with more than 64 tokens park their sums instead and copy the other one's half with plain stores, whole
+// rows at a time, and a cluster barrier (256 x 256 at 80 / 128 tokens: asynchronous 4.14 / 5.36 us, parked 3.90 / 4.94, 6144 x 2560
+// 7.01 / 8.06 and 6.76 / 7.59; with three CTAs the asynchronous stores are ahead, 2304 x 2304 at 128 tokens 6.04 against 6.30).
+// No global scratch, no atomics, and the summation order is fixed (peer 0, 1, ...), so
 // the result is reproducible.  For up to 32 tokens two CTAs fit on an SM, so that the
 // CTAs of the next kernel of the stream (the next layer's GEMM) are resident and streaming their weights
 // while this one finishes.
@@ -219,8 +222,9 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeBatch b) {
     // barrier only tells the peers that this CTA (and its bar_recv) is there before they push: arrive here, wait just
     // before the pushes, so that it costs nothing.
     const int n_own = split < p.M ? slot_of(p.M - split + splits - 1) : 0;
+    const bool parked = BN == 128 && splits == 2;   // two CTAs, more than 64 tokens: see the exchange
     if (splits > 1) {
-        if (threadIdx.x == 0) mbar_arrive_expect_tx(smem_u32(&bar_recv), static_cast<uint32_t>(n_own) * splits * 512u);
+        if (!parked && threadIdx.x == 0) mbar_arrive_expect_tx(smem_u32(&bar_recv), static_cast<uint32_t>(n_own) * splits * 512u);
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     }
     // set-up done: let the next kernel of the stream be scheduled (its launch latency then overlaps this
@@ -434,7 +438,9 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeBatch b) {
             if (trace && threadIdx.x == 64) trace[200] = clock64();
         }
         // Accumulator -> registers -> y (splits == 1), or straight into the receive buffers of the tokens' owners: token
-        // t belongs to CTA t mod splits, its slot there is t / splits, a receive buffer is [peer][slot][row].
+        // t belongs to CTA t mod splits, its slot there is t / splits, a receive buffer is [peer][slot][row].  (Or, of two CTAs,
+        // -> the pipeline's buffers, which nothing reads any more, token by token: the other one's tokens go from there to its
+        // receive buffer, this one's own are added from there.)
         if (splits > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // every peer is there
         if (mbar_wait(smem_u32(&bar_acc_full), 0, abort_flag)) {
             if (trace && threadIdx.x == 64) trace[192] = clock64();
@@ -460,6 +466,9 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeBatch b) {
                             }
                         }
                     }
+                } else if (parked) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) reinterpret_cast<float*>(smem)[(c * 16 + i) * 128 + q4 * 32 + lane] = __uint_as_float(v[i]);
                 } else {
                     // 4 x 4 transposes among the lanes of four weight rows: lane `sub` gets token 4 g + sub of those rows and
                     // sends them with one 16-byte asynchronous store, whose bytes are counted on the owner's barrier
@@ -490,8 +499,21 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeBatch b) {
         }
         tc_fence_before_sync();
         if (splits > 1) {
-            // all partial sums of this CTA's tokens have arrived (nobody writes to this CTA after that)
-            if (n_own > 0) mbar_wait(smem_u32(&bar_recv), 0, abort_flag);
+            if (parked) {
+                asm volatile("bar.sync 1, %0;" ::"n"(32 * C::kEpiWarps) : "memory");   // the parked tile is complete
+                for (int tok = abort_flag_s ? p.M : (split ^ 1) + 2 * ew; tok < p.M; tok += 2 * C::kEpiWarps) {
+                    uint4 v;
+                    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(smem_base + tok * 512 + lane * 16));
+                    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};"
+                                 ::"r"(peer_addr(recv_base + ((split * slots + (tok >> 1)) * 128 + 4 * lane) * 4, split ^ 1)), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+                }
+                __syncwarp();
+                asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+            } else if (n_own > 0) {
+                // all partial sums of this CTA's tokens have arrived (nobody writes to this CTA after that)
+                mbar_wait(smem_u32(&bar_recv), 0, abort_flag);
+            }
             // this CTA's tokens: split, split + splits, ...; a thread owns 4 consecutive weight rows and
             // every kEpiWarps-th slot; the sum runs in peer order
             const int n = n0 + 4 * lane;
@@ -505,7 +527,8 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeBatch b) {
                     if (peer < splits)
                         asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
                                      : "=f"(v[peer].x), "=f"(v[peer].y), "=f"(v[peer].z), "=f"(v[peer].w)
-                                     : "r"(recv_base + ((peer * slots + slot) * 128 + 4 * lane) * 4));
+                                     : "r"(parked && peer == split ? smem_base + tok * 512 + lane * 16
+                                                                   : recv_base + ((peer * slots + slot) * 128 + 4 * lane) * 4));
                 float4 sum = v[0];
 #pragma unroll
                 for (int peer = 1; peer < 8; ++peer)
@@ -533,11 +556,15 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeBatch b) {
         // A CTA that gave up pushes nothing and sums nothing, but healthy peers still deliver their partial
         // sums into its receive buffer and count them on its barrier: it stays until they have (bounded), so
         // that no store of a peer reaches the shared memory of a CTA that has left.
-        if (splits > 1 && abort_flag_s && n_own > 0 && threadIdx.x == 64)
+        if (splits > 1 && !parked && abort_flag_s && n_own > 0 && threadIdx.x == 64)
             mbar_wait_after_abort(smem_u32(&bar_recv), 0);
     }
     // the cluster barrier that the epilogue warps have passed
-    if (splits > 1 && warp < 2) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (splits > 1 && warp < 2) {
+        __syncwarp();
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (parked) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
 
     // ------------------------------------------------------------ teardown (normal and aborted)
     tc_fence_before_sync();

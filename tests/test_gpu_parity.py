@@ -450,6 +450,29 @@ def test_decode_several_ring_passes(prq, oracle, splits, monkeypatch):
     w.free()
 
 
+@pytest.mark.parametrize("y_dtype", ["f32", "bf16"])
+def test_decode_exchange_of_two_ctas(prq, oracle, y_dtype, monkeypatch):
+    """Two CTAs per cluster from 65 tokens on: even and odd token counts, one stage and several ring passes per CTA, a ragged last
+    tile of features."""
+    monkeypatch.setenv("PRQ_DECODE_SPLITS", "2")
+    for N, K, k in ((200, 256, 32), (328, 2592, 96)):
+        L = synth.layer(0, N, K, 128, T_cal=32, tag=931)
+        amax = oracle.channel_amax(L["zcal"])
+        w = prq.prepare_weights(L["W"], amax, 0.25, k)
+        o = oracle.prepare(L["W"], amax, float(np.float32(0.25)), k)
+        ca, sa = oracle.augment_act(*oracle.quantize_act(L["x"]), k)
+        y_ref = oracle.matmul(ca, sa, o["wcodes"], o["wscales"])
+        x = to_dev_bf16(L["x"])
+        for M in (65, 66, 79, 80, 97, 127, 128):
+            codes, _, sf = prq.quantize_act(w, x[:M], prq.ACT_IDENTITY)
+            y = prq.linear(w, codes, sf, M, prq.F32)
+            assert np.abs(y.cpu().numpy().astype(np.float64) - y_ref[:M]).max() <= prq_ref.tolerance(y_ref[:M]), M
+            if y_dtype == "bf16":
+                assert torch.equal(prq.linear(w, codes, sf, M, prq.BF16), y.bfloat16()), M
+        w.free()
+    assert prq.last_device_status() == 0
+
+
 def test_linear_fused_rejects_what_it_does_not_cover(prq, oracle):
     L = synth.layer(0, 128, 256, 4, T_cal=16, tag=950)
     w = prq.prepare_weights(L["W"], oracle.channel_amax(L["zcal"]), 0.5, 32)
