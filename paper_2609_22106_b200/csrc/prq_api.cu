@@ -243,7 +243,7 @@ constexpr int kAltWide = 1;
 bool alt_wanted(bool gated, int n_experts, int a) { return n_experts > 1 ? a == kAltWide : gated ? a == kAltGated : a != kAltGated; }
 
 // Weight-side tensor maps of a handle, encoded once at creation (cloning re-encodes: other addresses).
-int decode_splits_for(int n_tiles, int S, int M, DeviceInfo* di);
+int decode_splits_for(int n_tiles, int S, int M, bool two_calls, DeviceInfo* di);
 prq_status build_weight_maps(prq_weights* w) {
     w->maps_ready = false;
     const uint64_t Ka = static_cast<uint64_t>(w->K) + w->k_tail, E = w->n_experts;
@@ -263,7 +263,7 @@ prq_status build_weight_maps(prq_weights* w) {
         // costs 0.2 of 5.4 us)
         DeviceInfo* di;
         st = device_info(w->device, &di);
-        for (int M = 1; M <= 16 && st == PRQ_OK; ++M) w->splits16[M] = static_cast<uint8_t>(decode_splits_for((w->N + 127) / 128, w->plan.S, M, di));
+        for (int M = 1; M <= 16 && st == PRQ_OK; ++M) w->splits16[M] = static_cast<uint8_t>(decode_splits_for((w->N + 127) / 128, w->plan.S, M, false, di));
         w->maps_ready = st == PRQ_OK;   // (the dense calls refuse stacked experts)
     }
     return st;
@@ -303,14 +303,16 @@ int grouped_groups(int M, int n_groups) { return n_groups == 1 ? dense_groups(M)
 
 int decode_bn(int M) { return M <= 16 ? 16 : M <= 32 ? 32 : M <= 64 ? 64 : 128; }
 
-// Cluster size (= number of K-splits) of the decode kernel: the one that puts the most SMs to work in
-// the first wave, given how many clusters of each size the device can hold at once.
-int decode_splits_for(int n_tiles, int S, int M, DeviceInfo* di) {
+// Cluster size (= number of K-splits) of the decode kernel, given how many clusters of each size the device can hold at once.
+// Up to 32 tokens two CTAs share an SM, so that a launch is set up and has its weights while the one before it runs -- as far as
+// both fit: clusters that come up late pay set-up and weights behind the dependency.  From 33 tokens on a CTA fills an SM: the
+// size that puts the most SMs to work in the first wave.
+// `two_calls`: a quantiser stands in front.  (A single layer on up to 16 tokens is given false whichever form the call has:
+// prq_linear_fused promises the bits of the two calls, so both need the same splits.)
+int decode_splits_for(int n_tiles, int S, int M, bool two_calls, DeviceInfo* di) {
     const int bn = decode_bn(M);
     const int bi = bn == 16 ? 0 : bn == 32 ? 1 : bn == 64 ? 2 : 3;
-    const int forced = env_int("PRQ_DECODE_SPLITS", 0);
     const int limit = std::min(8, S);
-    if (forced > 0) return std::min(forced, limit);
     std::lock_guard<std::mutex> lock(g_dev_mutex);
     auto resident = [&](int s) {
         int& mc = di->max_clusters[bi][s];
@@ -318,22 +320,22 @@ int decode_splits_for(int n_tiles, int S, int M, DeviceInfo* di) {
         return mc;
     };
     if (bn <= 32) {
-        // Up to 32 tokens two CTAs share an SM, so that a launch is set up and has its weights while the one before it runs
-        // -- as far as both fit: clusters that come up late pay set-up and weights behind the dependency.  In hundredths of
-        // a microsecond: a stage costs about 23 and one per token (the quantiser, fused), half as much again beyond the
-        // ring, and late clusters 45 and up to 100 more with their share of the launch.  (us a launch, largest cluster that
-        // oversubscribes the SMs by a fifth at most -> this rule: 4096 x 2560 one / sixteen tokens 3.42 / 4.35 -> 2.74 / 4.21
-        // (5 -> 4 splits), 2560 x 4096 3.37 / 4.35 -> 2.74 / 4.19 (8 -> 6); quantise + multiply 32 tokens 6.34 -> 5.80, 9728 x 2560
-        // 7.76 -> 7.08 (2 -> 3); 2560 x 9728 stays at 8: 4.11, 6 would be 4.47.)
-        const bool two_calls = bn == 32;   // a quantiser stands in front, and hides part of what comes late
+        // In hundredths of a microsecond, the clusters of two launches against what fits.  One launch that quantises as well: a
+        // stage costs about 23 and one per token, 18 more beyond the ring, late clusters 45 and up to 100 more with their share of
+        // the launch (4096 x 2560 one / sixteen tokens 2.55 / 4.10 with four splits, five 3.30 / 4.20, 2560 x 4096 2.82 / 4.10 with
+        // six, eight 3.46 / 4.22; 2560 x 9728 stays at eight: 4.28, six 4.46).  With a quantiser in front, which hides part of
+        // what comes late: 15 a stage, 15 more beyond the ring, 10 and up to 60 more for late clusters (quantise + multiply at
+        // 1 / 16 / 32 tokens: two of 2560 x 4096 take four or five, 5.80 / 6.35 / 7.51, three 6.29 / 6.94 / 7.82, six 6.18 / 6.88 / 7.59;
+        // 9728 x 2560 three, 5.88 / 6.75 / 7.44, two 6.14 / 7.01 / 8.00; 12288 x 1024 at 32 one, 5.57, two 5.85).
         const int ring = bn == 16 ? 5 : 4;
+        const int per_stage = two_calls ? 15 : 23 + M, beyond_ring = two_calls ? 15 : 18, late_once = two_calls ? 10 : 45, late_share = two_calls ? 60 : 100;
         int best = 1, best_cost = 0;
         for (int s = 1; s <= limit; ++s) {
             const int mc = resident(s);
             if (s > 1 && n_tiles > mc) continue;   // more than one wave of clusters: not split (several waves cost far more)
             const int stages = (S + s - 1) / s, late = std::max(0, 2 * n_tiles - mc);
-            int cost = stages * (two_calls ? 25 : 23 + M) + std::max(0, stages - ring) * (two_calls ? 15 : 18);
-            if (late > 0) cost += two_calls ? 30 + 40 * std::min(late, n_tiles) / n_tiles : 45 + 100 * std::min(late, n_tiles) / n_tiles;
+            int cost = stages * per_stage + std::max(0, stages - ring) * beyond_ring;
+            if (late > 0) cost += late_once + late_share * std::min(late, n_tiles) / n_tiles;
             if (s == 1 || cost < best_cost) { best_cost = cost; best = s; }
         }
         return best;
@@ -350,9 +352,15 @@ int decode_splits_for(int n_tiles, int S, int M, DeviceInfo* di) {
     return best;
 }
 
+// developer switch: 0 = the rule
+int forced_decode_splits(int S) {
+    const int forced = env_int("PRQ_DECODE_SPLITS", 0);
+    return forced > 0 ? std::min(forced, std::min(8, S)) : 0;
+}
+
 int decode_splits(const prq_weights* w, int M, DeviceInfo* di) {
-    if (M <= 16 && !dev_knobs_enabled()) return w->splits16[M];
-    return decode_splits_for((w->N + 127) / 128, w->plan.S, M, di);
+    if (const int forced = forced_decode_splits(w->plan.S)) return forced;
+    return M <= 16 ? w->splits16[M] : decode_splits_for((w->N + 127) / 128, w->plan.S, M, true, di);
 }
 
 
@@ -1483,7 +1491,8 @@ prq_status prq_linear_multi(int n, const prq_weights* const* ws, const void* con
         b.lay[i] = DecodeLayer{static_cast<const uint8_t*>(scales_sf[i]), ws[i]->d_sf, y[i], ws[i]->N, ws[i]->w_groups,
                                ldy[i], tiles};
     }
-    b.splits = decode_splits_for(tiles, ws[0]->plan.S, M, di);
+    const int forced = forced_decode_splits(ws[0]->plan.S);
+    b.splits = forced ? forced : decode_splits_for(tiles, ws[0]->plan.S, M, true, di);
     cudaError_t e = launch_decode_batch(bn, maps, b, static_cast<cudaStream_t>(stream));
     g_launches.fetch_add(1);
     return e == cudaSuccess ? PRQ_OK : PRQ_ERR_CUDA;

@@ -33,7 +33,7 @@ std::map<const void*, size_t> g_symbol_bytes;
 std::map<const void*, const char*> g_names;
 int g_launches[2];
 const char* g_last_name = "";
-int g_last_grid = 0;
+int g_last_grid = 0, g_last_cluster = 0;
 unsigned g_fill = 1;
 int g_mallocs, g_frees;   // calls; of null pointers not counted
 int g_fail_in = 0;        // the allocation that fails, counted from the next one (0: none)
@@ -76,6 +76,11 @@ cudaError_t launch(const void* func, dim3 grid, size_t dynamic_smem) {
     g_last_grid = static_cast<int>(grid.x * grid.y * grid.z);
     return cudaSuccess;
 }
+int cluster_of(const cudaLaunchConfig_t* c) {
+    for (unsigned i = 0; i < c->numAttrs; ++i)
+        if (c->attrs[i].id == cudaLaunchAttributeClusterDimension) return static_cast<int>(c->attrs[i].val.clusterDim.x);
+    return 1;
+}
 CUresult encode_tiled() { return CUDA_SUCCESS; }
 thread_local struct { dim3 grid, block; size_t smem; cudaStream_t stream; } t_config;
 }  // namespace
@@ -84,6 +89,7 @@ extern "C" {
 int fake_launches(int device) { return g_launches[device]; }
 const char* fake_last_kernel() { return g_last_name; }   // mangled
 int fake_last_grid() { return g_last_grid; }             // CTAs
+int fake_last_cluster() { return g_last_cluster; }       // CTAs per cluster
 int fake_mallocs() { return g_mallocs; }
 int fake_frees() { return g_frees; }
 void fake_fail_malloc(int nth) { g_fail_in = nth; }
@@ -154,10 +160,13 @@ cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void* f, const cudaLaun
     std::lock_guard<std::mutex> lock(g_mu);
     auto it = g_dynamic_smem.find({t_device, f});
     if (c->dynamicSmemBytes > static_cast<size_t>(it == g_dynamic_smem.end() ? 48 * 1024 : it->second)) return cudaErrorInvalidValue;
-    *n = 74;
+    // what a B200 answers for one CTA and for two per SM
+    static const int two_per_sm[9] = {0, 296, 148, 93, 71, 56, 45, 37, 33};
+    const int size = cluster_of(c);
+    *n = size > 8 ? 0 : 2 * (c->dynamicSmemBytes + 1024) <= 233472 ? two_per_sm[size] : two_per_sm[size] / 2;
     return cudaSuccess;
 }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) { return launch(f, c->gridDim, c->dynamicSmemBytes); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) { g_last_cluster = cluster_of(c); return launch(f, c->gridDim, c->dynamicSmemBytes); }
 cudaError_t cudaLaunchKernel(const void* f, dim3 grid, dim3, void**, size_t smem, cudaStream_t) { return launch(f, grid, smem); }
 cudaError_t cudaGetSymbolAddress(void** p, const void* symbol) {
     std::lock_guard<std::mutex> lock(g_mu);

@@ -293,3 +293,44 @@ def _zero_weights(fake, N, K, k=0, gated=False):
     fake._check(fake.lib().prq_prepare_weights_device(W.ctypes.data, 1, N, K, amax.ctypes.data, 0.5, k, ctypes.cast(ctypes.pointer(o), ctypes.c_void_p), None,
                                                       ctypes.byref(h)), "prepare")
     return fake.Weights(h)
+
+
+def _cluster(fake, ws, M, fused=False):
+    """Cluster size of one decode launch over the layers `ws`."""
+    L, p, n = fake.lib(), lambda a: a.ctypes.data, len(ws)
+    some, arr = _aligned(16), ctypes.c_void_p * n    # (nothing is read or written: the kernels do not run)
+    if fused:
+        fake._check(L.prq_linear_fused(ws[0].handle, fake.ACT_IDENTITY, p(some), M, ws[0].K, p(some), ws[0].N, fake.F32, None), "fused")
+    elif n == 1:
+        fake._check(L.prq_linear(ws[0].handle, p(some), p(some), M, p(some), ws[0].N, fake.F32, None, 0, None), "linear")
+    else:
+        fake._check(L.prq_linear_multi(n, arr(*[w.handle.value for w in ws]), arr(*[p(some)] * n), arr(*[p(some)] * n), M, arr(*[p(some)] * n),
+                                       (ctypes.c_int * n)(*[w.N for w in ws]), fake.F32, None), "multi")
+    return L.fake_last_cluster()
+
+
+@pytest.mark.parametrize("want,Ns,K,k,M", [
+    (4, [4096], 2560, 128, 1), (4, [4096], 2560, 128, 16), (6, [2560], 4096, 256, 1), (8, [2560], 9728, 256, 16), (2, [9728], 2560, 256, 1),
+    (3, [9728], 2560, 256, 32), (1, [12288], 1024, 0, 32), (8, [2560], 9728, 256, 17), (1, [19456], 1024, 0, 32), (1, [256], 128, 0, 4),
+    # a quantiser in front of several layers
+    (4, [2560, 2560], 4096, 128, 1), (5, [2560, 2560], 4096, 128, 32), (3, [4096, 1024, 1024], 2560, 128, 16), (2, [4096, 4096], 1024, 64, 16),
+    # a CTA per SM
+    (2, [4096, 1024, 1024], 2560, 128, 64), (2, [256], 256, 32, 128), (8, [512], 2560, 0, 64)])
+def test_which_cluster_size_a_decode_call_takes(fake, want, Ns, K, k, M):
+    ws = [_zero_weights(fake, N, K, k) for N in Ns]
+    assert _cluster(fake, ws, M) == want
+    for w in ws:
+        w.free()
+
+
+@pytest.mark.parametrize("form", ["device", "host", "clone", "offline_copy"])
+@pytest.mark.parametrize("N,K,k", [(256, 256, 32), (2560, 4096, 256), (4096, 2560, 0), (5120, 512, 0)])
+def test_one_launch_and_two_split_alike(fake, form, N, K, k):
+    """prq_linear_fused gives the bits of the two calls: the same cluster size at every token count, whatever the handle's
+    origin."""
+    w = fake.prepare_weights(np.zeros((N, K), np.uint16), np.ones(K, np.float32), 0.5, k) if form == "host" else _zero_weights(fake, N, K, k)
+    c = getattr(w, form)() if form in ("clone", "offline_copy") else w
+    for M in range(1, fake.FUSED_MAX_M + 1):
+        assert _cluster(fake, [c], M) == _cluster(fake, [c], M, fused=True) == _cluster(fake, [w], M), M
+    for h in {c, w}:
+        h.free()
