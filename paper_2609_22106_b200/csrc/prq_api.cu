@@ -290,6 +290,12 @@ void note_use(const prq_weights* w, prq_stream_t stream) {
     if (stream != nullptr && w->legacy_stream_only.load(std::memory_order_relaxed)) w->legacy_stream_only.store(false, std::memory_order_relaxed);
 }
 
+// A product that reads the handle's prepared weights is about to be queued as well (see product_expected).
+void note_product(const prq_weights* w, prq_stream_t stream) {
+    note_use(w, stream);
+    if (w->quantised.load(std::memory_order_relaxed)) w->quantised.store(false, std::memory_order_relaxed);
+}
+
 // Online calls launch on the current device with pointers and tensor maps of the handle's device.
 bool handle_device_is_current(const prq_weights* w) {
     int dev = -1;
@@ -1196,15 +1202,30 @@ size_t prq_act_bytes(int M, int K, int k_tail, int n_groups, prq_buf which) {
     return 0;
 }
 
-// The weights that the decode product behind a quantiser of `n` layers will stream.  From 4 MB on: less than that the product's
-// own CTAs have requested by the time it starts (1024 x 2560, 1.4 MB, 16 / 128 tokens 4.43 / 7.01 without the hint, 4.78 /
-// 7.23 with it); up to 48 MB, a share of L2 that leaves room for what is in use.
+// Whether a quantiser launch for these layers asks in L2 for what follows it: not if the last one for any of them had no product
+// behind it yet, as where rows are quantised alone or ahead -- asking then costs it up to 80 % (27 MB) for nothing.  (Only how long a
+// call takes depends on this, so threads that share a handle need no order.)
+static bool product_expected(int n, const prq_weights* const* ws) {
+    bool yes = true;
+    for (int i = 0; i < n; ++i) yes = yes && !ws[i]->quantised.load(std::memory_order_relaxed);
+    for (int i = 0; yes && i < n; ++i) ws[i]->quantised.store(true, std::memory_order_relaxed);
+    return yes;
+}
+
+// The weights that the decode product behind a quantiser of `n` layers will stream: 5 to 20 MB of them.  Less than that the
+// product's own CTAs have requested by the time it starts (1024 x 2560, 1.4 MB, 16 / 128 tokens 4.43 / 7.01 without the hint, 4.78 / 7.23 with
+// it; two of 4096 x 1024, 4.5 MB, at 32 5.54 / 5.95); more keeps the memory busy longer than the quantiser runs, and its rows wait
+// behind them (two of 9728 x 2560, 27 MB, 1 / 16 / 64 tokens 8.5 / 9.0 / 11.0 -> 9.4 / 10.2 / 11.6; two of 6144 x 2560, 17 MB, 7.46 / 8.13 / 9.51 -> 7.46 /
+// 7.82 / 8.81).  Not for a gated producer, whose product reads other scale bytes in another order.
 static bool weight_hints(int n, const prq_weights* const* ws, int M, WeightHints* hints) {
     if (M > 128) return false;
     auto code_bytes = [&](const prq_weights* w) { return static_cast<size_t>(w->N) * (static_cast<size_t>(w->K) + w->k_tail) / 2; };
     size_t total = 0;
-    for (int i = 0; i < n; ++i) total += code_bytes(ws[i]);
-    if (total < (4u << 20) || total > (48u << 20)) return false;
+    for (int i = 0; i < n; ++i) {
+        if (ws[i]->gated) return false;
+        total += code_bytes(ws[i]);
+    }
+    if (total < (5u << 20) || total > (20u << 20)) return false;
     *hints = {};
     for (int i = 0; i < n; ++i)
         hints->lay[i] = {ws[i]->d_codes, ws[i]->d_sf, static_cast<uint32_t>(code_bytes(ws[i])),
@@ -1252,8 +1273,8 @@ prq_status prq_quantize_act(const prq_weights* w, prq_act_mode mode, const void*
     if (st != PRQ_OK) return st;
     p.status = di->status_ptr;
     WeightHints hints;
-    const bool ask = !expert_offsets && weight_hints(1, &w, M, &hints);
-    cudaError_t e = launch_quant_act(p, mode == PRQ_ACT_SCALE_PERM, p.act_groups, ask ? &hints : nullptr, static_cast<cudaStream_t>(stream));
+    const bool ask = !expert_offsets && product_expected(1, &w), weights = ask && weight_hints(1, &w, M, &hints);
+    cudaError_t e = launch_quant_act(p, mode == PRQ_ACT_SCALE_PERM, p.act_groups, ask, weights ? &hints : nullptr, static_cast<cudaStream_t>(stream));
     g_launches.fetch_add(1);
     return e == cudaSuccess ? PRQ_OK : PRQ_ERR_CUDA;
 }
@@ -1289,8 +1310,8 @@ prq_status prq_quantize_act_multi(int n, const prq_weights* const* ws, prq_act_m
     if (st != PRQ_OK) return st;
     b.status = di->status_ptr;
     WeightHints hints;
-    const bool ask = weight_hints(n, ws, M, &hints);
-    cudaError_t e = launch_quant_act_batch(b, mode == PRQ_ACT_SCALE_PERM, ask ? &hints : nullptr, static_cast<cudaStream_t>(stream));
+    const bool ask = product_expected(n, ws), weights = ask && weight_hints(n, ws, M, &hints);
+    cudaError_t e = launch_quant_act_batch(b, mode == PRQ_ACT_SCALE_PERM, ask, weights ? &hints : nullptr, static_cast<cudaStream_t>(stream));
     g_launches.fetch_add(1);
     return e == cudaSuccess ? PRQ_OK : PRQ_ERR_CUDA;
 }
@@ -1340,7 +1361,7 @@ prq_status prq_linear(const prq_weights* w, const void* codes, const void* scale
     if (st != PRQ_OK) return st;
     if (M < 0 || w->n_experts != 1 || !w->maps_ready) return PRQ_ERR_INVALID_ARG;
     if (!handle_device_is_current(w)) return PRQ_ERR_INVALID_ARG;
-    note_use(w, stream);
+    note_product(w, stream);
     DeviceInfo* di;
     st = device_info(w->device, &di);
     if (st != PRQ_OK) return st;
@@ -1470,7 +1491,7 @@ prq_status prq_linear_multi(int n, const prq_weights* const* ws, const void* con
     }
     if (M == 0) return PRQ_OK;
     if (!handle_device_is_current(ws[0])) return PRQ_ERR_INVALID_ARG;
-    for (int i = 0; i < n; ++i) note_use(ws[i], stream);
+    for (int i = 0; i < n; ++i) note_product(ws[i], stream);
     DeviceInfo* di;
     prq_status st = device_info(ws[0]->device, &di);
     if (st != PRQ_OK) return st;
@@ -1516,7 +1537,7 @@ prq_status prq_linear_gated(const prq_weights* w, const void* codes, const void*
     if (!aligned16(codes) || !aligned16(scales_sf) || !aligned16(out_codes) || !aligned16(out_scales_sf) || !aligned16(h_check))
         return PRQ_ERR_ALIGNMENT;
     if (!handle_device_is_current(w)) return PRQ_ERR_INVALID_ARG;
-    note_use(w, stream);
+    note_product(w, stream);
     DeviceInfo* di;
     prq_status st = device_info(w->device, &di);
     if (st != PRQ_OK) return st;
@@ -1561,7 +1582,7 @@ prq_status prq_linear_fused(const prq_weights* w, prq_act_mode mode, const void*
     if (y_dtype != PRQ_F32 && y_dtype != PRQ_BF16) return PRQ_ERR_INVALID_ARG;
     if (!aligned16(x) || !aligned16(y) || ldx % 8 || ldy % (y_dtype == PRQ_F32 ? 4 : 8)) return PRQ_ERR_ALIGNMENT;
     if (!handle_device_is_current(w)) return PRQ_ERR_INVALID_ARG;
-    note_use(w, stream);
+    note_product(w, stream);
     DeviceInfo* di;
     prq_status st = device_info(w->device, &di);
     if (st != PRQ_OK) return st;
@@ -1588,7 +1609,7 @@ prq_status prq_linear_grouped(const prq_weights* w, const void* codes, const voi
     if (st != PRQ_OK) return st;
     if (M_total < 0 || !expert_offsets || w->format != PRQ_FMT_MXFP4) return PRQ_ERR_INVALID_ARG;
     if (!handle_device_is_current(w)) return PRQ_ERR_INVALID_ARG;
-    note_use(w, stream);
+    note_product(w, stream);
     DeviceInfo* di;
     st = device_info(w->device, &di);
     if (st != PRQ_OK) return st;

@@ -195,5 +195,6 @@ struct prq_weights {
     uint8_t* d_scales_row = nullptr; // E x N x (K + k)/32 (layers prepared on the device)
     void* arena = nullptr;           // one allocation that holds all of the above (layers prepared on the device)
     mutable std::atomic<bool> legacy_stream_only{true};   // no work on the handle was queued on any other stream
+    mutable std::atomic<bool> quantised{false};   // rows were quantised for the handle since its last product
     size_t arena_bytes = 0;          // its size (a block out of the pool may be larger than what was asked for)
 };

@@ -44,8 +44,8 @@ struct WeightHints {
         uint32_t code_bytes, sf_bytes;
     } lay[kMaxBatch];
 };
-// `ask` may be null: the launch asks for nothing
-cudaError_t launch_quant_act(const QuantParams& p, bool scale_perm, int grid_groups, const WeightHints* ask, cudaStream_t stream);
+// `rows`: in identity mode the launch asks for its rows in L2 too; `weights` may be null
+cudaError_t launch_quant_act(const QuantParams& p, bool scale_perm, int grid_groups, bool rows, const WeightHints* weights, cudaStream_t stream);
 
 struct QuantLayer {                      // what differs per batched layer
     const int32_t* perm;
@@ -70,7 +70,7 @@ struct QuantBatch {
     QuantLayer lay[kMaxBatch];
     int* status;                         // device status word
 };
-cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, const WeightHints* ask, cudaStream_t stream);
+cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, bool rows, const WeightHints* weights, cudaStream_t stream);
 
 struct GemmParams {
     int M;                   // activation rows (all experts)

@@ -49,23 +49,24 @@ __device__ __forceinline__ uint32_t encode8(const float (&v)[8], uint32_t byte) 
 }
 
 // A launch on few rows leaves the memory idle, and the product behind it then waits for its weights: every CTA asks for its
-// share of them (`part` of `parts`) in L2.  Weights depend on no kernel, so this needs no wait.  Quantise + multiply, k = 256, us:
-// 2560 x 9728 at 16 / 64 / 128 tokens 7.16 / 9.20 / 11.35 -> 6.40 / 8.61 / 10.78, 4096 x 2560 5.33 / 7.06 / 8.92 -> 5.18 / 6.84 /
-// 8.11, 9728 x 2560 6.64 / 7.42 / 9.81 -> 6.33 / 6.95 / 9.01.  (Not for stacked experts: 89 MB keep the memory busy longer than the
+// share of them (`part` of `parts`) in L2.  Weights depend on no kernel, so this needs no wait.  Quantise + multiply, us:
+// 2560 x 9728, k = 256, at 16 / 64 / 128 tokens 7.13 / 9.21 / 11.33 -> 6.39 / 8.51 / 10.72, 4096 x 2560, k = 128, 5.26 / 7.01 / 8.86 -> 5.12 /
+// 6.78 / 7.99, 9728 x 2560, k = 256, 6.57 / 7.75 / 9.81 -> 6.42 / 7.01 / 9.04.  (Not for stacked experts: 89 MB keep the memory busy longer than the
 // quantiser runs, and its rows wait behind them; 64 tokens over 128 experts 27.5 -> 29.9.)
 __device__ __forceinline__ void ask_for(const uint8_t* base, uint32_t bytes, int part, int parts) {
     const uint32_t share = ((bytes + parts - 1) / parts + 127) & ~127u, at = share * part;
     if (at < bytes) prefetch_l2(base + at, min(share, (bytes - at)) & ~15u);
 }
 
-// The hints are parameters of instances of their own (kAsk): 100 bytes more in the parameters of every launch made the quantiser
+// The hints are parameters of instances of their own: 100 bytes more in the parameters of every launch made the quantiser
 // 0.06 - 0.1 us slower alone and up to 4 % at 2048 rows (2560 x 9728 10.7 -> 11.1 us, 256 x 256 at 16 tokens 1.54 -> 1.63).
-template <bool kAsk>
+constexpr int kAskNothing = 0, kAskRows = 1, kAskWeights = 2;   // (the last one: both)
+template <int kAsk>
 struct AskParam {};
 template <>
-struct AskParam<true> : WeightHints {};
+struct AskParam<kAskWeights> : WeightHints {};
 
-template <bool kScalePerm, bool kBatch, bool kAsk>
+template <bool kScalePerm, bool kBatch, int kAsk>
 __global__ void __launch_bounds__(kQuantThreads, kScalePerm ? 3 : 4)
 quant_act_kernel(const QuantBatch b, const AskParam<kAsk> ask) {
     __shared__ __align__(16) uint8_t sf_atom[512];
@@ -131,7 +132,7 @@ quant_act_kernel(const QuantBatch b, const AskParam<kAsk> ask) {
         }
     };
     const bool dense = p.expert_offsets == nullptr;
-    if constexpr (kAsk) {
+    if constexpr (kAsk == kAskWeights) {
         if (threadIdx.x == 0) {
             const int parts = static_cast<int>(gridDim.x * gridDim.z) * b.groups_per_lin;
             const int part = static_cast<int>(blockIdx.x + gridDim.x * (blockIdx.z + gridDim.z * (blockIdx.y - lin * b.groups_per_lin)));
@@ -144,8 +145,8 @@ quant_act_kernel(const QuantBatch b, const AskParam<kAsk> ask) {
     // before this launch (four per SM) thereby read memory while that computes.  A hint only: what an earlier kernel still writes
     // is read behind the wait.  Quantise + multiply, 2560 x 9728, 512 / 2048 (fp32 y) / 2048 / 4096 tokens: 23.4 / 33.2 / 32.3 / 65.5 ->
     // 22.2 / 32.0 / 31.2 / 62.0 us, 9728 x 2560 at 3000: 41.7 -> 41.0.  (Asking for the rows of the CTAs behind them too disturbs the
-    // one-wave GEMM: 33.6 with fp32 y.)
-    if (!kScalePerm && dense) {
+    // one-wave GEMM: 33.6 with fp32 y.)  Alone the quantiser only pays for it, 2 to 7 % (2560 x 9728 at 2048 tokens 7.41 -> 7.70).
+    if (!kScalePerm && kAsk) {
         const int row = group * kGroupRows + (threadIdx.x >> 1), col = atom * kAtomK + (threadIdx.x & 1) * 64;
         if (row < p.M && col < p.K) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.x + static_cast<size_t>(row) * p.ldx + col));
     }
@@ -727,7 +728,7 @@ cudaError_t launch_cols_impl(const QuantBatch& b, int sm_count, cudaStream_t str
 
 }  // namespace
 
-cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, const WeightHints* ask, cudaStream_t stream) {
+cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, bool rows, const WeightHints* weights, cudaStream_t stream) {
     const QuantBatch& p = b;
     const int grid_groups = b.groups_per_lin * b.n_lin;
     cudaLaunchConfig_t cfg = {};
@@ -785,10 +786,10 @@ cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, const W
         if (cols && !grouped) {
             const bool large = b.M >= 1500 && p.K >= 2048;
             if (b.M <= 128 && p.K <= 4096)
-                return ask ? launch_cols_impl<16, 1, false, 192, true>(b, sms, stream, ask) : launch_cols_impl<16, 1, false, 192>(b, sms, stream);
+                return weights ? launch_cols_impl<16, 1, false, 192, true>(b, sms, stream, weights) : launch_cols_impl<16, 1, false, 192>(b, sms, stream);
             if (large && p.K <= 8192) return launch_cols_impl<16, 4, false, 384>(b, sms, stream);
             if (large && fits(2)) return launch_cols_impl<16, 2, false, 640>(b, sms, stream);
-            if (fits(2)) return ask ? launch_cols_impl<16, 2, false, 320, true>(b, sms, stream, ask) : launch_cols_impl<16, 2, false, 320>(b, sms, stream);
+            if (fits(2)) return weights ? launch_cols_impl<16, 2, false, 320, true>(b, sms, stream, weights) : launch_cols_impl<16, 2, false, 320>(b, sms, stream);
         }
     }
     // the tail atoms of the scale + permute mode in shares of 16 rows (128 / 8), see the kernel
@@ -812,19 +813,20 @@ cudaError_t launch_quant_act_batch(const QuantBatch& b, bool scale_perm, const W
     cfg.numAttrs = 1;
     auto launch = [&](auto batch) {
         constexpr bool kBatch = decltype(batch)::value;
-        if (ask) {
-            AskParam<true> asked;
-            static_cast<WeightHints&>(asked) = *ask;
-            return scale_perm ? cudaLaunchKernelEx(&cfg, quant_act_kernel<true, kBatch, true>, bb, asked)
-                              : cudaLaunchKernelEx(&cfg, quant_act_kernel<false, kBatch, true>, bb, asked);
+        if (weights) {
+            AskParam<kAskWeights> asked;
+            static_cast<WeightHints&>(asked) = *weights;
+            return scale_perm ? cudaLaunchKernelEx(&cfg, quant_act_kernel<true, kBatch, kAskWeights>, bb, asked)
+                              : cudaLaunchKernelEx(&cfg, quant_act_kernel<false, kBatch, kAskWeights>, bb, asked);
         }
-        return scale_perm ? cudaLaunchKernelEx(&cfg, quant_act_kernel<true, kBatch, false>, bb, AskParam<false>{})
-                          : cudaLaunchKernelEx(&cfg, quant_act_kernel<false, kBatch, false>, bb, AskParam<false>{});
+        if (scale_perm) return cudaLaunchKernelEx(&cfg, quant_act_kernel<true, kBatch, kAskNothing>, bb, AskParam<kAskNothing>{});
+        return rows ? cudaLaunchKernelEx(&cfg, quant_act_kernel<false, kBatch, kAskRows>, bb, AskParam<kAskRows>{})
+                    : cudaLaunchKernelEx(&cfg, quant_act_kernel<false, kBatch, kAskNothing>, bb, AskParam<kAskNothing>{});
     };
     return b.n_lin > 1 ? launch(std::true_type{}) : launch(std::false_type{});
 }
 
-cudaError_t launch_quant_act(const QuantParams& p, bool scale_perm, int grid_groups, const WeightHints* ask, cudaStream_t stream) {
+cudaError_t launch_quant_act(const QuantParams& p, bool scale_perm, int grid_groups, bool rows, const WeightHints* weights, cudaStream_t stream) {
     QuantBatch b = {};
     b.x = p.x; b.expert_offsets = p.expert_offsets; b.M = p.M; b.ldx = p.ldx; b.K = p.K;
     b.n_experts = p.n_experts; b.act_groups = p.act_groups;
@@ -832,7 +834,7 @@ cudaError_t launch_quant_act(const QuantParams& p, bool scale_perm, int grid_gro
     b.groups_per_lin = grid_groups;
     b.lay[0] = QuantLayer{p.perm, p.inv_s_perm, p.codes, p.scales_row, p.scales_sf, p.k_tail};
     b.status = p.status;
-    return launch_quant_act_batch(b, scale_perm, ask, stream);
+    return launch_quant_act_batch(b, scale_perm, rows, weights, stream);
 }
 
 }  // namespace prq

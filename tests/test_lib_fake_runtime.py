@@ -265,24 +265,49 @@ def test_an_allocation_that_fails_is_tried_again_without_what_is_kept(fake, what
 
 
 def _asks(fake, ws, M, mode):
-    """One quantiser launch for the layers `ws`; whether it is an instance that takes hints (its last template argument)."""
+    """One quantiser launch for the layers `ws`: what its instance asks for in L2 (its last template argument)."""
     L, p, K, n = fake.lib(), lambda a: a.ctypes.data, ws[0].K, len(ws)
     some, arr = _aligned(16), ctypes.c_void_p * n    # (nothing is read or written: the kernels do not run)
     if n == 1:
         fake._check(L.prq_quantize_act(ws[0].handle, mode, p(some), M, K, None, p(some), None, p(some), None), "quantise")
     else:
         fake._check(L.prq_quantize_act_multi(n, arr(*[w.handle.value for w in ws]), mode, p(some), M, K, arr(*[p(some)] * n), arr(*[p(some)] * n), None), "multi")
-    return re.search(r"quant_act\w*_kernelI\w*?Lb([01])EE", L.fake_last_kernel().decode())[1] == "1"
+    cols, atoms = (re.search(rf"quant_act{kind}_kernelI\w*?L[bi](\d)EE", L.fake_last_kernel().decode()) for kind in ("_cols", ""))
+    return ("nothing", "weights")[int(cols[1])] if cols else ("nothing", "rows", "weights")[int(atoms[1])]
 
 
-@pytest.mark.parametrize("asks,Ns,K,M", [
-    (True, [2560], 4096, 1), (True, [2560], 4096, 128), (False, [2560], 4096, 129), (False, [2560], 4096, 2048), (False, [256], 256, 16), (False, [1024], 2560, 64),
-    (True, [4096, 1024, 1024], 2560, 64), (False, [512, 256], 1024, 64)])
-def test_which_quantisers_ask_for_weights(fake, asks, Ns, K, M):
-    """Everything else takes the instances without hints, whose launches carry no parameters for them."""
-    ws = [_zero_weights(fake, N, K) for N in Ns]
-    for mode in (fake.ACT_IDENTITY, fake.ACT_SCALE_PERM):
-        assert _asks(fake, ws, M, mode) == asks, mode
+@pytest.mark.parametrize("weights,Ns,K,M,gated", [
+    (True, [2560], 4096, 1, False), (True, [2560], 4096, 128, False), (False, [2560], 4096, 129, False), (False, [2560], 4096, 2048, False),
+    (False, [256], 256, 16, False), (False, [1024], 2560, 64, False), (False, [2560], 4064, 64, False), (True, [10240], 4096, 64, False),
+    (False, [10240], 4128, 64, False), (True, [4096, 1024, 1024], 2560, 64, False), (False, [512, 256], 1024, 64, False),
+    (False, [9728, 9728], 2560, 64, False), (False, [2560], 4096, 64, True)])
+def test_what_a_quantiser_asks_for(fake, weights, Ns, K, M, gated):
+    """5 to 20 MB of weights on up to 128 rows, not those of a gated producer; everything else takes the instances without hints, whose
+    launches carry no parameters for them."""
+    for mode, otherwise in ((fake.ACT_IDENTITY, "rows"), (fake.ACT_SCALE_PERM, "nothing")):
+        ws = [_zero_weights(fake, N, K, gated=gated) for N in Ns]
+        assert _asks(fake, ws, M, mode) == ("weights" if weights else otherwise), mode
+        for w in ws:
+            w.free()
+
+
+@pytest.mark.parametrize("several", [False, True])
+def test_a_quantiser_without_a_product_behind_it_asks_once(fake, several):
+    """... and again once a product has been called, in whichever form."""
+    ws = [_zero_weights(fake, N, 2560) for N in ((4096, 1024) if several else (4096,))]
+    asked = lambda mode=fake.ACT_SCALE_PERM: _asks(fake, ws, 16, mode)
+    products = [lambda: _cluster(fake, ws, 16)] + ([] if several else [lambda: _cluster(fake, ws, 16, fused=True)])
+    for product in products:
+        assert asked() == "weights"
+        assert asked() == "nothing" and asked(fake.ACT_IDENTITY) == "nothing"
+        product()
+        assert asked() == "weights"
+        product()
+        product()
+    if several:   # a product with one of the layers is not one with the other
+        assert asked() == "weights"
+        _cluster(fake, ws[:1], 16)
+        assert asked() == "nothing"
     for w in ws:
         w.free()
 
