@@ -373,8 +373,9 @@ prq_status prq_linear_fused(const prq_weights *w, prq_act_mode mode, const void 
 
 /* Several dense layers that read the same activation (q / k / v, gate / up), each with its own prepared
  * weights, served by one launch each of the quantiser and of the GEMM instead of n.  (Not in the paper: it
- * only saves launches; every layer's result is bit-for-bit the one of its own prq_quantize_act /
- * prq_linear calls.)  At decode batch sizes a launch costs as much as the work in it.
+ * only saves launches.)  At decode batch sizes a launch costs as much as the work in it.  Every layer's codes and scale
+ * bytes are bit-for-bit those of its own prq_quantize_act call.  Its y is that of its own prq_linear call up to the order of
+ * the fp32 sums: the launch cuts the reduction into one number of parts, chosen for all of its tiles together.
  *   n          1 .. PRQ_MULTI_MAX layers, all dense, on one device, with the same K
  *   ws         host array of n handles
  * prq_quantize_act_multi: x device, M x K bf16 (row stride ldx); codes[i], scales_sf[i] device out, sized by

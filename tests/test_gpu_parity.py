@@ -562,6 +562,25 @@ def test_multi_layer_launches_match_single_layer_calls(prq, oracle, M):
         w.free()
 
 
+@pytest.mark.parametrize("M", [1, 16, 32, 64])
+def test_multi_layer_launches_of_a_decoder_block(prq, M):
+    """q / k / v of a decoder block in one launch: the quantiser's bytes are those of the single-layer calls; the sums may be
+    grouped otherwise (three parts for 48 tiles, more for eight), which each side's distance to the exact result bounds."""
+    K, k, shapes = 2560, 128, (4096, 1024, 1024)
+    g = torch.Generator(device="cuda").manual_seed(11)
+    x = torch.randn(M, K, generator=g, device="cuda").to(torch.bfloat16)
+    ws = [prq.prepare_weights_device((torch.randn(N, K, generator=g, device="cuda") * 0.02).to(torch.bfloat16), np.ones(K, np.float32), 0.5, k) for N in shapes]
+    acts = prq.quantize_act_multi(ws, x, prq.ACT_SCALE_PERM)
+    ys = prq.linear_multi(ws, acts, M)
+    for w, (codes, sf), y in zip(ws, acts, ys):
+        c1, _, s1 = prq.quantize_act(w, x, prq.ACT_SCALE_PERM)
+        assert torch.equal(codes, c1) and torch.equal(sf, s1)
+        one = prq.linear(w, c1, s1, M).double().cpu().numpy()
+        assert np.abs(y.double().cpu().numpy() - one).max() <= 2 * prq_ref.tolerance(one)
+        w.free()
+    assert prq.last_device_status() == 0
+
+
 @pytest.mark.parametrize("N,K,k,alpha,search", [
     (256, 256, 32, 0.5, False),      # the tiny configuration's shape
     (100, 96, 0, 0.0, False),        # k = 0, alpha = 0: plain MXFP4 of W
@@ -940,3 +959,38 @@ def test_freed_device_memory_serves_the_next_handle(prq, oracle, side_streams):
     w.free()
     prq.release_cached_memory()
     assert torch.cuda.mem_get_info()[0] >= free0 - (4 << 20)
+
+
+def test_a_freed_layer_may_still_be_read(prq):
+    """Products queued on the default stream, their layer freed without a wait, the next one prepared in its memory: stream order
+    keeps them apart.  The memory stays until it is asked back."""
+    N, K, k, M = 2560, 9728, 256, 2048
+    g = torch.Generator(device="cuda").manual_seed(7)
+    Ws = [(torch.randn(N, K, generator=g, device="cuda") * 0.02).to(torch.bfloat16) for _ in range(2)]
+    amax = [np.abs(np.random.RandomState(i).randn(K)).astype(np.float32) + 0.1 for i in range(2)]
+    x = torch.randn(M, K, generator=g, device="cuda").to(torch.bfloat16)
+    out = [torch.empty((M, N), dtype=torch.float32, device="cuda") for _ in range(12)]
+    want, acts, ws = [], [], None
+    for W, a in zip(Ws, amax):
+        w = prq.prepare_weights_device(W, a, 0.5, k)
+        ws = prq.new_workspace(w, M) if ws is None else ws
+        codes, _, sf = prq.quantize_act(w, x, prq.ACT_SCALE_PERM)
+        acts.append((codes, sf))
+        want.append(prq.linear(w, codes, sf, M, workspace=ws))
+        w.free()
+    prq.release_cached_memory()
+    torch.cuda.synchronize()
+    w = prq.prepare_weights_device(Ws[0], amax[0], 0.5, k)
+    free = torch.cuda.mem_get_info()[0]
+    for y in out:
+        prq.linear(w, *acts[0], M, workspace=ws, out=y)
+    w.free()
+    w = prq.prepare_weights_device(Ws[1], amax[1], 0.5, k)
+    assert abs(torch.cuda.mem_get_info()[0] - free) < 4 << 20      # in the same memory
+    assert torch.equal(prq.linear(w, *acts[1], M, workspace=ws), want[1])
+    assert all(torch.equal(y, want[0]) for y in out)
+    free = torch.cuda.mem_get_info()[0]
+    w.free()
+    assert abs(torch.cuda.mem_get_info()[0] - free) < 4 << 20      # kept (the layer takes 16 MB)
+    prq.release_cached_memory()
+    assert torch.cuda.mem_get_info()[0] >= free + (12 << 20)

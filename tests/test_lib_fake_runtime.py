@@ -312,10 +312,10 @@ def test_a_quantiser_without_a_product_behind_it_asks_once(fake, several):
         w.free()
 
 
-def _zero_weights(fake, N, K, k=0, gated=False):
+def _zero_weights(fake, N, K, k=0, gated=False, stream=None):
     W, amax, h = np.zeros((N, K), np.uint16), np.ones(K, np.float32), ctypes.c_void_p()
     o = fake._opts(False, gated)
-    fake._check(fake.lib().prq_prepare_weights_device(W.ctypes.data, 1, N, K, amax.ctypes.data, 0.5, k, ctypes.cast(ctypes.pointer(o), ctypes.c_void_p), None,
+    fake._check(fake.lib().prq_prepare_weights_device(W.ctypes.data, 1, N, K, amax.ctypes.data, 0.5, k, ctypes.cast(ctypes.pointer(o), ctypes.c_void_p), stream,
                                                       ctypes.byref(h)), "prepare")
     return fake.Weights(h)
 
@@ -359,3 +359,91 @@ def test_one_launch_and_two_split_alike(fake, form, N, K, k):
         assert _cluster(fake, [c], M) == _cluster(fake, [c], M, fused=True) == _cluster(fake, [w], M), M
     for h in {c, w}:
         h.free()
+
+
+@pytest.fixture
+def empty_pool(fake):
+    fake.release_cached_memory()
+    yield fake.lib()
+    fake.release_cached_memory()
+
+
+def _allocates(fake, *a, **k):
+    """Whether preparing the layer on the device allocates; frees it again."""
+    before = fake.lib().fake_mallocs()
+    _zero_weights(fake, *a, **k).free()
+    return fake.lib().fake_mallocs() > before
+
+
+def test_a_freed_layers_memory_serves_the_next_one_of_about_its_size(fake, empty_pool):
+    assert _allocates(fake, 6400, 512)
+    assert not _allocates(fake, 6400, 512) and not _allocates(fake, 5120, 512)    # all of the block, four fifths of it
+    assert _allocates(fake, 4160, 512) and _allocates(fake, 12800, 512)           # two thirds, twice as much
+    assert not any(_allocates(fake, N, 512) for N in (4160, 6400, 12800))         # the smallest that is large enough
+    assert empty_pool.cudaSetDevice(1) == 0
+    try:
+        assert _allocates(fake, 6400, 512)                                        # another device's memory
+    finally:
+        empty_pool.cudaSetDevice(0)
+
+
+def test_what_freed_layers_leave_is_bounded(fake, empty_pool):
+    sizes = (64, 320, 1600, 8000, 40000)                       # none serves another one
+    for N in sizes:
+        assert _allocates(fake, N, 128)
+    frees = empty_pool.fake_frees()
+    assert not any(_allocates(fake, N, 128) for N in sizes[1:]) and _allocates(fake, sizes[0], 128)   # four blocks, the oldest went
+    assert empty_pool.fake_frees() == frees + 1                # ... and the next oldest for it
+    fake.release_cached_memory()
+    assert _allocates(fake, 8192, 9728) and _allocates(fake, 13312, 9728)   # 52 and 84 MB: the first one makes room
+    assert _allocates(fake, 8192, 9728)
+    assert _allocates(fake, 17408, 9728) and _allocates(fake, 17408, 9728)  # 106 MB: never kept
+    assert not _allocates(fake, 8192, 9728)
+
+
+def _side_uses(fake):
+    """Every call that queues work on a layer's memory, as (handles, call on a stream)."""
+    L, p, some = fake.lib(), lambda a: a.ctypes.data, _aligned(1 << 16)
+    two, ints = ctypes.c_void_p * 2, ctypes.c_int * 2
+    one = lambda **k: [_zero_weights(fake, 256, 256, **k)]
+    pair = lambda: [_zero_weights(fake, 256, 256) for _ in range(2)]
+    hs = lambda ws: two(*[w.handle.value for w in ws])
+    x = p(some)
+    down = fake.prepare_weights(np.zeros((64, 256), np.uint16), np.ones(256, np.float32), 0.5, 0)   # (memory of its own)
+    return {
+        "quantize": (one, lambda ws, s: L.prq_quantize_act(ws[0].handle, 1, x, 4, 256, None, x, None, x, s)),
+        "quantize_multi": (pair, lambda ws, s: L.prq_quantize_act_multi(2, hs(ws), 1, x, 4, 256, two(x, x), two(x, x), s)),
+        "linear": (one, lambda ws, s: L.prq_linear(ws[0].handle, x, x, 4, x, 256, 0, None, 0, s)),
+        "linear_multi": (pair, lambda ws, s: L.prq_linear_multi(2, hs(ws), two(x, x), two(x, x), 4, two(x, x), ints(256, 256), 0, s)),
+        "fused": (one, lambda ws, s: L.prq_linear_fused(ws[0].handle, 0, x, 4, 256, x, 256, 0, s)),
+        "grouped": (one, lambda ws, s: L.prq_linear_grouped(ws[0].handle, x, x, x, 4, x, 256, 0, s)),
+        "static_scratch": (one, lambda ws, s: L.prq_linear_static_scratch(ws[0].handle, x, x, 200, x, 256, 0, s)),
+        "gated": (lambda: [_zero_weights(fake, 512, 256, gated=True)],
+                  lambda ws, s: L.prq_linear_gated(ws[0].handle, x, x, 4, down.handle, x, None, x, None, s)),
+    }
+
+
+@pytest.mark.parametrize("use", ["quantize", "quantize_multi", "linear", "linear_multi", "fused", "grouped", "static_scratch", "gated", "prepare"])
+def test_memory_that_another_stream_may_read_is_not_kept(fake, empty_pool, use):
+    """A layer that was prepared or used on any stream but the legacy one goes back to the device when it is freed -- its memory is
+    not handed to a preparation that other stream's work is not ordered with -- and no preparation there gets kept memory."""
+    L, stream = empty_pool, ctypes.c_void_p()
+    assert L.cudaStreamCreateWithFlags(ctypes.byref(stream), 1) == 0
+    try:
+        if use == "prepare":
+            assert _allocates(fake, 256, 256) and not _allocates(fake, 256, 256)   # a block is kept
+            frees = L.fake_frees()
+            assert _allocates(fake, 256, 256, stream=stream)
+            assert L.fake_frees() == frees + 1
+            return
+        make, call = _side_uses(fake)[use]
+        for s, kept in ((None, True), (stream, False)):
+            fake.release_cached_memory()
+            ws = make()
+            assert call(ws, s) == 0
+            frees = L.fake_frees()
+            for w in ws:
+                w.free()
+            assert L.fake_frees() == frees + (0 if kept else len(ws)), s
+    finally:
+        L.cudaStreamDestroy(stream)
