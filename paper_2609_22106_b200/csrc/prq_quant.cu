@@ -68,7 +68,7 @@ struct AskParam<kAskWeights> : WeightHints {};
 
 template <bool kScalePerm, bool kBatch, int kAsk>
 __global__ void __launch_bounds__(kQuantThreads, kScalePerm ? 3 : 4)
-quant_act_kernel(const QuantBatch b, const AskParam<kAsk> ask) {
+quant_act_kernel(const QuantBatch b, const __grid_constant__ AskParam<kAsk> ask) {
     __shared__ __align__(16) uint8_t sf_atom[512];
     __shared__ int s_tile_start[kMaxExperts + 1];
 
@@ -376,26 +376,20 @@ struct ColsPlan {
 constexpr int kColsMaxStages = 8;
 constexpr size_t kColsSmem = 220 * 1024;   // shared memory of an SM that the rows in flight may take
 
-// With hints the plan stands in front, so that what every CTA reads first shares two 64-byte lines of parameters (2560 x 9728 at
-// 64 tokens 9.23 -> 8.49 us with the product behind it, 4096 x 2560 7.13 -> 6.78).
-template <bool kAsk>
-struct ColsParam {
-    QuantBatch b;
-    ColsPlan plan;
-};
-template <>
-struct ColsParam<true> {
-    ColsPlan plan;
-    QuantBatch b;
-    WeightHints ask;
-};
+__device__ __forceinline__ const QuantBatch& batch_of(const QuantBatch& b, const ColsPlan&) { return b; }
+__device__ __forceinline__ const QuantBatch& batch_of(const ColsPlan&, const QuantBatch& b) { return b; }
+__device__ __forceinline__ const ColsPlan& plan_of(const QuantBatch&, const ColsPlan& c) { return c; }
+__device__ __forceinline__ const ColsPlan& plan_of(const ColsPlan& c, const QuantBatch&) { return c; }
 
 // kCols: columns per lane, 8 or 16.  kRowsC: rows per slice, 1, 2 or 4.
+// With hints the plan stands in front of the batch, so that what every CTA reads first shares two 64-byte lines of parameters (2560 x
+// 9728 at 64 tokens 9.23 -> 8.49 us with the product behind it, 4096 x 2560 7.13 -> 6.78).
 template <int kCols, int kRowsC, bool kGrouped, int kMaxT, bool kAsk>
 __global__ void __launch_bounds__(kMaxT, 1)
-quant_act_cols_kernel(const __grid_constant__ ColsParam<kAsk> param) {
-    const QuantBatch& b = param.b;
-    const ColsPlan& plan_c = param.plan;
+quant_act_cols_kernel(const std::conditional_t<kAsk, ColsPlan, QuantBatch> first, const std::conditional_t<kAsk, QuantBatch, ColsPlan> second,
+                      const __grid_constant__ AskParam<kAsk ? kAskWeights : kAskNothing> ask) {
+    const QuantBatch& b = batch_of(first, second);
+    const ColsPlan& plan_c = plan_of(first, second);
     constexpr int kPairs = kCols / 2;
     constexpr int kBlkLanes = kBlock / kCols;            // lanes per 32-element block: 4 or 2
     constexpr int kAtomLanes = kAtomK / kCols;           // lanes per scale atom: 16 or 8
@@ -460,8 +454,8 @@ quant_act_cols_kernel(const __grid_constant__ ColsParam<kAsk> param) {
         if constexpr (kAsk) {
             if (loader && lane == 0) {
                 const int part = blockIdx.x + gridDim.x * blockIdx.y, parts = gridDim.x * gridDim.y;
-                ask_for(param.ask.lay[blockIdx.z].codes, param.ask.lay[blockIdx.z].code_bytes, part, parts);
-                ask_for(param.ask.lay[blockIdx.z].sf, param.ask.lay[blockIdx.z].sf_bytes, part, parts);
+                ask_for(ask.lay[blockIdx.z].codes, ask.lay[blockIdx.z].code_bytes, part, parts);
+                ask_for(ask.lay[blockIdx.z].sf, ask.lay[blockIdx.z].sf_bytes, part, parts);
             }
         }
         grid_dependency_wait();
@@ -722,8 +716,13 @@ cudaError_t launch_cols_impl(const QuantBatch& b, int sm_count, cudaStream_t str
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if constexpr (kAsk) return cudaLaunchKernelEx(&cfg, kernel, ColsParam<true>{cp, b, *ask});
-    else return cudaLaunchKernelEx(&cfg, kernel, ColsParam<false>{b, cp});
+    AskParam<kAsk ? kAskWeights : kAskNothing> asked;
+    if constexpr (kAsk) {
+        static_cast<WeightHints&>(asked) = *ask;
+        return cudaLaunchKernelEx(&cfg, kernel, cp, b, asked);
+    } else {
+        return cudaLaunchKernelEx(&cfg, kernel, b, cp, asked);
+    }
 }
 
 }  // namespace
