@@ -276,7 +276,7 @@ size_t prq_act_bytes_for(const prq_weights *w, int M, prq_buf which);
  * one ran out the kernel returns early and PRQ_ERR_TIMEOUT is recorded in the device status word
  * (prq_last_device_status); the output buffers are then incomplete.
  * For the product that normally follows, a dense launch also asks for data in L2: its rows in identity mode, and on up to 128 rows
- * the prepared weights of a layer (of the layers of one launch together) that takes 5 to 20 MB.  Such a launch takes up to 1.5
+ * the prepared weights of a layer (of the layers of one launch together) that takes 4 to 20 MB.  Such a launch takes up to 1.5
  * times as long by itself; where rows are quantised alone or ahead only the first one does: after a quantisation without a product
  * of the same handle behind it the next ones ask for nothing, until a product has been called.
  * M == 0 is a no-op. */

@@ -1212,20 +1212,22 @@ static bool product_expected(int n, const prq_weights* const* ws) {
     return yes;
 }
 
-// The weights that the decode product behind a quantiser of `n` layers will stream: 5 to 20 MB of them.  Less than that the
-// product's own CTAs have requested by the time it starts (1024 x 2560, 1.4 MB, 16 / 128 tokens 4.43 / 7.01 without the hint, 4.78 / 7.23 with
-// it; two of 4096 x 1024, 4.5 MB, at 32 5.54 / 5.95); more keeps the memory busy longer than the quantiser runs, and its rows wait
+// The weights that the decode product behind a quantiser of `n` layers will stream: 5 to 20 MB of them, from 33 tokens on, where a
+// product's CTA fills its SM, 4 to 20.  Less than that the product's own CTAs have requested by the time it starts (1024 x 2560, 1.4 MB,
+// 16 / 128 tokens 4.43 / 7.01 without the hint, 4.78 / 7.23 with it; two of 4096 x 1024, 4.5 MB, at 32 5.54 / 5.95, at 33 / 128 6.57 / 8.97 and
+// 6.42 / 7.98); more keeps the memory busy longer than the quantiser runs, and its rows wait
 // behind them (two of 9728 x 2560, 27 MB, 1 / 16 / 64 tokens 8.5 / 9.0 / 11.0 -> 9.4 / 10.2 / 11.6; two of 6144 x 2560, 17 MB, 7.46 / 8.13 / 9.51 -> 7.46 /
-// 7.82 / 8.81).  Not for a gated producer, whose product reads other scale bytes in another order.
+// 7.82 / 8.81).  Three or four layers on more than 96 rows fill the GPU with their quantiser's CTAs, and lose as well (q / k / v at 112 /
+// 128: 11.04 / 11.56 -> 11.64 / 12.42).  Not for a gated producer, whose product reads other scale bytes in another order.
 static bool weight_hints(int n, const prq_weights* const* ws, int M, WeightHints* hints) {
-    if (M > 128) return false;
+    if (M > 128 || (n > 2 && M > 96)) return false;
     auto code_bytes = [&](const prq_weights* w) { return static_cast<size_t>(w->N) * (static_cast<size_t>(w->K) + w->k_tail) / 2; };
     size_t total = 0;
     for (int i = 0; i < n; ++i) {
         if (ws[i]->gated) return false;
         total += code_bytes(ws[i]);
     }
-    if (total < (5u << 20) || total > (20u << 20)) return false;
+    if (total < ((M > 32 ? 4u : 5u) << 20) || total > (20u << 20)) return false;
     *hints = {};
     for (int i = 0; i < n; ++i)
         hints->lay[i] = {ws[i]->d_codes, ws[i]->d_sf, static_cast<uint32_t>(code_bytes(ws[i])),

@@ -238,7 +238,12 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeBatch b) {
     // small-CTA activation quantiser, whose blocks would squeeze in beside this kernel's CTAs and slow their chain for
     // nothing (they wait for this kernel's result anyway): there the trigger comes once the reduction has been issued
     // (quantise + GEMM step 9.1 -> 8.5 us at 64 tokens, 11.75 -> 11.67 at 128; GEMM-only loops unchanged).
-    if (BN < 64) grid_launch_dependents();
+    // So does a launch of whole reductions that fill the ring more than once (more tiles than clusters of two would find room for):
+    // the loads of the launch after next, which come up with the quantiser, only delay its own; there the trigger comes with the
+    // tokens (two of 9728 x 2560, quantise + multiply, 16 / 32 tokens: 9.12 / 10.23 -> 8.84 / 9.78 us, 19456 x 2560 alone 7.28 / 8.27 ->
+    // 6.17 / 7.37; 19456 x 1024, one ring pass, would lose: 3.62 -> 4.49).
+    const bool late_trigger = BN >= 64 || (!kFused && splits == 1 && n_st > kStages);
+    if (!late_trigger) grid_launch_dependents();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, tmem_slot, 0);
     long long* trace = (ptrace && blockIdx.x < 4) ? ptrace + blockIdx.x * 512 : nullptr;
     if (trace && threadIdx.x == 0) { trace[500] = clock64(); trace[502] = t_entry; trace[503] = t_setup; }
@@ -320,6 +325,7 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeBatch b) {
         // columns take 173 cycles, with one barrier probe per stage 260 - 320).
         int groups = 0, need = p.M + 15;
         if (!kFused) ok = ok && mbar_wait(smem_u32(&bar_t[0]), 0, abort_flag);
+        if (BN < 64 && late_trigger) grid_launch_dependents();
         if (trace && lane == 0) trace[64] = clock64();
 #pragma unroll 1
         for (int it = 0; it < pre && ok; ++it) {

@@ -278,11 +278,11 @@ def _asks(fake, ws, M, mode):
 
 @pytest.mark.parametrize("weights,Ns,K,M,gated", [
     (True, [2560], 4096, 1, False), (True, [2560], 4096, 128, False), (False, [2560], 4096, 129, False), (False, [2560], 4096, 2048, False),
-    (False, [256], 256, 16, False), (False, [1024], 2560, 64, False), (False, [2560], 4064, 64, False), (True, [10240], 4096, 64, False),
-    (False, [10240], 4128, 64, False), (True, [4096, 1024, 1024], 2560, 64, False), (False, [512, 256], 1024, 64, False),
+    (False, [256], 256, 16, False), (False, [1024], 2560, 64, False), (True, [2560], 4064, 64, False), (False, [2560], 4064, 32, False), (False, [2560], 3264, 64, False), (True, [2560], 4128, 32, False), (True, [10240], 4096, 64, False),
+    (False, [10240], 4128, 64, False), (True, [4096, 1024, 1024], 2560, 96, False), (False, [4096, 1024, 1024], 2560, 97, False), (False, [512, 256], 1024, 64, False),
     (False, [9728, 9728], 2560, 64, False), (False, [2560], 4096, 64, True)])
 def test_what_a_quantiser_asks_for(fake, weights, Ns, K, M, gated):
-    """5 to 20 MB of weights on up to 128 rows, not those of a gated producer; everything else takes the instances without hints, whose
+    """5 (from 33 rows on: 4) to 20 MB of weights on up to 128 rows, not those of a gated producer; everything else takes the instances without hints, whose
     launches carry no parameters for them."""
     for mode, otherwise in ((fake.ACT_IDENTITY, "rows"), (fake.ACT_SCALE_PERM, "nothing")):
         ws = [_zero_weights(fake, N, K, gated=gated) for N in Ns]
