@@ -27,7 +27,7 @@
 // its dependency, plus the hand-over to the next kernel.  Everything in it runs once per launch, so what counts is the
 // number of instructions and waits between the dependency and the last store.  What that gave (N = 2560, K = 9728, k = 256,
 // us a launch in a chain, before -> now): one token in one launch 4.53 -> 3.88 (N = 1024, K = 2560: 2.84 -> 2.40), quantise +
-// multiply 16 / 64 / 128 tokens 7.73 / 9.45 / 11.70 -> 7.11 / 9.20 / 11.31:
+// multiply 16 / 64 / 128 tokens 7.73 / 9.45 / 11.70 -> 7.13 / 9.21 / 11.33 (6.4 / 8.5 / 10.7 where the quantiser asks for the weights):
 //   * weight scales copied to tensor memory before the tokens are there; no wait, branch or commit between the stages of
 //     the first ring pass (393 -> 190 cycles per stage);
 //   * a few tokens' stages quantised side by side;
